@@ -141,6 +141,33 @@ struct rpbd_handle {
 
 namespace rpbd {
 
+// Programmatic dependent launch: a kernel launched with launch_pdl may start
+// while its predecessor on the stream is still finishing; it calls pdl_wait()
+// before it touches memory that any earlier kernel writes or reads, and the
+// wait ends when the predecessor has completed and its writes are visible.  The
+// predecessor lets it start early with pdl_trigger().  Every kernel of such a
+// chain waits, so completion stays in stream order.  Hides the ~2 us launch
+// gap between the short kernels of one call; also valid under stream capture.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// (a launch error is left for RPBD_LAUNCH_CHECK, as with <<<>>>)
+template <class... P, class... A>
+inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 int set_error(rpbd_handle* h, int code, const std::string& msg);
 // true the first time it is called for (h's device, key), false afterwards;
 // guards per-device one-time settings such as a kernel's shared-memory limit

@@ -65,7 +65,7 @@ struct SymItem {
     int home;   // home tile index (global, in records)
     int v0;     // first visitor record (multiple of VT)
     int ntile;  // visitor tiles
-    int slot;   // home-partial slot (0: diagonal item)
+    int slot;   // home-partial slot (one-home kernel: 0 is the diagonal item)
     int sys;    // system of a batch (0 for a single system)
 };
 
@@ -82,6 +82,7 @@ struct SymSys {
     int64_t S1;     // first double of the segment sums, divided by 3K
     int T;          // home tiles
     int chunk;      // visitors per off-diagonal item
+    int dslots;     // diagonal items per home tile (visitors of the tile itself, min(chunk, tile) each)
 };
 
 // system of global index x, given ascending starts base(s) (binary search)
@@ -523,6 +524,12 @@ static int run(rpbd_handle* h, int64_t n, const double* r, const In* F, Out* U, 
 // floats) so the 32 lanes' loads of different records hit distinct banks.
 
 constexpr int HT2 = 256;  // home blobs per CTA, two per thread
+// Work items per SM wanted of one launch (a CTA each, 4-8 resident).  Few long
+// items leave SMs idle in the last wave; an item's fixed cost (barriers, first
+// copy, home sums) only shows at one visitor tile per item.  4 -> 32 items per
+// SM: n = 30,720 1,151 -> 1,073 us (k = 1) and 1,542 -> 1,386 us (k = 2),
+// n = 65,535 4,783 -> 4,732 and 6,384 -> 6,114 us; 64: within 0.5% of 32.
+constexpr int64_t SYM2_ITEMS_PER_SM = 32;
 // beyond this many bytes of per-home-tile visitor partials a single system
 // always takes the fixed-point accumulation below
 constexpr double SYM_PARTIAL_LIMIT = 16.0 * (1ull << 30);
@@ -544,16 +551,47 @@ __host__ __device__ __forceinline__ int64_t rec2_off(int64_t i, int c, int len)
     return (i / VT) * VT * len + ((int64_t)c * VT + (i % VT)) * 4;
 }
 
+// Fixed-point accumulation of the packed symmetric kernel (acc == nullptr:
+// per-home-tile partials instead): [3K][records] accumulators, one largest
+// |force| per home tile and one non-finite flag per system.  The tiles' maxima
+// stand in for one maximum per system, so that pack2_kernel can write them
+// without an atomic, and the accumulators be cleared there as well: no memset
+// in front of the launch (a fourth launch cost ~2 us of a ~12 us call).
+struct Fixed2 {
+    unsigned long long* acc;
+    float* bmax;
+    unsigned* flag;
+};
+
+// exponent S of a system's scale 2^S from its T home tiles' maxima, by the
+// whole CTA of NT threads (red: NT / 32 words); *bad: a force is not finite
+template <int NT>
+__device__ __forceinline__ int fixed2_exponent(const float* __restrict__ bmax, int T, int64_t n, double cap, unsigned* red,
+                                               bool* bad)
+{
+    unsigned m = 0u;
+    for (int t = threadIdx.x; t < T; t += NT) m = max(m, __float_as_uint(__ldg(bmax + t)));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) m = max(m, red[w]);
+    *bad = m >= 0x7f800000u;
+    return fixed_exponent(*bad ? 0.0f : __uint_as_float(m), n, cap);
+}
+
 // One thread per record of the launch (all systems, padded to whole home
 // tiles); padding records sit far away with zero force.
 template <int K, class In>
-__global__ void pack2_kernel(int n_sys, const SymSys* __restrict__ sys, int64_t rec_end, int64_t n_tot, int k,
-                             const double* __restrict__ r, const In* __restrict__ F, double a, int wall, double s_min,
+__global__ void __launch_bounds__(HT2) pack2_kernel(int n_sys, const SymSys* __restrict__ sys, int64_t rec_end, int64_t n_tot, int k,
+                             const double* __restrict__ r, const In* __restrict__ F, double a, double ia, int wall,
+                             double s_min,
                              const int* __restrict__ active, float* __restrict__ rec, double* __restrict__ scale,
-                             unsigned* __restrict__ fmax_bits = nullptr)
+                             Fixed2 fx)
 {
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (j >= rec_end) return;
+    pdl_trigger();
+    // one block per home tile (rec_end is a whole number of them)
+    const int64_t j = blockIdx.x * (int64_t)HT2 + threadIdx.x;
     constexpr int NCH = Rec2<K>::NCH, LEN = Rec2<K>::LEN;
     const int sx = n_sys == 1 ? 0 : sys_of(n_sys, j, [&](int m) { return sys[m].B; });
     if (active && !active[sx]) return;  // a converged system of a batch: its records are not read
@@ -567,8 +605,11 @@ __global__ void pack2_kernel(int n_sys, const SymSys* __restrict__ sys, int64_t 
         const double z = r[2 * n_tot + i];
         if (wall) {
             zt = z > a ? z : a;
-            const double t = z / a;
-            s = t >= 1.0 ? 1.0 : (t <= s_min ? s_min : t);
+            s = 1.0;
+            if (z < a) {  // (the FP64 divide is ~40 instructions on a slow pipe: only blobs that overlap the wall)
+                const double t = z / a;
+                s = t >= 1.0 ? 1.0 : (t <= s_min ? s_min : t);
+            }
         } else {
             zt = z;
             s = 1.0;
@@ -578,8 +619,7 @@ __global__ void pack2_kernel(int n_sys, const SymSys* __restrict__ sys, int64_t 
     float v[2 * NCH];
 #pragma unroll
     for (int q = 0; q < 2 * NCH; ++q) v[q] = 0.0f;
-    // lengths in units of a (the packed pair form takes a = 1)
-    const double ia = 1.0 / a;
+    // lengths in units of a (the packed pair form takes a = 1; ia = 1 / a)
     x *= ia;
     y *= ia;
     zt *= ia;
@@ -600,9 +640,20 @@ __global__ void pack2_kernel(int n_sys, const SymSys* __restrict__ sys, int64_t 
 #pragma unroll
     for (int c = 0; c < NCH; ++c)
         *reinterpret_cast<float4*>(rec + rec2_off(j, c, LEN)) = make_float4(v[2 * c], v[2 * c], v[2 * c + 1], v[2 * c + 1]);
-    // largest |force| of the record's system and its non-finite flag (a warp never
-    // straddles two systems: each is padded to whole 256-record home tiles)
-    if (fmax_bits) fixed_force_max(fmax_bits + 2 * sx, fm);
+    if (!fx.acc) return;
+    // clear the record's accumulators, and leave the home tile's largest |force|
+    // (+inf: not finite) for the kernels that need the system's scale
+#pragma unroll
+    for (int q = 0; q < 3 * K; ++q) fx.acc[(int64_t)q * rec_end + j] = 0ull;
+    if (l == 0) fx.flag[sx] = 0u;
+    __shared__ unsigned wmax[HT2 / 32];
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(fm));
+    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x < HT2 / 32) {
+        const unsigned t = __reduce_max_sync((1u << (HT2 / 32)) - 1, wmax[threadIdx.x]);
+        if (threadIdx.x == 0) fx.bmax[blockIdx.x] = __uint_as_float(t);
+    }
 }
 
 // record j of a staged tile -> packed operands (both lanes equal); value m
@@ -676,8 +727,8 @@ __device__ __forceinline__ void pair_apply2(float2 dx, float2 dy, float2 dz, flo
     }
 }
 
-// pair_apply2 summed over the minimum image and its 8 nearest periodic images
-// in x, y (Sec. 4.2); Lx, Ly in units of a
+// pair_apply2, or the same with the block summed over the minimum image and its
+// 8 nearest periodic images in x, y (Sec. 4.2); Lx, Ly in units of a
 template <int K, bool BOTH, bool PER, bool FAR>
 __device__ __forceinline__ void pair_apply2_images(float2 dx, float2 dy, float2 dz, float2 hz, float2 zj,
                                                    const PairConstX2& pc, float Lx, float Ly, const float2* f,
@@ -728,9 +779,8 @@ struct Sym2Var {
 // thread, 64 threads, so each visitor record loaded and each visitor sum
 // handed on serves twice the pairs).  Warp w owns homes [64 HP w, 64 HP (w+1))
 // of the tile; pair p of a thread holds homes 64 HP w + 64 p + lane (.x) and
-// that + 32 (.y).  FAR: the cancellation-free far-field block.  ATOM (one
-// system): the visitor and home sums go into the fixed-point accumulators
-// (partial = [3K][n_pad] 64-bit integers, fmax_bits after them) instead of
+// that + 32 (.y).  FAR: the cancellation-free far-field block.  ATOM: the
+// visitor and home sums go into the fixed-point accumulators (fx) instead of
 // the per-home-tile partials.
 template <int K, bool PER, int UNR, int MINB, bool BATCH, int HP = 1, bool FAR = false, bool ATOM = false>
 __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float* __restrict__ rec,
@@ -739,8 +789,7 @@ __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float*
                                                               const SymSys* __restrict__ sys,
                                                               const int* __restrict__ active, float Lx, float Ly,
                                                               float* __restrict__ partial, int* __restrict__ err_flag,
-                                                              RingTest rt, const unsigned* __restrict__ fmax_bits = nullptr,
-                                                              int64_t acc_stride = 0)
+                                                              RingTest rt, Fixed2 fx, int64_t acc_stride)
 {
     constexpr int NT = HT2 / (2 * HP);  // threads
     constexpr int NW = NT / 32;          // warps
@@ -751,21 +800,18 @@ __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float*
     float* red = reinterpret_cast<float*>(smem_raw + NST * TILE_BYTES);  // [2 buffers][NW warps][VT][3K]
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + NST * TILE_BYTES + 2 * NW * VT * 3 * K * sizeof(float));
     const SymItem it = items[blockIdx.x];
+    pdl_wait();  // everything pack2_kernel wrote (the work list above is older)
+    pdl_trigger();
     if constexpr (BATCH)
         if (active && !active[it.sys]) return;  // a converged system: nothing in flight yet
     // a batch's layout is read again where partials are written (cached
     // loads), so none of it stays live in registers through the pair loop
     const SymSys* const sd = sys + it.sys;
-    const bool diag = it.slot == 0;
+    const bool diag = it.v0 / HT2 == it.home;  // visitors of the home tile itself
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t ib = (int64_t)it.home * HT2 + warp * 64 * HP + lane;  // home record of pair 0, lane .x
     const PairConstX2 pc = PairConstX2::make_unit();
     const float2 m1 = pc.m1;
-    // exponent S of the fixed-point scale 2^S of this item's system (ATOM)
-    const int fexp = ATOM ? fixed_exponent(__uint_as_float(__ldg(fmax_bits + (BATCH ? 2 * it.sys : 0))),
-                                           BATCH ? __ldg(&sd->n) : n, fixed_cap(PER))
-                          : 0;
-
     if (tid == 0) {
 #pragma unroll
         for (int s = 0; s < NST; ++s) mbar_init(&bar[s], 1);
@@ -777,6 +823,14 @@ __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float*
             mbar_expect_tx(&bar[s], TILE_BYTES);
             tma_load_1d(stage + (size_t)s * VT * LEN, rec + ((size_t)it.v0 + (size_t)s * VT) * LEN, TILE_BYTES, &bar[s]);
         }
+    // exponent S of the fixed-point scale 2^S of this item's system (red is free until the first tile's sums)
+    int fexp = 0;
+    if constexpr (ATOM) {
+        bool badf;
+        fexp = fixed2_exponent<NT>(fx.bmax + (BATCH ? __ldg(&sd->B) / HT2 : 0), BATCH ? __ldg(&sd->T) : n_home_tiles,
+                                   BATCH ? __ldg(&sd->n) : n, fixed_cap(PER), reinterpret_cast<unsigned*>(red), &badf);
+        __syncthreads();  // every thread has read red before the first tile's sums are written there
+    }
     float2 hxh[HP], hyh[HP], hxl[HP], hyl[HP], hz[HP], hf[HP][3 * K];
 #pragma unroll
     for (int p = 0; p < HP; ++p) {
@@ -872,8 +926,7 @@ __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float*
 #pragma unroll
                     for (int w = 1; w < NW; ++w) sum += rb[(w * VT + vl) * 3 * K + q];
                     if constexpr (ATOM)  // one fixed-point accumulator per record and component
-                        fixed_add(reinterpret_cast<unsigned long long*>(partial) + (int64_t)q * acc_stride + sB + vg,
-                                  sum, fexp, const_cast<unsigned*>(fmax_bits) + (BATCH ? 2 * it.sys : 0) + 1);
+                        fixed_add(fx.acc + (int64_t)q * acc_stride + sB + vg, sum, fexp, fx.flag + (BATCH ? it.sys : 0));
                     else
                         part[(hloc * 3 * K + q) * sn_pad + vg] = sum;
                 }
@@ -903,8 +956,8 @@ __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float*
 #pragma unroll
         for (int q = 0; q < 3 * K; ++q) {
             if constexpr (ATOM) {
-                unsigned long long* a64 = reinterpret_cast<unsigned long long*>(partial) + (int64_t)q * acc_stride + sB;
-                unsigned* const flag = const_cast<unsigned*>(fmax_bits) + (BATCH ? 2 * it.sys : 0) + 1;
+                unsigned long long* a64 = fx.acc + (int64_t)q * acc_stride + sB;
+                unsigned* const flag = fx.flag + (BATCH ? it.sys : 0);
                 if (l0 < sn) fixed_add(a64 + l0, acc[p][q].x, fexp, flag);
                 if (l1 < sn) fixed_add(a64 + l1, acc[p][q].y, fexp, flag);
             } else {
@@ -915,27 +968,30 @@ __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float*
     }
 }
 
-// U of a batch from its fixed-point accumulators ([3K][records], then two
-// words per system: largest |force|, non-finite flag): undo the system's 2^S,
-// scale and write; converged systems keep their U.  One thread per (blob,
-// component blockIdx.y).
+// U from the fixed-point accumulators: undo the system's 2^S, scale and write;
+// NaN throughout a system with a non-finite force or contribution; converged
+// systems of a batch keep their U.  One block per home tile and component
+// (blockIdx.y): a block never straddles two systems.
 template <class Out>
-__global__ void finish_fixed_batch_kernel(int n_sys, const SymSys* __restrict__ sys, int64_t n_tot, int k,
-                                          int64_t acc_stride, const int* __restrict__ active,
-                                          const unsigned long long* __restrict__ acc,
-                                          const unsigned* __restrict__ fmax_bits, const double* __restrict__ scale,
-                                          double inv8pieta, Out* __restrict__ U)
+__global__ void __launch_bounds__(HT2) finish2_kernel(int n_sys, const SymSys* __restrict__ sys, int64_t n_tot, int64_t acc_stride,
+                                                      double cap, const int* __restrict__ active, Fixed2 fx,
+                                                      const double* __restrict__ scale, double inv8pieta,
+                                                      Out* __restrict__ U)
 {
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    __shared__ unsigned red[HT2 / 32];
+    pdl_wait();
+    const int64_t j = blockIdx.x * (int64_t)HT2 + threadIdx.x;  // record
     const int q = blockIdx.y;
-    if (g >= n_tot || q >= 3 * k) return;
-    const int sx = sys_of(n_sys, g, [&](int m) { return sys[m].g0; });
-    if (active && !active[sx]) return;
+    const int sx = n_sys == 1 ? 0 : sys_of(n_sys, j, [&](int m) { return sys[m].B; });
+    if (active && !active[sx]) return;  // the whole block: one system
     const SymSys d = sys[sx];
-    const unsigned* fb = fmax_bits + 2 * sx;
-    const int S = fixed_exponent(__uint_as_float(fb[0]), d.n, fixed_cap(false));
-    const double v = fb[1] ? __longlong_as_double(0x7ff8000000000000LL)
-                           : ldexp((double)(long long)acc[(int64_t)q * acc_stride + d.B + (g - d.g0)], -S);
+    bool bad;
+    const int S = fixed2_exponent<HT2>(fx.bmax + d.B / HT2, d.T, d.n, cap, red, &bad);
+    const int64_t l = j - d.B;
+    if (l >= d.n) return;
+    const double v = bad || fx.flag[sx] ? __longlong_as_double(0x7ff8000000000000LL)
+                                        : ldexp((double)(long long)fx.acc[(int64_t)q * acc_stride + j], -S);
+    const int64_t g = d.g0 + l;
     U[(int64_t)q * n_tot + g] = (Out)(scale[g] * inv8pieta * v);
 }
 
@@ -1001,7 +1057,7 @@ __global__ void reduce2_kernel(int n_sys, const SymSys* __restrict__ sys, int64_
     const int h = (int)(l / HT2);
     const int nseg = (h + SEG - 1) / SEG;
     const int64_t vis = d.n_pad - (int64_t)(h + 1) * HT2;  // visitors of tile h
-    const int home_slots = 1 + (int)((vis + d.chunk - 1) / d.chunk);
+    const int home_slots = d.dslots + (int)((vis + d.chunk - 1) / d.chunk);
     const double* sg = segsum + (int64_t)3 * kt * d.S1 + l;
     const float* pt = partial + (int64_t)3 * kt * d.P1 + l;
     double sum = 0.0;
@@ -1049,18 +1105,22 @@ static int get_plan2(rpbd_handle* h, int n_sys, const int64_t* off, Sym2Plan** o
         }
     Sym2Plan* p = new Sym2Plan();
     p->off.assign(off, off + n_sys + 1);
-    // chunk: halved (down to one visitor tile) while the launch would have
-    // fewer than 4 items per SM
+    // chunk: halved (down to one visitor tile) while the launch would have fewer
+    // than SYM2_ITEMS_PER_SM items per SM.  The home tile's own visitors are
+    // split by the same chunk: a thread meets them one after another, and as one
+    // item of 256 they were the whole length of a small launch (n = 1,920,
+    // k = 1: 44 us of the kernel's 45 us).
     auto count = [&](int c) {
         int64_t m = 0;
         for (int s = 0; s < n_sys; ++s) {
             const int64_t np_ = (off[s + 1] - off[s] + HT2 - 1) / HT2 * HT2;
-            for (int64_t H = 0; H < np_ / HT2; ++H) m += 1 + (np_ - (H + 1) * HT2 + c - 1) / c;
+            for (int64_t H = 0; H < np_ / HT2; ++H) m += (HT2 + c - 1) / c + (np_ - (H + 1) * HT2 + c - 1) / c;
         }
         return m;
     };
     int chunk = CHUNK;
-    while (chunk > VT && count(chunk) < 4 * (int64_t)h->sm_count) chunk /= 2;
+    while (chunk > VT && count(chunk) < SYM2_ITEMS_PER_SM * (int64_t)h->sm_count) chunk /= 2;
+    const int dchunk = std::min(chunk, HT2), dslots = HT2 / dchunk;
     std::vector<SymItem> items;
     int64_t B = 0, P1 = 0, S1 = 0;
     for (int s = 0; s < n_sys; ++s) {
@@ -1073,12 +1133,13 @@ static int get_plan2(rpbd_handle* h, int n_sys, const int64_t* off, Sym2Plan** o
         d.chunk = chunk;
         d.P1 = P1;
         d.S1 = S1;
-        const int slots = d.T > 0 ? 1 + (int)((d.n_pad - HT2 + chunk - 1) / chunk) : 0;
+        d.dslots = dslots;
+        const int slots = d.T > 0 ? dslots + (int)((d.n_pad - HT2 + chunk - 1) / chunk) : 0;
         const int nseg = (d.T + SEG - 1) / SEG;
         for (int H = 0; H < d.T; ++H) {
             const int home = (int)(B / HT2) + H;
-            items.push_back(SymItem{home, (int)(B + (int64_t)H * HT2), HT2 / VT, 0, s});
-            int c = 1;
+            int c = 0;
+            for (; c < dslots; ++c) items.push_back(SymItem{home, (int)(B + (int64_t)H * HT2 + c * dchunk), dchunk / VT, c, s});
             for (int64_t v0 = (int64_t)(H + 1) * HT2; v0 < d.n_pad; v0 += chunk, ++c) {
                 const int64_t v1 = std::min<int64_t>(d.n_pad, v0 + chunk);
                 items.push_back(SymItem{home, (int)(B + v0), (int)((v1 - v0) / VT), c, s});
@@ -1125,7 +1186,7 @@ static int run2(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, 
     RPBD_TRY(get_plan2(h, n_sys, off, &pl));
     float* rec;
     double* scale;
-    float* partial;
+    float* partial = nullptr;
     double* segsum = nullptr;
     // fixed-point accumulation, one integer per record and component (memory
     // O(n), deterministic); per-home-tile partials with the fixed-order
@@ -1135,23 +1196,23 @@ static int run2(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, 
                       (n_sys == 1 && (h->far_field ||
                                       (double)pl->part_rows * 3 * K * sizeof(float) > SYM_PARTIAL_LIMIT));
     const int64_t acc_stride = pl->rec_end;
-    unsigned* fmax_bits = nullptr;
+    Fixed2 fx{nullptr, nullptr, nullptr};
     RPBD_TRY(ensure_t(h, b_rec, (size_t)pl->rec_end * LEN, &rec));
     RPBD_TRY(ensure_t(h, b_scale, (size_t)n_tot, &scale));
     if (atom) {
-        // [3K][records] accumulators, then two words per system (largest |force|, non-finite flag)
-        unsigned long long* acc;
-        const size_t words = (size_t)3 * K * acc_stride + (size_t)n_sys;
-        RPBD_TRY(ensure_t(h, b_part, words, &acc));
-        RPBD_CU(h, cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * words, st));
-        partial = reinterpret_cast<float*>(acc);
-        fmax_bits = reinterpret_cast<unsigned*>(acc + 3 * K * acc_stride);
+        // [3K][records] accumulators, one maximum per home tile, one flag per system; pack2_kernel
+        // initialises them
+        const size_t words = (size_t)3 * K * acc_stride, tiles = (size_t)(acc_stride / HT2);
+        RPBD_TRY(ensure_t(h, b_part, words + (tiles + n_sys + 1) / 2, &fx.acc));
+        fx.bmax = reinterpret_cast<float*>(fx.acc + words);
+        fx.flag = reinterpret_cast<unsigned*>(fx.bmax + tiles);
     } else {
         RPBD_TRY(ensure_t(h, b_part, (size_t)pl->part_rows * 3 * K, &partial));
         RPBD_TRY(ensure_t(h, b_seg, (size_t)std::max<int64_t>(1, pl->seg_rows) * 3 * K, &segsum));
     }
-    pack2_kernel<K, In><<<(unsigned)((pl->rec_end + 255) / 256), 256, 0, st>>>(
-        n_sys, pl->d_sys, pl->rec_end, n_tot, k, r, F, h->p.a, h->p.wall, h->p.s_min, active, rec, scale, fmax_bits);
+    const unsigned tiles_ = (unsigned)(pl->rec_end / HT2);
+    pack2_kernel<K, In><<<tiles_, HT2, 0, st>>>(n_sys, pl->d_sys, pl->rec_end, n_tot, k, r, F, h->p.a, 1.0 / h->p.a,
+                                                h->p.wall, h->p.s_min, active, rec, scale, fx);
     count_launch();
     const float Lxa = (float)(h->p.Lx / h->p.a), Lya = (float)(h->p.Ly / h->p.a);  // periodic cell in units of a
     if (h->profile) prof_begin(h, st);
@@ -1162,30 +1223,35 @@ static int run2(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, 
     const int64_t n1 = pl->sys[0].n, np1 = pl->sys[0].n_pad;
     const int T1 = pl->sys[0].T;
     const RingTest rt = ring_test(h);
-    // tuning variants, see Sym2Var; -1: the autotuner's usual pick at 65,535 blobs (k = 1: variant 3,
-    // k = 2: variant 5, k = 3..4: variant 4)
-    const int var = sv >= 0 ? sv : (K == 1 ? 3 : (K == 2 ? 5 : 4));
+    // tuning variants, see Sym2Var; -1: four home blobs per thread (half the visitor loads and
+    // hand-overs per pair) once the launch has more items than it needs, i.e. chunks longer than one
+    // visitor tile (about n > 8,800): k = 1 n = 30,720 1,055 vs 1,071 us, k = 2 1,385 vs 1,468, k = 4
+    // 2,190 vs 2,233.  Below that two per thread, twice the threads for the same pairs: k = 2 n = 3,840
+    // 43.5 vs 46.1 us, k = 4 60.1 vs 68.5; at n = 7,680 equal.  Periodic cell: two per thread, no unroll
+    // (nine images already are a long body; k = 1 n = 15,360 1,920 vs 2,146 us unrolled 4).
+    const int var = sv >= 0 ? sv : (PER ? 1 : (pl->sys[0].chunk > VT ? (K <= 2 ? 5 : 4) : 3));
 #define RPBD_SYM2_LAUNCH(V, FARV, ATOMV)                                                                          \
-    sym2_kernel<K, PER, Sym2Var<K, V, PER>::UNR, Sym2Var<K, V, PER>::MINB, false, Sym2Var<K, V, PER>::HP, FARV, ATOMV> \
-        <<<ni, Sym2Var<K, V, PER>::NT, Sym2Var<K, V, PER>::smem(LEN), st>>>(rec, items, n1, np1, T1, sys, nullptr,     \
-                                                                            Lxa, Lya, partial, h->dev_flag, rt,        \
-                                                                            fmax_bits, acc_stride)
+    launch_pdl(sym2_kernel<K, PER, Sym2Var<K, V, PER>::UNR, Sym2Var<K, V, PER>::MINB, false, Sym2Var<K, V, PER>::HP, FARV, \
+                           ATOMV>,                                                                                    \
+               ni, Sym2Var<K, V, PER>::NT, Sym2Var<K, V, PER>::smem(LEN), st, rec, items, n1, np1, T1, sys,            \
+               (const int*)nullptr, Lxa, Lya, partial, h->dev_flag, rt, fx, acc_stride)
     if (n_sys > 1) {  // batches: four home blobs per thread (variant 5's shape; 3-5% faster than two
                       // on 64 uneven suspensions of 480-22,500 blobs)
         if constexpr (!PER) {
             using V5 = Sym2Var<K, 5>;
             if (atom)
-                sym2_kernel<K, false, V5::UNR, V5::MINB, true, V5::HP, false, true><<<ni, V5::NT, V5::smem(LEN), st>>>(
-                    rec, items, 0, 0, 0, sys, active, Lxa, Lya, partial, h->dev_flag, rt, fmax_bits, acc_stride);
+                launch_pdl(sym2_kernel<K, false, V5::UNR, V5::MINB, true, V5::HP, false, true>, ni, V5::NT, V5::smem(LEN), st,
+                           rec, items, (int64_t)0, (int64_t)0, 0, sys, active, Lxa, Lya, partial, h->dev_flag, rt, fx,
+                           acc_stride);
             else
-                sym2_kernel<K, false, V5::UNR, V5::MINB, true, V5::HP><<<ni, V5::NT, V5::smem(LEN), st>>>(
-                    rec, items, 0, 0, 0, sys, active, Lxa, Lya, partial, h->dev_flag, rt);
+                launch_pdl(sym2_kernel<K, false, V5::UNR, V5::MINB, true, V5::HP>, ni, V5::NT, V5::smem(LEN), st, rec, items,
+                           (int64_t)0, (int64_t)0, 0, sys, active, Lxa, Lya, partial, h->dev_flag, rt, fx, acc_stride);
         } else
             return set_error(h, RPBD_BAD_ARG, "packed symmetric kernel: batches are open in x, y");
     } else if (h->far_field) {  // the cancellation-free block: one compiled variant per k
-        RPBD_SYM2_LAUNCH(K == 1 ? 3 : (K == 2 || !PER ? 5 : 3), true, true);  // (k > 2 periodic: no spill)
+        RPBD_SYM2_LAUNCH(PER ? 1 : (K == 1 ? 3 : 5), true, true);
     } else if (!atom) {  // per-home-tile partials and the fixed-order reduction: the default variant
-        RPBD_SYM2_LAUNCH(K == 1 ? 3 : (K == 2 ? 5 : 4), false, false);
+        RPBD_SYM2_LAUNCH(PER ? 1 : (K == 1 ? 3 : (K == 2 ? 5 : 4)), false, false);
     } else {
         switch (var) {
         case 1: RPBD_SYM2_LAUNCH(1, false, true); break;
@@ -1206,14 +1272,8 @@ static int run2(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, 
     // blocks were formed in units of a: M = M(a = 1) / a
     const double inv8pieta = 1.0 / (8.0 * 3.14159265358979323846 * h->p.eta * h->p.a);
     if (atom) {
-        const dim3 fgrid((unsigned)((n_tot + 255) / 256), (unsigned)(3 * k));
-        const auto* acc = reinterpret_cast<const unsigned long long*>(partial);
-        if (n_sys == 1)
-            finish_fixed_kernel<Out><<<fgrid, 256, 0, st>>>(n_tot, acc_stride, k, sym::fixed_cap(PER), acc, fmax_bits,
-                                                            scale, inv8pieta, U);
-        else
-            finish_fixed_batch_kernel<Out><<<fgrid, 256, 0, st>>>(n_sys, sys, n_tot, k, acc_stride, active, acc,
-                                                                  fmax_bits, scale, inv8pieta, U);
+        launch_pdl(finish2_kernel<Out>, dim3(tiles_, (unsigned)(3 * k)), HT2, 0, st, n_sys, sys, n_tot, acc_stride,
+                   fixed_cap(PER), active, fx, (const double*)scale, inv8pieta, U);
         count_launch();
         RPBD_LAUNCH_CHECK(h);
         return RPBD_OK;

@@ -1,0 +1,61 @@
+"""Pair kernels at the edges of their tiles: one blob more or less than a warp,
+a home tile or the size at which the work is cut differently, against the
+oracle (the tolerances of each precision: 1e-5 in FP32, 1e-12 in FP64)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import mobility as om
+from paper_1709_02410_gb300 import Handle, synth
+
+from gpu_util import rel2, to_dev
+
+pytestmark = pytest.mark.gpu
+
+CELL = 45.3
+
+
+def cloud(n, seed, side=None):
+    """n blobs at the boomerang suspensions' density, overlapping pairs and blobs below the wall height a among them."""
+    rng = np.random.default_rng(seed)
+    a = synth.A_BOOMERANG
+    side = 40.0 * np.sqrt(max(n, 60) / 1920) if side is None else side
+    r = np.empty((3, n))
+    r[:2] = rng.uniform(0.0, side, (2, n))
+    r[2] = 0.7 * a + rng.exponential(3.0 * a, n)
+    return r
+
+
+def rows_of(n):
+    """Sampled target blobs: all of a small system, else the tile edges and some between."""
+    if n <= 600:
+        return np.arange(n)
+    e = np.array([0, 31, 32, 63, 64, 127, 128, 255, 256, n - 257, n - 256, n - 33, n - 32, n - 1])
+    return np.unique(np.concatenate([e, np.linspace(0, n - 1, 40).astype(int)]))
+
+
+# 8,704 = 34 home tiles of 256: the last size with one visitor tile per item
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 64, 255, 257, 513, 8704, 8993])
+@pytest.mark.parametrize("cell", [0.0, CELL])
+def test_f32_symmetric_tiles(n, cell):
+    r = cloud(n, 700 + n, cell or None)
+    h = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT, Lx=cell, Ly=cell)
+    prm = om.Params(synth.ETA, synth.A_BOOMERANG, Lx=cell, Ly=cell)
+    rows = rows_of(n)
+    for k in (1, 2, 3):
+        F = synth.gaussian(701 + k, (k, 3, n), np.float32)
+        U = h.mobility_apply(to_dev(r), to_dev(F, torch.float32)).cpu().numpy()
+        assert rel2(U[:, :, rows], om.apply(r, F.astype(np.float64), prm, rows)) <= 1e-5
+
+
+def test_accumulators_are_cleared_between_calls():
+    """One handle, calls of other sizes, right-hand sides and a non-finite force between: every result as on a fresh handle."""
+    h = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT)
+    for n, k, bad in ((700, 2, False), (300, 1, True), (300, 1, False), (1100, 4, False), (40, 1, False), (700, 2, False)):
+        r, F = cloud(n, 710), synth.gaussian(711, (k, 3, n), np.float32)
+        if bad:
+            F[0, 1, 7] = np.inf
+        args = to_dev(r), to_dev(F, torch.float32)
+        U = h.mobility_apply(*args)
+        fresh = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT).mobility_apply(*args)
+        assert torch.isnan(U).all() if bad else torch.equal(U, fresh)
