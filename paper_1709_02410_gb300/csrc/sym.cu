@@ -606,7 +606,8 @@ __global__ void __launch_bounds__(HT2) pack2_kernel(int n_sys, const SymSys* __r
         if (wall) {
             zt = z > a ? z : a;
             s = 1.0;
-            if (z < a) {  // (the FP64 divide is ~40 instructions on a slow pipe: only blobs that overlap the wall)
+            if (!(z >= a)) {  // (the FP64 divide is ~40 instructions on a slow pipe: only where a blob
+                              // overlaps the wall, or is NaN, which stays NaN)
                 const double t = z / a;
                 s = t >= 1.0 ? 1.0 : (t <= s_min ? s_min : t);
             }

@@ -59,3 +59,13 @@ def test_accumulators_are_cleared_between_calls():
         U = h.mobility_apply(*args)
         fresh = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT).mobility_apply(*args)
         assert torch.isnan(U).all() if bad else torch.equal(U, fresh)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_nan_position_gives_nan(dtype):
+    """A NaN coordinate, the height too (clamped, but its overlap scale is NaN), shows in U."""
+    for c in range(3):
+        r, F = cloud(300, 720), synth.gaussian(721, (3, 300))
+        r[c, 40] = np.nan
+        U = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT).mobility_apply(to_dev(r), to_dev(F, dtype))
+        assert torch.isnan(U[:, 40]).all()
