@@ -741,12 +741,21 @@ __device__ __forceinline__ void pair_apply2_images(float2 dx, float2 dy, float2 
         const float iLx = 1.0f / Lx, iLy = 1.0f / Ly;
         dx = make_float2(dx.x - Lx * rintf(dx.x * iLx), dx.y - Lx * rintf(dx.y * iLx));
         dy = make_float2(dy.x - Ly * rintf(dy.x * iLy), dy.y - Ly * rintf(dy.y * iLy));
+        ImageBlock2 M;
+        pair_image_sum_x2<FAR>(dx, dy, dz, hz, zj, Lx, Ly, pc, M);
 #pragma unroll
-        for (int ia = -1; ia <= 1; ++ia)
-#pragma unroll
-            for (int ib = -1; ib <= 1; ++ib)
-                pair_apply2<K, BOTH, FAR>(add2(dx, bc2((float)ia * Lx)), add2(dy, bc2((float)ib * Ly)), dz, hz, zj, pc,
-                                     f, hf, acc, vacc);
+        for (int m = 0; m < K; ++m) {
+            const float2 fx = f[3 * m], fy = f[3 * m + 1], fz = f[3 * m + 2];
+            acc[3 * m + 0] = fma2(M.xz, fz, fma2(M.xy, fy, fma2(M.xx, fx, acc[3 * m + 0])));
+            acc[3 * m + 1] = fma2(M.yz, fz, fma2(M.yy, fy, fma2(M.xy, fx, acc[3 * m + 1])));
+            acc[3 * m + 2] = fma2(M.zz, fz, fma2(M.zy, fy, fma2(M.zx, fx, acc[3 * m + 2])));
+            if constexpr (BOTH) {
+                const float2 gx = hf[3 * m], gy = hf[3 * m + 1], gz = hf[3 * m + 2];
+                vacc[3 * m + 0] = fma2(M.zx, gz, fma2(M.xy, gy, fma2(M.xx, gx, vacc[3 * m + 0])));
+                vacc[3 * m + 1] = fma2(M.zy, gz, fma2(M.yy, gy, fma2(M.xy, gx, vacc[3 * m + 1])));
+                vacc[3 * m + 2] = fma2(M.zz, gz, fma2(M.yz, gy, fma2(M.xz, gx, vacc[3 * m + 2])));
+            }
+        }
     }
 }
 
@@ -1229,7 +1238,8 @@ static int run2(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, 
     // visitor tile (about n > 8,800): k = 1 n = 30,720 1,055 vs 1,071 us, k = 2 1,385 vs 1,468, k = 4
     // 2,190 vs 2,233.  Below that two per thread, twice the threads for the same pairs: k = 2 n = 3,840
     // 43.5 vs 46.1 us, k = 4 60.1 vs 68.5; at n = 7,680 equal.  Periodic cell: two per thread, no unroll
-    // (nine images already are a long body; k = 1 n = 15,360 1,920 vs 2,146 us unrolled 4).
+    // (nine images already are a long body; k = 1 n = 15,360 1,561 vs 1,645 us unrolled
+    // 4 and 1,613-1,766 with four per thread, k = 2 1,666 vs 1,782 and 1,784-2,076).
     const int var = sv >= 0 ? sv : (PER ? 1 : (pl->sys[0].chunk > VT ? (K <= 2 ? 5 : 4) : 3));
 #define RPBD_SYM2_LAUNCH(V, FARV, ATOMV)                                                                          \
     launch_pdl(sym2_kernel<K, PER, Sym2Var<K, V, PER>::UNR, Sym2Var<K, V, PER>::MINB, false, Sym2Var<K, V, PER>::HP, FARV, \

@@ -161,4 +161,114 @@ __device__ __forceinline__ void pair_factors_x2(float2 dx, float2 dy, float2 dz,
     Mzz = fma2(v, iZ, fma2(dz, base, alpha));
 }
 
+// Sum of the pair block over the nine images of the pseudo-periodic cell, two
+// pairs per call, applied once.  The images of a pair share its heights, so
+// dz, Rz, zi zj and their products leave the image loop, and the block entries
+// are summed instead of applying every image's block to the forces: with
+//   gx, gz = dz c2v -+ Rz v Pn,   Mzz = alpha + dz^2 c2v + v Z
+// (c2v, Pn, Z as in pair_factors_x2) the sums over images of alpha, c2v, v Z,
+// beta {dx^2, dx dy, dy^2} and {c2v, v Pn} {dx, dy} determine all of them; the
+// dx factors are taken out of the inner loop over the images in y.  ~40 packed
+// operations per image instead of ~60 (block and both applies).
+struct ImageBlock2 {
+    float2 xx, xy, yy, xz, yz, zx, zy, zz;
+};
+
+template <bool FAR>
+__device__ __forceinline__ void pair_image_sum_x2(float2 dx0, float2 dy0, float2 dz, float2 zi, float2 zj, float Lx, float Ly,
+                                                  const PairConstX2& c, ImageBlock2& M)
+{
+    const float2 zero = bc2(0.0f);
+    const float2 Rz = add2(zi, zj), q = mul2(Rz, Rz), dz2 = mul2(dz, dz), u = mul2(zi, zj);
+    const float2 cu1 = fma2(bc2(6.0f), u, bc2(2.0f));           // 6 zi zj + 2
+    const float2 cu2 = fma2(bc2(-2.0f), u, bc2(-2.0f / 3.0f));  // -2 zi zj - 2/3
+    float2 dy[3], dyy[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        dy[b] = add2(dy0, bc2((float)(b - 1) * Ly));
+        dyy[b] = mul2(dy[b], dy[b]);
+    }
+    float2 al = zero, cs = zero, zs = zero, bxx = zero, bxy = zero, byy = zero;
+    float2 cx = zero, cy = zero, px = zero, py = zero;  // sums of c2v d, v Pn d
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float2 dx = add2(dx0, bc2((float)(a - 1) * Lx));
+        const float2 dxx = mul2(dx, dx);
+        float2 rb = zero, rby = zero, rc = zero, rp = zero;  // sums over the images in y
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const float2 rho2 = add2(dxx, dyy[b]);
+            const float2 r2 = add2(rho2, dz2), R2 = add2(rho2, q);
+            const float2 rinv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+            const float2 Rinv = make_float2(rsqrtf(R2.x), rsqrtf(R2.y));
+            const float2 rinv2 = mul2(rinv, rinv), rinv3 = mul2(rinv, rinv2);
+            const float2 w = mul2(Rinv, Rinv), v = mul2(Rinv, w);
+            float2 X1, c2v;  // c1 - 1/R and c2 - 1/R^3
+            if constexpr (FAR) {
+                const float2 rR = mul2(rinv, Rinv);
+                const float2 sR = fma2(r2, rinv, mul2(R2, Rinv));  // r + R
+                const float2 isR = make_float2(rcp_approx(sR.x), rcp_approx(sR.y));
+                const float2 D1 = mul2(mul2(mul2(bc2(4.0f), u), rR), isR);
+                const float2 D3 = mul2(D1, add2(add2(rinv2, w), rR));
+                X1 = fma2(c.a23, rinv3, D1);
+                c2v = fma2(c.m2a2, mul2(rinv3, rinv2), D3);
+                if (r2.x < c.four_a2 || r2.y < c.four_a2) {
+                    if (r2.x < c.four_a2) {
+                        float c1x = 0.0f, c2x = 0.0f;
+                        overlap_fix(r2.x, rinv.x, c, c1x, c2x);
+                        X1.x = c1x - Rinv.x;
+                        c2v.x = c2x - v.x;
+                    }
+                    if (r2.y < c.four_a2) {
+                        float c1y = 0.0f, c2y = 0.0f;
+                        overlap_fix(r2.y, rinv.y, c, c1y, c2y);
+                        X1.y = c1y - Rinv.y;
+                        c2v.y = c2y - v.y;
+                    }
+                }
+            } else {
+                float2 c1 = fma2(c.a23, rinv3, rinv);
+                float2 c2 = mul2(rinv3, fma2(c.m2a2, rinv2, c.one));
+                if (r2.x < c.four_a2 || r2.y < c.four_a2) {
+                    overlap_fix(r2.x, rinv.x, c, c1.x, c2.x);
+                    overlap_fix(r2.y, rinv.y, c, c1.y, c2.y);
+                }
+                X1 = fma2(c.m1, Rinv, c1);
+                c2v = fma2(c.m1, v, c2);
+            }
+            const float2 y = mul2(q, w);  // e_z^2
+            const float2 h1 = fma2(w, fma2(bc2(70.0f / 3.0f), y, bc2(-10.0f / 3.0f)), fma2(bc2(-10.0f), y, cu1));
+            const float2 iA = fma2(w, fma2(bc2(-10.0f / 3.0f), y, c.a23), fma2(bc2(2.0f), y, cu2));
+            const float2 Bp = mul2(w, h1);  // B + 1
+            const float2 tz = fma2(bc2(20.0f), w, fma2(c.m1, h1, bc2(-4.0f)));
+            const float2 iZ = fma2(y, tz, mul2(bc2(-8.0f / 3.0f), w));
+            const float2 vP = mul2(v, fma2(mul2(w, bc2(-20.0f / 3.0f)), w, Bp));  // -v P
+            const float2 be = fma2(v, Bp, c2v);
+            al = add2(al, fma2(v, iA, X1));
+            zs = fma2(v, iZ, zs);
+            rb = add2(rb, be);
+            rby = fma2(be, dy[b], rby);
+            byy = fma2(be, dyy[b], byy);
+            rc = add2(rc, c2v);
+            cy = fma2(c2v, dy[b], cy);
+            rp = add2(rp, vP);
+            py = fma2(vP, dy[b], py);
+        }
+        bxx = fma2(rb, dxx, bxx);
+        bxy = fma2(rby, dx, bxy);
+        cx = fma2(rc, dx, cx);
+        cs = add2(cs, rc);
+        px = fma2(rp, dx, px);
+    }
+    M.xx = add2(al, bxx);
+    M.xy = bxy;
+    M.yy = add2(al, byy);
+    const float2 tx = mul2(dz, cx), ty = mul2(dz, cy), mRz = mul2(c.m1, Rz);
+    M.xz = fma2(mRz, px, tx);
+    M.yz = fma2(mRz, py, ty);
+    M.zx = fma2(Rz, px, tx);
+    M.zy = fma2(Rz, py, ty);
+    M.zz = add2(fma2(dz2, cs, al), zs);
+}
+
 }  // namespace rpbd
