@@ -31,6 +31,7 @@
 #include <vector>
 
 #include "accum.cuh"
+#include "ring.cuh"
 #include "rpbd_internal.cuh"
 #include "wall_rpy.cuh"
 #include "fixed_point.cuh"
@@ -98,42 +99,7 @@ __device__ __forceinline__ int sys_of(int n_sys, int64_t x, F base)
     return lo;
 }
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t c)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(c) : "memory");
-}
-__device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void tma_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(ok)
-                 : "r"(smem_u32(bar)), "r"(parity)
-                 : "memory");
-    return ok != 0;
-}
-// bounded wait: `limit` SM clock cycles at most (default ~2 s); false on timeout
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, long long limit = 4000000000LL)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity))
-        if (clock64() - t0 > limit) return false;
-    return true;
-}
+using namespace ring;
 
 template <int K, class In>
 __global__ void pack_kernel(int64_t n, int64_t n_pad, int k, const double* __restrict__ r, const In* __restrict__ F,
@@ -530,6 +496,9 @@ constexpr int HT2 = 256;  // home blobs per CTA, two per thread
 // SM: n = 30,720 1,151 -> 1,073 us (k = 1) and 1,542 -> 1,386 us (k = 2),
 // n = 65,535 4,783 -> 4,732 and 6,384 -> 6,114 us; 64: within 0.5% of 32.
 constexpr int64_t SYM2_ITEMS_PER_SM = 32;
+// visitors per item at most: 2,048 -> 512 n = 65,535 4,667 -> 4,638 us (k = 1),
+// 6,109 -> 6,082 (k = 2), 9,633 -> 9,656 (k = 4); 128 to 1,024 within 0.5%
+constexpr int CHUNK2 = 512;
 // beyond this many bytes of per-home-tile visitor partials a single system
 // always takes the fixed-point accumulation below
 constexpr double SYM_PARTIAL_LIMIT = 16.0 * (1ull << 30);
@@ -1128,10 +1097,14 @@ static int get_plan2(rpbd_handle* h, int n_sys, const int64_t* off, Sym2Plan** o
         }
         return m;
     };
-    int chunk = CHUNK;
+    int chunk = CHUNK2;
     while (chunk > VT && count(chunk) < SYM2_ITEMS_PER_SM * (int64_t)h->sm_count) chunk /= 2;
     const int dchunk = std::min(chunk, HT2), dslots = HT2 / dchunk;
-    std::vector<SymItem> items;
+    // longest items first so the hardware scheduler fills the tail with short ones: one bucket per length
+    std::vector<std::vector<SymItem>> bucket(std::max(chunk, dchunk) / VT + 1);
+    auto push = [&](int home, int64_t v0, int64_t nv, int slot, int s) {
+        bucket[nv / VT].push_back(SymItem{home, (int)v0, (int)(nv / VT), slot, s});
+    };
     int64_t B = 0, P1 = 0, S1 = 0;
     for (int s = 0; s < n_sys; ++s) {
         SymSys d;
@@ -1149,10 +1122,9 @@ static int get_plan2(rpbd_handle* h, int n_sys, const int64_t* off, Sym2Plan** o
         for (int H = 0; H < d.T; ++H) {
             const int home = (int)(B / HT2) + H;
             int c = 0;
-            for (; c < dslots; ++c) items.push_back(SymItem{home, (int)(B + (int64_t)H * HT2 + c * dchunk), dchunk / VT, c, s});
+            for (; c < dslots; ++c) push(home, B + (int64_t)H * HT2 + c * dchunk, dchunk, c, s);
             for (int64_t v0 = (int64_t)(H + 1) * HT2; v0 < d.n_pad; v0 += chunk, ++c) {
-                const int64_t v1 = std::min<int64_t>(d.n_pad, v0 + chunk);
-                items.push_back(SymItem{home, (int)(B + v0), (int)((v1 - v0) / VT), c, s});
+                push(home, B + v0, std::min<int64_t>(d.n_pad, v0 + chunk) - v0, c, s);
             }
         }
         p->max_nseg = std::max(p->max_nseg, nseg);
@@ -1161,8 +1133,8 @@ static int get_plan2(rpbd_handle* h, int n_sys, const int64_t* off, Sym2Plan** o
         S1 += (int64_t)nseg * d.n_pad;
         p->sys.push_back(d);
     }
-    // longest items first so the hardware scheduler fills the tail with short ones
-    std::stable_sort(items.begin(), items.end(), [](const SymItem& a, const SymItem& b) { return a.ntile > b.ntile; });
+    std::vector<SymItem> items;
+    for (size_t len = bucket.size(); len-- > 0;) items.insert(items.end(), bucket[len].begin(), bucket[len].end());
     p->n_items = (int)items.size();
     p->rec_end = B;
     p->part_rows = P1;
