@@ -563,6 +563,10 @@ int mobility_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* 
     // targets per thread) for k = 1, 3, 4; k = 2 keeps its own K = 2 tile
     if (dtype == RPBD_F32 && h->use_packed && h->p.wall && !(h->p.Lx > 0.0) && k <= 4 && k != 2)
         return single_packed_apply_impl(h, n, r, F, U, k, io_double, st);
+    // FP64: the symmetric kernel; the one-direction kernel for many right-hand
+    // sides and for systems whose partials would not fit
+    if (dtype == RPBD_F64 && sym64_takes(h, n, k))
+        return sym64_apply_impl(h, n, r, (const double*)F, (double*)U, k, st);
     if (io_double || dtype == RPBD_F64)
         return apply_typed<double, double>(h, n, r, (const double*)F, (double*)U, k, dtype, st);
     return apply_typed<float, float>(h, n, r, (const float*)F, (float*)U, k, dtype, st);

@@ -262,6 +262,14 @@ int precond_build_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, co
 int sym_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* F, void* U, int k, bool io_double,
                    cudaStream_t st);
 
+// symmetric FP64 matvec: whether it takes (n, k), and the matvec itself
+bool sym64_takes(const rpbd_handle* h, int64_t n, int k);
+int sym64_apply_impl(rpbd_handle* h, int64_t n, const double* r, const double* F, double* U, int k, cudaStream_t st);
+
+// FP64 gradient of sum_m u_m^T M F_m
+int adjoint64_impl(rpbd_handle* h, int64_t n, const double* r, const double* u, const double* F, int nr, double* grad,
+                   cudaStream_t st);
+
 // batched systems (concatenated SoA; host offsets)
 int batched_apply_impl(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, const void* F, void* U,
                        int k, bool io_double, const int* active, cudaStream_t st);

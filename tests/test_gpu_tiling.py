@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from oracle import mobility as om
-from paper_1709_02410_gb300 import Handle, synth
+from paper_1709_02410_gb300 import F32, F64, Handle, synth
 
 from gpu_util import rel2, to_dev
 
@@ -69,3 +69,33 @@ def test_nan_position_gives_nan(dtype):
         r[c, 40] = np.nan
         U = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT).mobility_apply(to_dev(r), to_dev(F, dtype))
         assert torch.isnan(U[:, 40]).all()
+
+
+# 4,096 / 4,097: one and four warps per CTA
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 65, 255, 1937, 4096, 4097, 4225])
+@pytest.mark.parametrize("wall,cell", [(True, 0.0), (True, CELL), (False, 0.0)])
+def test_f64_symmetric_tiles(n, wall, cell):
+    r = cloud(n, 730 + n, cell or None)
+    h = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT, wall=wall, Lx=cell, Ly=cell)
+    prm = om.Params(synth.ETA, synth.A_BOOMERANG, wall=wall, Lx=cell, Ly=cell)
+    rows = rows_of(n)
+    for k in (1, 2, 3) if n > 600 else (1, 2, 4, 7, 9):
+        F = synth.gaussian(731 + k, (k, 3, n))
+        U = h.mobility_apply(to_dev(r), to_dev(F)).cpu().numpy()
+        assert rel2(U[:, :, rows], om.apply(r, F, prm, rows)) <= 1e-12
+
+
+# FP64: 32 homes a warp, four warps past 4,096; FP32: 64 homes a warp, four warps past 8,192
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 64, 65, 255, 1937, 4097, 8193])
+@pytest.mark.parametrize("wall,cell", [(True, 0.0), (True, CELL), (False, 0.0)])
+def test_adjoint_tiles(n, wall, cell):
+    r = cloud(n, 740 + n, cell or None)
+    h = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT, wall=wall, Lx=cell, Ly=cell)
+    prm = om.Params(synth.ETA, synth.A_BOOMERANG, wall=wall, Lx=cell, Ly=cell)
+    rows = rows_of(n)
+    for k in (1,) if n > 600 else (1, 2, 3, 6):
+        u, F = synth.gaussian(741 + k, (2, k, 3, n))
+        go = sum(om.grad(r, u[m], F[m], prm, rows) for m in range(k))
+        for dtype, tol in ((F64, 1e-11), (F32, 1e-5)):
+            g = h.mobility_adjoint(to_dev(r), to_dev(u), to_dev(F), dtype=dtype).cpu().numpy()
+            assert np.linalg.norm(g[:, rows] - go) <= tol * np.linalg.norm(go)  # (a lone unbounded blob has none)
