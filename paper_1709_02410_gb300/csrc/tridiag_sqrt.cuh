@@ -1,8 +1,25 @@
-// T^{1/2} e_1 for the Lanczos square root (Sec. 2.2): the symmetric
-// tridiagonal T_m (diagonal alpha, off-diagonal beta) is diagonalised by
-// cyclic Jacobi on one warp, T = Q diag(lambda) Q^T, and
-//   c = T^{1/2} e_1 = Q diag(sqrt(max(lambda, 0))) Q^T e_1.
+// T^{1/2} e_1 for the Lanczos square root (Sec. 2.2), T_m symmetric tridiagonal
+// (diagonal alpha, off-diagonal beta), by one warp.
 //
+// Positive definite T (every Lanczos run on an SPD mobility): the contour-
+// integral quadrature of Hale, Higham & Trefethen (SIAM J. Numer. Anal. 46,
+// 2008, method 3 for the square root).  From
+//   T^{1/2} = (2/pi) int_0^inf T (T + t^2)^{-1} dt,  t = sqrt(lo) sc(u | k'),
+// the midpoint rule in u over (0, K') with N nodes converges as
+// exp(-2 pi^2 N / (log(hi/lo) + 3)) for a spectrum in [lo, hi]: N = 32, one node
+// per lane, is below 1e-16 up to hi/lo = 1e6, and 64, two per lane, up to 1e12.
+// Each node is one tridiagonal solve (T + t^2) z = T e_1 (no cancellation), so the
+// chain is ~2 m steps; Jacobi needs 5-6 sweeps of ~m dependent rounds (129 us per
+// call, mean over the iterations of a time step, now 39 us, and 1e-16 instead of
+// 1e-15 off at condition 1e4).  hi is Gershgorin's bound; lo the largest of 32
+// trial shifts hi 2^{-47 j/32} with T - shift positive definite.  The elliptic
+// functions come from the arithmetic-geometric mean and Gauss' transformation
+// (Abramowitz & Stegun 16.12, 17.6), nodes beyond K'/2 from those below by
+// sc(K' - u) = 1 / (k sc(u)).
+//
+// Otherwise (an eigenvalue below ~1e-14 of the largest, or negative) T is
+// diagonalised by cyclic Jacobi, T = Q diag(lambda) Q^T, and
+//   c = T^{1/2} e_1 = Q diag(sqrt(max(lambda, 0))) Q^T e_1.
 // The rotations of one sweep are ordered as a round-robin tournament: in each
 // of the N - 1 rounds (N = m1 rounded up to even) the indices form N/2
 // disjoint pairs, so the round's rotations commute and are applied together
@@ -19,7 +36,119 @@ namespace rpbd {
 constexpr int TRIDIAG_MAX_PAIRS = 48;
 
 // shared memory (doubles) the routine needs for order m1
-__host__ __device__ inline int tridiag_sqrt_smem_doubles(int m1) { return 2 * m1 * m1 + 6 * TRIDIAG_MAX_PAIRS; }
+__host__ __device__ inline int tridiag_sqrt_smem_doubles(int m1)
+{
+    const int jacobi = 2 * m1 * m1 + 6 * TRIDIAG_MAX_PAIRS, quad = 66 * m1;
+    return jacobi > quad ? jacobi : quad;
+}
+
+// the quadrature; false (nothing written) when T is not safely positive definite
+__device__ inline bool tridiag_sqrt_quadrature(int m1, const double* __restrict__ alpha, const double* __restrict__ beta,
+                                               double* sm, double* __restrict__ c)
+{
+    const int lane = threadIdx.x & 31;
+    double* al = sm;            // m1
+    double* be = al + m1;       // m1 (m1 - 1 used)
+    double* dinv = be + m1;     // [m1][32]: 1 / pivot of each lane's node
+    double* y = dinv + 32 * m1; // [m1][32]
+    for (int i = lane; i < m1; i += 32) {
+        al[i] = alpha[i];
+        be[i] = i + 1 < m1 ? beta[i] : 0.0;
+    }
+    __syncwarp();
+    double hi = 0.0;
+    bool fine = true;
+    for (int i = lane; i < m1; i += 32) {
+        const double g = al[i] + fabs(be[i]) + (i ? fabs(be[i - 1]) : 0.0);
+        fine = fine && g > 0.0 && g < 1e300;
+        hi = fmax(hi, g);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    if (!__all_sync(0xffffffffu, fine)) return false;
+    // T - x positive definite? (pivots of L D L^T), lane 0: x = hi 2^-47
+    const double x = hi * exp2(-47.0 / 32.0 * (32 - lane));
+    {
+        double d = al[0] - x;
+        bool pos = d > 0.0;
+        for (int i = 1; i < m1; ++i) {
+            d = al[i] - x - be[i - 1] * be[i - 1] / d;
+            pos = pos && d > 0.0;
+        }
+        const unsigned ok = __ballot_sync(0xffffffffu, pos);
+        if (!(ok & 1u)) return false;
+        hi = __shfl_sync(0xffffffffu, hi, 0);
+        const int best = __popc(ok & ~(ok + 1u)) - 1;  // last of the leading run of lanes
+        const double lo = __shfl_sync(0xffffffffu, x, best);
+        // K' and Gauss' transformation for modulus k' (complement k = sqrt(lo / hi))
+        const double k = sqrt(lo / hi);
+        double a = 1.0, b = k, km[12];  // km[n]: modulus after n + 1 steps
+        int steps = 0;
+#pragma unroll
+        for (int n = 0; n < 12; ++n) {
+            km[n] = 0.0;
+            if (a - b > 1e-15 * a) {  // (uniform)
+                const double an = 0.5 * (a + b), cn = 0.5 * (a - b);
+                b = sqrt(a * b);
+                a = an;
+                km[n] = cn / an;
+                steps = n + 1;
+            }
+        }
+        const double Kp = 1.5707963267948966 / a;
+        const int N = hi <= 1e6 * lo ? 32 : 64;
+        double ci = 0.0, cj = 0.0, ck = 0.0;  // components lane, lane + 32, lane + 64
+        for (int half = 0; half < N / 32; ++half) {
+            const int j = lane + 32 * half, jj = j < N / 2 ? j : N - 1 - j;
+            double u = (jj + 0.5) * Kp / N, sn, cn, dn = 1.0;
+            sincos(u * a, &sn, &cn);  // a = the mean: u divided by every 1 + km
+#pragma unroll
+            for (int n = 11; n >= 0; --n)
+                if (n < steps) {
+                    const double t = km[n] * sn * sn, rr = 1.0 / (1.0 + t);
+                    cn = cn * dn * rr;
+                    sn = (1.0 + km[n]) * sn * rr;
+                    dn = (1.0 - t) * rr;
+                }
+            double sc = sn / cn, w = dn / (cn * cn);
+            if (j != jj) {
+                w /= k * sc * sc;
+                sc = 1.0 / (k * sc);
+            }
+            w *= 2.0 * Kp * sqrt(lo) / (3.14159265358979323846 * N);
+            const double sig = lo * sc * sc;
+            // (T + sig) z = T e_1
+            double di = 1.0 / (al[0] + sig), yi = al[0];
+            dinv[lane] = di;
+            y[lane] = yi;
+            for (int i = 1; i < m1; ++i) {
+                const double bb = be[i - 1], l = bb * di;
+                di = 1.0 / (al[i] + sig - l * bb);
+                yi = (i == 1 ? bb : 0.0) - l * yi;
+                dinv[i * 32 + lane] = di;
+                y[i * 32 + lane] = yi;
+            }
+            double z = 0.0;
+            for (int i = m1 - 1; i >= 0; --i) {
+                z = (y[i * 32 + lane] - be[i] * z) * dinv[i * 32 + lane];
+                y[i * 32 + lane] = w * z;
+            }
+            __syncwarp();
+            for (int s = 0; s < 32; ++s) {  // (rotated: every lane its own bank)
+                const int q = (lane + s) & 31;
+                if (lane < m1) ci += y[lane * 32 + q];
+                if (lane + 32 < m1) cj += y[(lane + 32) * 32 + q];
+                if (lane + 64 < m1) ck += y[(lane + 64) * 32 + q];
+            }
+            __syncwarp();
+        }
+        if (lane < m1) c[lane] = ci;
+        if (lane + 32 < m1) c[lane + 32] = cj;
+        if (lane + 64 < m1) c[lane + 64] = ck;
+    }
+    __syncwarp();
+    return true;
+}
 
 // One warp (all 32 lanes call it).  sm: tridiag_sqrt_smem_doubles(m1)
 // doubles of shared memory; m1 <= 2 * TRIDIAG_MAX_PAIRS.  On return c[i]
@@ -29,6 +158,7 @@ __device__ inline void tridiag_sqrt_e1(int m1, const double* __restrict__ alpha,
                                        double* sm, double* __restrict__ c)
 {
     const int lane = threadIdx.x & 31;
+    if (tridiag_sqrt_quadrature(m1, alpha, beta, sm, c)) return;
     double* A = sm;                    // m1 x m1, row-major
     double* Q = A + m1 * m1;           // eigenvectors (columns)
     double* rc = Q + m1 * m1;          // per pair: cos, sin, t, apq, app, aqq
