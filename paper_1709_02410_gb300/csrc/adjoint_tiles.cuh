@@ -77,7 +77,7 @@ __device__ __forceinline__ double overlap_scale(double z, double a, double s_min
 
 // adds the rows of blob tile `home` (all threads of the CTA), writes g when complete
 template <class S>
-__device__ void finish_tile(const Cut& c, const Out& o, int home, const S* __restrict__ partial, const double* __restrict__ r,
+__device__ void finish_tile(const Cut& c, const Out& o, int home, const S* partial, const double* r,
                             double a, int wall, double s_min)
 {
     const bool own = home >= c.h0 && home < c.h0 + c.hg;
@@ -115,9 +115,8 @@ __device__ void finish_tile(const Cut& c, const Out& o, int home, const S* __res
 // one visitor tile into shared memory.  FP64: fields x, y, z~, s F, s u of [32]
 // doubles, straight from the caller's arrays; FP32: the packed records.
 template <class V, int K>
-__device__ __forceinline__ void load_tile(const Cut& c, int tile, int nr, const double* __restrict__ r,
-                                          const double* __restrict__ u, const double* __restrict__ F,
-                                          const float4* __restrict__ rec, double a, int wall, double s_min, void* st)
+__device__ __forceinline__ void load_tile(const Cut& c, int tile, int nr, const double* r, const double* u, const double* F,
+                                          const float4* rec, double a, int wall, double s_min, void* st)
 {
     if constexpr (std::is_same<V, double>::value) {
         double* o = static_cast<double*>(st);
@@ -145,11 +144,11 @@ __device__ __forceinline__ void load_tile(const Cut& c, int tile, int nr, const 
 }
 
 template <class V, int K, bool WALL, bool PER, class C>
-__global__ void __launch_bounds__(128) adjoint_kernel(Cut c, int nr, const double* __restrict__ r, const double* __restrict__ u,
-                                                      const double* __restrict__ F, const float4* __restrict__ rec, C k,
+__global__ void __launch_bounds__(128) adjoint_kernel(Cut c, int nr, const double* r, const double* u,
+                                                      const double* F, const float4* rec, C k,
                                                       double a, double s_min, typename Scalar<V>::S Lx,
                                                       typename Scalar<V>::S Ly,
-                                                      typename Scalar<V>::S* __restrict__ partial, Out out)
+                                                      typename Scalar<V>::S* partial, Out out)
 {
     using S = typename Scalar<V>::S;
     constexpr bool D = std::is_same<V, double>::value;

@@ -12,10 +12,12 @@
 //    rotations and the Hessenberg least-squares solve in a device kernel.
 //
 // The host drives the iteration and reads one FP64 scalar per iteration (the
-// residual estimate or the Lanczos change) to decide whether to stop; every
-// arithmetic step runs in the kernels below.
+// residual estimate or the Lanczos change, which the iteration's last kernel
+// writes to pinned host memory) to decide whether to stop; every arithmetic
+// step runs in the kernels below.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "rpbd_internal.cuh"
@@ -71,17 +73,6 @@ __global__ void reduce_partials_kernel(int nblocks, const double* __restrict__ p
     }
 }
 
-// w -= sum_i h[i] V_i
-__global__ void multiaxpy_kernel(int64_t n, const double* __restrict__ V, int64_t ld, int nv,
-                                 const double* __restrict__ h, double* __restrict__ w)
-{
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        double s = w[e];
-        for (int i = 0; i < nv; ++i) s -= h[i] * V[(int64_t)i * ld + e];
-        w[e] = s;
-    }
-}
-
 // out = scale * sum_i y[i] V_i   (scale = *scale_dev when scale_dev != NULL)
 __global__ void lincomb_kernel(int64_t n, const double* __restrict__ V, int64_t ld, int nv,
                                const double* __restrict__ y, double scale, const double* __restrict__ scale_dev,
@@ -111,25 +102,48 @@ __global__ void add_kernel(int64_t n, const double* __restrict__ x, double* __re
         y[e] += x[e];
 }
 
-// saddle operator pieces: lamout -= K U ; Uout = -K^T lam (done with launch_KT then negate)
-__global__ void K_sub_kernel(int64_t nb, int nper, const double* __restrict__ r, const double* __restrict__ q,
-                             const double* __restrict__ U, double* __restrict__ out)
+// Saddle products of up to four processes (blockIdx.y): w = [M lam - K U; -K^T lam]
+// given M lam (Ml, which may be w itself).  One warp per body.
+struct SaddleProd {
+    const double *Ml, *lam, *U;
+    double* w;
+};
+struct SaddleBatch {
+    SaddleProd p[4];
+};
+__global__ void saddle_kernel(int64_t nb, int nper, const double* r, const double* q, SaddleBatch B)
 {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    pdl_wait();
+    pdl_trigger();
+    const int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (b >= nb) return;
+    const SaddleProd P = B.p[blockIdx.y];
+    const int lane = threadIdx.x & 31;
     const int64_t n = nb * nper;
-    if (i >= n) return;
-    const int64_t p = i / nper;
-    const double d0 = r[i] - q[3 * p], d1 = r[n + i] - q[3 * p + 1], d2 = r[2 * n + i] - q[3 * p + 2];
-    const double* u = U + 6 * p;
-    out[i] -= u[0] + (u[4] * d2 - u[5] * d1);
-    out[n + i] -= u[1] + (u[5] * d0 - u[3] * d2);
-    out[2 * n + i] -= u[2] + (u[3] * d1 - u[4] * d0);
-}
-
-__global__ void negate_kernel(int64_t n, double* __restrict__ x)
-{
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-        x[e] = -x[e];
+    const double q0 = q[3 * b], q1 = q[3 * b + 1], q2 = q[3 * b + 2];
+    double u[6], s[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll
+    for (int c = 0; c < 6; ++c) u[c] = P.U[6 * b + c];
+    for (int k = lane; k < nper; k += 32) {
+        const int64_t i = b * nper + k;
+        const double d0 = r[i] - q0, d1 = r[n + i] - q1, d2 = r[2 * n + i] - q2;
+        const double l0 = P.lam[i], l1 = P.lam[n + i], l2 = P.lam[2 * n + i];
+        P.w[i] = P.Ml[i] - (u[0] + (u[4] * d2 - u[5] * d1));
+        P.w[n + i] = P.Ml[n + i] - (u[1] + (u[5] * d0 - u[3] * d2));
+        P.w[2 * n + i] = P.Ml[2 * n + i] - (u[2] + (u[3] * d1 - u[4] * d0));
+        s[0] += l0;
+        s[1] += l1;
+        s[2] += l2;
+        s[3] += d1 * l2 - d2 * l1;
+        s[4] += d2 * l0 - d0 * l2;
+        s[5] += d0 * l1 - d1 * l0;
+    }
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
+        if (lane == 0) P.w[3 * n + 6 * b + c] = -s[c];
+    }
 }
 
 static unsigned vgrid(int64_t n)
@@ -150,82 +164,222 @@ static int multidot(rpbd_handle* h, int64_t n, const double* V, int64_t ld, int 
 }
 
 // ---------------------------------------------------------------------------
-// small GMRES kernels (one thread)
+// Orthogonalisation of w against a Krylov basis V_0..V_{nv-1}: classical
+// Gram-Schmidt twice, the norm, and v_nv = w / |w|, for up to four processes at
+// once (blockIdx.y), in four kernels that start under each other's tail.  As
+// separate dot, reduction, update, add, norm and normalisation launches the step
+// was eleven launches, ~60 us of a ~140 us GMRES iteration at 1,920 blobs whose
+// arithmetic takes ~3 us.  Each block keeps its slice of w in shared memory
+// through an update and the dot products that follow it, and sums the previous
+// kernel's per-block partials itself (the same fixed order in every block).
+struct OrthoProc {
+    const double* V;
+    double *w, *part, *h, *vnext;  // part: ortho_part doubles; h: nv coefficients of both passes
+    int nv;
+    // GMRES: H column, rotations, residual; Lanczos: the tridiagonal's end
+    double *H, *cs, *sn, *g, *sc;
+    double *alpha, *beta, *c, *c_prev;
+    double* host;  // two scalars for the host
+};
+struct OrthoBatch {
+    OrthoProc p[4];
+};
 
-// H column j from hcol[0..j] and hcol[j+1] = |w|^2; rotations; residual estimate
-__global__ void gmres_column_kernel(int j, int mdim, const double* __restrict__ hcol, double* __restrict__ H,
-                                    double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g,
-                                    const double* __restrict__ bnorm, double* __restrict__ res)
+// blocks of w: 128 elements each while that does not fill two blocks per SM of
+// this GPU's 152, at most 4,096 (the slice in shared memory)
+static int ortho_blocks(int64_t len)
 {
-    double* col = H + (int64_t)j * (mdim + 1);
-    for (int i = 0; i <= j; ++i) col[i] = hcol[i];
-    col[j + 1] = sqrt(hcol[j + 1]);
-    for (int i = 0; i < j; ++i) {
-        const double t = cs[i] * col[i] + sn[i] * col[i + 1];
-        col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-        col[i] = t;
+    const int64_t small = (len + 127) / 128;
+    if (small <= 304) return (int)small;
+    return (int)std::max<int64_t>(304, (len + 4095) / 4096);
+}
+static size_t ortho_part(int64_t len, int nv) { return (size_t)ortho_blocks(len) * (2 * nv + 1); }
+
+// h[i] = sum of the blocks' partials of dot i, i < nv (shared memory, all threads)
+__device__ __forceinline__ void ortho_gather(int nv, int nblk, const double* part, double* h)
+{
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < nv; i += blockDim.x >> 5) {
+        double s = 0.0;
+#pragma unroll 4
+        for (int b = lane; b < nblk; b += 32) s += part[(int64_t)i * nblk + b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) h[i] = s;
     }
-    const double den = hypot(col[j], col[j + 1]);
-    if (den > 0.0) {
-        cs[j] = col[j] / den;
-        sn[j] = col[j + 1] / den;
-    } else {
-        cs[j] = 1.0;
-        sn[j] = 0.0;
-    }
-    col[j] = den;
-    col[j + 1] = 0.0;
-    g[j + 1] = -sn[j] * g[j];
-    g[j] = cs[j] * g[j];
-    res[0] = fabs(g[j + 1]) / bnorm[0];
+    __syncthreads();
 }
 
-// y = H(0:k,0:k)^-1 g(0:k), upper triangular back substitution
+// PASS 0: partials of V^T w.  1: w -= V h with h from pass 0's partials, then
+// partials of V^T w.  2: w -= V h with pass 1's, then the partials of |w|^2.
+template <int PASS>
+__global__ void ortho_kernel(int64_t len, int64_t ld, int slice, OrthoBatch B)
+{
+    extern __shared__ double sm[];
+    double* ws = sm;           // slice
+    double* h = sm + slice;    // nv
+    pdl_wait();
+    pdl_trigger();
+    const OrthoProc P = B.p[blockIdx.y];
+    const int nblk = gridDim.x, lane = threadIdx.x & 31;
+    const int64_t e0 = (int64_t)blockIdx.x * slice;
+    const int cnt = (int)max((int64_t)0, min((int64_t)slice, len - e0));
+    const double* V = P.V + e0;
+    double* in = P.part + (PASS == 2 ? (int64_t)P.nv * nblk : 0);
+    double* out = P.part + (PASS == 0 ? 0 : PASS == 1 ? (int64_t)P.nv * nblk : 2 * (int64_t)P.nv * nblk);
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) ws[e] = P.w[e0 + e];
+    if (PASS > 0) {
+        ortho_gather(P.nv, nblk, in, h);
+        if (blockIdx.x == 0)
+            for (int i = threadIdx.x; i < P.nv; i += blockDim.x) P.h[i] = PASS == 1 ? h[i] : P.h[i] + h[i];
+        for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+            double s = ws[e];
+#pragma unroll 8
+            for (int i = 0; i < P.nv; ++i) s -= h[i] * V[(int64_t)i * ld + e];
+            ws[e] = s;
+            P.w[e0 + e] = s;
+        }
+    }
+    __syncthreads();
+    const int nd = PASS == 2 ? 1 : P.nv;
+    for (int i = threadIdx.x >> 5; i < nd; i += blockDim.x >> 5) {
+        const double* v = PASS == 2 ? ws : V + (int64_t)i * ld;
+        double s = 0.0;
+#pragma unroll 8
+        for (int e = lane; e < cnt; e += 32) s += v[e] * ws[e];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) out[(int64_t)i * nblk + blockIdx.x] = s;
+    }
+}
+
+// |w|^2 from the partials of pass 2, in every thread
+__device__ __forceinline__ double ortho_norm2(const OrthoProc& P, int nblk, double* h)
+{
+    ortho_gather(1, nblk, P.part + 2 * (int64_t)P.nv * nblk, h);
+    return h[0];
+}
+
+// v_nv = w / |w| of the block's slice (0 when the norm vanishes)
+__device__ __forceinline__ void ortho_normalize(const OrthoProc& P, int64_t len, int slice, double nrm2)
+{
+    const double nv = sqrt(nrm2), inv = nv > 0.0 ? 1.0 / nv : 0.0;
+    const int64_t e0 = (int64_t)blockIdx.x * slice;
+    const int cnt = (int)max((int64_t)0, min((int64_t)slice, len - e0));
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) P.vnext[e0 + e] = P.w[e0 + e] * inv;
+}
+
+// GMRES: v_{j+1}, and in one block more H's column j = nv - 1, the rotations and
+// the residual estimate.  sc: [1] |b|, [2] residual estimate
+__global__ void gmres_finish_kernel(int64_t len, int slice, int mdim, OrthoBatch B)
+{
+    extern __shared__ double sm[];  // 3 (mdim + 2)
+    pdl_wait();
+    pdl_trigger();
+    const OrthoProc P = B.p[blockIdx.y];
+    const int nblk = gridDim.x - 1, j = P.nv - 1;
+    const double nrm2 = ortho_norm2(P, nblk, sm);
+    if ((int)blockIdx.x < nblk) {
+        ortho_normalize(P, len, slice, nrm2);
+        return;
+    }
+    __syncthreads();
+    double *col = sm, *cs = sm + mdim + 2, *sn = cs + mdim + 2;
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+        col[i] = P.h[i];
+        cs[i] = P.cs[i];
+        sn[i] = P.sn[i];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double last = sqrt(nrm2), cur = col[0];  // rotate down the column
+        for (int i = 0; i < j; ++i) {
+            const double nx = col[i + 1];
+            col[i] = cs[i] * cur + sn[i] * nx;
+            cur = -sn[i] * cur + cs[i] * nx;
+        }
+        const double den = hypot(cur, last);
+        const double c = den > 0.0 ? cur / den : 1.0, sv = den > 0.0 ? last / den : 0.0;
+        P.cs[j] = c;
+        P.sn[j] = sv;
+        col[j] = den;
+        const double gj = P.g[j], gn = -sv * gj;
+        P.g[j + 1] = gn;
+        P.g[j] = c * gj;
+        const double res = fabs(gn) / P.sc[1];
+        P.sc[2] = res;
+        P.host[0] = P.sc[1];
+        P.host[1] = res;
+    }
+    __syncthreads();
+    double* H = P.H + (int64_t)j * (mdim + 1);
+    for (int i = threadIdx.x; i <= j + 1; i += blockDim.x) H[i] = i <= j ? col[i] : 0.0;
+}
+
+// y = H(0:k,0:k)^-1 g(0:k), back substitution by columns: one block, the
+// right-hand side in shared memory (k doubles)
 __global__ void gmres_backsolve_kernel(int k, int mdim, const double* __restrict__ H, const double* __restrict__ g,
                                        double* __restrict__ y)
 {
+    extern __shared__ double s[];
+    for (int i = threadIdx.x; i < k; i += blockDim.x) s[i] = g[i];
+    __syncthreads();
     for (int i = k - 1; i >= 0; --i) {
-        double s = g[i];
-        for (int c = i + 1; c < k; ++c) s -= H[(int64_t)c * (mdim + 1) + i] * y[c];
-        const double d = H[(int64_t)i * (mdim + 1) + i];
-        y[i] = d != 0.0 ? s / d : 0.0;
+        const double* col = H + (int64_t)i * (mdim + 1);
+        const double d = col[i];
+        const double v = d != 0.0 ? s[i] / d : 0.0;
+        __syncthreads();
+        for (int c = threadIdx.x; c < i; c += blockDim.x) s[c] -= col[c] * v;
+        if (threadIdx.x == 0) y[i] = v;
+        __syncthreads();
     }
 }
 
-// g = [sqrt(nrm2), 0, ...]; bnorm (when first) = sqrt(nrm2); res = sqrt(nrm2)/bnorm
+// g = [sqrt(nrm2), 0, ...]; bnorm = sc[1] (when first) = sqrt(nrm2); sc[2] = sqrt(nrm2)/bnorm
 __global__ void gmres_start_kernel(int mdim, const double* __restrict__ nrm2, double* __restrict__ g,
-                                   double* __restrict__ bnorm, int first, double* __restrict__ res)
+                                   double* __restrict__ sc, int first, double* __restrict__ host)
 {
     const double b = sqrt(nrm2[0]);
-    for (int i = 0; i <= mdim; ++i) g[i] = 0.0;
-    g[0] = b;
-    if (first) bnorm[0] = b;
-    res[0] = bnorm[0] > 0.0 ? b / bnorm[0] : 0.0;
+    for (int i = threadIdx.x; i <= mdim; i += blockDim.x) g[i] = i == 0 ? b : 0.0;
+    if (threadIdx.x == 0) {
+        const double bn = first ? b : sc[1];
+        sc[1] = bn;
+        sc[2] = bn > 0.0 ? b / bn : 0.0;
+        host[0] = bn;
+        host[1] = sc[2];
+    }
 }
 
 // ---------------------------------------------------------------------------
 // Lanczos small kernels
 
-// alpha/beta bookkeeping: alpha[m] = h[m] (after both passes), beta[m] = |w|
-__global__ void lanczos_coef_kernel(int m, const double* __restrict__ h, const double* __restrict__ nrm2,
-                                    double* __restrict__ alpha, double* __restrict__ beta)
-{
-    alpha[m] = h[m];
-    beta[m] = sqrt(nrm2[0]);
-}
-
-// One warp: c = T^{1/2} e_1 of the (m+1) x (m+1) tridiagonal T
-// (tridiag_sqrt.cuh), change = |c - [c_prev; 0]| / |c|.
-__global__ void lanczos_sqrt_kernel(int m1, const double* __restrict__ alpha, const double* __restrict__ beta,
-                                    double* __restrict__ c, double* __restrict__ c_prev, double* __restrict__ change)
+// v_{m+1}, and in one block more alpha_m = h[m], beta_m = |w|, c = T^{1/2} e_1 of
+// the (m+1) x (m+1) tridiagonal T (tridiag_sqrt.cuh, its shared memory) and the
+// change |c - [c_prev; 0]| / |c|; nv = m + 1.  host: |w|^2, change
+__global__ void lanczos_finish_kernel(int64_t len, int slice, OrthoBatch B)
 {
     extern __shared__ double sm[];
-    const int lane = threadIdx.x;
-    tridiag_sqrt_e1(m1, alpha, beta, sm, c);
+    pdl_wait();
+    pdl_trigger();
+    const OrthoProc P = B.p[blockIdx.y];
+    const int nblk = gridDim.x - 1, m1 = P.nv, lane = threadIdx.x & 31;
+    const double nrm2 = ortho_norm2(P, nblk, sm);
+    if ((int)blockIdx.x < nblk) {
+        ortho_normalize(P, len, slice, nrm2);
+        return;
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    if (lane == 0) {
+        P.alpha[m1 - 1] = P.h[m1 - 1];
+        P.beta[m1 - 1] = sqrt(nrm2);
+    }
+    __syncwarp();
+    tridiag_sqrt_e1(m1, P.alpha, P.beta, sm, P.c);
     double nc = 0.0, nd = 0.0;
     for (int i = lane; i < m1; i += 32) {
-        const double v = c[i];
-        const double prev = i < m1 - 1 ? c_prev[i] : 0.0;
+        const double v = P.c[i];
+        const double prev = i < m1 - 1 ? P.c_prev[i] : 0.0;
         nc += v * v;
         nd += (v - prev) * (v - prev);
     }
@@ -235,8 +389,11 @@ __global__ void lanczos_sqrt_kernel(int m1, const double* __restrict__ alpha, co
         nd += __shfl_xor_sync(0xffffffffu, nd, o);
     }
     __syncwarp();
-    for (int i = lane; i < m1; i += 32) c_prev[i] = c[i];
-    if (lane == 0) change[0] = nc > 0.0 ? sqrt(nd / nc) : 0.0;
+    for (int i = lane; i < m1; i += 32) P.c_prev[i] = P.c[i];
+    if (lane == 0) {
+        P.host[0] = nrm2;
+        P.host[1] = nc > 0.0 ? sqrt(nd / nc) : 0.0;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -262,12 +419,37 @@ struct Small {
     double* y() { return g() + mdim + 1; }                         // mdim + 1
     double* hcol() { return y() + mdim + 1; }                      // mdim + 2
     double* scal() { return hcol() + mdim + 2; }                   // 8 scalars
-    double* partial() { return scal() + 8; }                       // DOT_BLOCKS * (mdim + 2)
-    static size_t count(int mdim)
+    double* partial() { return scal() + 8; }                       // DOT_BLOCKS, or ortho_part(len, mdim)
+    static size_t count(int mdim, int64_t len)
     {
-        return (size_t)(mdim + 1) * mdim + 2 * mdim + 3 * (mdim + 1) + 1 + 8 + (size_t)DOT_BLOCKS * (mdim + 2);
+        return (size_t)(mdim + 1) * mdim + 2 * mdim + 3 * (mdim + 1) + 1 + 8 +
+               std::max<size_t>(DOT_BLOCKS, ortho_part(len, mdim));
     }
 };
+
+// orthogonalises the batch's np processes (the first three kernels; the caller
+// launches the finishing one with the returned grid and slice)
+struct OrthoGrid {
+    int blocks, slice, threads;
+};
+static OrthoGrid launch_ortho(int64_t len, int np, const OrthoBatch& B, cudaStream_t st)
+{
+    OrthoGrid G;
+    G.blocks = ortho_blocks(len);
+    G.slice = (int)((len + G.blocks - 1) / G.blocks);
+    G.threads = G.slice > 512 ? 512 : 256;
+    int nv = 0;
+    for (int a = 0; a < np; ++a) nv = std::max(nv, B.p[a].nv);
+    const dim3 grid((unsigned)G.blocks, (unsigned)np);
+    const size_t smem = (size_t)(G.slice + nv) * sizeof(double);
+    launch_pdl(ortho_kernel<0>, grid, G.threads, smem, st, len, len, G.slice, B);
+    count_launch();
+    launch_pdl(ortho_kernel<1>, grid, G.threads, smem, st, len, len, G.slice, B);
+    count_launch();
+    launch_pdl(ortho_kernel<2>, grid, G.threads, smem, st, len, len, G.slice, B);
+    count_launch();
+    return G;
+}
 
 // ---------------------------------------------------------------------------
 // Lanczos
@@ -300,14 +482,14 @@ int lanczos_multi_impl(rpbd_handle* h, int64_t n, const double* r, int nsys, con
     RPBD_TRY(check_finite(h, 3 * n, r, st));
     const int64_t len = 3 * n;
     const int mdim = LANCZOS_MAX + 1;
-    const size_t small_count = Small::count(mdim) + 4 * (size_t)mdim;
+    const size_t small_count = Small::count(mdim, len) + 4 * (size_t)mdim;
     double *Vall, *vall, *small, *mv = nullptr;
     RPBD_TRY(ensure_t(h, BUF_KRYLOV, (size_t)nsys * (max_iter + 1) * len, &Vall));
     RPBD_TRY(ensure_t(h, BUF_VEC, (size_t)nsys * 3 * len, &vall));
     RPBD_TRY(ensure_t(h, BUF_SMALL, (size_t)nsys * small_count, &small));
     if (nsys > 1) RPBD_TRY(ensure_t(h, BUF_GMRES_MV, (size_t)2 * nsys * len, &mv));
-    if (once_per_device(h, reinterpret_cast<const void*>(lanczos_sqrt_kernel)))
-        RPBD_CU(h, cudaFuncSetAttribute(lanczos_sqrt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (once_per_device(h, reinterpret_cast<const void*>(lanczos_finish_kernel)))
+        RPBD_CU(h, cudaFuncSetAttribute(lanczos_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         tridiag_sqrt_smem_doubles(LANCZOS_MAX + 1) * (int)sizeof(double)));
     RPBD_CU(h, cudaMemsetAsync(h->dev_flag, 0, sizeof(int), st));
     const unsigned g = vgrid(len);
@@ -318,11 +500,12 @@ int lanczos_multi_impl(rpbd_handle* h, int64_t n, const double* r, int nsys, con
         p.W = W[s];
         p.out = out[s];
         p.V = Vall + (int64_t)s * (max_iter + 1) * len;
-        p.z = vall + (int64_t)s * 3 * len;
-        p.y = p.z + len;
-        p.w = p.z + 2 * len;
+        // z and y of all processes lie side by side: a k-RHS matvec takes them as they are
+        p.z = vall + (int64_t)s * len;
+        p.y = vall + (int64_t)(nsys + s) * len;
+        p.w = vall + (int64_t)(2 * nsys + s) * len;
         p.S = Small{small + (int64_t)s * small_count, mdim};
-        p.alpha = p.S.partial() + (size_t)DOT_BLOCKS * (mdim + 2);
+        p.alpha = small + (int64_t)(s + 1) * small_count - 4 * (size_t)mdim;
         p.beta = p.alpha + mdim;
         p.cvec = p.beta + mdim;
         p.cprev = p.cvec + mdim;
@@ -349,41 +532,44 @@ int lanczos_multi_impl(rpbd_handle* h, int64_t n, const double* r, int nsys, con
             if (P[s].active) act[k++] = s;
         if (k == 0) break;
         // w = G v_m for every active process, one k-RHS matvec
+        const bool side = act[k - 1] - act[0] == k - 1;  // their z and y are side by side
         for (int a = 0; a < k; ++a) {
             LanczosProc& p = P[act[a]];
             const double* vm = p.V + (int64_t)p.m * len;
-            double* dst = k == 1 ? p.z : mv + (int64_t)a * len;
+            double* dst = side ? p.z : mv + (int64_t)a * len;
             if (use_precond) RPBD_TRY(precond_apply_impl(h, 2, vm, dst, st));
-            else RPBD_CU(h, cudaMemcpyAsync(dst, vm, sizeof(double) * len, cudaMemcpyDeviceToDevice, st));
+            else if (k > 1) RPBD_CU(h, cudaMemcpyAsync(dst, vm, sizeof(double) * len, cudaMemcpyDeviceToDevice, st));
         }
-        if (k == 1) {
-            LanczosProc& p = P[act[0]];
-            RPBD_TRY(mobility_apply_impl(h, n, r, p.z, p.y, 1, dtype, true, st));
-        } else {
-            RPBD_TRY(mobility_apply_impl(h, n, r, mv, mv + (int64_t)k * len, k, dtype, true, st));
-        }
+        LanczosProc& p0 = P[act[0]];
+        const double* Fm = !use_precond && k == 1 ? p0.V + (int64_t)p0.m * len : side ? p0.z : mv;
+        double* Um = !use_precond && k == 1 ? p0.w : side ? p0.y : mv + (int64_t)k * len;
+        RPBD_TRY(mobility_apply_impl(h, n, r, Fm, Um, k, dtype, true, st));
+        OrthoBatch B = {};
+        int mmax = 0;
         for (int a = 0; a < k; ++a) {
             LanczosProc& p = P[act[a]];
-            const double* my = k == 1 ? p.y : mv + (int64_t)(k + a) * len;
+            const double* my = Um + (int64_t)a * len;
             if (use_precond) RPBD_TRY(precond_apply_impl(h, 1, my, p.w, st));
-            else RPBD_CU(h, cudaMemcpyAsync(p.w, my, sizeof(double) * len, cudaMemcpyDeviceToDevice, st));
+            else if (k > 1) RPBD_CU(h, cudaMemcpyAsync(p.w, my, sizeof(double) * len, cudaMemcpyDeviceToDevice, st));
             ++p.matvecs;
-            // full reorthogonalisation, classical Gram-Schmidt twice
-            const int m = p.m;
-            RPBD_TRY(multidot(h, len, p.V, len, m + 1, p.w, p.S.hcol(), 0, p.S.partial(), st));
-            multiaxpy_kernel<<<g, 256, 0, st>>>(len, p.V, len, m + 1, p.S.hcol(), p.w); count_launch();
-            RPBD_TRY(multidot(h, len, p.V, len, m + 1, p.w, p.S.y(), 0, p.S.partial(), st));
-            multiaxpy_kernel<<<g, 256, 0, st>>>(len, p.V, len, m + 1, p.S.y(), p.w); count_launch();
-            add_kernel<<<1, 128, 0, st>>>(m + 1, p.S.y(), p.S.hcol()); count_launch();
-            RPBD_TRY(multidot(h, len, p.w, 0, 1, p.w, &p.sc[1], 0, p.S.partial(), st));
-            lanczos_coef_kernel<<<1, 1, 0, st>>>(m, p.S.hcol(), &p.sc[1], p.alpha, p.beta); count_launch();
-            const int m1 = m + 1;
-            lanczos_sqrt_kernel<<<1, 32, tridiag_sqrt_smem_doubles(m1) * sizeof(double), st>>>(
-                m1, p.alpha, p.beta, p.cvec, p.cprev, &p.sc[2]);
-            count_launch();
-            normalize_kernel<<<g, 256, 0, st>>>(len, p.w, &p.sc[1], p.V + (int64_t)(m + 1) * len); count_launch();
-            RPBD_CU(h, cudaMemcpyAsync(h->host_small + 2 * a, &p.sc[1], 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
+            OrthoProc& o = B.p[a];
+            o.V = p.V;
+            o.w = p.w;
+            o.part = p.S.partial();
+            o.h = p.S.hcol();
+            o.vnext = p.V + (int64_t)(p.m + 1) * len;
+            o.nv = p.m + 1;
+            o.alpha = p.alpha;
+            o.beta = p.beta;
+            o.c = p.cvec;
+            o.c_prev = p.cprev;
+            o.host = h->host_small + 2 * a;
+            mmax = std::max(mmax, p.m + 1);
         }
+        const OrthoGrid G = launch_ortho(len, k, B, st);
+        launch_pdl(lanczos_finish_kernel, dim3((unsigned)G.blocks + 1, (unsigned)k), 256,
+                   tridiag_sqrt_smem_doubles(mmax) * sizeof(double), st, len, G.slice, B);
+        count_launch();
         RPBD_LAUNCH_CHECK(h);
         RPBD_CU(h, cudaStreamSynchronize(st));
         for (int a = 0; a < k; ++a) {
@@ -437,24 +623,14 @@ int lanczos_impl(rpbd_handle* h, int64_t n, const double* r, const double* W, do
 // number of processes needing one), and reads every process's residual with
 // one host synchronisation per iteration.
 
-// out = [M lam - K U; -K^T lam] given Mlam = M lam already in out[0:3n]
-static void saddle_finish(rpbd_handle* h, int64_t nb, int nper, const double* r, const double* q, const double* x,
-                          double* out, cudaStream_t st)
-{
-    const int64_t n = nb * nper;
-    K_sub_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(nb, nper, r, q, x + 3 * n, out); count_launch();
-    launch_KT(nb, nper, r, q, x, out + 3 * n, st);
-    negate_kernel<<<vgrid(6 * nb), 256, 0, st>>>(6 * nb, out + 3 * n); count_launch();
-}
-
 struct GmresProc {
     GmresProblem pb;
-    double *V, *x, *b, *w, *z, *sc;
+    double *V, *x, *b, *w, *zl, *zU, *sc;
     Small S{nullptr, 0};
     enum Phase { NEED_RESID, NEED_ARNOLDI, READ_START, READ_ITER, DONE } phase = DONE;
     int j = 0, total = 0, matvecs = 0, status = RPBD_NOT_CONVERGED;
     double res = 1.0;
-    const double* req = nullptr;  // vector whose saddle product is wanted
+    const double *req_l = nullptr, *req_U = nullptr;  // vector whose saddle product is wanted
 };
 
 int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, const double* q, int nsys,
@@ -478,7 +654,8 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
     double *Vall, *vall, *small, *mv = nullptr;
     RPBD_TRY(ensure_t(h, BUF_KRYLOV, (size_t)nsys * (mdim + 1) * len, &Vall));
     RPBD_TRY(ensure_t(h, BUF_VEC, (size_t)nsys * 4 * len, &vall));
-    RPBD_TRY(ensure_t(h, BUF_SMALL, (size_t)nsys * Small::count(mdim), &small));
+    const size_t small_count = Small::count(mdim, len);
+    RPBD_TRY(ensure_t(h, BUF_SMALL, (size_t)nsys * small_count, &small));
     if (nsys > 1) RPBD_TRY(ensure_t(h, BUF_GMRES_MV, (size_t)2 * nsys * 3 * n, &mv));
     GmresProc P[4];
     const unsigned g = vgrid(len);
@@ -487,7 +664,8 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
     // r0 = w: |r0|, g, residual estimate, v_0 (first: |b| = |r0|)
     auto begin_cycle = [&](GmresProc& p, int first) -> int {
         RPBD_TRY(multidot(h, len, p.w, 0, 1, p.w, &p.sc[0], 0, p.S.partial(), st));
-        gmres_start_kernel<<<1, 1, 0, st>>>(mdim, &p.sc[0], p.S.g(), &p.sc[1], first, &p.sc[2]); count_launch();
+        gmres_start_kernel<<<1, 64, 0, st>>>(mdim, &p.sc[0], p.S.g(), p.sc, first, h->host_small + 2 * (&p - P));
+        count_launch();
         normalize_kernel<<<g, 256, 0, st>>>(len, p.w, &p.sc[0], p.V); count_launch();
         RPBD_LAUNCH_CHECK(h);
         p.phase = GmresProc::READ_START;
@@ -495,29 +673,32 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
     };
     // x += P^-1 V y over the cycle's jn Arnoldi vectors
     auto end_cycle = [&](GmresProc& p, int jn) -> int {
-        gmres_backsolve_kernel<<<1, 1, 0, st>>>(jn, mdim, p.S.H(), p.S.g(), p.S.y()); count_launch();
+        gmres_backsolve_kernel<<<1, 64, jn * sizeof(double), st>>>(jn, mdim, p.S.H(), p.S.g(), p.S.y()); count_launch();
         lincomb_kernel<<<g, 256, 0, st>>>(len, p.V, len, jn, p.S.y(), 1.0, nullptr, p.w); count_launch();
-        RPBD_TRY(precond_saddle_impl(h, p.w, p.w + 3 * n, p.z, p.z + 3 * n, st));
-        add_kernel<<<g, 256, 0, st>>>(len, p.z, p.x); count_launch();
+        const PrecSaddle ps{p.w, p.w + 3 * n, p.zl, p.zU};
+        RPBD_TRY(precond_saddle_impl(h, 1, &ps, st));
+        add_kernel<<<g, 256, 0, st>>>(3 * n, p.zl, p.x); count_launch();
+        add_kernel<<<vgrid(6 * nb), 256, 0, st>>>(6 * nb, p.zU, p.x + 3 * n); count_launch();
         RPBD_LAUNCH_CHECK(h);
         return RPBD_OK;
     };
-    auto want_arnoldi = [&](GmresProc& p) -> int {
-        RPBD_TRY(precond_saddle_impl(h, p.V + (int64_t)p.j * len, p.V + (int64_t)p.j * len + 3 * n, p.z, p.z + 3 * n, st));
-        p.req = p.z;
-        p.phase = GmresProc::NEED_ARNOLDI;
-        return RPBD_OK;
+    auto want_resid = [&](GmresProc& p) {  // the product with x
+        p.req_l = p.x;
+        p.req_U = p.x + 3 * n;
+        p.phase = GmresProc::NEED_RESID;
     };
 
     for (int s = 0; s < nsys; ++s) {
         GmresProc& p = P[s];
         p.pb = probs[s];
         p.V = Vall + (int64_t)s * (mdim + 1) * len;
-        p.x = vall + (int64_t)s * 4 * len;
+        p.x = vall + (int64_t)s * 3 * len;
         p.b = p.x + len;
         p.w = p.x + 2 * len;
-        p.z = p.x + 3 * len;
-        p.S = Small{small + (int64_t)s * Small::count(mdim), mdim};
+        // the blob parts of all processes' z lie side by side: a k-RHS matvec takes them as they are
+        p.zl = vall + (int64_t)nsys * 3 * len + (int64_t)s * 3 * n;
+        p.zU = vall + (int64_t)nsys * (3 * len + 3 * n) + (int64_t)s * 6 * nb;
+        p.S = Small{small + (int64_t)s * small_count, mdim};
         p.sc = p.S.scal();  // [0] |.|^2, [1] |b|, [2] residual estimate
         // b = [-slip; -FT]
         if (p.pb.slip) launch_scale_copy(3 * n, -1.0, p.pb.slip, p.b, st);
@@ -529,9 +710,8 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
             RPBD_CU(h, cudaMemcpyAsync(p.x, p.pb.lambda, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, st));
             RPBD_CU(h, cudaMemcpyAsync(p.x + 3 * n, p.pb.U, sizeof(double) * 6 * nb, cudaMemcpyDeviceToDevice, st));
             RPBD_TRY(multidot(h, len, p.b, 0, 1, p.b, &p.sc[0], 0, p.S.partial(), st));
-            gmres_start_kernel<<<1, 1, 0, st>>>(mdim, &p.sc[0], p.S.g(), &p.sc[1], 1, &p.sc[2]); count_launch();
-            p.req = p.x;
-            p.phase = GmresProc::NEED_RESID;
+            gmres_start_kernel<<<1, 64, 0, st>>>(mdim, &p.sc[0], p.S.g(), p.sc, 1, h->host_small + 2 * s); count_launch();
+            want_resid(p);
         } else {
             RPBD_CU(h, cudaMemsetAsync(p.x, 0, sizeof(double) * len, st));
             launch_scale_copy(len, 1.0, p.b, p.w, st);
@@ -541,14 +721,19 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
 
     for (;;) {
         // residuals of every process waiting for one: one synchronisation
-        int nread = 0;
+        bool read = false;
         for (int s = 0; s < nsys; ++s)
-            if (P[s].phase == GmresProc::READ_START || P[s].phase == GmresProc::READ_ITER) {
-                RPBD_CU(h, cudaMemcpyAsync(h->host_small + 2 * s, &P[s].sc[1], 2 * sizeof(double),
-                                           cudaMemcpyDeviceToHost, st));
-                ++nread;
-            }
-        if (nread) RPBD_CU(h, cudaStreamSynchronize(st));
+            read = read || P[s].phase == GmresProc::READ_START || P[s].phase == GmresProc::READ_ITER;
+        if (read) RPBD_CU(h, cudaStreamSynchronize(st));
+        PrecSaddle ps[4];
+        int nps = 0;
+        auto want_arnoldi = [&](GmresProc& p) {  // z = P^-1 v_j, and the product with it
+            const double* v = p.V + (int64_t)p.j * len;
+            ps[nps++] = PrecSaddle{v, v + 3 * n, p.zl, p.zU};
+            p.req_l = p.zl;
+            p.req_U = p.zU;
+            p.phase = GmresProc::NEED_ARNOLDI;
+        };
         for (int s = 0; s < nsys; ++s) {
             GmresProc& p = P[s];
             const double bn = h->host_small[2 * s], res = h->host_small[2 * s + 1];
@@ -566,7 +751,7 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
                     p.phase = GmresProc::DONE;
                 } else {
                     p.j = 0;
-                    RPBD_TRY(want_arnoldi(p));
+                    want_arnoldi(p);
                 }
             } else if (p.phase == GmresProc::READ_ITER) {
                 p.res = res;
@@ -580,58 +765,70 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
                     } else if (p.total >= p.pb.max_iter) {
                         p.phase = GmresProc::DONE;
                     } else {
-                        p.req = p.x;  // restart: r0 = b - A x
-                        p.phase = GmresProc::NEED_RESID;
+                        want_resid(p);  // restart: r0 = b - A x
                     }
                 } else {
                     p.j = jn;
-                    RPBD_TRY(want_arnoldi(p));
+                    want_arnoldi(p);
                 }
             }
         }
+        if (nps) RPBD_TRY(precond_saddle_impl(h, nps, ps, st));
         // one matvec for every process that needs one
         int act[4], k = 0;
         for (int s = 0; s < nsys; ++s)
             if (P[s].phase == GmresProc::NEED_RESID || P[s].phase == GmresProc::NEED_ARNOLDI) act[k++] = s;
         if (k == 0) break;
-        if (k == 1) {
-            GmresProc& p = P[act[0]];
-            RPBD_TRY(mobility_apply_impl(h, n, r, p.req, p.w, 1, dtype, true, st));
-        } else {
-            double* Fm = mv;
-            double* Um = mv + (int64_t)k * 3 * n;
+        const double* Fm = P[act[0]].req_l;
+        double* Um = k == 1 ? P[act[0]].w : mv;
+        bool side = true;  // operands already side by side
+        for (int a = 1; a < k; ++a) side = side && P[act[a]].req_l == Fm + (int64_t)a * 3 * n;
+        if (!side) {
             for (int a = 0; a < k; ++a)
-                RPBD_CU(h, cudaMemcpyAsync(Fm + (int64_t)a * 3 * n, P[act[a]].req, sizeof(double) * 3 * n,
+                RPBD_CU(h, cudaMemcpyAsync(mv + (int64_t)(k + a) * 3 * n, P[act[a]].req_l, sizeof(double) * 3 * n,
                                            cudaMemcpyDeviceToDevice, st));
-            RPBD_TRY(mobility_apply_impl(h, n, r, Fm, Um, k, dtype, true, st));
-            for (int a = 0; a < k; ++a)
-                RPBD_CU(h, cudaMemcpyAsync(P[act[a]].w, Um + (int64_t)a * 3 * n, sizeof(double) * 3 * n,
-                                           cudaMemcpyDeviceToDevice, st));
+            Fm = mv + (int64_t)k * 3 * n;
         }
+        RPBD_TRY(mobility_apply_impl(h, n, r, Fm, Um, k, dtype, true, st));
+        SaddleBatch SB = {};
+        OrthoBatch B = {};
+        int no = 0;
         for (int a = 0; a < k; ++a) {
             GmresProc& p = P[act[a]];
-            saddle_finish(h, nb, nper, r, q, p.req, p.w, st);
+            SB.p[a] = SaddleProd{Um + (int64_t)a * 3 * n, p.req_l, p.req_U, p.w};
+        }
+        launch_pdl(saddle_kernel, dim3((unsigned)((nb + 3) / 4), (unsigned)k), 128, 0, st, nb, nper, r, q, SB);
+        count_launch();
+        for (int a = 0; a < k; ++a) {
+            GmresProc& p = P[act[a]];
             ++p.matvecs;
             if (p.phase == GmresProc::NEED_RESID) {
                 launch_axpby(len, 1.0, p.b, -1.0, p.w, p.w, st);
                 RPBD_TRY(begin_cycle(p, 0));
             } else {
                 // Arnoldi: classical Gram-Schmidt twice, Givens, residual estimate
-                const int j = p.j;
-                RPBD_TRY(multidot(h, len, p.V, len, j + 1, p.w, p.S.hcol(), 0, p.S.partial(), st));
-                multiaxpy_kernel<<<g, 256, 0, st>>>(len, p.V, len, j + 1, p.S.hcol(), p.w); count_launch();
-                RPBD_TRY(multidot(h, len, p.V, len, j + 1, p.w, p.S.y(), 0, p.S.partial(), st));
-                multiaxpy_kernel<<<g, 256, 0, st>>>(len, p.V, len, j + 1, p.S.y(), p.w); count_launch();
-                add_kernel<<<1, 256, 0, st>>>(j + 1, p.S.y(), p.S.hcol()); count_launch();
-                RPBD_TRY(multidot(h, len, p.w, 0, 1, p.w, p.S.hcol() + j + 1, 0, p.S.partial(), st));
-                normalize_kernel<<<g, 256, 0, st>>>(len, p.w, p.S.hcol() + j + 1, p.V + (int64_t)(j + 1) * len);
-                count_launch();
-                gmres_column_kernel<<<1, 1, 0, st>>>(j, mdim, p.S.hcol(), p.S.H(), p.S.cs(), p.S.sn(), p.S.g(),
-                                                      &p.sc[1], &p.sc[2]);
-                count_launch();
-                RPBD_LAUNCH_CHECK(h);
+                OrthoProc& o = B.p[no++];
+                o.V = p.V;
+                o.w = p.w;
+                o.part = p.S.partial();
+                o.h = p.S.hcol();
+                o.vnext = p.V + (int64_t)(p.j + 1) * len;
+                o.nv = p.j + 1;
+                o.H = p.S.H();
+                o.cs = p.S.cs();
+                o.sn = p.S.sn();
+                o.g = p.S.g();
+                o.sc = p.sc;
+                o.host = h->host_small + 2 * act[a];
                 p.phase = GmresProc::READ_ITER;
             }
+        }
+        if (no) {
+            const OrthoGrid G = launch_ortho(len, no, B, st);
+            launch_pdl(gmres_finish_kernel, dim3((unsigned)G.blocks + 1, (unsigned)no), 256,
+                       3 * (size_t)(mdim + 2) * sizeof(double), st, len, G.slice, mdim, B);
+            count_launch();
+            RPBD_LAUNCH_CHECK(h);
         }
     }
     RPBD_TRY(check_flag(h, st));

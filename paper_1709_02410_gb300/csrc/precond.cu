@@ -193,17 +193,24 @@ __global__ void __launch_bounds__(PREC_THREADS) prec_build_kernel(int nper, int6
     for (int e = tid; e < 36; e += blockDim.x) gN[p * 36 + e] = NN[e];
 }
 
+// Rows of the stored factors' products, one CTA per body, entries read straight
+// from global memory, every one once.  The threads split a row's columns into
+// APPLY_THREADS / span pieces, so a chain is ~m / 4 loads, issued eight at a
+// time; with half the threads, the factor staged in shared memory first and
+// loads one by one a 45-row product took ~10 us, most of it latency.
+constexpr int APPLY_THREADS = 256;
+
 // out = A_p x_p per body, A_p one of the stored factors.
 // mode 0: L (lower), 1: L^-1 (lower), 2: L^-T, 3: M^-1.  With `active`
 // (batches: systems at blob offsets off[0..n_sys]), bodies of inactive
 // systems are skipped and their out left as it is.
-__global__ void __launch_bounds__(PREC_THREADS) prec_apply_kernel(int mode, int nper, int64_t n,
-                                                                  const double* __restrict__ Mat,
-                                                                  const double* __restrict__ x, double* __restrict__ out,
-                                                                  const int* __restrict__ active,
-                                                                  const int64_t* __restrict__ off, int n_sys)
+__global__ void __launch_bounds__(APPLY_THREADS) prec_apply_kernel(int mode, int nper, int64_t n,
+                                                                   const double* Mat, const double* x, double* out,
+                                                                   const int* active, const int64_t* off, int n_sys)
 {
-    extern __shared__ double sm[];
+    __shared__ double v[PREC_MAX_M], part[APPLY_THREADS];
+    pdl_wait();
+    pdl_trigger();
     const int m = 3 * nper;
     const int64_t p = blockIdx.x;
     if (active) {
@@ -216,101 +223,89 @@ __global__ void __launch_bounds__(PREC_THREADS) prec_apply_kernel(int mode, int 
         }
         if (!active[lo]) return;
     }
-    double* A = sm;
-    double* v = sm + m * m;
-    const double* src = Mat + p * m * m;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) A[e] = src[e];
-    for (int e = threadIdx.x; e < m; e += blockDim.x) {
-        const int b = e / 3, c = e % 3;
-        v[e] = x[c * n + p * nper + b];
-    }
+    const double* A = Mat + p * m * m;
+    const int tid = threadIdx.x;
+    for (int e = tid; e < m; e += APPLY_THREADS) v[e] = x[(e % 3) * n + p * nper + e / 3];
     __syncthreads();
-    // row i's sum over its column range [j0, j1) split into `parts` pieces
-    // over the CTA's threads, then added in order
-    double* part = v + m;  // parts * span
-    const int span = (m + 31) & ~31, parts = PREC_THREADS / span;
-    const int q = threadIdx.x / span, i = threadIdx.x % span;
+    if (mode == 2) {  // (L^-1)^T: sum_j Linv(j, i) v_j, j >= i: column i is contiguous, one warp per row
+        const int lane = tid & 31;
+        for (int i = tid >> 5; i < m; i += APPLY_THREADS / 32) {
+            double acc = 0.0;
+            for (int j = i + lane; j < m; j += 32) acc += A[i * m + j] * v[j];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane == 0) out[(i % 3) * n + p * nper + i / 3] = acc;
+        }
+        return;
+    }
+    // M^-1, or lower triangular (j <= i): row i's columns j = q, q + parts, ...
+    const int span = (m + 31) & ~31, parts = APPLY_THREADS / span;
+    const int q = tid / span, i = tid % span;
     if (q < parts && i < m) {
-        const int j0 = mode == 2 ? i : 0, j1 = mode == 2 || mode == 3 ? m : i + 1;
-        const int per = (j1 - j0 + parts - 1) / parts;
-        const int a0 = j0 + q * per, a1 = a0 + per < j1 ? a0 + per : j1;
+        const int j1 = mode == 3 ? m : i + 1;
         double acc = 0.0;
-        if (mode == 2)  // (L^-1)^T: sum_j Linv(j, i) v_j, j >= i
-            for (int j = a0; j < a1; ++j) acc += A[i * m + j] * v[j];
-        else            // M^-1, or lower triangular (j <= i)
-            for (int j = a0; j < a1; ++j) acc += A[j * m + i] * v[j];
+#pragma unroll 8
+        for (int j = q; j < j1; j += parts) acc += A[j * m + i] * v[j];
         part[q * span + i] = acc;
     }
     __syncthreads();
-    if (threadIdx.x < m) {
-        double acc = part[threadIdx.x];
-        for (int q2 = 1; q2 < parts; ++q2) acc += part[q2 * span + threadIdx.x];
-        const int b = threadIdx.x / 3, c = threadIdx.x % 3;
-        out[c * n + p * nper + b] = acc;
+    if (tid < m) {
+        double acc = part[tid];
+        for (int q2 = 1; q2 < parts; ++q2) acc += part[q2 * span + tid];
+        out[(tid % 3) * n + p * nper + tid / 3] = acc;
     }
 }
 
 // exact body-block saddle solve: [M(pp) -K_p; -K_p^T 0][lam; U] = [a; b]
 //   t = (M^-1 K)^T a + b,  U = -N t,  lam = M^-1 a + (M^-1 K) U
-// One CTA per body.  M^-1 and M^-1 K are read straight from global memory
-// (each entry once, coalesced along the row index); the six dot products of
-// t use one warp each with a shuffle reduction, and the m-row product is split
-// into column halves over the CTA's threads, then added.
-__global__ void __launch_bounds__(PREC_THREADS) prec_saddle_kernel(int nper, int64_t n, const double* __restrict__ Minv,
-                                                                   const double* __restrict__ MinvK,
-                                                                   const double* __restrict__ N,
-                                                                   const double* __restrict__ a,
-                                                                   const double* __restrict__ b,
-                                                                   double* __restrict__ lam, double* __restrict__ U)
+// for up to four vectors (blockIdx.y).  M^-1 a does not wait for U.
+struct SaddleArgs {
+    PrecSaddle p[4];
+};
+__global__ void __launch_bounds__(APPLY_THREADS) prec_saddle_kernel(int nper, int64_t n, const double* Minv,
+                                                                    const double* MinvK, const double* N, SaddleArgs S)
 {
-    extern __shared__ double sm[];
+    __shared__ double va[PREC_MAX_M], part[APPLY_THREADS], t6[6], u6[6];
+    pdl_wait();
+    pdl_trigger();
+    const PrecSaddle P = S.p[blockIdx.y];
     const int m = 3 * nper;
     const int64_t p = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int NW = PREC_THREADS / 32;
-    const int span = (m + 31) & ~31;           // threads per column part
-    const int parts = PREC_THREADS / span;     // >= 1 since m <= PREC_MAX_M <= PREC_THREADS
-    double* va = sm;                           // m
-    double* part = va + m;                     // parts * span
-    __shared__ double t6[6], u6[6];
+    const int span = (m + 31) & ~31, parts = APPLY_THREADS / span;
     const double* A = Minv + p * m * m;        // column-major: (i, j) at j * m + i
     const double* MK = MinvK + p * 6 * m;      // (M^-1 K)^T rows: column c at c * m
-    for (int e = tid; e < m; e += PREC_THREADS) {
-        const int bb = e / 3, c = e % 3;
-        va[e] = a ? a[c * n + p * nper + bb] : 0.0;
-    }
+    for (int e = tid; e < m; e += APPLY_THREADS) va[e] = P.a ? P.a[(e % 3) * n + p * nper + e / 3] : 0.0;
     __syncthreads();
-    for (int e = warp; e < 6; e += NW) {
+    if (warp < 6) {
         double v = 0.0;
-        for (int k = lane; k < m; k += 32) v += MK[e * m + k] * va[k];
+        for (int k = lane; k < m; k += 32) v += MK[warp * m + k] * va[k];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) t6[e] = v + (b ? b[6 * p + e] : 0.0);
+        if (lane == 0) t6[warp] = v + (P.b ? P.b[6 * p + warp] : 0.0);
+    }
+    const int q = tid / span, i = tid % span;
+    if (q < parts && i < m) {
+        double v = 0.0;
+#pragma unroll 8
+        for (int j = q; j < m; j += parts) v += A[j * m + i] * va[j];
+        part[q * span + i] = v;
     }
     __syncthreads();
     if (tid < 6) {
         double v = 0.0;
+#pragma unroll
         for (int c = 0; c < 6; ++c) v -= N[p * 36 + c * 6 + tid] * t6[c];
         u6[tid] = v;
-        U[6 * p + tid] = v;
-    }
-    __syncthreads();
-    const int q = tid / span, i = tid % span;
-    if (q < parts && i < m) {
-        const int per = (m + parts - 1) / parts;
-        const int j0 = q * per, j1 = j0 + per < m ? j0 + per : m;
-        double v = 0.0;
-        for (int j = j0; j < j1; ++j) v += A[j * m + i] * va[j];
-        if (q == 0)
-            for (int c = 0; c < 6; ++c) v += MK[c * m + i] * u6[c];
-        part[q * span + i] = v;
+        P.U[6 * p + tid] = v;
     }
     __syncthreads();
     if (tid < m) {
         double v = part[tid];
         for (int q2 = 1; q2 < parts; ++q2) v += part[q2 * span + tid];
-        const int bb = tid / 3, c = tid % 3;
-        lam[c * n + p * nper + bb] = v;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) v += MK[c * m + tid] * u6[c];
+        P.lam[(tid % 3) * n + p * nper + tid / 3] = v;
     }
 }
 
@@ -328,14 +323,11 @@ int precond_build_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, co
     RPBD_TRY(ensure_t(h, BUF_PREC_N, (size_t)nb * 36, &N));
     const size_t smem = (size_t)(2 * m * m + 6 * m + 5 * nper) * sizeof(double);
     const double inv8pieta = 1.0 / (8.0 * 3.14159265358979323846 * h->p.eta);
-    if (once_per_device(h, reinterpret_cast<const void*>(prec_apply_kernel))) {
+    if (once_per_device(h, reinterpret_cast<const void*>(prec_build_kernel<true, false>))) {
         const int mx = (2 * PREC_MAX_M * PREC_MAX_M + 6 * PREC_MAX_M + 5 * 32) * (int)sizeof(double);
         RPBD_CU(h, cudaFuncSetAttribute(prec_build_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
         RPBD_CU(h, cudaFuncSetAttribute(prec_build_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
         RPBD_CU(h, cudaFuncSetAttribute(prec_build_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-        const int mx2 = (PREC_MAX_M * PREC_MAX_M + 7 * PREC_MAX_M) * (int)sizeof(double);
-        RPBD_CU(h, cudaFuncSetAttribute(prec_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mx2));
-        RPBD_CU(h, cudaFuncSetAttribute(prec_saddle_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mx2));
     }
     RPBD_CU(h, cudaMemsetAsync(h->dev_flag, 0, sizeof(int), st));
     const double Lx = h->p.Lx, Ly = h->p.Ly;
@@ -361,26 +353,25 @@ int precond_apply_impl(rpbd_handle* h, int mode, const double* x, double* out, c
 {
     if (!h->prec_valid) return set_error(h, RPBD_BAD_ARG, "preconditioner not built");
     if (mode < 0 || mode > 3 || !x || !out) return set_error(h, RPBD_BAD_ARG, "precond_apply: bad arguments");
-    const int m = 3 * h->prec_nper;
     const double* Mat = mode == 0 ? (const double*)h->buf[BUF_PREC_L]
                         : mode == 3 ? (const double*)h->buf[BUF_PREC_MINV]
                                     : (const double*)h->buf[BUF_PREC_LINV];
-    const size_t smem = (size_t)(m * m + m + PREC_THREADS) * sizeof(double);
-    prec_apply_kernel<<<(unsigned)h->prec_nb, PREC_THREADS, smem, st>>>(
-        mode, h->prec_nper, h->prec_nb * h->prec_nper, Mat, x, out, active, off, n_sys);
+    launch_pdl(prec_apply_kernel, (unsigned)h->prec_nb, APPLY_THREADS, 0, st, mode, h->prec_nper,
+               h->prec_nb * h->prec_nper, Mat, x, out, active, off, n_sys);
     count_launch();
     RPBD_LAUNCH_CHECK(h);
     return RPBD_OK;
 }
 
-int precond_saddle_impl(rpbd_handle* h, const double* a, const double* b, double* lam, double* U, cudaStream_t st)
+int precond_saddle_impl(rpbd_handle* h, int np, const PrecSaddle* ps, cudaStream_t st)
 {
     if (!h->prec_valid) return set_error(h, RPBD_BAD_ARG, "preconditioner not built");
-    const int m = 3 * h->prec_nper;
-    const size_t smem = (size_t)(m + PREC_THREADS) * sizeof(double);
-    prec_saddle_kernel<<<(unsigned)h->prec_nb, PREC_THREADS, smem, st>>>(
-        h->prec_nper, h->prec_nb * h->prec_nper, (const double*)h->buf[BUF_PREC_MINV],
-        (const double*)h->buf[BUF_PREC_MINVK], (const double*)h->buf[BUF_PREC_N], a, b, lam, U); count_launch();
+    SaddleArgs S = {};
+    for (int a = 0; a < np; ++a) S.p[a] = ps[a];
+    launch_pdl(prec_saddle_kernel, dim3((unsigned)h->prec_nb, (unsigned)np), APPLY_THREADS, 0, st, h->prec_nper,
+               h->prec_nb * h->prec_nper, (const double*)h->buf[BUF_PREC_MINV], (const double*)h->buf[BUF_PREC_MINVK],
+               (const double*)h->buf[BUF_PREC_N], S);
+    count_launch();
     RPBD_LAUNCH_CHECK(h);
     return RPBD_OK;
 }

@@ -148,6 +148,8 @@ namespace rpbd {
 // predecessor lets it start early with pdl_trigger().  Every kernel of such a
 // chain waits, so completion stays in stream order.  Hides the ~2 us launch
 // gap between the short kernels of one call; also valid under stream capture.
+// Pointers to what earlier kernels write are not __restrict__ in such a kernel:
+// that would let the compiler move their loads above the wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -228,9 +230,12 @@ int check_finite(rpbd_handle* h, int64_t n, const double* x, cudaStream_t st);
 // systems at device blob offsets off[0..n_sys]
 int precond_apply_impl(rpbd_handle* h, int mode, const double* x, double* out, cudaStream_t st,
                        const int* active = nullptr, const int64_t* off = nullptr, int n_sys = 0);
-// saddle block solve: (lam, U) = P^-1 (a, b)
-int precond_saddle_impl(rpbd_handle* h, const double* a, const double* b, double* lam,
-                        double* U, cudaStream_t st);
+// saddle block solves: (lam, U) = P^-1 (a, b) for np <= 4 vectors
+struct PrecSaddle {
+    const double *a, *b;
+    double *lam, *U;
+};
+int precond_saddle_impl(rpbd_handle* h, int np, const PrecSaddle* ps, cudaStream_t st);
 
 int lanczos_impl(rpbd_handle* h, int64_t n, const double* r, const double* W, double* out,
                  double tol, int max_iter, int dtype, int use_precond, rpbd_stats* stats,

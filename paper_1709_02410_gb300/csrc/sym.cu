@@ -535,11 +535,11 @@ struct Fixed2 {
 // exponent S of a system's scale 2^S from its T home tiles' maxima, by the
 // whole CTA of NT threads (red: NT / 32 words); *bad: a force is not finite
 template <int NT>
-__device__ __forceinline__ int fixed2_exponent(const float* __restrict__ bmax, int T, int64_t n, double cap, unsigned* red,
+__device__ __forceinline__ int fixed2_exponent(const float* bmax, int T, int64_t n, double cap, unsigned* red,
                                                bool* bad)
 {
     unsigned m = 0u;
-    for (int t = threadIdx.x; t < T; t += NT) m = max(m, __float_as_uint(__ldg(bmax + t)));
+    for (int t = threadIdx.x; t < T; t += NT) m = max(m, __float_as_uint(bmax[t]));
     m = __reduce_max_sync(0xffffffffu, m);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
     __syncthreads();
@@ -553,11 +553,12 @@ __device__ __forceinline__ int fixed2_exponent(const float* __restrict__ bmax, i
 // tiles); padding records sit far away with zero force.
 template <int K, class In>
 __global__ void __launch_bounds__(HT2) pack2_kernel(int n_sys, const SymSys* __restrict__ sys, int64_t rec_end, int64_t n_tot, int k,
-                             const double* __restrict__ r, const In* __restrict__ F, double a, double ia, int wall,
+                             const double* r, const In* F, double a, double ia, int wall,
                              double s_min,
-                             const int* __restrict__ active, float* __restrict__ rec, double* __restrict__ scale,
+                             const int* active, float* rec, double* scale,
                              Fixed2 fx)
 {
+    pdl_wait();
     pdl_trigger();
     // one block per home tile (rec_end is a whole number of them)
     const int64_t j = blockIdx.x * (int64_t)HT2 + threadIdx.x;
@@ -762,12 +763,12 @@ struct Sym2Var {
 // visitor and home sums go into the fixed-point accumulators (fx) instead of
 // the per-home-tile partials.
 template <int K, bool PER, int UNR, int MINB, bool BATCH, int HP = 1, bool FAR = false, bool ATOM = false>
-__global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float* __restrict__ rec,
+__global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float* rec,
                                                               const SymItem* __restrict__ items, int64_t n,
                                                               int64_t n_pad, int n_home_tiles,
                                                               const SymSys* __restrict__ sys,
-                                                              const int* __restrict__ active, float Lx, float Ly,
-                                                              float* __restrict__ partial, int* __restrict__ err_flag,
+                                                              const int* active, float Lx, float Ly,
+                                                              float* partial, int* __restrict__ err_flag,
                                                               RingTest rt, Fixed2 fx, int64_t acc_stride)
 {
     constexpr int NT = HT2 / (2 * HP);  // threads
@@ -953,12 +954,12 @@ __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float*
 // (blockIdx.y): a block never straddles two systems.
 template <class Out>
 __global__ void __launch_bounds__(HT2) finish2_kernel(int n_sys, const SymSys* __restrict__ sys, int64_t n_tot, int64_t acc_stride,
-                                                      double cap, const int* __restrict__ active, Fixed2 fx,
-                                                      const double* __restrict__ scale, double inv8pieta,
-                                                      Out* __restrict__ U)
+                                                      double cap, const int* active, Fixed2 fx, const double* scale,
+                                                      double inv8pieta, Out* U)
 {
     __shared__ unsigned red[HT2 / 32];
     pdl_wait();
+    pdl_trigger();
     const int64_t j = blockIdx.x * (int64_t)HT2 + threadIdx.x;  // record
     const int q = blockIdx.y;
     const int sx = n_sys == 1 ? 0 : sys_of(n_sys, j, [&](int m) { return sys[m].B; });
@@ -1193,8 +1194,8 @@ static int run2(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, 
         RPBD_TRY(ensure_t(h, b_seg, (size_t)std::max<int64_t>(1, pl->seg_rows) * 3 * K, &segsum));
     }
     const unsigned tiles_ = (unsigned)(pl->rec_end / HT2);
-    pack2_kernel<K, In><<<tiles_, HT2, 0, st>>>(n_sys, pl->d_sys, pl->rec_end, n_tot, k, r, F, h->p.a, 1.0 / h->p.a,
-                                                h->p.wall, h->p.s_min, active, rec, scale, fx);
+    launch_pdl(pack2_kernel<K, In>, tiles_, HT2, 0, st, n_sys, (const SymSys*)pl->d_sys, pl->rec_end, n_tot, k, r, F, h->p.a,
+               1.0 / h->p.a, h->p.wall, h->p.s_min, active, rec, scale, fx);
     count_launch();
     const float Lxa = (float)(h->p.Lx / h->p.a), Lya = (float)(h->p.Ly / h->p.a);  // periodic cell in units of a
     if (h->profile) prof_begin(h, st);

@@ -199,9 +199,10 @@ __device__ __forceinline__ void image_sum(double dx0, double dy0, double zi, dou
 // Records: field f of blob i at ((i / 32) NF + f) 32 + i % 32, fields x, y,
 // z~, s F(0, x..z), ...; padding blobs sit far away with zero force.
 template <int K>
-__global__ void pack64_kernel(int64_t n, int64_t n_pad, int k, const double* __restrict__ r, const double* __restrict__ F,
-                              double a, int wall, double s_min, double* __restrict__ rec, double* __restrict__ scale)
+__global__ void pack64_kernel(int64_t n, int64_t n_pad, int k, const double* r, const double* F, double a, int wall,
+                              double s_min, double* rec, double* scale)
 {
+    pdl_wait();
     pdl_trigger();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n_pad) return;
@@ -234,8 +235,8 @@ __global__ void pack64_kernel(int64_t n, int64_t n_pad, int k, const double* __r
 // Grid: (home tile, item of `chunk` visitor tiles, part of the steps).  Partial
 // rows of [3K][n_pad]: T * parts visitor rows, then items * parts home rows.
 template <int K, bool WALL, bool PER, int NW>
-__global__ void __launch_bounds__(32 * NW) sym64_kernel(const double* __restrict__ rec, int64_t n_pad, int chunk, Const c,
-                                                        double* __restrict__ partial, int* __restrict__ err_flag, RingTest rt)
+__global__ void __launch_bounds__(32 * NW) sym64_kernel(const double* rec, int64_t n_pad, int chunk, Const c,
+                                                        double* partial, int* err_flag, RingTest rt)
 {
     constexpr int NF = 3 + 3 * K, NT = 32 * NW;
     constexpr uint32_t TILE_BYTES = VT * NF * sizeof(double);
@@ -381,12 +382,12 @@ __global__ void __launch_bounds__(32 * NW) sym64_kernel(const double* __restrict
 constexpr int RS = 8;
 template <int K>
 __global__ void __launch_bounds__(32 * RS) reduce64_kernel(int64_t n, int64_t n_pad, int nw, int T, int parts, int chunk,
-                                                           const double* __restrict__ partial,
-                                                           const double* __restrict__ scale, double inv8pieta,
-                                                           double* __restrict__ U)
+                                                           const double* partial, const double* scale,
+                                                           double inv8pieta, double* U)
 {
     __shared__ double sm[RS][32];
     pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31, y = threadIdx.x >> 5, q = blockIdx.y;
     const int64_t tile = blockIdx.x, i = tile * VT + lane;
     const int home = (int)(tile / nw), sub = (int)(tile % nw);
@@ -454,8 +455,8 @@ static int run(rpbd_handle* h, const Cut& c, int64_t n, const double* r, const d
     RPBD_TRY(ensure_t(h, BUF_PACK, (size_t)c.n_pad * (3 + 3 * K), &rec));
     RPBD_TRY(ensure_t(h, BUF_SCALE, (size_t)c.n_pad, &scale));
     RPBD_TRY(ensure_t(h, BUF_PARTIAL, (size_t)c.rows() * 3 * K * c.n_pad, &partial));
-    pack64_kernel<K><<<(unsigned)((c.n_pad + 127) / 128), 128, 0, st>>>(n, c.n_pad, k, r, F, h->p.a, h->p.wall, h->p.s_min,
-                                                                        rec, scale);
+    launch_pdl(pack64_kernel<K>, (unsigned)((c.n_pad + 127) / 128), 128, 0, st, n, c.n_pad, k, r, F, h->p.a, h->p.wall,
+               h->p.s_min, rec, scale);
     count_launch();
     if (h->profile) prof_begin(h, st);
     const bool per = h->p.Lx > 0.0;
