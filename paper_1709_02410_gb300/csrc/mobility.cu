@@ -28,6 +28,7 @@
 #include "fixed_point.cuh"
 #include "rpbd_internal.cuh"
 #include "wall_rpy.cuh"
+#include "wall_rpy_x2.cuh"
 
 namespace rpbd {
 
@@ -501,6 +502,273 @@ static int apply_k(rpbd_handle* h, int64_t n, const double* r, const In* F, Out*
     return RPBD_OK;
 }
 
+// ---------------------------------------------------------------------------
+// Five to sixteen right-hand sides with the wall, FP32: two targets per thread.
+//
+// With one target per thread every pair's 14 16-byte record loads returned as
+// many bytes as shared memory delivers in the time of its FMAs (k = 16: 224
+// against 219 cycles per 128 pairs), and the block was formed by scalar
+// instructions.  Two targets share each loaded record; their blocks are formed
+// together by packed two-wide instructions (wall_rpy_x2.cuh, lengths in units of
+// a), then each target's entry is broadcast into a register pair and applied to
+// the right-hand sides two at a time.  Consecutive FMAs share the force operand,
+// which spares register-file reads.  65,535 blobs: k = 16 27.9 -> 23.7 ms (90% of
+// the FMA pipe by instruction count), k = 8 18.6 -> 15.7 ms.  Three CTAs per SM
+// (168 registers) against two without spills: 23.7 / 24.9 ms.
+namespace wide {
+
+constexpr int BT = 128;   // threads; 2 BT targets per CTA
+constexpr int TS = 64;    // sources per stage
+constexpr int NST = 3;
+
+// source record: x_hi x_hi y_hi y_hi | x_lo x_lo y_lo y_lo | z~ z~ - - | forces as in Rec<float, K>
+template <int K>
+struct WRec {
+    static constexpr int LEN = 12 + 3 * K;
+    static_assert(K % 4 == 0, "whole 16-byte chunks");
+};
+
+template <int K, class In>
+__global__ void pack_kernel(int64_t n, int64_t n_pad, int k, const double* r, const In* F, double a, double ia, double s_min,
+                            float* rec, double* scale, unsigned* fmax_bits)
+{
+    pdl_trigger();
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n_pad) return;
+    float* o = rec + i * WRec<K>::LEN;
+    double x = 1.0e7, y = 1.0e7, zt = a, s = 0.0;  // padding: far away, zero force
+    if (i < n) {
+        x = r[i] * ia;
+        y = r[n + i] * ia;
+        const double z = r[2 * n + i];
+        zt = z > a ? z : a;
+        s = 1.0;
+        if (!(z >= a)) {  // (NaN stays NaN)
+            const double t = z / a;
+            s = t >= 1.0 ? 1.0 : (t <= s_min ? s_min : t);
+        }
+        scale[i] = s;
+    }
+    const float xh = (float)x, yh = (float)y, xl = (float)(x - (double)xh), yl = (float)(y - (double)yh), z = (float)(zt * ia);
+    float4* o4 = reinterpret_cast<float4*>(o);
+    o4[0] = make_float4(xh, xh, yh, yh);
+    o4[1] = make_float4(xl, xl, yl, yl);
+    o4[2] = make_float4(z, z, 0.0f, 0.0f);
+    float fm = 0.0f;  // largest |stored force| of this blob (+inf: not finite)
+#pragma unroll
+    for (int m = 0; m < K; ++m)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            float v = 0.0f;
+            if (i < n && m < k) {
+                v = (float)(s * (double)F[((int64_t)m * 3 + c) * n + i]);
+                fm = isfinite(v) ? fmaxf(fm, fabsf(v)) : INFINITY;
+            }
+            o[12 + 6 * (m / 2) + 2 * c + (m & 1)] = v;
+        }
+    if (fmax_bits) fixed_force_max(fmax_bits, fm);
+}
+
+template <int K, bool PER, bool FX, int MINB>
+__global__ void __launch_bounds__(BT, MINB) pair_kernel(const float* rec, int64_t n, int64_t n_pad, int tiles_per_chunk,
+                                                        int n_tiles, float Lx, float Ly, float* partial, int* err_flag,
+                                                        RingTest rt, FixedAcc fx)
+{
+    constexpr int LEN = WRec<K>::LEN;
+    constexpr uint32_t TILE_BYTES = TS * LEN * sizeof(float);
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    float* stage = reinterpret_cast<float*>(smem_raw);
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + NST * TILE_BYTES);
+    const int tid = threadIdx.x, chunk = blockIdx.y;
+    const int tile0 = chunk * tiles_per_chunk;
+    const int ntile = min(tiles_per_chunk, n_tiles - tile0);
+    const int64_t i0 = blockIdx.x * (int64_t)(2 * BT) + tid, i1 = i0 + BT;
+    pdl_wait();
+    pdl_trigger();
+    if (tid == 0) {
+#pragma unroll
+        for (int s = 0; s < NST; ++s) mbar_init(&bar[s], 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    if (tid == 0)  // (failure-path test: stage 0 gets no copy, so its wait runs out)
+        for (int s = rt.skip_first ? 1 : 0; s < NST && s < ntile; ++s) {
+            mbar_expect_tx(&bar[s], TILE_BYTES);
+            tma_load_1d(stage + (size_t)s * TS * LEN, rec + (size_t)(tile0 + s) * TS * LEN, TILE_BYTES, &bar[s]);
+        }
+    const float* r0 = rec + (i0 < n ? i0 : n - 1) * LEN;
+    const float* r1 = rec + (i1 < n ? i1 : n - 1) * LEN;
+    const float2 xh = make_float2(r0[0], r1[0]), yh = make_float2(r0[2], r1[2]);
+    const float2 xl = make_float2(r0[4], r1[4]), yl = make_float2(r0[6], r1[6]), zi = make_float2(r0[8], r1[8]);
+    const PairConstX2 pc = PairConstX2::make_unit();
+    const float2 m1 = pc.m1;
+    float2 acc[2][3 * K / 2];  // [target][3 p + c]: right-hand sides 2p, 2p + 1
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int q = 0; q < 3 * K / 2; ++q) acc[t][q] = make_float2(0.0f, 0.0f);
+    int t = 0;
+    bool bad = false;
+    for (; t < ntile; ++t) {
+        const int s = t % NST;
+        const bool ok = mbar_wait_bounded(&bar[s], (t / NST) & 1, rt.limit);
+        if (ok) {
+            const float* st = stage + (size_t)s * TS * LEN;
+#pragma unroll 1
+            for (int jj = 0; jj < TS; ++jj) {
+                const float4* rj = reinterpret_cast<const float4*>(st + jj * LEN);
+                const float4 p0 = rj[0], p1 = rj[1], p2 = rj[2];
+                float2 dx = add2(fma2(m1, make_float2(p0.x, p0.y), xh), fma2(m1, make_float2(p1.x, p1.y), xl));
+                float2 dy = add2(fma2(m1, make_float2(p0.z, p0.w), yh), fma2(m1, make_float2(p1.z, p1.w), yl));
+                const float2 zj = make_float2(p2.x, p2.y);
+                const float2 dz = fma2(m1, zj, zi);
+                ImageBlock2 M;
+                if constexpr (PER) {
+                    const float iLx = 1.0f / Lx, iLy = 1.0f / Ly;
+                    dx = make_float2(dx.x - Lx * rintf(dx.x * iLx), dx.y - Lx * rintf(dx.y * iLx));
+                    dy = make_float2(dy.x - Ly * rintf(dy.x * iLy), dy.y - Ly * rintf(dy.y * iLy));
+                    pair_image_sum_x2<false>(dx, dy, dz, zi, zj, Lx, Ly, pc, M);
+                } else {
+                    float2 al, be, gx, gz;
+                    pair_factors_x2<false>(dx, dy, dz, zi, zj, pc, al, be, gx, gz, M.zz);
+                    const float2 bx = mul2(be, dx), by = mul2(be, dy);
+                    M.xx = fma2(bx, dx, al);
+                    M.xy = mul2(bx, dy);
+                    M.yy = fma2(by, dy, al);
+                    M.xz = mul2(dx, gx);
+                    M.yz = mul2(dy, gx);
+                    M.zx = mul2(dx, gz);
+                    M.zy = mul2(dy, gz);
+                }
+                const float2 xx0 = bc2(M.xx.x), xy0 = bc2(M.xy.x), yy0 = bc2(M.yy.x), xz0 = bc2(M.xz.x), yz0 = bc2(M.yz.x);
+                const float2 zx0 = bc2(M.zx.x), zy0 = bc2(M.zy.x), zz0 = bc2(M.zz.x);
+                const float2 xx1 = bc2(M.xx.y), xy1 = bc2(M.xy.y), yy1 = bc2(M.yy.y), xz1 = bc2(M.xz.y), yz1 = bc2(M.yz.y);
+                const float2 zx1 = bc2(M.zx.y), zy1 = bc2(M.zy.y), zz1 = bc2(M.zz.y);
+                const float2* f = reinterpret_cast<const float2*>(st + jj * LEN + 12);
+#pragma unroll
+                for (int p = 0; p < K / 2; ++p) {
+                    float2 *a = acc[0] + 3 * p, *b = acc[1] + 3 * p;
+                    const float2 fx = f[3 * p], fy = f[3 * p + 1], fz = f[3 * p + 2];
+                    a[0] = fma2(xx0, fx, a[0]);
+                    a[1] = fma2(xy0, fx, a[1]);
+                    a[2] = fma2(zx0, fx, a[2]);
+                    b[0] = fma2(xx1, fx, b[0]);
+                    b[1] = fma2(xy1, fx, b[1]);
+                    b[2] = fma2(zx1, fx, b[2]);
+                    a[0] = fma2(xy0, fy, a[0]);
+                    a[1] = fma2(yy0, fy, a[1]);
+                    a[2] = fma2(zy0, fy, a[2]);
+                    b[0] = fma2(xy1, fy, b[0]);
+                    b[1] = fma2(yy1, fy, b[1]);
+                    b[2] = fma2(zy1, fy, b[2]);
+                    a[0] = fma2(xz0, fz, a[0]);
+                    a[1] = fma2(yz0, fz, a[1]);
+                    a[2] = fma2(zz0, fz, a[2]);
+                    b[0] = fma2(xz1, fz, b[0]);
+                    b[1] = fma2(yz1, fz, b[1]);
+                    b[2] = fma2(zz1, fz, b[2]);
+                }
+            }
+        }
+        if (__syncthreads_or(!ok)) {
+            bad = true;
+            break;
+        }
+        if (tid == 0 && t + NST < ntile) {
+            fence_proxy_async();
+            mbar_expect_tx(&bar[s], TILE_BYTES);
+            tma_load_1d(stage + (size_t)s * TS * LEN, rec + (size_t)(tile0 + t + NST) * TS * LEN, TILE_BYTES, &bar[s]);
+        }
+    }
+    if (bad) {  // record the timeout, then let copies still in flight land (bounded)
+        if (tid == 0) {
+            atomicExch(err_flag, 1);
+            for (int u = t + 1; u < ntile && u < t + NST; ++u) mbar_wait_bounded(&bar[u % NST], (u / NST) & 1);
+        }
+        return;
+    }
+    const int S = FX ? fixed_exponent(__uint_as_float(*fx.fmax_bits), n, fx.cap) : 0;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+        const int64_t i = g ? i1 : i0;
+        if (i >= n) continue;
+#pragma unroll
+        for (int p = 0; p < K / 2; ++p)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float2 v = acc[g][3 * p + c];
+                const int64_t q = 6 * p + c;  // component c of right-hand side 2p; of 2p + 1: q + 3
+                if constexpr (FX) {
+                    fixed_add(fx.acc + q * n_pad + i, v.x, S, fx.fmax_bits + 1);
+                    fixed_add(fx.acc + (q + 3) * n_pad + i, v.y, S, fx.fmax_bits + 1);
+                } else {
+                    partial[((int64_t)chunk * 3 * K + q) * n_pad + i] = v.x;
+                    partial[((int64_t)chunk * 3 * K + q + 3) * n_pad + i] = v.y;
+                }
+            }
+    }
+}
+
+template <int K, bool PER, class In, class Out>
+static int apply(rpbd_handle* h, int64_t n, const double* r, const In* F, Out* U, int k, cudaStream_t st)
+{
+    constexpr int LEN = WRec<K>::LEN;
+    constexpr int MINB = K == 16 ? (PER ? 2 : 3) : (PER ? 2 : 4);
+    const int64_t n_pad = (n + TS - 1) / TS * TS;
+    const int n_tiles = (int)(n_pad / TS);
+    const int64_t tgt_tiles = (n + 2 * BT - 1) / (2 * BT);
+    // chunks: enough CTAs to fill the GPU several times over, at most 2,048
+    // sources summed in FP32
+    const int64_t S = std::max<int64_t>(1, ((int64_t)h->sm_count * 8 + tgt_tiles - 1) / tgt_tiles);
+    const int tiles_per_chunk = (int)std::max<int64_t>(1, std::min<int64_t>(2048 / TS, (n_tiles + S - 1) / S));
+    const int n_chunks = (n_tiles + tiles_per_chunk - 1) / tiles_per_chunk;
+    float *rec, *partial = nullptr;
+    double* scale;
+    RPBD_TRY(ensure_t(h, BUF_PACK, (size_t)n_pad * LEN, &rec));
+    RPBD_TRY(ensure_t(h, BUF_SCALE, (size_t)n_pad, &scale));
+    const bool fixed = !h->sym_partials;
+    FixedAcc fx{nullptr, nullptr, PER ? 36.0 : 4.0};
+    if (fixed) {
+        RPBD_TRY(ensure_t(h, BUF_PARTIAL, (size_t)3 * K * n_pad + 1, &fx.acc));
+        RPBD_CU(h, cudaMemsetAsync(fx.acc, 0, sizeof(unsigned long long) * (3 * K * n_pad + 1), st));
+        fx.fmax_bits = reinterpret_cast<unsigned*>(fx.acc + 3 * K * n_pad);
+    } else {
+        RPBD_TRY(ensure_t(h, BUF_PARTIAL, (size_t)n_chunks * 3 * K * n_pad, &partial));
+    }
+    pack_kernel<K, In><<<(unsigned)((n_pad + 127) / 128), 128, 0, st>>>(n, n_pad, k, r, F, h->p.a, 1.0 / h->p.a, h->p.s_min,
+                                                                        rec, scale, fx.fmax_bits);
+    count_launch();
+    auto kern = fixed ? pair_kernel<K, PER, true, MINB> : pair_kernel<K, PER, false, MINB>;
+    const size_t smem = (size_t)NST * TS * LEN * sizeof(float) + NST * sizeof(uint64_t);
+    if (once_per_device(h, reinterpret_cast<const void*>(kern)))
+        RPBD_CU(h, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (h->profile) prof_begin(h, st);
+    launch_pdl(kern, dim3((unsigned)tgt_tiles, (unsigned)n_chunks), BT, smem, st, rec, n, n_pad, tiles_per_chunk, n_tiles,
+               (float)(h->p.Lx / h->p.a), (float)(h->p.Ly / h->p.a), partial, h->dev_flag, ring_test(h), fx);
+    count_launch();
+    if (h->profile) prof_end(h, st, RPBD_F32, K, (double)n * (double)n);
+    RPBD_LAUNCH_CHECK(h);
+    // blocks were formed in units of a: M = M(a = 1) / a
+    const double inv8pieta = 1.0 / (8.0 * 3.14159265358979323846 * h->p.eta * h->p.a);
+    const dim3 rgrid((unsigned)((n + 255) / 256), (unsigned)(3 * k));
+    if (fixed)
+        finish_fixed_kernel<Out><<<rgrid, 256, 0, st>>>(n, n_pad, k, fx.cap, fx.acc, fx.fmax_bits, scale, inv8pieta, U);
+    else
+        reduce_kernel<float, Out><<<rgrid, 256, 0, st>>>(n, n_pad, k, K, n_chunks, partial, scale, inv8pieta, U);
+    count_launch();
+    RPBD_LAUNCH_CHECK(h);
+    return RPBD_OK;
+}
+
+template <class In, class Out>
+static int dispatch(rpbd_handle* h, int64_t n, const double* r, const In* F, Out* U, int k, cudaStream_t st)
+{
+    if (h->p.Lx > 0.0) return k <= 8 ? apply<8, true>(h, n, r, F, U, k, st) : apply<16, true>(h, n, r, F, U, k, st);
+    return k <= 8 ? apply<8, false>(h, n, r, F, U, k, st) : apply<16, false>(h, n, r, F, U, k, st);
+}
+
+}  // namespace wide
+
 template <class R, bool WALL, bool PER, class In, class Out>
 static int apply_dispatch(rpbd_handle* h, int64_t n, const double* r, const In* F, Out* U, int k, cudaStream_t st)
 {
@@ -563,6 +831,10 @@ int mobility_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* 
     // targets per thread) for k = 1, 3, 4; k = 2 keeps its own K = 2 tile
     if (dtype == RPBD_F32 && h->use_packed && h->p.wall && !(h->p.Lx > 0.0) && k <= 4 && k != 2)
         return single_packed_apply_impl(h, n, r, F, U, k, io_double, st);
+    if (dtype == RPBD_F32 && h->use_packed && h->p.wall && k > 4) {
+        if (io_double) return wide::dispatch(h, n, r, (const double*)F, (double*)U, k, st);
+        return wide::dispatch(h, n, r, (const float*)F, (float*)U, k, st);
+    }
     // FP64: the symmetric kernel; the one-direction kernel for many right-hand
     // sides and for systems whose partials would not fit
     if (dtype == RPBD_F64 && sym64_takes(h, n, k))

@@ -99,3 +99,20 @@ def test_adjoint_tiles(n, wall, cell):
         for dtype, tol in ((F64, 1e-11), (F32, 1e-5)):
             g = h.mobility_adjoint(to_dev(r), to_dev(u), to_dev(F), dtype=dtype).cpu().numpy()
             assert np.linalg.norm(g[:, rows] - go) <= tol * np.linalg.norm(go)  # (a lone unbounded blob has none)
+
+
+# two targets per thread (256 a CTA), 64 sources a stage
+@pytest.mark.parametrize("n", [1, 63, 65, 128, 129, 257, 2113])
+@pytest.mark.parametrize("cell", [0.0, CELL])
+def test_f32_many_right_hand_sides(n, cell):
+    r = cloud(n, 750 + n, cell or None)
+    h = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT, Lx=cell, Ly=cell)
+    prm = om.Params(synth.ETA, synth.A_BOOMERANG, Lx=cell, Ly=cell)
+    rows = rows_of(n)
+    for k in (5, 8, 9, 16):
+        F = synth.gaussian(751 + k, (k, 3, n), np.float32)
+        ref = om.apply(r, F.astype(np.float64), prm, rows)
+        for partials in (False, True):
+            h.set_sym_partials(partials)
+            U = h.mobility_apply(to_dev(r), to_dev(F, torch.float32)).cpu().numpy()
+            assert rel2(U[:, :, rows], ref) <= 1e-5
