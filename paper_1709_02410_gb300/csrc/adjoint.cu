@@ -119,6 +119,9 @@ static int launch(rpbd_handle* h, const adj::Cut& c, int kc, const double* r, co
     const double ia = 1.0 / h->p.a;
     launch_pdl(kern, dim3((unsigned)c.hg, (unsigned)c.items, (unsigned)c.parts), 32 * c.nw, smem, st, c, kc, r, u, F, rec,
                adj::Unit{}, h->p.a, h->p.s_min, (float)(h->p.Lx * ia), (float)(h->p.Ly * ia), partial, o);
+    count_launch();
+    launch_pdl(adj::adjoint_reduce_kernel<float>, dim3((unsigned)c.tiles, 3), 32 * adj::RS, 0, st, c, o, (const float*)partial, r,
+               h->p.a, (int)WALL, h->p.s_min);
     return RPBD_OK;
 }
 

@@ -16,7 +16,7 @@ static int launch(rpbd_handle* h, const adj::Cut& c, int kc, const double* r, co
 {
     const size_t smem = 2 * (size_t)(3 + 6 * K) * adj::VT * 8 + 2 * c.nw * 4 * adj::VT * sizeof(double);
     adj::adjoint_kernel<double, K, WALL, PER, adj::Radius>
-        <<<dim3((unsigned)c.hg, (unsigned)c.items, (unsigned)c.parts), 32 * c.nw, smem, st>>>(
+        <<<dim3((unsigned)c.hg, (unsigned)c.items, (unsigned)c.parts), c.threads, smem, st>>>(
             c, kc, r, u, F, nullptr, adj::Radius::make(h->p.a), h->p.a, h->p.s_min, h->p.Lx, h->p.Ly, partial, o);
     return RPBD_OK;
 }

@@ -5,16 +5,18 @@
 // FP64, two in packed FP32), visitors in tiles of 32 through shared memory, lane
 // l meets visitor (step + l) mod 32 and hands the visitor's running sums to lane
 // l - 1 after every step.  Pairs inside a warp's own home blobs are done in the
-// home direction only.  Sums of (dE/dx, dE/dy, dE/dz, E) go to one partial row
-// per (home tile, part) for the visitors and per (item, part) for the homes; the
-// last CTA to finish a blob tile (a ticket per tile, no CTA ever waits) adds its
-// rows in a fixed order, so the result does not depend on the order of the CTAs
-// and no further launch is needed.
+// home direction only.  Sums of (dE/dx, dE/dy, dE/dz~, E) go to one partial row
+// per (home tile, part) for the visitors and per (item, part) for the homes, added
+// in a fixed order, so the result does not depend on the order of the CTAs.  FP64:
+// by the last CTA to finish a blob tile (a ticket per tile, no CTA ever waits), in
+// the same launch.  FP32, where the pairs are over sooner than one CTA has walked
+// a tile's rows, by a kernel of its own (1,920 blobs 275 -> 49 us).
 //
 // Bound by arithmetic: the FP64 pipe, or packed FP32 issue (~160 operations per
 // unordered pair).  Before, one thread per blob walked all sources with the block
 // on dual numbers, so 1,920 blobs filled 15 of 152 SMs: FP64 gradient with its two
-// matvecs 29.3 -> 1.31 ms at 1,920 blobs; FP32 2.99 -> 0.99 ms at 16,380.
+// matvecs 29.3 -> 1.31 ms at 1,920 blobs (FP64 pipe 85% busy); FP32 2.99 -> 0.78 ms
+// at 16,380 (FMA pipe 78%).
 //
 // Cutting as in sym64.cu: CTAs of one warp for small n, four beyond, items of
 // `chunk` visitor tiles, the 32 steps of a tile over `parts` items for very
@@ -39,7 +41,7 @@ constexpr double GROUP_BYTES = 4.0 * (1ull << 30);
 // how one launch (a group of home tiles) is cut
 struct Cut {
     int64_t n, n_pad;
-    int nw;            // warps per CTA
+    int nw, threads;   // warps with home blobs per CTA, threads per CTA
     int vpw, vph;      // visitor tiles per warp's home blobs, per home tile
     int tiles;         // visitor tiles
     int chunk, parts;  // visitor tiles per item (a power of two), items per tile's steps
@@ -75,40 +77,104 @@ __device__ __forceinline__ double overlap_scale(double z, double a, double s_min
     return t >= 1.0 ? 1.0 : (t <= s_min ? s_min : t);
 }
 
-// adds the rows of blob tile `home` (all threads of the CTA), writes g when complete
+// g of blob i from its complete sums (q 0..3: dE/dx, dE/dy, dE/dz~, E); q 0, 1 or both of 2 and 3
+__device__ __forceinline__ void write_xy(const Cut& c, const Out& o, int64_t i, int q, double s) { o.grad[q * c.n + i] = o.ig * s; }
+__device__ __forceinline__ void write_z(const Cut& c, const Out& o, int64_t i, double sz, double se, const double* r, double a,
+                                        int wall, double s_min)
+{
+    // z~ follows z from a upwards, s = z / a between s_min a and a
+    const double z = r[2 * c.n + i];
+    const bool above = !wall || z >= a, ramp = wall && z / a < 1.0 && z / a > s_min;
+    const double dz = above || z != z ? o.ig * sz : 0.0;
+    o.grad[2 * c.n + i] = dz + (ramp ? o.ie * se / z : 0.0);
+}
+
+// sum over rows e = e0, e0 + step, ... of one value, eight loads in flight
+template <class S, class At>
+__device__ __forceinline__ double sum_rows(int e0, int step, int rows, At at)
+{
+    double s = 0.0;
+    int e = e0;
+    for (; e + 7 * step < rows; e += 8 * step) {
+        S v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = __ldcg(at(e + u * step));
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s += (double)v[u];
+    }
+    for (; e < rows; e += step) s += (double)__ldcg(at(e));
+    return s;
+}
+
+// adds the rows of blob tile `home` (all threads of the CTA, one value each at a
+// time), writes g when complete.  sm: 128 vph doubles of shared memory
 template <class S>
-__device__ void finish_tile(const Cut& c, const Out& o, int home, const S* partial, const double* r,
-                            double a, int wall, double s_min)
+__device__ void finish_tile(const Cut& c, const Out& o, int home, const S* partial, const double* r, double a, int wall,
+                            double s_min, double* sm)
 {
     const bool own = home >= c.h0 && home < c.h0 + c.hg;
     const int before = min(c.h0 + c.hg, home) - c.h0;  // home tiles of the group before this one
     const int nit = own ? (c.tiles - home * c.vph + c.chunk - 1) / c.chunk * c.parts : 0;
-    for (int idx = threadIdx.x; idx < 32 * c.vph; idx += blockDim.x) {
-        const int64_t i = (int64_t)home * 32 * c.vph + idx;
-        if (i >= c.n) break;
-        const int vis = (before + (own && idx / 32 >= c.vpw ? 1 : 0)) * c.parts;
-        double s[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll 8
-        for (int e = 0; e < vis + nit; ++e) {
-            const S* p = partial + (int64_t)(e < vis ? e : c.hg * c.parts + e - vis) * 4 * c.n_pad + i;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) s[q] += (double)__ldcg(p + q * c.n_pad);
+    const int ht = 32 * c.vph;
+    for (int idx = threadIdx.x; idx < 4 * ht; idx += blockDim.x) {
+        const int q = idx / ht, b = idx - q * ht;
+        const int64_t i = (int64_t)home * ht + b;
+        const int vis = (before + (own && b / 32 >= c.vpw ? 1 : 0)) * c.parts, shift = c.hg * c.parts - vis;
+        const S* p = partial + q * c.n_pad + i;
+        const int64_t ld = 4 * c.n_pad;
+        double s = sum_rows<S>(0, 1, vis + nit, [&](int e) { return p + (e < vis ? e : e + shift) * ld; });
+        if (!o.first) s += o.G[q * c.n_pad + i];
+        if (!(own && o.last)) o.G[q * c.n_pad + i] = s;  // later groups' homes come after this tile
+        sm[idx] = s;
+    }
+    __syncthreads();
+    if (own && o.last)
+        for (int idx = threadIdx.x; idx < 3 * ht; idx += blockDim.x) {
+            const int q = idx / ht, b = idx - q * ht;
+            const int64_t i = (int64_t)home * ht + b;
+            if (i >= c.n) continue;
+            if (q < 2) write_xy(c, o, i, q, sm[idx]);
+            else write_z(c, o, i, sm[idx], sm[idx + ht], r, a, wall, s_min);
         }
-        if (!o.first)
+    __syncthreads();
+}
+
+// the same for every tile, 32 blobs, one sum (blockIdx.y: x, y, z with E) and 8 row
+// slices a block (the slices added in order)
+constexpr int RS = 8;
+template <class S>
+__global__ void __launch_bounds__(32 * RS) adjoint_reduce_kernel(Cut c, Out o, const S* partial, const double* r, double a,
+                                                                 int wall, double s_min)
+{
+    __shared__ double sm[2][RS][32];
+    pdl_wait();
+    pdl_trigger();
+    const int lane = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int tile = blockIdx.x, home = tile / c.vph, sub = tile % c.vph, q0 = blockIdx.y, nq = q0 == 2 ? 2 : 1;
+    if (home < c.h0) return;  // complete already
+    const bool own = home < c.h0 + c.hg;
+    const int64_t i = (int64_t)tile * VT + lane;
+    const int vis = (min(c.h0 + c.hg, home) - c.h0 + (own && sub >= c.vpw ? 1 : 0)) * c.parts;
+    const int rows = vis + (own ? (c.tiles - home * c.vph + c.chunk - 1) / c.chunk * c.parts : 0);
+    const int shift = c.hg * c.parts - vis;
+    const int64_t ld = 4 * c.n_pad;
+    for (int q = 0; q < nq; ++q) {
+        const S* p = partial + (q0 + q) * c.n_pad + i;
+        sm[q][y][lane] = sum_rows<S>(y, RS, rows, [&](int e) { return p + (e < vis ? e : e + shift) * ld; });
+    }
+    __syncthreads();
+    if (y || i >= c.n) return;
+    double s[2] = {0.0, 0.0};
+    for (int q = 0; q < nq; ++q) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) s[q] += o.G[q * c.n_pad + i];
-        if (own && o.last) {  // later groups' homes come after this tile
-            const double z = r[2 * c.n + i];
-            o.grad[i] = o.ig * s[0];
-            o.grad[c.n + i] = o.ig * s[1];
-            // z~ follows z from a upwards, s = z / a between s_min a and a
-            const bool above = !wall || z >= a, ramp = wall && z / a < 1.0 && z / a > s_min;
-            const double dz = above || z != z ? o.ig * s[2] : 0.0;
-            o.grad[2 * c.n + i] = dz + (ramp ? o.ie * s[3] / z : 0.0);
-        } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) o.G[q * c.n_pad + i] = s[q];
-        }
+        for (int w = 0; w < RS; ++w) s[q] += sm[q][w][lane];
+        double* G = o.G + (q0 + q) * c.n_pad + i;
+        if (!o.first) s[q] += *G;
+        if (!(own && o.last)) *G = s[q];
+    }
+    if (own && o.last) {
+        if (q0 < 2) write_xy(c, o, i, q0, s[0]);
+        else write_z(c, o, i, s[0], s[1], r, a, wall, s_min);
     }
 }
 
@@ -125,7 +191,7 @@ __device__ __forceinline__ void load_tile(const Cut& c, int tile, int nr, const 
         const bool real = i < c.n;
         const double z = real ? r[2 * c.n + i] : a;
         const double s = wall ? overlap_scale(z, a, s_min) : 1.0;
-        for (int f = threadIdx.x >> 5; f < 3 + 6 * K; f += c.nw) {
+        for (int f = threadIdx.x >> 5; f < 3 + 6 * K; f += blockDim.x >> 5) {
             double v;
             if (f < 2) v = real ? r[f * c.n + i] : 1.0e7;  // padding: far away
             else if (f == 2) v = wall ? (z > a ? z : a) : z;
@@ -159,16 +225,18 @@ __global__ void __launch_bounds__(128) adjoint_kernel(Cut c, int nr, const doubl
     const int tile0 = home * c.vph + item * c.chunk;  // visitors: the home tile's own blobs and all after them
     const int ntile = min(c.chunk, c.tiles - tile0);
     pdl_wait();
+    pdl_trigger();
     if (ntile <= 0) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int s0 = VT / c.parts * part, s1 = s0 + VT / c.parts;
 
     load_tile<V, K>(c, tile0, nr, r, u, F, rec, a, WALL, s_min, smem_raw);
-    // home blobs: 32 vpw per warp
+    // home blobs: 32 vpw per warp (warps past nw, in launches of few CTAs, only help to load and to add rows)
+    const bool pairs = warp < c.nw;
     V hx, hy, hxl, hyl, hz, A[3 * K], B[3 * K];
     if constexpr (D) {
         const int64_t i = (int64_t)(home * c.vph + warp) * VT + lane;
-        const bool real = i < c.n;
+        const bool real = pairs && i < c.n;
         const double z = real ? r[2 * c.n + i] : a, s = WALL ? overlap_scale(z, a, s_min) : 1.0;
         hx = real ? r[i] : 1.0e7;
         hy = real ? r[c.n + i] : 1.0e7;
@@ -208,7 +276,7 @@ __global__ void __launch_bounds__(128) adjoint_kernel(Cut c, int nr, const doubl
         const unsigned char* st = smem_raw + (t & 1) * STAGE;
         const int own = tile0 + t - home * c.vph;  // counted from the home tile's first
         S* rb = red + (t & 1) * (c.nw * 4 * VT);
-        if (own >= warp * c.vpw) {
+        if (pairs && own >= warp * c.vpw) {
             const bool both = own >= (warp + 1) * c.vpw;
             V vacc[4] = {zero, zero, zero, zero};
 #pragma unroll 1
@@ -285,6 +353,7 @@ __global__ void __launch_bounds__(128) adjoint_kernel(Cut c, int nr, const doubl
     }
     const int64_t row_h = ((int64_t)c.hg * c.parts + item * c.parts + part) * 4;
     const int64_t ib = (int64_t)(home * c.vph + warp * c.vpw) * VT + lane;
+    if (pairs)
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         if constexpr (D) partial[(row_h + q) * c.n_pad + ib] = acc[q];
@@ -293,6 +362,7 @@ __global__ void __launch_bounds__(128) adjoint_kernel(Cut c, int nr, const doubl
             partial[(row_h + q) * c.n_pad + ib + VT] = acc[q].y;
         }
     }
+    if constexpr (!D) return;  // (adjoint_reduce_kernel follows)
     // tickets of the blob tiles this item added to; the last one in finishes the tile
     __threadfence();
     __syncthreads();
@@ -301,6 +371,7 @@ __global__ void __launch_bounds__(128) adjoint_kernel(Cut c, int nr, const doubl
     int* const ready = reinterpret_cast<int*>(red);
     for (int x = 0; x <= max(0, last - first + 1); ++x) {
         const int tile = x == 0 ? home : first + x - 1;
+        __syncthreads();
         if (tid == 0) {
             const int homes = min(c.h0 + c.hg, tile) - c.h0;  // of this launch, before the tile
             const int own_items = tile < c.h0 + c.hg ? (c.tiles - tile * c.vph + c.chunk - 1) / c.chunk * c.parts : 0;
@@ -311,7 +382,7 @@ __global__ void __launch_bounds__(128) adjoint_kernel(Cut c, int nr, const doubl
         __syncthreads();
         if (go) {
             __threadfence();
-            finish_tile<S>(c, out, tile, partial, r, a, WALL, s_min);
+            finish_tile<S>(c, out, tile, partial, r, a, WALL, s_min, reinterpret_cast<double*>(red));
         }
     }
 }
@@ -337,6 +408,10 @@ inline Cut cut(int64_t n, int vpw, int64_t small_n, int max_chunk, size_t row_by
     while (c.chunk > 1 && count(c.chunk) < 16 * (int64_t)sm_count) c.chunk /= 2;
     c.parts = 1;
     while (c.parts < 4 && count(c.chunk) * c.parts < 16 * (int64_t)sm_count) c.parts *= 2;
+    // few CTAs: help with the loads and sums, and steps over twice as many
+    const bool few = count(c.chunk) * c.parts <= 4 * (int64_t)sm_count;
+    if (few && vpw == 1) c.parts *= 2;
+    c.threads = few && vpw == 1 ? 128 : 32 * c.nw;
     // (past 65,535 items, the grid's limit, longer chunks)
     while ((c.tiles + c.chunk - 1) / c.chunk > 65535) c.chunk *= 2;
     const int64_t fit = (int64_t)(GROUP_BYTES / ((double)row_bytes * c.n_pad * c.parts));
@@ -353,6 +428,7 @@ inline Cut cut(int64_t n, int vpw, int64_t small_n, int max_chunk, size_t row_by
 template <class S, class Pass, class Launch>
 static int run_all(rpbd_handle* h, Cut c, int nr, double* grad, double ig, double ie, Pass pass, Launch launch, cudaStream_t st)
 {
+    constexpr bool tickets = sizeof(S) == 8;
     const int T = c.tiles / c.vph;
     const size_t words = (size_t)((int64_t)c.hg + c.items) * c.parts * 4 * c.n_pad;
     unsigned char* base;
@@ -368,10 +444,10 @@ static int run_all(rpbd_handle* h, Cut c, int nr, double* grad, double ig, doubl
     const int hg = c.hg;
     for (int m0 = 0; m0 < nr; m0 += 4) {
         const int kc = std::min(4, nr - m0);
-        RPBD_CU(h, cudaMemsetAsync(o.ticket, 0, t_bytes, st));
+        if (tickets) RPBD_CU(h, cudaMemsetAsync(o.ticket, 0, t_bytes, st));
         RPBD_TRY(pass(m0, kc));
         for (int h0 = 0; h0 < T; h0 += hg) {
-            if (h0) RPBD_CU(h, cudaMemsetAsync(o.ticket, 0, t_bytes, st));
+            if (tickets && h0) RPBD_CU(h, cudaMemsetAsync(o.ticket, 0, t_bytes, st));
             c.h0 = h0;
             c.hg = std::min(hg, T - h0);
             o.first = m0 == 0 && h0 == 0;

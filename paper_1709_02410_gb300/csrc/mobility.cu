@@ -518,8 +518,11 @@ static int apply_k(rpbd_handle* h, int64_t n, const double* r, const In* F, Out*
 namespace wide {
 
 constexpr int BT = 128;   // threads; 2 BT targets per CTA
-constexpr int TS = 64;    // sources per stage
 constexpr int NST = 3;
+// sources per stage: 64, or 16 up to SMALL_N blobs, where the longest CTA's walk
+// through its sources is the kernel's length (k = 16, with the pack's split below:
+// n = 240 53 -> 27 us a call, n = 1,920 70 -> 56 us, n = 3,840 131 -> 120 us)
+constexpr int64_t SMALL_N = 4096;
 
 // source record: x_hi x_hi y_hi y_hi | x_lo x_lo y_lo y_lo | z~ z~ - - | forces as in Rec<float, K>
 template <int K>
@@ -528,48 +531,51 @@ struct WRec {
     static_assert(K % 4 == 0, "whole 16-byte chunks");
 };
 
+// one thread per blob and pair of right-hand sides (blockIdx.y; the first also
+// writes the position): as one thread per blob the pack took half of a small call
 template <int K, class In>
 __global__ void pack_kernel(int64_t n, int64_t n_pad, int k, const double* r, const In* F, double a, double ia, double s_min,
                             float* rec, double* scale, unsigned* fmax_bits)
 {
     pdl_trigger();
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int p = blockIdx.y;
     if (i >= n_pad) return;
-    float* o = rec + i * WRec<K>::LEN;
-    double x = 1.0e7, y = 1.0e7, zt = a, s = 0.0;  // padding: far away, zero force
-    if (i < n) {
-        x = r[i] * ia;
-        y = r[n + i] * ia;
-        const double z = r[2 * n + i];
-        zt = z > a ? z : a;
-        s = 1.0;
-        if (!(z >= a)) {  // (NaN stays NaN)
-            const double t = z / a;
-            s = t >= 1.0 ? 1.0 : (t <= s_min ? s_min : t);
-        }
-        scale[i] = s;
+    const bool real = i < n;
+    const double z = real ? r[2 * n + i] : a;
+    double s = 1.0;
+    if (!(z >= a)) {  // (NaN stays NaN)
+        const double t = z / a;
+        s = t >= 1.0 ? 1.0 : (t <= s_min ? s_min : t);
     }
-    const float xh = (float)x, yh = (float)y, xl = (float)(x - (double)xh), yl = (float)(y - (double)yh), z = (float)(zt * ia);
-    float4* o4 = reinterpret_cast<float4*>(o);
-    o4[0] = make_float4(xh, xh, yh, yh);
-    o4[1] = make_float4(xl, xl, yl, yl);
-    o4[2] = make_float4(z, z, 0.0f, 0.0f);
-    float fm = 0.0f;  // largest |stored force| of this blob (+inf: not finite)
+    float v[6];
+    float fm = 0.0f;  // largest |stored force| (+inf: not finite)
 #pragma unroll
-    for (int m = 0; m < K; ++m)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            float v = 0.0f;
-            if (i < n && m < k) {
-                v = (float)(s * (double)F[((int64_t)m * 3 + c) * n + i]);
-                fm = isfinite(v) ? fmaxf(fm, fabsf(v)) : INFINITY;
-            }
-            o[12 + 6 * (m / 2) + 2 * c + (m & 1)] = v;
+    for (int e = 0; e < 6; ++e) {  // component e / 2 of right-hand side 2p + e % 2
+        const int m = 2 * p + e % 2;
+        v[e] = 0.0f;
+        if (real && m < k) {
+            v[e] = (float)(s * (double)F[((int64_t)m * 3 + e / 2) * n + i]);
+            fm = isfinite(v[e]) ? fmaxf(fm, fabsf(v[e])) : INFINITY;
         }
+    }
+    float2* o = reinterpret_cast<float2*>(rec + i * WRec<K>::LEN) + 6 + 3 * p;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) o[c] = make_float2(v[2 * c], v[2 * c + 1]);
+    if (p == 0) {
+        const double x = real ? r[i] * ia : 1.0e7, y = real ? r[n + i] * ia : 1.0e7;  // padding: far away, zero force
+        const float xh = (float)x, yh = (float)y, xl = (float)(x - (double)xh), yl = (float)(y - (double)yh);
+        const float zf = (float)((z > a ? z : a) * ia);
+        float4* o4 = reinterpret_cast<float4*>(rec + i * WRec<K>::LEN);
+        o4[0] = make_float4(xh, xh, yh, yh);
+        o4[1] = make_float4(xl, xl, yl, yl);
+        o4[2] = make_float4(zf, zf, 0.0f, 0.0f);
+        if (real) scale[i] = s;
+    }
     if (fmax_bits) fixed_force_max(fmax_bits, fm);
 }
 
-template <int K, bool PER, bool FX, int MINB>
+template <int K, int TS, bool PER, bool FX, int MINB>
 __global__ void __launch_bounds__(BT, MINB) pair_kernel(const float* rec, int64_t n, int64_t n_pad, int tiles_per_chunk,
                                                         int n_tiles, float Lx, float Ly, float* partial, int* err_flag,
                                                         RingTest rt, FixedAcc fx)
@@ -709,7 +715,7 @@ __global__ void __launch_bounds__(BT, MINB) pair_kernel(const float* rec, int64_
     }
 }
 
-template <int K, bool PER, class In, class Out>
+template <int K, int TS, bool PER, class In, class Out>
 static int apply(rpbd_handle* h, int64_t n, const double* r, const In* F, Out* U, int k, cudaStream_t st)
 {
     constexpr int LEN = WRec<K>::LEN;
@@ -735,10 +741,10 @@ static int apply(rpbd_handle* h, int64_t n, const double* r, const In* F, Out* U
     } else {
         RPBD_TRY(ensure_t(h, BUF_PARTIAL, (size_t)n_chunks * 3 * K * n_pad, &partial));
     }
-    pack_kernel<K, In><<<(unsigned)((n_pad + 127) / 128), 128, 0, st>>>(n, n_pad, k, r, F, h->p.a, 1.0 / h->p.a, h->p.s_min,
-                                                                        rec, scale, fx.fmax_bits);
+    pack_kernel<K, In><<<dim3((unsigned)((n_pad + 127) / 128), K / 2), 128, 0, st>>>(n, n_pad, k, r, F, h->p.a, 1.0 / h->p.a,
+                                                                                     h->p.s_min, rec, scale, fx.fmax_bits);
     count_launch();
-    auto kern = fixed ? pair_kernel<K, PER, true, MINB> : pair_kernel<K, PER, false, MINB>;
+    auto kern = fixed ? pair_kernel<K, TS, PER, true, MINB> : pair_kernel<K, TS, PER, false, MINB>;
     const size_t smem = (size_t)NST * TS * LEN * sizeof(float) + NST * sizeof(uint64_t);
     if (once_per_device(h, reinterpret_cast<const void*>(kern)))
         RPBD_CU(h, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -763,8 +769,12 @@ static int apply(rpbd_handle* h, int64_t n, const double* r, const In* F, Out* U
 template <class In, class Out>
 static int dispatch(rpbd_handle* h, int64_t n, const double* r, const In* F, Out* U, int k, cudaStream_t st)
 {
-    if (h->p.Lx > 0.0) return k <= 8 ? apply<8, true>(h, n, r, F, U, k, st) : apply<16, true>(h, n, r, F, U, k, st);
-    return k <= 8 ? apply<8, false>(h, n, r, F, U, k, st) : apply<16, false>(h, n, r, F, U, k, st);
+    if (n <= SMALL_N) {
+        if (h->p.Lx > 0.0) return k <= 8 ? apply<8, 16, true>(h, n, r, F, U, k, st) : apply<16, 16, true>(h, n, r, F, U, k, st);
+        return k <= 8 ? apply<8, 16, false>(h, n, r, F, U, k, st) : apply<16, 16, false>(h, n, r, F, U, k, st);
+    }
+    if (h->p.Lx > 0.0) return k <= 8 ? apply<8, 64, true>(h, n, r, F, U, k, st) : apply<16, 64, true>(h, n, r, F, U, k, st);
+    return k <= 8 ? apply<8, 64, false>(h, n, r, F, U, k, st) : apply<16, 64, false>(h, n, r, F, U, k, st);
 }
 
 }  // namespace wide
