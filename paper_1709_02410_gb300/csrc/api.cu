@@ -372,11 +372,31 @@ int rpbd_autotune(rpbd_handle* h, int64_t n, const double* r, int k, double* bes
             best_c = c;
         }
     }
+    // a small system's default is a kernel of its own (direct.cu), not one of the variants: kept
+    // where it is the fastest, as the variant that the default would be for larger systems
+    bool keep_default = false;
+    if (nsym == 6 && direct_takes(h, n, k) && !h->sym_partials && !h->far_field) {
+        h->use_sym[cls] = 1;
+        h->sym_variant[cls] = -1;
+        int s = mobility_apply_impl(h, n, r, F, U, k, RPBD_F32, false, st);
+        if (s != RPBD_OK) { h->profile = prof; return s; }
+        RPBD_CU(h, cudaEventRecord(e0, st));
+        for (int rep = 0; rep < 2; ++rep) RPBD_TRY(mobility_apply_impl(h, n, r, F, U, k, RPBD_F32, false, st));
+        RPBD_CU(h, cudaEventRecord(e1, st));
+        RPBD_CU(h, cudaEventSynchronize(e1));
+        float ms = 0.0f;
+        RPBD_CU(h, cudaEventElapsedTime(&ms, e0, e1));
+        if (ms / 2.0 < best) {
+            best = ms / 2.0;
+            best_c = h->p.Lx > 0.0 ? 1 : 3;
+            keep_default = true;
+        }
+    }
     h->profile = prof;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     h->use_sym[cls] = best_c >= 0;
-    h->sym_variant[cls] = best_c >= 0 ? best_c : -1;
+    h->sym_variant[cls] = best_c >= 0 && !keep_default ? best_c : -1;
     if (best_ms) *best_ms = best;
     return best_c + 1;
 }

@@ -835,6 +835,12 @@ int mobility_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* 
     // the packed symmetric kernel takes any n (past the partials' limit it sums in FP64
     // atomics); the one-home kernel only while its partials fit
     const bool packed_sym = h->use_packed && h->p.wall;
+    // a small system on the default settings: one launch (the failure-path test
+    // wants the bounded waits of the ring kernels, the partials option their
+    // partials, a chosen variant that variant)
+    if (dtype == RPBD_F32 && packed_sym && k <= 4 && h->use_sym[sym_class(k)] && h->sym_variant[sym_class(k)] < 0 &&
+        !h->sym_partials && !h->test_stall && direct_takes(h, n, k))
+        return direct_apply_impl(h, n, r, F, U, k, io_double, st);
     if (dtype == RPBD_F32 && k <= 4 && h->use_sym[sym_class(k)] && (packed_sym || sym_bytes <= 16.0 * (1ull << 30)))
         return sym_apply_impl(h, n, r, F, U, k, io_double, st);
     // one direction with the wall in the open cell: the packed tile (two

@@ -267,6 +267,10 @@ int precond_build_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, co
 int sym_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* F, void* U, int k, bool io_double,
                    cudaStream_t st);
 
+// FP32 matvec of a small system in one launch: whether it takes (n, k), and the matvec itself
+bool direct_takes(const rpbd_handle* h, int64_t n, int k);
+int direct_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* F, void* U, int k, bool io_double, cudaStream_t st);
+
 // symmetric FP64 matvec: whether it takes (n, k), and the matvec itself
 bool sym64_takes(const rpbd_handle* h, int64_t n, int k);
 int sym64_apply_impl(rpbd_handle* h, int64_t n, const double* r, const double* F, double* U, int k, cudaStream_t st);

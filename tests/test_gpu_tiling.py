@@ -34,12 +34,15 @@ def rows_of(n):
     return np.unique(np.concatenate([e, np.linspace(0, n - 1, 40).astype(int)]))
 
 
-# 8,704 = 34 home tiles of 256: the last size with one visitor tile per item
-@pytest.mark.parametrize("n", [1, 2, 31, 33, 64, 255, 257, 513, 8704, 8993])
+# 8,704 = 34 home tiles of 256: the last size with one visitor tile per item; variant 3: those kernels below
+# 960 blobs too, where the default is one launch (640 with three or four right-hand sides)
+@pytest.mark.parametrize("n,variant", [(n, v) for v in (-1, 3) for n in (1, 2, 31, 33, 64, 255, 257, 513, 8704, 8993)
+                                       if v == -1 or n < 8000] + [(n, -1) for n in (304, 305, 609, 640, 641, 960, 961)])
 @pytest.mark.parametrize("cell", [0.0, CELL])
-def test_f32_symmetric_tiles(n, cell):
+def test_f32_symmetric_tiles(n, variant, cell):
     r = cloud(n, 700 + n, cell or None)
     h = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT, Lx=cell, Ly=cell)
+    h.set_sym_variant(variant)
     prm = om.Params(synth.ETA, synth.A_BOOMERANG, Lx=cell, Ly=cell)
     rows = rows_of(n)
     for k in (1, 2, 3):
@@ -51,13 +54,16 @@ def test_f32_symmetric_tiles(n, cell):
 def test_accumulators_are_cleared_between_calls():
     """One handle, calls of other sizes, right-hand sides and a non-finite force between: every result as on a fresh handle."""
     h = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT)
+    h.set_sym_variant(3)  # (small systems default to a kernel without accumulators)
     for n, k, bad in ((700, 2, False), (300, 1, True), (300, 1, False), (1100, 4, False), (40, 1, False), (700, 2, False)):
         r, F = cloud(n, 710), synth.gaussian(711, (k, 3, n), np.float32)
         if bad:
             F[0, 1, 7] = np.inf
         args = to_dev(r), to_dev(F, torch.float32)
         U = h.mobility_apply(*args)
-        fresh = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT).mobility_apply(*args)
+        g = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT)
+        g.set_sym_variant(3)
+        fresh = g.mobility_apply(*args)
         assert torch.isnan(U).all() if bad else torch.equal(U, fresh)
 
 
@@ -116,3 +122,11 @@ def test_f32_many_right_hand_sides(n, cell):
             h.set_sym_partials(partials)
             U = h.mobility_apply(to_dev(r), to_dev(F, torch.float32)).cpu().numpy()
             assert rel2(U[:, :, rows], ref) <= 1e-5
+
+
+def test_small_system_non_finite_force():
+    """A force that is not finite makes every velocity NaN, as with the accumulators of larger systems."""
+    r, F = cloud(200, 760), synth.gaussian(761, (2, 3, 200), np.float32)
+    F[1, 2, 11] = np.inf
+    U = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT).mobility_apply(to_dev(r), to_dev(F, torch.float32))
+    assert torch.isnan(U).all()
