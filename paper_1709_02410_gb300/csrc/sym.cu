@@ -759,10 +759,11 @@ struct Sym2Var {
 // thread, 64 threads, so each visitor record loaded and each visitor sum
 // handed on serves twice the pairs).  Warp w owns homes [64 HP w, 64 HP (w+1))
 // of the tile; pair p of a thread holds homes 64 HP w + 64 p + lane (.x) and
-// that + 32 (.y).  FAR: the cancellation-free far-field block.  ATOM: the
+// that + 32 (.y).  PARTS: the item's steps (of every tile) are those of part
+// blockIdx.y of PARTS.  FAR: the cancellation-free far-field block.  ATOM: the
 // visitor and home sums go into the fixed-point accumulators (fx) instead of
 // the per-home-tile partials.
-template <int K, bool PER, int UNR, int MINB, bool BATCH, int HP = 1, bool FAR = false, bool ATOM = false>
+template <int K, bool PER, int UNR, int MINB, bool BATCH, int HP = 1, bool FAR = false, bool ATOM = false, int PARTS = 1>
 __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float* rec,
                                                               const SymItem* __restrict__ items, int64_t n,
                                                               int64_t n_pad, int n_home_tiles,
@@ -774,6 +775,8 @@ __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float*
     constexpr int NT = HT2 / (2 * HP);  // threads
     constexpr int NW = NT / 32;          // warps
     constexpr int LEN = Rec2<K>::LEN;
+    constexpr int STEPS = VT / PARTS;
+    const int s0 = PARTS > 1 ? STEPS * (int)blockIdx.y : 0;
     constexpr uint32_t TILE_BYTES = VT * LEN * sizeof(float);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float* stage = reinterpret_cast<float*>(smem_raw);
@@ -846,7 +849,7 @@ __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float*
         if (ok && diag) {
             // one direction, every lane on the same source (broadcast reads)
 #pragma unroll 2
-            for (int jj = 0; jj < VT; ++jj) {
+            for (int jj = s0; jj < s0 + STEPS; ++jj) {
                 float2 xh, yh, xl, yl, zj, f[3 * K];
                 load_rec2<K>(st, jj, xh, yh, xl, yl, zj, f);
 #pragma unroll
@@ -864,8 +867,8 @@ __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float*
 #pragma unroll
             for (int q = 0; q < 3 * K; ++q) vacc[q] = make_float2(0.0f, 0.0f);
 #pragma unroll UNR
-            for (int step = 0; step < VT; ++step) {
-                const int v = (step + lane) & (VT - 1);
+            for (int step = 0; step < STEPS; ++step) {
+                const int v = (s0 + step + lane) & (VT - 1);
                 float2 xh, yh, xl, yl, zj, f[3 * K];
                 load_rec2<K>(st, v, xh, yh, xl, yl, zj, f);
 #pragma unroll
@@ -882,10 +885,10 @@ __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float*
                     vacc[q].y = __shfl_sync(0xffffffffu, vacc[q].y, (lane + 1) & 31);
                 }
             }
-            // lane l now holds visitor l's sums over this warp's 64 HP homes
+            // lane l now holds the sums of visitor (l + s0 + STEPS) mod 32 over this warp's 64 HP homes
             float* rb = red + (t & 1) * (NW * VT * 3 * K);  // double-buffered: one barrier per tile
 #pragma unroll
-            for (int q = 0; q < 3 * K; ++q) rb[(warp * VT + lane) * 3 * K + q] = vacc[q].x + vacc[q].y;
+            for (int q = 0; q < 3 * K; ++q) rb[(warp * VT + ((lane + s0 + STEPS) & (VT - 1))) * 3 * K + q] = vacc[q].x + vacc[q].y;
         }
         if (__syncthreads_or(!ok)) {
             bad = true;
@@ -1237,6 +1240,22 @@ static int run2(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, 
     } else if (!atom) {  // per-home-tile partials and the fixed-order reduction: the default variant
         RPBD_SYM2_LAUNCH(PER ? 1 : (K == 1 ? 3 : (K == 2 ? 5 : 4)), false, false);
     } else {
+        // periodic cell, few items of one visitor tile: the tile's 32 steps over two or four items
+        // (k = 1, a call: n = 975 33.9 -> 25.3 us in four, 1,920 49.0 -> 44.4 in four (46.8 in two), 3,840
+        // 125.8 -> 116.6 in two, 4,800 no gain; in the open cell, whose steps are nine times shorter, 0-10%
+        // either way)
+        constexpr bool SPLIT = PER;
+        const int64_t few = SPLIT && sv < 0 && pl->sys[0].chunk == VT ? h->sm_count : 0;
+        if constexpr (SPLIT) {
+            using V1 = Sym2Var<K, 1, PER>;
+            auto split = [&](auto kern, unsigned parts) {
+                launch_pdl(kern, dim3((unsigned)ni, parts), V1::NT, V1::smem(LEN), st, rec, items, n1, np1, T1, sys,
+                           (const int*)nullptr, Lxa, Lya, partial, h->dev_flag, rt, fx, acc_stride);
+            };
+            if (ni <= 2 * few) split(sym2_kernel<K, PER, V1::UNR, V1::MINB, false, 1, false, true, 4>, 4);
+            else if (ni <= 8 * few) split(sym2_kernel<K, PER, V1::UNR, V1::MINB, false, 1, false, true, 2>, 2);
+        }
+        if (ni > 8 * few)
         switch (var) {
         case 1: RPBD_SYM2_LAUNCH(1, false, true); break;
         case 2: RPBD_SYM2_LAUNCH(2, false, true); break;
