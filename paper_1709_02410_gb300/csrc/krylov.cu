@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "precond.cuh"
 #include "rpbd_internal.cuh"
 #include "tridiag_sqrt.cuh"
 
@@ -177,7 +178,7 @@ struct OrthoProc {
     double *w, *part, *h, *vnext;  // part: ortho_part doubles; h: nv coefficients of both passes
     int nv;
     // GMRES: H column, rotations, residual; Lanczos: the tridiagonal's end
-    double *H, *cs, *sn, *g, *sc;
+    double *H, *cs, *sn, *g, *sc, *zl, *zU;
     double *alpha, *beta, *c, *c_prev;
     double* host;  // two scalars for the host
 };
@@ -195,18 +196,43 @@ static int ortho_blocks(int64_t len)
 }
 static size_t ortho_part(int64_t len, int nv) { return (size_t)ortho_blocks(len) * (2 * nv + 1); }
 
+// d[i] = sum_e at(i, e), i < nd, e < cnt, by the block's warps, U sums at a time
+// each (independent chains: one FP64 addition takes tens of cycles here)
+template <int U, class At, class Put>
+__device__ __forceinline__ void ortho_sums(int nd, int cnt, At at, Put put)
+{
+    const int lane = threadIdx.x & 31;
+    for (int i0 = (threadIdx.x >> 5) * U; i0 < nd; i0 += (blockDim.x >> 5) * U) {
+        double s[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) s[u] = 0.0;
+#pragma unroll 4
+        for (int e = lane; e < cnt; e += 32)
+#pragma unroll
+            for (int u = 0; u < U; ++u) s[u] += at(min(i0 + u, nd - 1), e);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int u = 0; u < U; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+        if (lane == 0)
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (i0 + u < nd) put(i0 + u, s[u]);
+    }
+}
+template <class At, class Put>
+__device__ __forceinline__ void ortho_sums(int nd, int cnt, At at, Put put)
+{
+    const int nw = blockDim.x >> 5;
+    if (nd <= nw) ortho_sums<1>(nd, cnt, at, put);
+    else if (nd <= 2 * nw) ortho_sums<2>(nd, cnt, at, put);
+    else ortho_sums<4>(nd, cnt, at, put);
+}
+
 // h[i] = sum of the blocks' partials of dot i, i < nv (shared memory, all threads)
 __device__ __forceinline__ void ortho_gather(int nv, int nblk, const double* part, double* h)
 {
-    const int lane = threadIdx.x & 31;
-    for (int i = threadIdx.x >> 5; i < nv; i += blockDim.x >> 5) {
-        double s = 0.0;
-#pragma unroll 4
-        for (int b = lane; b < nblk; b += 32) s += part[(int64_t)i * nblk + b];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) h[i] = s;
-    }
+    ortho_sums(nv, nblk, [&](int i, int b) { return part[(int64_t)i * nblk + b]; }, [&](int i, double s) { h[i] = s; });
     __syncthreads();
 }
 
@@ -221,7 +247,7 @@ __global__ void ortho_kernel(int64_t len, int64_t ld, int slice, OrthoBatch B)
     pdl_wait();
     pdl_trigger();
     const OrthoProc P = B.p[blockIdx.y];
-    const int nblk = gridDim.x, lane = threadIdx.x & 31;
+    const int nblk = gridDim.x;
     const int64_t e0 = (int64_t)blockIdx.x * slice;
     const int cnt = (int)max((int64_t)0, min((int64_t)slice, len - e0));
     const double* V = P.V + e0;
@@ -233,24 +259,24 @@ __global__ void ortho_kernel(int64_t len, int64_t ld, int slice, OrthoBatch B)
         if (blockIdx.x == 0)
             for (int i = threadIdx.x; i < P.nv; i += blockDim.x) P.h[i] = PASS == 1 ? h[i] : P.h[i] + h[i];
         for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
-            double s = ws[e];
-#pragma unroll 8
-            for (int i = 0; i < P.nv; ++i) s -= h[i] * V[(int64_t)i * ld + e];
+            double s4[4] = {0.0, 0.0, 0.0, 0.0};
+            int i = 0;
+            for (; i + 4 <= P.nv; i += 4)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s4[u] += h[i + u] * V[(int64_t)(i + u) * ld + e];
+            for (; i < P.nv; ++i) s4[0] += h[i] * V[(int64_t)i * ld + e];
+            const double s = ws[e] - ((s4[0] + s4[1]) + (s4[2] + s4[3]));
             ws[e] = s;
             P.w[e0 + e] = s;
         }
     }
     __syncthreads();
-    const int nd = PASS == 2 ? 1 : P.nv;
-    for (int i = threadIdx.x >> 5; i < nd; i += blockDim.x >> 5) {
-        const double* v = PASS == 2 ? ws : V + (int64_t)i * ld;
-        double s = 0.0;
-#pragma unroll 8
-        for (int e = lane; e < cnt; e += 32) s += v[e] * ws[e];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) out[(int64_t)i * nblk + blockIdx.x] = s;
-    }
+    if (PASS == 2)
+        ortho_sums<1>(1, cnt, [&](int, int e) { return ws[e] * ws[e]; },
+                      [&](int, double x) { out[blockIdx.x] = x; });
+    else
+        ortho_sums(P.nv, cnt, [&](int i, int e) { return V[(int64_t)i * ld + e] * ws[e]; },
+                   [&](int i, double x) { out[(int64_t)i * nblk + blockIdx.x] = x; });
 }
 
 // |w|^2 from the partials of pass 2, in every thread
@@ -269,18 +295,34 @@ __device__ __forceinline__ void ortho_normalize(const OrthoProc& P, int64_t len,
     for (int e = threadIdx.x; e < cnt; e += blockDim.x) P.vnext[e0 + e] = P.w[e0 + e] * inv;
 }
 
-// GMRES: v_{j+1}, and in one block more H's column j = nv - 1, the rotations and
-// the residual estimate.  sc: [1] |b|, [2] residual estimate
-__global__ void gmres_finish_kernel(int64_t len, int slice, int mdim, OrthoBatch B)
+// GMRES: v_{j+1} = w / |w| and at once z = P^-1 v_{j+1} for the next iteration (the
+// body-block solve of precond.cuh, a block per body: two launches' work in one, and
+// the residual is on its way to the host meanwhile); in one block more H's column
+// j = nv - 1, the rotations and the residual estimate.  sc: [1] |b|, [2] residual
+// estimate
+__global__ void __launch_bounds__(APPLY_THREADS) gmres_finish_kernel(int nper, int64_t n, int nblk, int mdim, PrecFactors M,
+                                                                     OrthoBatch B)
 {
     extern __shared__ double sm[];  // 3 (mdim + 2)
     pdl_wait();
     pdl_trigger();
     const OrthoProc P = B.p[blockIdx.y];
-    const int nblk = gridDim.x - 1, j = P.nv - 1;
+    const int j = P.nv - 1;
     const double nrm2 = ortho_norm2(P, nblk, sm);
-    if ((int)blockIdx.x < nblk) {
-        ortho_normalize(P, len, slice, nrm2);
+    if (blockIdx.x + 1 < gridDim.x) {
+        const double nv = sqrt(nrm2), inv = nv > 0.0 ? 1.0 / nv : 0.0;
+        prec_saddle_body(nper, n, M, blockIdx.x,
+                         [&](int64_t e) {
+                             const double v = P.w[e] * inv;
+                             P.vnext[e] = v;
+                             return v;
+                         },
+                         [&](int64_t e) {
+                             const double v = P.w[3 * n + e] * inv;
+                             P.vnext[3 * n + e] = v;
+                             return v;
+                         },
+                         P.zl, P.zU);
         return;
     }
     __syncthreads();
@@ -631,6 +673,7 @@ struct GmresProc {
     int j = 0, total = 0, matvecs = 0, status = RPBD_NOT_CONVERGED;
     double res = 1.0;
     const double *req_l = nullptr, *req_U = nullptr;  // vector whose saddle product is wanted
+    bool z_ready = false;                             // z = P^-1 v_j already there
 };
 
 int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, const double* q, int nsys,
@@ -676,6 +719,7 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
         gmres_backsolve_kernel<<<1, 64, jn * sizeof(double), st>>>(jn, mdim, p.S.H(), p.S.g(), p.S.y()); count_launch();
         lincomb_kernel<<<g, 256, 0, st>>>(len, p.V, len, jn, p.S.y(), 1.0, nullptr, p.w); count_launch();
         const PrecSaddle ps{p.w, p.w + 3 * n, p.zl, p.zU};
+        p.z_ready = false;
         RPBD_TRY(precond_saddle_impl(h, 1, &ps, st));
         add_kernel<<<g, 256, 0, st>>>(3 * n, p.zl, p.x); count_launch();
         add_kernel<<<vgrid(6 * nb), 256, 0, st>>>(6 * nb, p.zU, p.x + 3 * n); count_launch();
@@ -729,7 +773,8 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
         int nps = 0;
         auto want_arnoldi = [&](GmresProc& p) {  // z = P^-1 v_j, and the product with it
             const double* v = p.V + (int64_t)p.j * len;
-            ps[nps++] = PrecSaddle{v, v + 3 * n, p.zl, p.zU};
+            if (!p.z_ready) ps[nps++] = PrecSaddle{v, v + 3 * n, p.zl, p.zU};
+            p.z_ready = false;
             p.req_l = p.zl;
             p.req_U = p.zU;
             p.phase = GmresProc::NEED_ARNOLDI;
@@ -819,14 +864,17 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
                 o.sn = p.S.sn();
                 o.g = p.S.g();
                 o.sc = p.sc;
+                o.zl = p.zl;
+                o.zU = p.zU;
+                p.z_ready = true;
                 o.host = h->host_small + 2 * act[a];
                 p.phase = GmresProc::READ_ITER;
             }
         }
         if (no) {
             const OrthoGrid G = launch_ortho(len, no, B, st);
-            launch_pdl(gmres_finish_kernel, dim3((unsigned)G.blocks + 1, (unsigned)no), 256,
-                       3 * (size_t)(mdim + 2) * sizeof(double), st, len, G.slice, mdim, B);
+            launch_pdl(gmres_finish_kernel, dim3((unsigned)nb + 1, (unsigned)no), APPLY_THREADS,
+                       3 * (size_t)(mdim + 2) * sizeof(double), st, nper, n, G.blocks, mdim, prec_factors(h), B);
             count_launch();
             RPBD_LAUNCH_CHECK(h);
         }

@@ -14,12 +14,12 @@
 #include <cuda_runtime.h>
 
 #include "pair64.cuh"
+#include "precond.cuh"
 #include "rpbd_internal.cuh"
 
 namespace rpbd {
 
 constexpr int PREC_THREADS = 256;
-constexpr int PREC_MAX_M = 96;  // 3 * nper <= 96
 
 // One CTA per body, bound by FP64 instructions (about 19 cycles a warp instruction
 // per SM) and, for few bodies, by the chain of m pivots.  Pair blocks are formed
@@ -205,13 +205,6 @@ __global__ void __launch_bounds__(PREC_THREADS) prec_build_kernel(int nper, int6
     }
 }
 
-// Rows of the stored factors' products, one CTA per body, entries read straight
-// from global memory, every one once.  The threads split a row's columns into
-// APPLY_THREADS / span pieces, so a chain is ~m / 4 loads, issued eight at a
-// time; with half the threads, the factor staged in shared memory first and
-// loads one by one a 45-row product took ~10 us, most of it latency.
-constexpr int APPLY_THREADS = 256;
-
 // out = A_p x_p per body, A_p one of the stored factors.
 // mode 0: L (lower), 1: L^-1 (lower), 2: L^-T, 3: M^-1.  With `active`
 // (batches: systems at blob offsets off[0..n_sys]), bodies of inactive
@@ -268,57 +261,17 @@ __global__ void __launch_bounds__(APPLY_THREADS) prec_apply_kernel(int mode, int
     }
 }
 
-// exact body-block saddle solve: [M(pp) -K_p; -K_p^T 0][lam; U] = [a; b]
-//   t = (M^-1 K)^T a + b,  U = -N t,  lam = M^-1 a + (M^-1 K) U
-// for up to four vectors (blockIdx.y).  M^-1 a does not wait for U.
+// for up to four vectors (blockIdx.y)
 struct SaddleArgs {
     PrecSaddle p[4];
 };
-__global__ void __launch_bounds__(APPLY_THREADS) prec_saddle_kernel(int nper, int64_t n, const double* Minv,
-                                                                    const double* MinvK, const double* N, SaddleArgs S)
+__global__ void __launch_bounds__(APPLY_THREADS) prec_saddle_kernel(int nper, int64_t n, PrecFactors M, SaddleArgs S)
 {
-    __shared__ double va[PREC_MAX_M], part[APPLY_THREADS], t6[6], u6[6];
     pdl_wait();
     pdl_trigger();
     const PrecSaddle P = S.p[blockIdx.y];
-    const int m = 3 * nper;
-    const int64_t p = blockIdx.x;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int span = (m + 31) & ~31, parts = APPLY_THREADS / span;
-    const double* A = Minv + p * m * m;        // column-major: (i, j) at j * m + i
-    const double* MK = MinvK + p * 6 * m;      // (M^-1 K)^T rows: column c at c * m
-    for (int e = tid; e < m; e += APPLY_THREADS) va[e] = P.a ? P.a[(e % 3) * n + p * nper + e / 3] : 0.0;
-    __syncthreads();
-    if (warp < 6) {
-        double v = 0.0;
-        for (int k = lane; k < m; k += 32) v += MK[warp * m + k] * va[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) t6[warp] = v + (P.b ? P.b[6 * p + warp] : 0.0);
-    }
-    const int q = tid / span, i = tid % span;
-    if (q < parts && i < m) {
-        double v = 0.0;
-#pragma unroll 8
-        for (int j = q; j < m; j += parts) v += A[j * m + i] * va[j];
-        part[q * span + i] = v;
-    }
-    __syncthreads();
-    if (tid < 6) {
-        double v = 0.0;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) v -= N[p * 36 + c * 6 + tid] * t6[c];
-        u6[tid] = v;
-        P.U[6 * p + tid] = v;
-    }
-    __syncthreads();
-    if (tid < m) {
-        double v = part[tid];
-        for (int q2 = 1; q2 < parts; ++q2) v += part[q2 * span + tid];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) v += MK[c * m + tid] * u6[c];
-        P.lam[(tid % 3) * n + p * nper + tid / 3] = v;
-    }
+    prec_saddle_body(nper, n, M, blockIdx.x, [&](int64_t e) { return P.a ? P.a[e] : 0.0; },
+                     [&](int64_t e) { return P.b ? P.b[e] : 0.0; }, P.lam, P.U);
 }
 
 int precond_build_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, const double* q, cudaStream_t st)
@@ -382,8 +335,7 @@ int precond_saddle_impl(rpbd_handle* h, int np, const PrecSaddle* ps, cudaStream
     SaddleArgs S = {};
     for (int a = 0; a < np; ++a) S.p[a] = ps[a];
     launch_pdl(prec_saddle_kernel, dim3((unsigned)h->prec_nb, (unsigned)np), APPLY_THREADS, 0, st, h->prec_nper,
-               h->prec_nb * h->prec_nper, (const double*)h->buf[BUF_PREC_MINV], (const double*)h->buf[BUF_PREC_MINVK],
-               (const double*)h->buf[BUF_PREC_N], S);
+               h->prec_nb * h->prec_nper, prec_factors(h), S);
     count_launch();
     RPBD_LAUNCH_CHECK(h);
     return RPBD_OK;

@@ -31,6 +31,8 @@
 
 #include <cuda_runtime.h>
 
+#include "wall_rpy.cuh"
+
 namespace rpbd {
 
 constexpr int TRIDIAG_MAX_PAIRS = 48;
@@ -70,10 +72,10 @@ __device__ inline bool tridiag_sqrt_quadrature(int m1, const double* __restrict_
     const double x = hi * exp2(-47.0 / 32.0 * (32 - lane));
     {
         double d = al[0] - x;
-        bool pos = d > 0.0;
+        bool pos = d > 1e-280;
         for (int i = 1; i < m1; ++i) {
-            d = al[i] - x - be[i - 1] * be[i - 1] / d;
-            pos = pos && d > 0.0;
+            d = al[i] - x - be[i - 1] * be[i - 1] * rcp3(d);  // (0, tiny or NaN pivots: not positive)
+            pos = pos && d > 1e-280 && d < 1e300;
         }
         const unsigned ok = __ballot_sync(0xffffffffu, pos);
         if (!(ok & 1u)) return false;
@@ -89,7 +91,7 @@ __device__ inline bool tridiag_sqrt_quadrature(int m1, const double* __restrict_
             km[n] = 0.0;
             if (a - b > 1e-15 * a) {  // (uniform)
                 const double an = 0.5 * (a + b), cn = 0.5 * (a - b);
-                b = sqrt(a * b);
+                b = a * b * rsqrt3(a * b);
                 a = an;
                 km[n] = cn / an;
                 steps = n + 1;
@@ -105,7 +107,7 @@ __device__ inline bool tridiag_sqrt_quadrature(int m1, const double* __restrict_
 #pragma unroll
             for (int n = 11; n >= 0; --n)
                 if (n < steps) {
-                    const double t = km[n] * sn * sn, rr = 1.0 / (1.0 + t);
+                    const double t = km[n] * sn * sn, rr = rcp3(1.0 + t);
                     cn = cn * dn * rr;
                     sn = (1.0 + km[n]) * sn * rr;
                     dn = (1.0 - t) * rr;
@@ -118,12 +120,12 @@ __device__ inline bool tridiag_sqrt_quadrature(int m1, const double* __restrict_
             w *= 2.0 * Kp * sqrt(lo) / (3.14159265358979323846 * N);
             const double sig = lo * sc * sc;
             // (T + sig) z = T e_1
-            double di = 1.0 / (al[0] + sig), yi = al[0];
+            double di = rcp3(al[0] + sig), yi = al[0];
             dinv[lane] = di;
             y[lane] = yi;
             for (int i = 1; i < m1; ++i) {
                 const double bb = be[i - 1], l = bb * di;
-                di = 1.0 / (al[i] + sig - l * bb);
+                di = rcp3(al[i] + sig - l * bb);
                 yi = (i == 1 ? bb : 0.0) - l * yi;
                 dinv[i * 32 + lane] = di;
                 y[i * 32 + lane] = yi;

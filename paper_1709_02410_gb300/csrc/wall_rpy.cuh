@@ -93,6 +93,14 @@ __device__ __forceinline__ double rsqrt3(double x)
     const double e = fma(-x * y, y, 1.0);
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
+// 1/x for normal x, the same way: y (1 + e + e^2), e = 1 - x y
+__device__ __forceinline__ double rcp3(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
 __device__ __forceinline__ float val_(float x) { return x; }
 __device__ __forceinline__ double val_(double x) { return x; }
 
