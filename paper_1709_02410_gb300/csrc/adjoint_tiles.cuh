@@ -430,10 +430,16 @@ static int run_all(rpbd_handle* h, Cut c, int nr, double* grad, double ig, doubl
 {
     constexpr bool tickets = sizeof(S) == 8;
     const int T = c.tiles / c.vph;
-    const size_t words = (size_t)((int64_t)c.hg + c.items) * c.parts * 4 * c.n_pad;
     unsigned char* base;
     const size_t g_bytes = sizeof(double) * 4 * c.n_pad, t_bytes = ((size_t)T * sizeof(int) + 15) / 16 * 16;
-    RPBD_TRY(ensure_t(h, BUF_PARTIAL, words * sizeof(S) + g_bytes + t_bytes, &base));
+    for (;;) {  // smaller groups where the memory left is short
+        const size_t words = (size_t)((int64_t)c.hg + c.items) * c.parts * 4 * c.n_pad;
+        const int s = ensure_t(h, BUF_PARTIAL, words * sizeof(S) + g_bytes + t_bytes, &base);
+        if (s == RPBD_OK) break;
+        if (s != RPBD_NO_MEM || c.hg == 1) return s;
+        cudaGetLastError();
+        c.hg = (c.hg + 1) / 2;
+    }
     Out o;
     o.G = reinterpret_cast<double*>(base);
     o.ticket = reinterpret_cast<int*>(base + g_bytes);

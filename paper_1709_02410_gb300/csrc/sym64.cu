@@ -42,7 +42,7 @@ constexpr int VT = 32;           // visitor tile (records)
 constexpr int NST = 4;           // ring stages
 constexpr int MAX_CHUNK = 64;    // visitor tiles per item
 constexpr int64_t SMALL_N = 4096;
-constexpr double PARTIAL_LIMIT = 16.0 * (1ull << 30);
+constexpr double PARTIAL_LIMIT = 4.0 * (1ull << 30);
 
 using namespace pair64;
 
@@ -332,13 +332,18 @@ static int run(rpbd_handle* h, const Cut& c, int64_t n, const double* r, const d
 // Instructions per ordered pair (above): passes of up to four right-hand sides
 // cost 36, 46 or 66 each, the one-direction kernel 66 + 9 K with K = 8 or 16:
 // fewer up to k = 8.  The partials, about n^2/128 rows beyond SMALL_N, have to
-// stay under PARTIAL_LIMIT (n about 290,000 for k = 1).
-bool sym64_takes(const rpbd_handle* h, int64_t n, int k)
+// stay under PARTIAL_LIMIT (n about 145,000 for k = 1), and fit the memory left:
+// where they do not, the one-direction kernel, which needs a tenth of it, runs.
+bool sym64_takes(rpbd_handle* h, int64_t n, int k)
 {
-    if (k > 8 || n > (int64_t)1 << 24) return false;
+    if (k > 8 || n > (int64_t)1 << 20) return false;
     const sym64::Cut c = sym64::cut(n, h->sm_count);
-    return c.T <= 0x7fffffff && c.items <= 65535 &&
-           c.rows() * 3.0 * (k <= 2 ? k : 4) * (double)c.n_pad * sizeof(double) <= sym64::PARTIAL_LIMIT;
+    const double bytes = c.rows() * 3.0 * (k <= 2 ? k : 4) * (double)c.n_pad * sizeof(double);
+    if (c.items > 65535 || bytes > sym64::PARTIAL_LIMIT) return false;
+    void* p;
+    if (ensure(h, BUF_PARTIAL, (size_t)bytes, &p) == RPBD_OK) return true;
+    cudaGetLastError();  // (the failed allocation is not the one-direction kernel's)
+    return false;
 }
 
 int sym64_apply_impl(rpbd_handle* h, int64_t n, const double* r, const double* F, double* U, int k, cudaStream_t st)

@@ -130,3 +130,16 @@ def test_small_system_non_finite_force():
     F[1, 2, 11] = np.inf
     U = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT).mobility_apply(to_dev(r), to_dev(F, torch.float32))
     assert torch.isnan(U).all()
+
+
+@pytest.mark.parametrize("dtype,n,tol", [(F32, 217_001, 1e-5), (F64, 127_003, 1e-11)])
+def test_adjoint_in_groups(dtype, n, tol):
+    """Past the partials' bound the home tiles run in several launches whose sums are carried over."""
+    r = cloud(n, 770)
+    u, F = synth.gaussian(771, (2, 3, n))
+    h = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT)
+    rows = rows_of(n)
+    before = h.lib.rpbd_launch_count()
+    g = h.mobility_adjoint(to_dev(r), to_dev(u), to_dev(F), dtype=dtype).cpu().numpy()
+    assert h.lib.rpbd_launch_count() - before > (1 if dtype == F64 else 3)  # more than one group
+    assert rel2(g[:, rows], om.grad(r, u, F, om.Params(synth.ETA, synth.A_BOOMERANG), rows)) <= tol
