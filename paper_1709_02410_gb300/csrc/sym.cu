@@ -1222,11 +1222,20 @@ static int run2(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, 
                            ATOMV>,                                                                                    \
                ni, Sym2Var<K, V, PER>::NT, Sym2Var<K, V, PER>::smem(LEN), st, rec, items, n1, np1, T1, sys,            \
                (const int*)nullptr, Lxa, Lya, partial, h->dev_flag, rt, fx, acc_stride)
-    if (n_sys > 1) {  // batches: four home blobs per thread (variant 5's shape; 3-5% faster than two
-                      // on 64 uneven suspensions of 480-22,500 blobs)
+    if (n_sys > 1) {
+        // batches: four home blobs per thread (variant 5's shape; 2-5% faster than two on 64 uneven
+        // suspensions of 480-22,500 blobs), two while the items are short: k = 2, 64 systems of 120-1,920
+        // blobs 172.8 -> 157.5 us, 8 of them 43.0 -> 34.8; k = 4 292 -> 234 us, 64 systems of 240-4,500
+        // 1,083 -> 909; k = 1 0-14%
         if constexpr (!PER) {
             using V5 = Sym2Var<K, 5>;
-            if (atom)
+            using V3 = Sym2Var<K, 3>;
+            const int chunk1 = pl->sys[0].chunk;  // one for all systems
+            if (atom && (K <= 2 ? chunk1 == VT : chunk1 < CHUNK2))
+                launch_pdl(sym2_kernel<K, false, V3::UNR, V3::MINB, true, V3::HP, false, true>, ni, V3::NT, V3::smem(LEN), st,
+                           rec, items, (int64_t)0, (int64_t)0, 0, sys, active, Lxa, Lya, partial, h->dev_flag, rt, fx,
+                           acc_stride);
+            else if (atom)
                 launch_pdl(sym2_kernel<K, false, V5::UNR, V5::MINB, true, V5::HP, false, true>, ni, V5::NT, V5::smem(LEN), st,
                            rec, items, (int64_t)0, (int64_t)0, 0, sys, active, Lxa, Lya, partial, h->dev_flag, rt, fx,
                            acc_stride);

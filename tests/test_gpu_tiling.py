@@ -51,6 +51,23 @@ def test_f32_symmetric_tiles(n, variant, cell):
         assert rel2(U[:, :, rows], om.apply(r, F.astype(np.float64), prm, rows)) <= 1e-5
 
 
+# (the last: items of several visitor tiles, four homes per thread)
+@pytest.mark.parametrize("sizes", [(1, 255, 256, 257), (33, 513, 64), (300,) * 40, (6000, 12, 7001)])
+@pytest.mark.parametrize("k", [1, 2, 3])
+def test_f32_symmetric_batches(sizes, k):
+    """Batches of short items, two home blobs per thread, and of longer ones, four, each system against the oracle."""
+    rs = [cloud(n, 770 + i) for i, n in enumerate(sizes)]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    h = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT)
+    h.set_batch_variant(4)
+    prm = om.Params(synth.ETA, synth.A_BOOMERANG)
+    F = synth.gaussian(771, (k, 3, off[-1]), np.float32)
+    U = h.mobility_apply_batched(off, to_dev(np.concatenate(rs, axis=1)), to_dev(F, torch.float32)).cpu().numpy()
+    for s, r in enumerate(rs):
+        sl, rows = slice(off[s], off[s + 1]), rows_of(r.shape[1])
+        assert rel2(U[:, :, sl][:, :, rows], om.apply(r, F[:, :, sl].astype(np.float64), prm, rows)) <= 1e-5
+
+
 def test_accumulators_are_cleared_between_calls():
     """One handle, calls of other sizes, right-hand sides and a non-finite force between: every result as on a fresh handle."""
     h = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT)
