@@ -44,7 +44,7 @@ __device__ __forceinline__ void split(double x, float& hi, float& lo)
 }
 
 template <int K, bool PER, class In, class Out>
-__global__ void __launch_bounds__(NT) direct_kernel(int n, int k, int tp, const double* r, const In* F, double a, float ia,
+__global__ void __launch_bounds__(NT) direct_kernel(int n, int k, int tp, const double* r, const In* F, double a, double ia,
                                                     double s_min, float Lx, float Ly, double inv8pieta, Out* U)
 {
     extern __shared__ float sm[];  // fields x_hi, y_hi, x_lo, y_lo, z~/a, s F of [n]
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(NT) direct_kernel(int n, int k, int tp, const 
         sm[n + i] = h;
         sm[3 * n + i] = l;
         const double z = r[2 * n + i];
-        sm[4 * n + i] = (float)(z > a ? z : a) * ia;
+        sm[4 * n + i] = (float)((z > a ? z : a) * ia);
         double s = 1.0;
         if (!(z >= a)) {  // overlaps the wall, or NaN (stays NaN)
             const double t = z / a;
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(NT) direct_kernel(int n, int k, int tp, const 
     }
     bad = __syncthreads_or(bad);  // a force that is not finite: U is NaN everywhere, as in sym.cu
     const PairConstX2 pc = PairConstX2::make_unit();
-    const float2 m1 = pc.m1, ia2 = bc2(ia);
+    const float2 m1 = pc.m1, ia2 = bc2((float)ia);
     const int wp = NT / 32 / tp;                                     // warps per pair of targets
     const int t0 = ((int)blockIdx.x * tp + warp / wp) * 2, t1 = t0 + 1;
     const int c0 = min(t0, n - 1), c1 = min(t1, n - 1);
@@ -167,7 +167,7 @@ static int run(rpbd_handle* h, int n, const double* r, const In* F, Out* U, int 
     while (tp < 8 && n > 2 * tp * h->sm_count) tp *= 2;
     const double inv8pieta = 1.0 / (8.0 * 3.14159265358979323846 * h->p.eta * h->p.a);  // blocks in units of a
     if (h->profile) prof_begin(h, st);
-    launch_pdl(kern, (unsigned)((n + 2 * tp - 1) / (2 * tp)), NT, smem, st, n, k, tp, r, F, h->p.a, (float)(1.0 / h->p.a),
+    launch_pdl(kern, (unsigned)((n + 2 * tp - 1) / (2 * tp)), NT, smem, st, n, k, tp, r, F, h->p.a, 1.0 / h->p.a,
                h->p.s_min, (float)(h->p.Lx / h->p.a), (float)(h->p.Ly / h->p.a), inv8pieta, U);
     count_launch();
     if (h->profile) prof_end(h, st, PER ? 3 : 4, K, (double)n * (double)n);
