@@ -104,7 +104,9 @@ __global__ void add_kernel(int64_t n, const double* __restrict__ x, double* __re
 }
 
 // Saddle products of up to four processes (blockIdx.y): w = [M lam - K U; -K^T lam]
-// given M lam (Ml, which may be w itself).  One warp per body.
+// given M lam (Ml, which may be w itself).  G lanes per body, the smallest of 8,
+// 16 and 32 that has one per blob: the FP64 pipe bounds it, at one warp per body
+// and six separate sums 75 instructions a body of 15 blobs, now 26.
 struct SaddleProd {
     const double *Ml, *lam, *U;
     double* w;
@@ -112,12 +114,15 @@ struct SaddleProd {
 struct SaddleBatch {
     SaddleProd p[4];
 };
+constexpr int SADDLE_THREADS = 32;  // (few bodies: one warp per SM)
+template <int G>
 __global__ void saddle_kernel(int64_t nb, int nper, const double* r, const double* q, SaddleBatch B)
 {
     pdl_wait();
     pdl_trigger();
-    const int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (b >= nb) return;
+    const int64_t bi = (blockIdx.x * (int64_t)SADDLE_THREADS + threadIdx.x) / G;
+    const bool on = bi < nb;
+    const int64_t b = on ? bi : nb - 1;
     const SaddleProd P = B.p[blockIdx.y];
     const int lane = threadIdx.x & 31;
     const int64_t n = nb * nper;
@@ -125,7 +130,7 @@ __global__ void saddle_kernel(int64_t nb, int nper, const double* r, const doubl
     double u[6], s[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
     for (int c = 0; c < 6; ++c) u[c] = P.U[6 * b + c];
-    for (int k = lane; k < nper; k += 32) {
+    for (int k = on ? lane % G : nper; k < nper; k += G) {
         const int64_t i = b * nper + k;
         const double d0 = r[i] - q0, d1 = r[n + i] - q1, d2 = r[2 * n + i] - q2;
         const double l0 = P.lam[i], l1 = P.lam[n + i], l2 = P.lam[2 * n + i];
@@ -139,12 +144,9 @@ __global__ void saddle_kernel(int64_t nb, int nper, const double* r, const doubl
         s[4] += d2 * l0 - d0 * l2;
         s[5] += d0 * l1 - d1 * l0;
     }
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
-        if (lane == 0) P.w[3 * n + 6 * b + c] = -s[c];
-    }
+    const double v = group_sum6<G>(s, lane);
+    const int c = sum6_of<G>(lane);
+    if (on && c >= 0) P.w[3 * n + 6 * b + c] = -v;
 }
 
 static unsigned vgrid(int64_t n)
@@ -210,14 +212,20 @@ __device__ __forceinline__ void ortho_sums(int nd, int cnt, At at, Put put)
         for (int e = lane; e < cnt; e += 32)
 #pragma unroll
             for (int u = 0; u < U; ++u) s[u] += at(min(i0 + u, nd - 1), e);
+        // half of the sums to each half of the lanes while there are several
+        int o = 16, mine = 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
+        for (int c = U / 2; c > 0; c >>= 1, o >>= 1) {
+            const bool up = lane & o;
 #pragma unroll
-            for (int u = 0; u < U; ++u) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
-        if (lane == 0)
+            for (int u = 0; u < c; ++u)
+                s[u] = (up ? s[u + c] : s[u]) + __shfl_xor_sync(0xffffffffu, up ? s[u] : s[u + c], o);
+            if (up) mine += c;
+        }
+        const int first = 2 * o - 1;
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (i0 + u < nd) put(i0 + u, s[u]);
+        for (; o > 0; o >>= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+        if ((lane & first) == 0 && i0 + mine < nd) put(i0 + mine, s[0]);
     }
 }
 template <class At, class Put>
@@ -279,17 +287,25 @@ __global__ void ortho_kernel(int64_t len, int64_t ld, int slice, OrthoBatch B)
                    [&](int i, double x) { out[(int64_t)i * nblk + blockIdx.x] = x; });
 }
 
-// |w|^2 from the partials of pass 2, in every thread
-__device__ __forceinline__ double ortho_norm2(const OrthoProc& P, int nblk, double* h)
+// h[0..2] = |w|^2 from the partials of pass 2, |w| and 1/|w| (0 when it vanishes):
+// by one thread, a square root and a division in every one keep the FP64 pipe
+// busy longer than the rest of the finishing kernels
+__device__ __forceinline__ void ortho_norm(const OrthoProc& P, int nblk, double* h)
 {
-    ortho_gather(1, nblk, P.part + 2 * (int64_t)P.nv * nblk, h);
-    return h[0];
+    const double* part = P.part + 2 * (int64_t)P.nv * nblk;
+    ortho_sums<1>(1, nblk, [&](int, int b) { return part[b]; },
+                  [&](int, double s) {
+                      const double nv = sqrt(s);
+                      h[0] = s;
+                      h[1] = nv;
+                      h[2] = nv > 0.0 ? 1.0 / nv : 0.0;
+                  });
+    __syncthreads();
 }
 
 // v_nv = w / |w| of the block's slice (0 when the norm vanishes)
-__device__ __forceinline__ void ortho_normalize(const OrthoProc& P, int64_t len, int slice, double nrm2)
+__device__ __forceinline__ void ortho_normalize(const OrthoProc& P, int64_t len, int slice, double inv)
 {
-    const double nv = sqrt(nrm2), inv = nv > 0.0 ? 1.0 / nv : 0.0;
     const int64_t e0 = (int64_t)blockIdx.x * slice;
     const int cnt = (int)max((int64_t)0, min((int64_t)slice, len - e0));
     for (int e = threadIdx.x; e < cnt; e += blockDim.x) P.vnext[e0 + e] = P.w[e0 + e] * inv;
@@ -308,9 +324,9 @@ __global__ void __launch_bounds__(APPLY_THREADS) gmres_finish_kernel(int nper, i
     pdl_trigger();
     const OrthoProc P = B.p[blockIdx.y];
     const int j = P.nv - 1;
-    const double nrm2 = ortho_norm2(P, nblk, sm);
+    ortho_norm(P, nblk, sm);
+    const double nv = sm[1], inv = sm[2];
     if (blockIdx.x + 1 < gridDim.x) {
-        const double nv = sqrt(nrm2), inv = nv > 0.0 ? 1.0 / nv : 0.0;
         prec_saddle_body(nper, n, M, blockIdx.x,
                          [&](int64_t e) {
                              const double v = P.w[e] * inv;
@@ -334,7 +350,7 @@ __global__ void __launch_bounds__(APPLY_THREADS) gmres_finish_kernel(int nper, i
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double last = sqrt(nrm2), cur = col[0];  // rotate down the column
+        double last = nv, cur = col[0];  // rotate down the column
         for (int i = 0; i < j; ++i) {
             const double nx = col[i + 1];
             col[i] = cs[i] * cur + sn[i] * nx;
@@ -405,16 +421,17 @@ __global__ void lanczos_finish_kernel(int64_t len, int slice, OrthoBatch B)
     pdl_trigger();
     const OrthoProc P = B.p[blockIdx.y];
     const int nblk = gridDim.x - 1, m1 = P.nv, lane = threadIdx.x & 31;
-    const double nrm2 = ortho_norm2(P, nblk, sm);
+    ortho_norm(P, nblk, sm);
+    const double nrm2 = sm[0], nv = sm[1], inv = sm[2];
     if ((int)blockIdx.x < nblk) {
-        ortho_normalize(P, len, slice, nrm2);
+        ortho_normalize(P, len, slice, inv);
         return;
     }
     __syncthreads();
     if (threadIdx.x >= 32) return;
     if (lane == 0) {
         P.alpha[m1 - 1] = P.h[m1 - 1];
-        P.beta[m1 - 1] = sqrt(nrm2);
+        P.beta[m1 - 1] = nv;
     }
     __syncwarp();
     tridiag_sqrt_e1(m1, P.alpha, P.beta, sm, P.c);
@@ -842,7 +859,9 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
             GmresProc& p = P[act[a]];
             SB.p[a] = SaddleProd{Um + (int64_t)a * 3 * n, p.req_l, p.req_U, p.w};
         }
-        launch_pdl(saddle_kernel, dim3((unsigned)((nb + 3) / 4), (unsigned)k), 128, 0, st, nb, nper, r, q, SB);
+        const int G = nper <= 8 ? 8 : nper <= 16 ? 16 : 32, per = SADDLE_THREADS / G;
+        launch_pdl(G == 8 ? saddle_kernel<8> : G == 16 ? saddle_kernel<16> : saddle_kernel<32>,
+                   dim3((unsigned)((nb + per - 1) / per), (unsigned)k), SADDLE_THREADS, 0, st, nb, nper, r, q, SB);
         count_launch();
         for (int a = 0; a < k; ++a) {
             GmresProc& p = P[act[a]];

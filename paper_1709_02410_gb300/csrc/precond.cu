@@ -232,31 +232,31 @@ __global__ void __launch_bounds__(APPLY_THREADS) prec_apply_kernel(int mode, int
     const int tid = threadIdx.x;
     for (int e = tid; e < m; e += APPLY_THREADS) v[e] = x[(e % 3) * n + p * nper + e / 3];
     __syncthreads();
-    const int span = (m + 31) & ~31, parts = APPLY_THREADS / span;
-    const int q = tid / span, i = tid % span;
+    const int parts = apply_parts(m, APPLY_THREADS);
+    const int q = tid / m, i = tid - q * m;
     if (mode == 2) {  // (L^-1)^T: sum_j Linv(j, i) v_j, j >= i: through shared memory, rows of odd length
         extern __shared__ double sA[];
         const int ld = m | 1, lane = tid & 31;
         for (int c = tid >> 5; c < m; c += APPLY_THREADS / 32)
             for (int j = c + lane; j < m; j += 32) sA[c * ld + j] = A[c * m + j];
         __syncthreads();
-        if (q < parts && i < m) {
+        if (q < parts) {
             double acc = 0.0;
 #pragma unroll 4
             for (int j = i + q; j < m; j += parts) acc += sA[i * ld + j] * v[j];
-            part[q * span + i] = acc;
+            part[tid] = acc;
         }
-    } else if (q < parts && i < m) {  // M^-1, or lower triangular (j <= i): row i's columns j = q, q + parts, ...
+    } else if (q < parts) {  // M^-1, or lower triangular (j <= i): row i's columns j = q, q + parts, ...
         const int j1 = mode == 3 ? m : i + 1;
         double acc = 0.0;
 #pragma unroll 8
         for (int j = q; j < j1; j += parts) acc += A[j * m + i] * v[j];
-        part[q * span + i] = acc;
+        part[tid] = acc;
     }
     __syncthreads();
     if (tid < m) {
         double acc = part[tid];
-        for (int q2 = 1; q2 < parts; ++q2) acc += part[q2 * span + tid];
+        for (int q2 = 1; q2 < parts; ++q2) acc += part[q2 * m + tid];
         out[(tid % 3) * n + p * nper + tid / 3] = acc;
     }
 }

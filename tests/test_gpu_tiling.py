@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 import torch
 
-from oracle import mobility as om
+from oracle import mobility as om, saddle
 from paper_1709_02410_gb300 import F32, F64, Handle, synth
 
 from gpu_util import rel2, to_dev
@@ -160,3 +160,22 @@ def test_adjoint_in_groups(dtype, n, tol):
     g = h.mobility_adjoint(to_dev(r), to_dev(u), to_dev(F), dtype=dtype).cpu().numpy()
     assert h.lib.rpbd_launch_count() - before > (1 if dtype == F64 else 3)  # more than one group
     assert rel2(g[:, rows], om.grad(r, u, F, om.Params(synth.ETA, synth.A_BOOMERANG), rows)) <= tol
+
+
+@pytest.mark.parametrize("nper", [3, 8, 9, 16, 17, 32])
+def test_saddle_solve_by_blobs_per_body(nper):
+    """Bodies of 3 to 32 blobs (8, 16 or 32 lanes of a warp each, an odd number of bodies) against the dense solution."""
+    a = synth.A_BOOMERANG
+    L = np.zeros((nper, 3))
+    L[:, 0] = np.maximum(nper // 2 - np.arange(nper), 0)  # one arm along x, one along y
+    L[:, 1] = np.maximum(np.arange(nper) - nper // 2, 0)
+    rng = np.random.default_rng(780 + nper)
+    q = np.stack([40.0 * a * np.arange(5), rng.uniform(0, 9 * a, 5), a * rng.uniform(1.5, 4.0, 5)], 1)
+    r = (q[:, None] + 2.1 * a * L).reshape(-1, 3).T.copy()
+    slip, FT = rng.standard_normal(r.shape), rng.standard_normal((5, 6)) * 1e-2
+    prm = om.Params(synth.ETA, a)
+    lam_d, U_d, _ = saddle.dense_solution(r, q, nper, prm, slip, FT)
+    h = Handle(synth.ETA, a, synth.KT)
+    lam, U, st = h.gmres_rigid_solve(nper, to_dev(r), to_dev(q), to_dev(slip), to_dev(FT), tol=1e-12, max_iter=200)
+    assert st["status"] == 0
+    assert rel2(U.cpu().numpy(), U_d) <= 1e-9 and rel2(lam.cpu().numpy(), lam_d) <= 1e-8
