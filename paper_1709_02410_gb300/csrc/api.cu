@@ -10,6 +10,7 @@
 #include <utility>
 
 #include "rpbd_internal.cuh"
+#include "tridiag_sqrt.cuh"
 
 namespace rpbd {
 
@@ -106,6 +107,18 @@ const char* rpbd_status_string(int status)
 
 const char* rpbd_last_error(const rpbd_handle* h) { return h ? h->err.c_str() : "null handle"; }
 
+// 33 KB on the device, the same for every handle; computed by the first one
+struct SqrtTable {
+    SqrtNode node[SQRT_TABLE];
+    SqrtTable() { sqrt_nodes(node); }
+};
+static bool put_sqrt_nodes(rpbd_handle* h)
+{
+    static const SqrtTable t;
+    return cudaMalloc(&h->sqrt_nodes, sizeof(t)) == cudaSuccess &&
+           cudaMemcpy(h->sqrt_nodes, &t, sizeof(t), cudaMemcpyHostToDevice) == cudaSuccess;
+}
+
 int rpbd_create(rpbd_handle** out, const rpbd_params* p)
 {
     if (!out || !p) return RPBD_BAD_ARG;
@@ -121,8 +134,10 @@ int rpbd_create(rpbd_handle** out, const rpbd_params* p)
         return RPBD_CUDA;
     }
     if (cudaMalloc(&h->dev_flag, sizeof(int)) != cudaSuccess || cudaMemset(h->dev_flag, 0, sizeof(int)) != cudaSuccess ||
-        cudaMallocHost(&h->host_small, 4096 * sizeof(double)) != cudaSuccess) {
+        cudaMallocHost(&h->host_small, 4096 * sizeof(double)) != cudaSuccess || !put_sqrt_nodes(h)) {
         if (h->dev_flag) cudaFree(h->dev_flag);
+        if (h->host_small) cudaFreeHost(h->host_small);
+        if (h->sqrt_nodes) cudaFree(h->sqrt_nodes);
         delete h;
         return RPBD_CUDA;
     }
@@ -143,6 +158,7 @@ int rpbd_destroy(rpbd_handle* h)
     for (int b = 0; b < BUF_COUNT; ++b)
         if (h->buf[b]) cudaFree(h->buf[b]);
     if (h->dev_flag) cudaFree(h->dev_flag);
+    if (h->sqrt_nodes) cudaFree(h->sqrt_nodes);
     if (h->host_small) cudaFreeHost(h->host_small);
     delete h;
     return RPBD_OK;

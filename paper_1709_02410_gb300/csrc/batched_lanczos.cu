@@ -109,7 +109,8 @@ __global__ void blz_init_kernel(int n_sys, const double* __restrict__ W2, int* _
 }
 
 // one warp per system: alpha_m, beta_m; T^{1/2} e_1 (tridiag_sqrt.cuh); stop test
-__global__ void blz_sqrt_kernel(int m, int max_iter, double tol, int mdim, const double* __restrict__ H,
+__global__ void blz_sqrt_kernel(int m, int max_iter, double tol, int mdim, const SqrtNode* __restrict__ nodes,
+                                const double* __restrict__ H,
                                 const double* __restrict__ nrm2, const double* __restrict__ W2,
                                 double* __restrict__ alpha, double* __restrict__ beta, double* __restrict__ c,
                                 double* __restrict__ cprev, double* __restrict__ change, int* __restrict__ active,
@@ -128,7 +129,7 @@ __global__ void blz_sqrt_kernel(int m, int max_iter, double tol, int mdim, const
     }
     __syncwarp();
     double* cs = c + s * mdim;
-    tridiag_sqrt_e1(m1, al, be, sm, cs);
+    tridiag_sqrt_e1(m1, nodes, al, be, sm, cs);
     double nc = 0.0, nd = 0.0;
     double* cp = cprev + s * mdim;
     for (int i = lane; i < m1; i += 32) {
@@ -249,7 +250,8 @@ static int blz_body(rpbd_handle* h, int n_sys, const int64_t* off, int64_t n, co
         seg_dot_kernel<<<dim3(n_sys, 1), 256, 0, st>>>(n, B.doff, B.w, 0, B.w, B.nrm2, 1, B.active);
         count_launch();
         const int m1 = m + 1;
-        blz_sqrt_kernel<<<n_sys, 32, tridiag_sqrt_smem_doubles(m1) * sizeof(double), st>>>(m, max_iter, tol, mdim, B.H1, B.nrm2, B.W2,
+        blz_sqrt_kernel<<<n_sys, 32, tridiag_sqrt_smem_doubles(m1) * sizeof(double), st>>>(m, max_iter, tol, mdim,
+                                                                         (const SqrtNode*)h->sqrt_nodes, B.H1, B.nrm2, B.W2,
                                                                          B.alpha, B.beta, B.c, B.cprev, B.change,
                                                                          B.active, B.iters);
         count_launch();

@@ -414,7 +414,7 @@ __global__ void gmres_start_kernel(int mdim, const double* __restrict__ nrm2, do
 // v_{m+1}, and in one block more alpha_m = h[m], beta_m = |w|, c = T^{1/2} e_1 of
 // the (m+1) x (m+1) tridiagonal T (tridiag_sqrt.cuh, its shared memory) and the
 // change |c - [c_prev; 0]| / |c|; nv = m + 1.  host: |w|^2, change
-__global__ void lanczos_finish_kernel(int64_t len, int slice, OrthoBatch B)
+__global__ void lanczos_finish_kernel(int64_t len, int slice, const SqrtNode* nodes, OrthoBatch B)
 {
     extern __shared__ double sm[];
     pdl_wait();
@@ -434,7 +434,7 @@ __global__ void lanczos_finish_kernel(int64_t len, int slice, OrthoBatch B)
         P.beta[m1 - 1] = nv;
     }
     __syncwarp();
-    tridiag_sqrt_e1(m1, P.alpha, P.beta, sm, P.c);
+    tridiag_sqrt_e1(m1, nodes, P.alpha, P.beta, sm, P.c);
     double nc = 0.0, nd = 0.0;
     for (int i = lane; i < m1; i += 32) {
         const double v = P.c[i];
@@ -627,7 +627,8 @@ int lanczos_multi_impl(rpbd_handle* h, int64_t n, const double* r, int nsys, con
         }
         const OrthoGrid G = launch_ortho(len, k, B, st);
         launch_pdl(lanczos_finish_kernel, dim3((unsigned)G.blocks + 1, (unsigned)k), 256,
-                   tridiag_sqrt_smem_doubles(mmax) * sizeof(double), st, len, G.slice, B);
+                   tridiag_sqrt_smem_doubles(mmax) * sizeof(double), st, len, G.slice,
+                   (const SqrtNode*)h->sqrt_nodes, B);
         count_launch();
         RPBD_LAUNCH_CHECK(h);
         RPBD_CU(h, cudaStreamSynchronize(st));

@@ -108,6 +108,8 @@ struct rpbd_handle {
     double* host_small = nullptr;
     // device error flag (bounded waits in kernels)
     int* dev_flag = nullptr;
+    // the Lanczos square root's quadrature nodes (tridiag_sqrt.cuh), written once
+    void* sqrt_nodes = nullptr;
     // pair-kernel timing
     bool profile = false;
     std::vector<rpbd::ProfRec> prof;

@@ -10,12 +10,13 @@
 // per lane, is below 1e-16 up to hi/lo = 1e6, and 64, two per lane, up to 1e12.
 // Each node is one tridiagonal solve (T + t^2) z = T e_1 (no cancellation), so the
 // chain is ~2 m steps; Jacobi needs 5-6 sweeps of ~m dependent rounds (129 us per
-// call, mean over the iterations of a time step, now 39 us, and 1e-16 instead of
-// 1e-15 off at condition 1e4).  hi is Gershgorin's bound; lo the largest of 32
-// trial shifts hi 2^{-47 j/32} with T - shift positive definite.  The elliptic
-// functions come from the arithmetic-geometric mean and Gauss' transformation
-// (Abramowitz & Stegun 16.12, 17.6), nodes beyond K'/2 from those below by
-// sc(K' - u) = 1 / (k sc(u)).
+// call, mean over the iterations of a time step, against 39 for the quadrature
+// with everything on the device, and 1e-15 instead of 1e-16 off at condition 1e4).  hi is Gershgorin's bound; lo the largest of 32
+// trial shifts hi 2^{-47 j/32} with T - shift positive definite.  The shifts' and
+// weights' ratios to hi and sqrt(hi) depend on j alone: a table of 32 KB that the
+// host fills once (sqrt_nodes), since one FP64 operation after another takes the
+// warp ~0.04 us (with the elliptic functions on the device 21.6 us of a Lanczos
+// iteration at 7 vectors, now 10.3).
 //
 // Otherwise (an eigenvalue below ~1e-14 of the largest, or negative) T is
 // diagonalised by cyclic Jacobi, T = Q diag(lambda) Q^T, and
@@ -31,6 +32,8 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "wall_rpy.cuh"
 
 namespace rpbd {
@@ -44,9 +47,59 @@ __host__ __device__ inline int tridiag_sqrt_smem_doubles(int m1)
     return jacobi > quad ? jacobi : quad;
 }
 
+constexpr int SQRT_TRIALS = 32, SQRT_NODES = 64;
+struct SqrtNode {
+    double shift, weight;  // over hi, over sqrt(hi)
+};
+// lo / hi of trial j; with 32 nodes from this ratio on, below it with 64
+__host__ __device__ constexpr bool sqrt_32_nodes(double ratio) { return ratio >= 1e-6; }
+
+// SQRT_TRIALS rows of SQRT_NODES nodes, then one of the trials' ratios (as shifts).
+// The elliptic functions sc, dn for modulus k', k = sqrt(lo / hi), from the
+// arithmetic-geometric mean and Gauss' transformation (Abramowitz & Stegun 16.12,
+// 17.6), nodes beyond K'/2 from those below by sc(K' - u) = 1 / (k sc(u)).
+constexpr int SQRT_TABLE = (SQRT_TRIALS + 1) * SQRT_NODES;
+inline void sqrt_nodes(SqrtNode* t)
+{
+    for (int i = 0; i < SQRT_TABLE; ++i) t[i] = SqrtNode{0.0, 0.0};
+    const double pi = 3.14159265358979323846;
+    for (int j = 0; j < SQRT_TRIALS; ++j) {
+        const double ratio = std::exp2(-47.0 / SQRT_TRIALS * (SQRT_TRIALS - j)), k = std::sqrt(ratio);
+        t[SQRT_TRIALS * SQRT_NODES + j].shift = ratio;
+        double a = 1.0, b = k, km[12], kc[12];  // modulus after n + 1 steps, and one minus it
+        int steps = 0;
+        while (steps < 12 && a - b > 1e-15 * a) {
+            const double an = 0.5 * (a + b), cn = 0.5 * (a - b);
+            km[steps] = cn / an;
+            kc[steps++] = b / an;
+            b = std::sqrt(a * b);
+            a = an;
+        }
+        const double Kp = 0.5 * pi / a;
+        const int N = sqrt_32_nodes(ratio) ? 32 : 64;
+        for (int i = 0; i < N; ++i) {
+            const int ii = i < N / 2 ? i : N - 1 - i;
+            const double u = (ii + 0.5) * Kp / N;
+            double sn = std::sin(u * a), cn = std::cos(u * a), dn = 1.0;  // a = the mean: u divided by every 1 + km
+            for (int n = steps - 1; n >= 0; --n) {
+                const double q = 1.0 + km[n] * sn * sn, p = kc[n] + km[n] * cn * cn;  // p = 2 - q, without the cancellation
+                cn = cn * dn / q;
+                sn = (1.0 + km[n]) * sn / q;
+                dn = p / q;
+            }
+            double sc = sn / cn, w = dn / (cn * cn);
+            if (i != ii) {
+                w /= k * sc * sc;
+                sc = 1.0 / (k * sc);
+            }
+            t[j * SQRT_NODES + i] = SqrtNode{ratio * sc * sc, w * 2.0 * Kp * k / (pi * N)};
+        }
+    }
+}
+
 // the quadrature; false (nothing written) when T is not safely positive definite
-__device__ inline bool tridiag_sqrt_quadrature(int m1, const double* __restrict__ alpha, const double* __restrict__ beta,
-                                               double* sm, double* __restrict__ c)
+__device__ inline bool tridiag_sqrt_quadrature(int m1, const SqrtNode* __restrict__ nodes,
+                                               const double* __restrict__ alpha, const double* __restrict__ beta, double* sm, double* __restrict__ c)
 {
     const int lane = threadIdx.x & 31;
     double* al = sm;            // m1
@@ -68,64 +121,31 @@ __device__ inline bool tridiag_sqrt_quadrature(int m1, const double* __restrict_
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
     if (!__all_sync(0xffffffffu, fine)) return false;
-    // T - x positive definite? (pivots of L D L^T), lane 0: x = hi 2^-47
-    const double x = hi * exp2(-47.0 / 32.0 * (32 - lane));
+    // T - x positive definite? (pivots of L D L^T)
+    const double ratio = nodes[SQRT_TRIALS * SQRT_NODES + lane].shift, x = hi * ratio;
     {
         double d = al[0] - x;
         bool pos = d > 1e-280;
         for (int i = 1; i < m1; ++i) {
-            d = al[i] - x - be[i - 1] * be[i - 1] * rcp3(d);  // (0, tiny or NaN pivots: not positive)
+            d = fma(-(be[i - 1] * be[i - 1]), rcp3(d), al[i] - x);  // (0, tiny or NaN pivots: not positive)
             pos = pos && d > 1e-280 && d < 1e300;
         }
         const unsigned ok = __ballot_sync(0xffffffffu, pos);
         if (!(ok & 1u)) return false;
         hi = __shfl_sync(0xffffffffu, hi, 0);
         const int best = __popc(ok & ~(ok + 1u)) - 1;  // last of the leading run of lanes
-        const double lo = __shfl_sync(0xffffffffu, x, best);
-        // K' and Gauss' transformation for modulus k' (complement k = sqrt(lo / hi))
-        const double k = sqrt(lo / hi);
-        double a = 1.0, b = k, km[12];  // km[n]: modulus after n + 1 steps
-        int steps = 0;
-#pragma unroll
-        for (int n = 0; n < 12; ++n) {
-            km[n] = 0.0;
-            if (a - b > 1e-15 * a) {  // (uniform)
-                const double an = 0.5 * (a + b), cn = 0.5 * (a - b);
-                b = a * b * rsqrt3(a * b);
-                a = an;
-                km[n] = cn / an;
-                steps = n + 1;
-            }
-        }
-        const double Kp = 1.5707963267948966 / a;
-        const int N = hi <= 1e6 * lo ? 32 : 64;
+        const int N = sqrt_32_nodes(__shfl_sync(0xffffffffu, ratio, best)) ? 32 : 64;
         double ci = 0.0, cj = 0.0, ck = 0.0;  // components lane, lane + 32, lane + 64
         for (int half = 0; half < N / 32; ++half) {
-            const int j = lane + 32 * half, jj = j < N / 2 ? j : N - 1 - j;
-            double u = (jj + 0.5) * Kp / N, sn, cn, dn = 1.0;
-            sincos(u * a, &sn, &cn);  // a = the mean: u divided by every 1 + km
-#pragma unroll
-            for (int n = 11; n >= 0; --n)
-                if (n < steps) {
-                    const double t = km[n] * sn * sn, rr = rcp3(1.0 + t);
-                    cn = cn * dn * rr;
-                    sn = (1.0 + km[n]) * sn * rr;
-                    dn = (1.0 - t) * rr;
-                }
-            double sc = sn / cn, w = dn / (cn * cn);
-            if (j != jj) {
-                w /= k * sc * sc;
-                sc = 1.0 / (k * sc);
-            }
-            w *= 2.0 * Kp * sqrt(lo) / (3.14159265358979323846 * N);
-            const double sig = lo * sc * sc;
+            const SqrtNode nd = nodes[best * SQRT_NODES + 32 * half + lane];
+            const double sig = hi * nd.shift, w = sqrt(hi) * nd.weight;
             // (T + sig) z = T e_1
             double di = rcp3(al[0] + sig), yi = al[0];
             dinv[lane] = di;
             y[lane] = yi;
             for (int i = 1; i < m1; ++i) {
                 const double bb = be[i - 1], l = bb * di;
-                di = rcp3(al[i] + sig - l * bb);
+                di = rcp3(fma(-(bb * bb), di, al[i] + sig));
                 yi = (i == 1 ? bb : 0.0) - l * yi;
                 dinv[i * 32 + lane] = di;
                 y[i * 32 + lane] = yi;
@@ -152,15 +172,15 @@ __device__ inline bool tridiag_sqrt_quadrature(int m1, const double* __restrict_
     return true;
 }
 
-// One warp (all 32 lanes call it).  sm: tridiag_sqrt_smem_doubles(m1)
+// One warp (all 32 lanes call it).  nodes: the table of sqrt_nodes(); sm: tridiag_sqrt_smem_doubles(m1)
 // doubles of shared memory; m1 <= 2 * TRIDIAG_MAX_PAIRS.  On return c[i]
 // (global or shared, i < m1) holds T^{1/2} e_1; the return value is valid
 // in every lane.
-__device__ inline void tridiag_sqrt_e1(int m1, const double* __restrict__ alpha, const double* __restrict__ beta,
-                                       double* sm, double* __restrict__ c)
+__device__ inline void tridiag_sqrt_e1(int m1, const SqrtNode* __restrict__ nodes, const double* __restrict__ alpha,
+                                       const double* __restrict__ beta, double* sm, double* __restrict__ c)
 {
     const int lane = threadIdx.x & 31;
-    if (tridiag_sqrt_quadrature(m1, alpha, beta, sm, c)) return;
+    if (tridiag_sqrt_quadrature(m1, nodes, alpha, beta, sm, c)) return;
     double* A = sm;                    // m1 x m1, row-major
     double* Q = A + m1 * m1;           // eigenvectors (columns)
     double* rc = Q + m1 * m1;          // per pair: cos, sin, t, apq, app, aqq

@@ -179,3 +179,17 @@ def test_saddle_solve_by_blobs_per_body(nper):
     lam, U, st = h.gmres_rigid_solve(nper, to_dev(r), to_dev(q), to_dev(slip), to_dev(FT), tol=1e-12, max_iter=200)
     assert st["status"] == 0
     assert rel2(U.cpu().numpy(), U_d) <= 1e-9 and rel2(lam.cpu().numpy(), lam_d) <= 1e-8
+
+
+@pytest.mark.parametrize("gap", [1.0, 1e-3, 1e-5, 1e-7, 1e-10])
+def test_lanczos_root_by_condition(gap):
+    """Two blobs a distance gap a apart (the smallest eigenvalue is proportional to it) among four others, run to the
+    full space: 32 quadrature nodes, 64, and the diagonalisation.  Rounding of M moves the root by ~1e-16 sqrt(condition)."""
+    a = synth.A_BOOMERANG
+    r = a * np.array([[0, 0, 2], [gap, 0, 2], [3, 1, 3], [0, 4, 2.5], [5, 5, 4], [-3, 2, 2]], float).T
+    W = synth.gaussian(790, r.shape)
+    lam, Q = np.linalg.eigh(om.dense(r, om.Params(synth.ETA, a)))
+    ref = om.blob_to_soa(Q @ (np.sqrt(np.maximum(lam, 0)) * (Q.T @ om.soa_to_blob(W))))
+    h = Handle(synth.ETA, a, synth.KT)
+    out, _ = h.lanczos_sqrt_apply(to_dev(r), to_dev(W), tol=1e-14, max_iter=18, use_precond=False)
+    assert rel2(out.cpu().numpy(), ref) <= 1e-9
