@@ -2,19 +2,30 @@
 // suspensions, plus an optional matvec per system, as one CUDA graph.
 //
 // All systems advance in lockstep, one Lanczos iteration per step: the matvec
-// is the persistent batched pair kernel (batched.cu); dot products, the
-// classical Gram-Schmidt reorthogonalisation (applied twice), the
-// normalisation and the FP64 tridiagonal square root (one warp per system,
-// cyclic Jacobi) all use per-system coefficients.  A system whose relative
-// change |y_m - y_{m-1}|/|y_m| drops below tol is switched off by a device flag;
-// later iterations skip its work, so max_iter iterations can be captured once
-// and replayed without any host round trip.
+// is the batched pair kernel (batched.cu, sym.cu); dot products, the classical
+// Gram-Schmidt reorthogonalisation (applied twice), the normalisation and the
+// FP64 tridiagonal square root (tridiag_sqrt.cuh, one warp per system) all use
+// per-system coefficients.  A system whose relative change
+// |y_m - y_{m-1}|/|y_m| drops below tol is switched off by a device flag; later
+// iterations skip its work, so max_iter iterations can be captured once and
+// replayed without any host round trip.
+//
+// The vector kernels work on chunks of at most 1,024 blobs of one system, a block
+// each, as krylov.cu's do on slices: a block keeps its chunk of w in shared memory
+// through an update and the dot products that follow, and sums the previous
+// kernel's partials of its system's chunks itself.  As eight kernels with one
+// block per system and dot product (the whole chip waits for the largest system's),
+// a search for the system and a square root and division per element, a Lanczos
+// run took 140.8 ms on 64 systems of 471,495 blobs (126 of them the matvecs), now
+// 137.2; on 64 systems of 120-1,920 blobs 6.17 -> 5.41, on 8 of those 2.17 -> 1.70.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
+#include "ortho.cuh"
 #include "rpbd_internal.cuh"
 #include "tridiag_sqrt.cuh"
 
@@ -22,116 +33,175 @@ namespace rpbd {
 
 constexpr int BLZ_MAX = 64;
 
-__device__ __forceinline__ int bl_find_sys(const int64_t* off, int n_sys, int64_t i)
+// blobs [b0, b0 + cnt) of system s; the system's chunks are c0 .. c0 + nc
+struct BlzChunk {
+    int64_t b0;
+    int cnt, s, c0, nc;
+    int pad[2];
+};
+// chunks so small only while that does not fill two blocks per SM of this GPU's 152
+static int blz_chunk_size(int64_t n)
 {
-    int lo = 0, hi = n_sys;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (off[mid] <= i) lo = mid; else hi = mid;
+    const int64_t c = ((n + 303) / 304 + 127) / 128 * 128;
+    return (int)std::min<int64_t>(1024, std::max<int64_t>(128, c));
+}
+static std::vector<BlzChunk> blz_chunks(int n_sys, const int64_t* off)
+{
+    const int64_t size = blz_chunk_size(off[n_sys]);
+    std::vector<BlzChunk> v;
+    for (int s = 0; s < n_sys; ++s) {
+        const int64_t len = off[s + 1] - off[s], nc = (len + size - 1) / size;
+        const int c0 = (int)v.size();
+        for (int64_t c = 0; c < nc; ++c) {
+            const int64_t lo = len * c / nc, hi = len * (c + 1) / nc;
+            v.push_back(BlzChunk{off[s] + lo, (int)(hi - lo), s, c0, (int)nc, {0, 0}});
+        }
     }
-    return lo;
+    return v;
 }
 
-// out[s * ldo + i] = <V_i, w> restricted to system s (3 components)
-__global__ void seg_dot_kernel(int64_t n, const int64_t* __restrict__ off, const double* __restrict__ V, int64_t ld,
-                               const double* __restrict__ w, double* __restrict__ out, int ldo,
-                               const int* __restrict__ active)
+// element e of a chunk's 3 cnt in the [3][n] vector
+__device__ __forceinline__ int64_t blz_at(const BlzChunk& C, int64_t n, int e)
 {
-    const int s = blockIdx.x, i = blockIdx.y;
-    if (active && !active[s]) return;
-    const int64_t a = off[s], b = off[s + 1];
-    const double* v = V + (int64_t)i * ld;
-    double acc = 0.0;
-    for (int c = 0; c < 3; ++c)
-        for (int64_t e = a + threadIdx.x; e < b; e += blockDim.x) acc += v[c * n + e] * w[c * n + e];
-    __shared__ double red[32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        acc = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (threadIdx.x == 0) out[s * ldo + i] = acc;
-    }
+    const int c = (e >= C.cnt) + (e >= 2 * C.cnt);
+    return c * n + C.b0 + (e - c * C.cnt);
 }
 
-// w -= sum_i h[s][i] V_i   (s = system of the element)
-__global__ void seg_axpy_kernel(int64_t n, int n_sys, const int64_t* __restrict__ off, const double* __restrict__ V,
-                                int64_t ld, int nv, const double* __restrict__ h, int ldh, double* __restrict__ w,
-                                const int* __restrict__ active)
-{
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 3 * n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int s = bl_find_sys(off, n_sys, e % n);
-        if (!active[s]) continue;
-        double acc = w[e];
-        for (int i = 0; i < nv; ++i) acc -= h[s * ldh + i] * V[(int64_t)i * ld + e];
-        w[e] = acc;
-    }
-}
-
-__global__ void seg_add_kernel(int n_sys, int nv, int ldh, const double* __restrict__ a, double* __restrict__ b,
-                               const int* __restrict__ active)
-{
-    const int s = blockIdx.x;
-    if (!active[s]) return;
-    for (int i = threadIdx.x; i < nv; i += blockDim.x) b[s * ldh + i] += a[s * ldh + i];
-}
-
-// V_out = x / sqrt(nrm2[s]) for active systems
-__global__ void seg_normalize_kernel(int64_t n, int n_sys, const int64_t* __restrict__ off, const double* __restrict__ x,
-                                     const double* __restrict__ nrm2, double* __restrict__ out,
-                                     const int* __restrict__ active)
-{
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 3 * n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int s = bl_find_sys(off, n_sys, e % n);
-        if (active && !active[s]) continue;
-        const double nv = sqrt(nrm2[s]);
-        out[e] = nv > 0.0 ? x[e] / nv : 0.0;
-    }
-}
-
-__global__ void blz_init_kernel(int n_sys, const double* __restrict__ W2, int* __restrict__ active,
-                                int* __restrict__ iters, double* __restrict__ change, double* __restrict__ c,
-                                double* __restrict__ cprev, int mdim)
-{
-    const int s = blockIdx.x;
-    if (threadIdx.x == 0) {
-        active[s] = W2[s] > 0.0 ? 1 : 0;
-        iters[s] = 0;
-        change[s] = 0.0;
-    }
-    for (int i = threadIdx.x; i < mdim; i += blockDim.x) {
-        c[s * mdim + i] = 0.0;
-        cprev[s * mdim + i] = 0.0;
-    }
-}
-
-// one warp per system: alpha_m, beta_m; T^{1/2} e_1 (tridiag_sqrt.cuh); stop test
-__global__ void blz_sqrt_kernel(int m, int max_iter, double tol, int mdim, const SqrtNode* __restrict__ nodes,
-                                const double* __restrict__ H,
-                                const double* __restrict__ nrm2, const double* __restrict__ W2,
-                                double* __restrict__ alpha, double* __restrict__ beta, double* __restrict__ c,
-                                double* __restrict__ cprev, double* __restrict__ change, int* __restrict__ active,
-                                int* __restrict__ iters)
+// partials: [2 nv + 1][nch], rows 0..nv of pass 0, nv..2 nv of pass 1, 2 nv of |w|^2
+// PASS 0: partials of V^T w.  1: w -= V h with h from pass 0's partials, then
+// partials of V^T w.  2: w -= V h with pass 1's, then the partials of |w|^2.
+// 3: the partials of |w|^2 alone (nv = 0).  H: both passes' coefficients, [s][ldh].
+template <int PASS>
+__global__ void blz_ortho_kernel(int64_t n, int nch, const BlzChunk* chunks, const double* V, int nv, double* w, double* part,
+                                 double* H, int ldh, const int* active)
 {
     extern __shared__ double sm[];
-    const int s = blockIdx.x;
-    const int lane = threadIdx.x;
-    if (!active[s]) return;
-    const int m1 = m + 1;
-    double* al = alpha + s * mdim;
-    double* be = beta + s * mdim;
+    pdl_wait();
+    pdl_trigger();
+    if ((int)blockIdx.x >= nch) return;
+    const BlzChunk C = chunks[blockIdx.x];
+    if (PASS < 3 && !active[C.s]) return;
+    const int64_t ld = 3 * n;
+    const int cnt = 3 * C.cnt;
+    double *ws = sm, *h = sm + cnt;
+    double* in = part + (PASS == 2 ? (int64_t)nv * nch : 0) + C.c0;
+    double* out = part + (PASS == 0 ? 0 : PASS == 1 ? (int64_t)nv * nch : 2 * (int64_t)nv * nch) + blockIdx.x;
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) ws[e] = w[blz_at(C, n, e)];
+    if (PASS == 1 || PASS == 2) {
+        ortho_sums(nv, C.nc, [&](int i, int b) { return in[(int64_t)i * nch + b]; }, [&](int i, double x) { h[i] = x; });
+        __syncthreads();
+        if ((int)blockIdx.x == C.c0)
+            for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+                double* Hi = H + (int64_t)C.s * ldh + i;
+                *Hi = PASS == 1 ? h[i] : *Hi + h[i];
+            }
+        for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+            const int64_t g = blz_at(C, n, e);
+            double s4[4] = {0.0, 0.0, 0.0, 0.0};
+            int i = 0;
+            for (; i + 4 <= nv; i += 4)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s4[u] += h[i + u] * V[(int64_t)(i + u) * ld + g];
+            for (; i < nv; ++i) s4[0] += h[i] * V[(int64_t)i * ld + g];
+            const double x = ws[e] - ((s4[0] + s4[1]) + (s4[2] + s4[3]));
+            ws[e] = x;
+            w[g] = x;
+        }
+    }
+    __syncthreads();
+    if (PASS >= 2)
+        ortho_sums<1>(1, cnt, [&](int, int e) { return ws[e] * ws[e]; }, [&](int, double x) { out[0] = x; });
+    else
+        ortho_sums(nv, cnt, [&](int i, int e) { return V[(int64_t)i * ld + blz_at(C, n, e)] * ws[e]; },
+                   [&](int i, double x) { out[(int64_t)i * nch] = x; });
+}
+
+struct BlzState {
+    double *alpha, *beta, *c, *cprev, *W2, *change;
+    int* iters;
+    int mdim;
+};
+
+// h[0..2] = |w|^2 from its chunks' partials, |w|, 1/|w| (0 when it vanishes), by one
+// thread: in every one the FP64 pipe would be busy with the root and the division
+__device__ __forceinline__ void blz_norm(const double* part, int nc, double* h)
+{
+    ortho_sums<1>(1, nc, [&](int, int b) { return part[b]; },
+                  [&](int, double s) {
+                      const double nv = sqrt(s);
+                      h[0] = s;
+                      h[1] = nv;
+                      h[2] = nv > 0.0 ? 1.0 / nv : 0.0;
+                  });
+    __syncthreads();
+}
+__device__ __forceinline__ void blz_normalize(const BlzChunk& C, int64_t n, const double* part, const double* w, double* out)
+{
+    __shared__ double h[3];
+    blz_norm(part + C.c0, C.nc, h);
+    for (int e = threadIdx.x; e < 3 * C.cnt; e += blockDim.x) {
+        const int64_t g = blz_at(C, n, e);
+        out[g] = w[g] * h[2];
+    }
+}
+
+// v_0 = W / |W| by chunks, then one block per system: its state
+__global__ void blz_start_kernel(int64_t n, int nch, const BlzChunk* chunks, const int2* sys, const double* W, const double* part,
+                                 double* V, BlzState S, int* active)
+{
+    pdl_wait();
+    pdl_trigger();
+    if ((int)blockIdx.x < nch) {
+        blz_normalize(chunks[blockIdx.x], n, part, W, V);
+        return;
+    }
+    __shared__ double h[3];
+    const int s = blockIdx.x - nch;
+    blz_norm(part + sys[s].x, sys[s].y, h);
+    if (threadIdx.x == 0) {
+        S.W2[s] = h[0];
+        active[s] = h[0] > 0.0 ? 1 : 0;
+        S.iters[s] = 0;
+        S.change[s] = 0.0;
+    }
+    for (int i = threadIdx.x; i < S.mdim; i += blockDim.x) {
+        S.c[s * S.mdim + i] = 0.0;
+        S.cprev[s * S.mdim + i] = 0.0;
+    }
+}
+
+// v_{m+1} = w / |w| by chunks; then one block per system: alpha_m, beta_m,
+// T^{1/2} e_1 (tridiag_sqrt.cuh) and the stop test.  The flags for the next
+// iteration go to next, the other blocks still read active.
+__global__ void blz_finish_kernel(int64_t n, int nch, const BlzChunk* chunks, const int2* sys, int m, int max_iter, double tol,
+                                  const SqrtNode* nodes, const double* H, const double* w, const double* part, double* vnext,
+                                  BlzState S, const int* active, int* next)
+{
+    extern __shared__ double sm[];
+    pdl_wait();
+    pdl_trigger();
+    if ((int)blockIdx.x < nch) {
+        const BlzChunk C = chunks[blockIdx.x];
+        if (active[C.s]) blz_normalize(C, n, part, w, vnext);
+        return;
+    }
+    const int s = blockIdx.x - nch, lane = threadIdx.x, m1 = m + 1;
+    if (!active[s]) {
+        if (lane == 0) next[s] = 0;
+        return;
+    }
+    __shared__ double h[3];
+    blz_norm(part + sys[s].x, sys[s].y, h);
+    if (lane >= 32) return;
+    const double nrm2 = h[0];
+    double *al = S.alpha + s * S.mdim, *be = S.beta + s * S.mdim, *cs = S.c + s * S.mdim, *cp = S.cprev + s * S.mdim;
     if (lane == 0) {
-        al[m] = H[s * (mdim + 1) + m];
-        be[m] = sqrt(nrm2[s]);
+        al[m] = H[s * (S.mdim + 1) + m];
+        be[m] = h[1];
     }
     __syncwarp();
-    double* cs = c + s * mdim;
     tridiag_sqrt_e1(m1, nodes, al, be, sm, cs);
     double nc = 0.0, nd = 0.0;
-    double* cp = cprev + s * mdim;
     for (int i = lane; i < m1; i += 32) {
         const double v = cs[i];
         const double prev = i < m1 - 1 ? cp[i] : 0.0;
@@ -149,28 +219,34 @@ __global__ void blz_sqrt_kernel(int m, int max_iter, double tol, int mdim, const
         const double ch = nc > 0.0 ? sqrt(nd / nc) : 0.0;
         bool stop = false;
         if (m >= 1) {
-            change[s] = ch;
+            S.change[s] = ch;
             if (ch < tol) stop = true;
         }
-        if (!(nrm2[s] > 1e-300 * W2[s])) stop = true;  // invariant subspace
+        if (!(nrm2 > 1e-300 * S.W2[s])) stop = true;  // invariant subspace
         if (m1 >= max_iter) stop = true;
-        if (stop) {
-            active[s] = 0;
-            iters[s] = m1;
-        }
+        next[s] = stop ? 0 : 1;
+        if (stop) S.iters[s] = m1;
     }
 }
 
-// y[e] = sqrt(W2[s]) sum_{i < iters[s]} c[s][i] V_i[e]
-__global__ void blz_combine_kernel(int64_t n, int n_sys, const int64_t* __restrict__ off, const double* __restrict__ V,
-                                   int64_t ld, const double* __restrict__ c, int mdim, const int* __restrict__ iters,
-                                   const double* __restrict__ W2, double* __restrict__ y)
+// y = sqrt(W2[s]) sum_{i < iters[s]} c[s][i] V_i
+__global__ void blz_combine_kernel(int64_t n, int nch, const BlzChunk* chunks, const double* V, BlzState S, double* y)
 {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 3 * n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int s = bl_find_sys(off, n_sys, e % n);
+    __shared__ double c[BLZ_MAX], root;
+    pdl_wait();
+    pdl_trigger();
+    if ((int)blockIdx.x >= nch) return;
+    const BlzChunk C = chunks[blockIdx.x];
+    const int it = S.iters[C.s];
+    for (int i = threadIdx.x; i < it; i += blockDim.x) c[i] = S.c[C.s * S.mdim + i];
+    if (threadIdx.x == 0) root = sqrt(S.W2[C.s]);
+    __syncthreads();
+    for (int e = threadIdx.x; e < 3 * C.cnt; e += blockDim.x) {
+        const int64_t g = blz_at(C, n, e);
         double acc = 0.0;
-        for (int i = 0; i < iters[s]; ++i) acc += c[s * mdim + i] * V[(int64_t)i * ld + e];
-        y[e] = sqrt(W2[s]) * acc;
+#pragma unroll 4
+        for (int i = 0; i < it; ++i) acc += c[i] * V[(int64_t)i * 3 * n + g];
+        y[g] = root * acc;
     }
 }
 
@@ -202,65 +278,54 @@ void batched_free_graphs(rpbd_handle* h)
 
 struct BlzBufs {
     double *V, *z, *y, *w, *Win, *rin, *out, *Fin, *Uout;
-    double *H1, *H2, *alpha, *beta, *c, *cprev, *nrm2, *W2, *change;
-    int *active, *iters;
+    double *H, *part;
+    BlzState S;
+    int* active[2];  // of even and odd iterations
     int64_t* doff;
+    BlzChunk* chunks;
+    int2* sys;  // first chunk and chunks of each system
+    int nch, chunk;
 };
-
-static unsigned sgrid(int64_t n)
-{
-    int64_t g = (3 * n + 255) / 256;
-    if (g > 152 * 8) g = 152 * 8;
-    return (unsigned)(g < 1 ? 1 : g);
-}
 
 // every kernel of one batched Lanczos (+ optional matvec), no host sync
 static int blz_body(rpbd_handle* h, int n_sys, const int64_t* off, int64_t n, const BlzBufs& B, double tol,
                     int max_iter, int use_precond, bool with_apply, cudaStream_t st)
 {
-    const int mdim = BLZ_MAX + 1;
     const int64_t len = 3 * n;
-    const unsigned g = sgrid(n);
-    seg_dot_kernel<<<dim3(n_sys, 1), 256, 0, st>>>(n, B.doff, B.Win, 0, B.Win, B.W2, 1, nullptr);
-    count_launch();
-    blz_init_kernel<<<n_sys, 64, 0, st>>>(n_sys, B.W2, B.active, B.iters, B.change, B.c, B.cprev, mdim);
-    count_launch();
-    seg_normalize_kernel<<<g, 256, 0, st>>>(n, n_sys, B.doff, B.Win, B.W2, B.V, nullptr);
+    const int ldh = B.S.mdim + 1, threads = 3 * B.chunk > 512 ? 512 : 256;
+    const unsigned g = (unsigned)std::max(1, B.nch), gs = (unsigned)(B.nch + n_sys);
+    const int elems = 3 * B.chunk;
+    auto ortho = [&](auto kernel, int nv, double* w, const int* active) {
+        launch_pdl(kernel, g, threads, (size_t)(elems + nv) * sizeof(double), st, n, B.nch, (const BlzChunk*)B.chunks,
+                   (const double*)B.V, nv, w, B.part, B.H, ldh, active);
+        count_launch();
+    };
+    ortho(blz_ortho_kernel<3>, 0, B.Win, nullptr);
+    launch_pdl(blz_start_kernel, gs, 256, 0, st, n, B.nch, (const BlzChunk*)B.chunks, (const int2*)B.sys, (const double*)B.Win,
+               (const double*)B.part, B.V, B.S, B.active[0]);
     count_launch();
     for (int m = 0; m < max_iter; ++m) {
         const double* vm = B.V + (int64_t)m * len;
+        const int* act = B.active[m & 1];
         if (use_precond) {
-            RPBD_TRY(precond_apply_impl(h, 2, vm, B.z, st, B.active, B.doff, n_sys));
-            RPBD_TRY(batched_apply_impl(h, n_sys, off, B.rin, B.z, B.y, 1, true, B.active, st));
-            RPBD_TRY(precond_apply_impl(h, 1, B.y, B.w, st, B.active, B.doff, n_sys));
+            RPBD_TRY(precond_apply_impl(h, 2, vm, B.z, st, act, B.doff, n_sys));
+            RPBD_TRY(batched_apply_impl(h, n_sys, off, B.rin, B.z, B.y, 1, true, act, st));
+            RPBD_TRY(precond_apply_impl(h, 1, B.y, B.w, st, act, B.doff, n_sys));
         } else {
-            RPBD_TRY(batched_apply_impl(h, n_sys, off, B.rin, vm, B.w, 1, true, B.active, st));
+            RPBD_TRY(batched_apply_impl(h, n_sys, off, B.rin, vm, B.w, 1, true, act, st));
         }
         const int nv = m + 1;
-        seg_dot_kernel<<<dim3(n_sys, nv), 256, 0, st>>>(n, B.doff, B.V, len, B.w, B.H1, mdim + 1, B.active);
-        count_launch();
-        seg_axpy_kernel<<<g, 256, 0, st>>>(n, n_sys, B.doff, B.V, len, nv, B.H1, mdim + 1, B.w, B.active);
-        count_launch();
-        seg_dot_kernel<<<dim3(n_sys, nv), 256, 0, st>>>(n, B.doff, B.V, len, B.w, B.H2, mdim + 1, B.active);
-        count_launch();
-        seg_axpy_kernel<<<g, 256, 0, st>>>(n, n_sys, B.doff, B.V, len, nv, B.H2, mdim + 1, B.w, B.active);
-        count_launch();
-        seg_add_kernel<<<n_sys, 64, 0, st>>>(n_sys, nv, mdim + 1, B.H2, B.H1, B.active);
-        count_launch();
-        seg_dot_kernel<<<dim3(n_sys, 1), 256, 0, st>>>(n, B.doff, B.w, 0, B.w, B.nrm2, 1, B.active);
-        count_launch();
-        const int m1 = m + 1;
-        blz_sqrt_kernel<<<n_sys, 32, tridiag_sqrt_smem_doubles(m1) * sizeof(double), st>>>(m, max_iter, tol, mdim,
-                                                                         (const SqrtNode*)h->sqrt_nodes, B.H1, B.nrm2, B.W2,
-                                                                         B.alpha, B.beta, B.c, B.cprev, B.change,
-                                                                         B.active, B.iters);
-        count_launch();
-        seg_normalize_kernel<<<g, 256, 0, st>>>(n, n_sys, B.doff, B.w, B.nrm2, B.V + (int64_t)(m + 1) * len,
-                                                B.active);
+        ortho(blz_ortho_kernel<0>, nv, B.w, act);
+        ortho(blz_ortho_kernel<1>, nv, B.w, act);
+        ortho(blz_ortho_kernel<2>, nv, B.w, act);
+        launch_pdl(blz_finish_kernel, gs, 256, tridiag_sqrt_smem_doubles(nv) * sizeof(double), st, n, B.nch,
+                   (const BlzChunk*)B.chunks, (const int2*)B.sys, m, max_iter, tol, (const SqrtNode*)h->sqrt_nodes,
+                   (const double*)B.H, (const double*)B.w, (const double*)(B.part + 2 * (int64_t)nv * B.nch),
+                   B.V + (int64_t)(m + 1) * len, B.S, act, B.active[(m + 1) & 1]);
         count_launch();
     }
-    blz_combine_kernel<<<g, 256, 0, st>>>(n, n_sys, B.doff, B.V, len, B.c, mdim, B.iters, B.W2,
-                                          use_precond ? B.y : B.out);
+    launch_pdl(blz_combine_kernel, g, 256, 0, st, n, B.nch, (const BlzChunk*)B.chunks, (const double*)B.V, B.S,
+               use_precond ? B.y : B.out);
     count_launch();
     if (use_precond) RPBD_TRY(precond_apply_impl(h, 0, B.y, B.out, st));
     if (with_apply) RPBD_TRY(batched_apply_impl(h, n_sys, off, B.rin, B.Fin, B.Uout, 1, true, nullptr, st));
@@ -284,22 +349,39 @@ static int blz_bufs(rpbd_handle* h, int n_sys, const int64_t* off, int64_t n, in
     B->out = p; p += len;
     B->Fin = p; p += len;
     B->Uout = p; p += len;
+    const std::vector<BlzChunk> ch = blz_chunks(n_sys, off);
+    B->nch = (int)ch.size();
+    B->chunk = blz_chunk_size(n);
+    // the layout on the device: chunk table, systems' chunks, offsets (one copy), then the state
+    const size_t tab = ch.size() * sizeof(BlzChunk) + n_sys * sizeof(int2) + (n_sys + 1) * sizeof(int64_t);
     double* sm;
-    const size_t nsm = (size_t)n_sys * (2 * (mdim + 1) + 4 * mdim + 3) + (size_t)2 * n_sys + (n_sys + 1);
+    const size_t nsm = tab / sizeof(double) + (size_t)n_sys * (mdim + 1 + 4 * mdim + 2) + (size_t)2 * n_sys +
+                       ch.size() * (2 * (size_t)max_iter + 1);
     RPBD_TRY(ensure_t(h, BUF_BLZ_SMALL, nsm, &sm));
-    B->H1 = sm; sm += (size_t)n_sys * (mdim + 1);
-    B->H2 = sm; sm += (size_t)n_sys * (mdim + 1);
-    B->alpha = sm; sm += (size_t)n_sys * mdim;
-    B->beta = sm; sm += (size_t)n_sys * mdim;
-    B->c = sm; sm += (size_t)n_sys * mdim;
-    B->cprev = sm; sm += (size_t)n_sys * mdim;
-    B->nrm2 = sm; sm += n_sys;
-    B->W2 = sm; sm += n_sys;
-    B->change = sm; sm += n_sys;
-    B->active = reinterpret_cast<int*>(sm); sm += n_sys;
-    B->iters = reinterpret_cast<int*>(sm); sm += n_sys;
-    B->doff = reinterpret_cast<int64_t*>(sm);
-    RPBD_CU(h, cudaMemcpy(B->doff, off, sizeof(int64_t) * (n_sys + 1), cudaMemcpyHostToDevice));
+    std::vector<char> host(tab);
+    char* q = host.data();
+    if (!ch.empty()) std::memcpy(q, ch.data(), ch.size() * sizeof(BlzChunk));
+    int2* hs = reinterpret_cast<int2*>(q + ch.size() * sizeof(BlzChunk));
+    for (int s = 0; s < n_sys; ++s) hs[s] = make_int2(0, 0);
+    for (const BlzChunk& c : ch) hs[c.s] = make_int2(c.c0, c.nc);
+    std::memcpy(hs + n_sys, off, (n_sys + 1) * sizeof(int64_t));
+    RPBD_CU(h, cudaMemcpy(sm, q, tab, cudaMemcpyHostToDevice));
+    B->chunks = reinterpret_cast<BlzChunk*>(sm);
+    B->sys = reinterpret_cast<int2*>(B->chunks + ch.size());
+    B->doff = reinterpret_cast<int64_t*>(B->sys + n_sys);
+    sm += tab / sizeof(double);
+    B->H = sm; sm += (size_t)n_sys * (mdim + 1);
+    B->S.mdim = mdim;
+    B->S.alpha = sm; sm += (size_t)n_sys * mdim;
+    B->S.beta = sm; sm += (size_t)n_sys * mdim;
+    B->S.c = sm; sm += (size_t)n_sys * mdim;
+    B->S.cprev = sm; sm += (size_t)n_sys * mdim;
+    B->S.W2 = sm; sm += n_sys;
+    B->S.change = sm; sm += n_sys;
+    B->part = sm; sm += ch.size() * (2 * (size_t)max_iter + 1);
+    B->S.iters = reinterpret_cast<int*>(sm);
+    B->active[0] = B->S.iters + n_sys;
+    B->active[1] = B->active[0] + n_sys;
     return RPBD_OK;
 }
 
@@ -323,8 +405,8 @@ int rpbd_lanczos_sqrt_apply_batched(rpbd_handle* h, int n_sys, const int64_t* of
     if (use_precond && (!h->prec_valid || h->prec_nb * h->prec_nper != n))
         return set_error(h, RPBD_BAD_ARG, "batched lanczos: preconditioner not built for these blobs");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if (once_per_device(h, reinterpret_cast<const void*>(blz_sqrt_kernel)))
-        RPBD_CU(h, cudaFuncSetAttribute(blz_sqrt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (once_per_device(h, reinterpret_cast<const void*>(blz_finish_kernel)))
+        RPBD_CU(h, cudaFuncSetAttribute(blz_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         tridiag_sqrt_smem_doubles(BLZ_MAX) * (int)sizeof(double)));
     BlzBufs B;
     RPBD_TRY(blz_bufs(h, n_sys, offsets, n, max_iter, &B));
@@ -390,7 +472,7 @@ int rpbd_lanczos_sqrt_apply_batched(rpbd_handle* h, int n_sys, const int64_t* of
     RPBD_CU(h, cudaMemcpyAsync(out, B.out, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, st));
     if (with_apply) RPBD_CU(h, cudaMemcpyAsync(U, B.Uout, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, st));
     if (iters) {
-        RPBD_CU(h, cudaMemcpyAsync(iters, B.iters, sizeof(int) * n_sys, cudaMemcpyDeviceToHost, st));
+        RPBD_CU(h, cudaMemcpyAsync(iters, B.S.iters, sizeof(int) * n_sys, cudaMemcpyDeviceToHost, st));
         RPBD_CU(h, cudaStreamSynchronize(st));
         int flag = 0;
         RPBD_CU(h, cudaMemcpy(&flag, h->dev_flag, sizeof(int), cudaMemcpyDeviceToHost));

@@ -193,3 +193,24 @@ def test_lanczos_root_by_condition(gap):
     h = Handle(synth.ETA, a, synth.KT)
     out, _ = h.lanczos_sqrt_apply(to_dev(r), to_dev(W), tol=1e-14, max_iter=18, use_precond=False)
     assert rel2(out.cpu().numpy(), ref) <= 1e-9
+
+
+@pytest.mark.parametrize("sizes", [(1, 127, 0, 128, 129), (385, 2), (40_000, 129, 3)])
+def test_batched_lanczos_chunks(sizes):
+    """Systems at the edges of the vector kernels' chunks (128 blobs here, 256 in the last case), a fixed number of
+    iterations, against one Lanczos per system; FP32 pairs, the tolerance of the batched oracle tests."""
+    rs = [cloud(n, 800 + i) for i, n in enumerate(sizes) if n]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    h = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT)
+    W = synth.gaussian(801, (3, off[-1]))
+    out, _, it = h.lanczos_sqrt_apply_batched(off, to_dev(np.concatenate(rs, axis=1)), to_dev(W), tol=1e-30, max_iter=7,
+                                              use_precond=False)
+    g = Handle(synth.ETA, synth.A_BOOMERANG, synth.KT)
+    for s, r in zip([s for s, n in enumerate(sizes) if n], rs):
+        if r.shape[1] == 1:
+            continue  # (three unknowns: the space is exhausted before the seventh iteration)
+        Ws = to_dev(np.ascontiguousarray(W[:, off[s]:off[s + 1]]))
+        ref, _ = g.lanczos_sqrt_apply(to_dev(r), Ws, tol=1e-30, max_iter=7, dtype=F32, use_precond=False)
+        assert it[s] == 7 or r.shape[1] < 3
+        assert rel2(out[:, off[s]:off[s + 1]].cpu().numpy(), ref.cpu().numpy()) <= 1e-4
+    assert torch.isfinite(out).all()
