@@ -23,15 +23,16 @@ namespace rpbd {
 
 // S from the largest finite |force| of the launch; in FP64, where the bound
 // stays finite for every finite FP32 force (S then lies within about
-// [-130, 210])
+// [-130, 210]).  Every thread of every CTA asks for it, and a warp's FP64
+// instruction holds an SM's pipe for ~19 cycles: the exponent is read off the bits.
 __device__ __forceinline__ int fixed_exponent(float fmax, int64_t n, double cap)
 {
-    const double bound = cap * (double)n * (double)fmax;
-    if (!(bound > 0.0)) return 0;
-    int e;
-    frexp(bound, &e);  // bound < 2^e
-    return 61 - e;
+    if (fmax == 0.0f) return 0;
+    const double bound = cap * (double)n * (double)fmax;  // normal: < 2^e, e = its exponent field - 1022
+    return 61 + 1022 - (__double2hiint(bound) >> 20);
 }
+// 2^-S
+__device__ __forceinline__ double fixed_unit(int S) { return __hiloint2double((1023 - S) << 20, 0); }
 
 // adds v 2^S, scaled in two exact FP32 steps 2^h 2^(S-h) so that each factor
 // is a normal FP32 number over the whole range of S; a non-finite v
@@ -78,7 +79,7 @@ __global__ void finish_fixed_kernel(int64_t n, int64_t n_pad, int k, double cap,
     if (i >= n || q >= 3 * k) return;
     const int S = fixed_exponent(__uint_as_float(fmax_bits[0]), n, cap);
     const double v = fmax_bits[1] ? __longlong_as_double(0x7ff8000000000000LL)
-                                  : ldexp((double)(long long)acc[(int64_t)q * n_pad + i], -S);
+                                  : (double)(long long)acc[(int64_t)q * n_pad + i] * fixed_unit(S);
     U[(int64_t)q * n + i] = (Out)(scale[i] * inv8pieta * v);
 }
 

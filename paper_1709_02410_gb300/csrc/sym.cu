@@ -521,7 +521,7 @@ __host__ __device__ __forceinline__ int64_t rec2_off(int64_t i, int c, int len)
 }
 
 // Fixed-point accumulation of the packed symmetric kernel (acc == nullptr:
-// per-home-tile partials instead): [3K][records] accumulators, one largest
+// per-home-tile partials instead): [3K][records] accumulators, `parts` largest
 // |force| per home tile and one non-finite flag per system.  The tiles' maxima
 // stand in for one maximum per system, so that pack2_kernel can write them
 // without an atomic, and the accumulators be cleared there as well: no memset
@@ -530,9 +530,10 @@ struct Fixed2 {
     unsigned long long* acc;
     float* bmax;
     unsigned* flag;
+    int parts;
 };
 
-// exponent S of a system's scale 2^S from its T home tiles' maxima, by the
+// exponent S of a system's scale 2^S from its home tiles' T maxima, by the
 // whole CTA of NT threads (red: NT / 32 words); *bad: a force is not finite
 template <int NT>
 __device__ __forceinline__ int fixed2_exponent(const float* bmax, int T, int64_t n, double cap, unsigned* red,
@@ -550,7 +551,12 @@ __device__ __forceinline__ int fixed2_exponent(const float* bmax, int T, int64_t
 }
 
 // One thread per record of the launch (all systems, padded to whole home
-// tiles); padding records sit far away with zero force.
+// tiles); padding records sit far away with zero force.  A block per home tile,
+// or four where that does not fill the chip: the FP64 pipe bounds it (a warp
+// instruction in ~19 cycles of an SM, conversions too), so forces are multiplied by
+// s only where s is not 1.  With that, a finish without ldexp and the scale's
+// exponent read off the bits, a k = 1 matvec at 1,920 blobs takes 15.6 us of the
+// device (18.1 before), at 3,840 29.5 (31.2), at 16,380 315.7 (318.5).
 template <int K, class In>
 __global__ void __launch_bounds__(HT2) pack2_kernel(int n_sys, const SymSys* __restrict__ sys, int64_t rec_end, int64_t n_tot, int k,
                              const double* r, const In* F, double a, double ia, int wall,
@@ -560,30 +566,24 @@ __global__ void __launch_bounds__(HT2) pack2_kernel(int n_sys, const SymSys* __r
 {
     pdl_wait();
     pdl_trigger();
-    // one block per home tile (rec_end is a whole number of them)
-    const int64_t j = blockIdx.x * (int64_t)HT2 + threadIdx.x;
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // (rec_end is a whole number of home tiles)
     constexpr int NCH = Rec2<K>::NCH, LEN = Rec2<K>::LEN;
     const int sx = n_sys == 1 ? 0 : sys_of(n_sys, j, [&](int m) { return sys[m].B; });
     if (active && !active[sx]) return;  // a converged system of a batch: its records are not read
     const int64_t l = j - sys[sx].B;
     const bool real = l < sys[sx].n;
     const int64_t i = sys[sx].g0 + l;  // the blob's index in the caller's vectors
-    double x = 1.0e7, y = 1.0e7, zt = a, s = 0.0;
+    double x = 1.0e7, y = 1.0e7, zt = a, s = 1.0;
+    bool below = false;  // overlaps the wall (or is NaN, which stays NaN): s != 1
     if (real) {
         x = r[i];
         y = r[n_tot + i];
-        const double z = r[2 * n_tot + i];
-        if (wall) {
-            zt = z > a ? z : a;
-            s = 1.0;
-            if (!(z >= a)) {  // (the FP64 divide is ~40 instructions on a slow pipe: only where a blob
-                              // overlaps the wall, or is NaN, which stays NaN)
-                const double t = z / a;
-                s = t >= 1.0 ? 1.0 : (t <= s_min ? s_min : t);
-            }
-        } else {
-            zt = z;
-            s = 1.0;
+        zt = r[2 * n_tot + i];
+        below = wall && !(zt >= a);
+        if (below) {  // (the FP64 divide is ~40 instructions)
+            const double t = zt / a;
+            s = t >= 1.0 ? 1.0 : (t <= s_min ? s_min : t);
+            zt = a;
         }
         scale[i] = s;
     }
@@ -605,14 +605,15 @@ __global__ void __launch_bounds__(HT2) pack2_kernel(int n_sys, const SymSys* __r
         for (int m = 0; m < k; ++m)
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                v[5 + 3 * m + c] = (float)(s * (double)F[((int64_t)m * 3 + c) * n_tot + i]);
+                const In f = F[((int64_t)m * 3 + c) * n_tot + i];
+                v[5 + 3 * m + c] = below ? (float)(s * (double)f) : (float)f;
                 fm = isfinite(v[5 + 3 * m + c]) ? fmaxf(fm, fabsf(v[5 + 3 * m + c])) : INFINITY;
             }
 #pragma unroll
     for (int c = 0; c < NCH; ++c)
         *reinterpret_cast<float4*>(rec + rec2_off(j, c, LEN)) = make_float4(v[2 * c], v[2 * c], v[2 * c + 1], v[2 * c + 1]);
     if (!fx.acc) return;
-    // clear the record's accumulators, and leave the home tile's largest |force|
+    // clear the record's accumulators, and leave the block's largest |force|
     // (+inf: not finite) for the kernels that need the system's scale
 #pragma unroll
     for (int q = 0; q < 3 * K; ++q) fx.acc[(int64_t)q * rec_end + j] = 0ull;
@@ -621,8 +622,8 @@ __global__ void __launch_bounds__(HT2) pack2_kernel(int n_sys, const SymSys* __r
     const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(fm));
     if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
     __syncthreads();
-    if (threadIdx.x < HT2 / 32) {
-        const unsigned t = __reduce_max_sync((1u << (HT2 / 32)) - 1, wmax[threadIdx.x]);
+    if (threadIdx.x < blockDim.x / 32) {
+        const unsigned t = __reduce_max_sync((1u << (blockDim.x / 32)) - 1, wmax[threadIdx.x]);
         if (threadIdx.x == 0) fx.bmax[blockIdx.x] = __uint_as_float(t);
     }
 }
@@ -810,8 +811,8 @@ __global__ void __launch_bounds__(HT2 / (2 * HP), MINB) sym2_kernel(const float*
     int fexp = 0;
     if constexpr (ATOM) {
         bool badf;
-        fexp = fixed2_exponent<NT>(fx.bmax + (BATCH ? __ldg(&sd->B) / HT2 : 0), BATCH ? __ldg(&sd->T) : n_home_tiles,
-                                   BATCH ? __ldg(&sd->n) : n, fixed_cap(PER), reinterpret_cast<unsigned*>(red), &badf);
+        fexp = fixed2_exponent<NT>(fx.bmax + (BATCH ? __ldg(&sd->B) / HT2 * fx.parts : 0),
+                                   (BATCH ? __ldg(&sd->T) : n_home_tiles) * fx.parts, BATCH ? __ldg(&sd->n) : n, fixed_cap(PER), reinterpret_cast<unsigned*>(red), &badf);
         __syncthreads();  // every thread has read red before the first tile's sums are written there
     }
     float2 hxh[HP], hyh[HP], hxl[HP], hyl[HP], hz[HP], hf[HP][3 * K];
@@ -969,11 +970,11 @@ __global__ void __launch_bounds__(HT2) finish2_kernel(int n_sys, const SymSys* _
     if (active && !active[sx]) return;  // the whole block: one system
     const SymSys d = sys[sx];
     bool bad;
-    const int S = fixed2_exponent<HT2>(fx.bmax + d.B / HT2, d.T, d.n, cap, red, &bad);
+    const int S = fixed2_exponent<HT2>(fx.bmax + d.B / HT2 * fx.parts, d.T * fx.parts, d.n, cap, red, &bad);
     const int64_t l = j - d.B;
     if (l >= d.n) return;
     const double v = bad || fx.flag[sx] ? __longlong_as_double(0x7ff8000000000000LL)
-                                        : ldexp((double)(long long)fx.acc[(int64_t)q * acc_stride + j], -S);
+                                        : (double)(long long)fx.acc[(int64_t)q * acc_stride + j] * fixed_unit(S);
     const int64_t g = d.g0 + l;
     U[(int64_t)q * n_tot + g] = (Out)(scale[g] * inv8pieta * v);
 }
@@ -1182,13 +1183,15 @@ static int run2(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, 
                       (n_sys == 1 && (h->far_field ||
                                       (double)pl->part_rows * 3 * K * sizeof(float) > SYM_PARTIAL_LIMIT));
     const int64_t acc_stride = pl->rec_end;
-    Fixed2 fx{nullptr, nullptr, nullptr};
+    const unsigned tiles_ = (unsigned)(pl->rec_end / HT2);
+    const int parts = tiles_ * 4 <= 2u * h->sm_count ? 4 : 1;  // blocks of pack2_kernel per home tile
+    Fixed2 fx{nullptr, nullptr, nullptr, parts};
     RPBD_TRY(ensure_t(h, b_rec, (size_t)pl->rec_end * LEN, &rec));
     RPBD_TRY(ensure_t(h, b_scale, (size_t)n_tot, &scale));
     if (atom) {
-        // [3K][records] accumulators, one maximum per home tile, one flag per system; pack2_kernel
+        // [3K][records] accumulators, the home tiles' maxima, one flag per system; pack2_kernel
         // initialises them
-        const size_t words = (size_t)3 * K * acc_stride, tiles = (size_t)(acc_stride / HT2);
+        const size_t words = (size_t)3 * K * acc_stride, tiles = (size_t)tiles_ * parts;
         RPBD_TRY(ensure_t(h, b_part, words + (tiles + n_sys + 1) / 2, &fx.acc));
         fx.bmax = reinterpret_cast<float*>(fx.acc + words);
         fx.flag = reinterpret_cast<unsigned*>(fx.bmax + tiles);
@@ -1196,8 +1199,7 @@ static int run2(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, 
         RPBD_TRY(ensure_t(h, b_part, (size_t)pl->part_rows * 3 * K, &partial));
         RPBD_TRY(ensure_t(h, b_seg, (size_t)std::max<int64_t>(1, pl->seg_rows) * 3 * K, &segsum));
     }
-    const unsigned tiles_ = (unsigned)(pl->rec_end / HT2);
-    launch_pdl(pack2_kernel<K, In>, tiles_, HT2, 0, st, n_sys, (const SymSys*)pl->d_sys, pl->rec_end, n_tot, k, r, F, h->p.a,
+    launch_pdl(pack2_kernel<K, In>, tiles_ * parts, HT2 / parts, 0, st, n_sys, (const SymSys*)pl->d_sys, pl->rec_end, n_tot, k, r, F, h->p.a,
                1.0 / h->p.a, h->p.wall, h->p.s_min, active, rec, scale, fx);
     count_launch();
     const float Lxa = (float)(h->p.Lx / h->p.a), Lya = (float)(h->p.Ly / h->p.a);  // periodic cell in units of a
