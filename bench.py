@@ -41,9 +41,9 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12   # SMs x FP32 lanes x FMA x m
 # DRAM bytes (read + write) per launch from one ncu capture of the current
 # kernels (profiles/pair_kernel_f32_k16_boomerangs_65535.md, profiles/sym_kernel_f32_k*_boomerangs_65535.md);
 # None when not captured
-NCU_TRAFFIC = {"f32symf_k1": 5897216 + 0, "f32symf_k2": 9592576 + 0, "f32_k16": 39866880 + 470016}
+NCU_TRAFFIC = {"f32symf_k1": 6134272 + 0, "f32symf_k2": 9827328 + 0, "f32_k16": 41184768 + 1390592}
 # FMA-pipe activity (sm__pipe_fma_cycles_active) from the same captures
-NCU_FMA_PIPE = {"f32symf_k1": 0.778, "f32symf_k2": 0.769, "f32_k16": 0.795}
+NCU_FMA_PIPE = {"f32symf_k1": 0.787, "f32symf_k2": 0.778, "f32_k16": 0.917}
 
 
 F_ASSEMBLY = 12             # flops of forming the 9 entries from the block's 5 scalars

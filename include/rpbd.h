@@ -47,7 +47,8 @@ extern "C" {
 
 /* arithmetic of the pair kernels */
 #define RPBD_F64 0 /* FP64 pair math, FP64 accumulation */
-#define RPBD_F32 1 /* FP32 pair math; FP32 tile partials summed as compensated float pairs (two-sum, ~48 bits), then FP64 */
+#define RPBD_F32 1 /* FP32 pair math; FP32 tile sums accumulated in 64-bit fixed point (or, see RPBD_OPT_SYM_PARTIALS,
+                      as compensated float pairs), then FP64 */
 
 typedef struct rpbd_handle rpbd_handle;
 
@@ -127,9 +128,10 @@ int rpbd_blobs_from_bodies(rpbd_handle* h, int64_t nb, int nper, const double* s
 
 /* ---- a2: wall-RPY matvec (Sec. 2.1; the dense GPU sum of Sec. 2.1/4.2) -- */
 
-/* U = M(r) F for k right-hand sides (1 <= k <= 16; k in {1,2,4,8,16} hit
- * specialised kernels, other k run as the next larger one).  F and U are
- * [k][3][n] of type double (dtype RPBD_F64) or float (RPBD_F32).
+/* U = M(r) F for k right-hand sides (1 <= k <= 16; FP32: k in {1,2,4,8,16} hit
+ * specialised kernels, other k run as the next larger one; FP64: k <= 8 runs
+ * in passes of up to four).  F and U are [k][3][n] of type double (dtype
+ * RPBD_F64) or float (RPBD_F32).
  * M_ij = s_i s_j [M_RPY(r~_i - r~_j) + M_wall(r~_i, r~_j)], r~ = (x, y, max(z, a)). */
 int rpbd_mobility_apply(rpbd_handle* h, int64_t n, const double* r, const void* F, void* U,
                         int k, int dtype, void* stream);
@@ -179,10 +181,11 @@ int rpbd_mobility_adjoint_f32(rpbd_handle* h, int64_t n, const double* r, const 
 
 /* grad[3][n] = d( sum_m u_m^T M(r) F_m )/dr for k right-hand-side pairs
  * (1 <= k <= 16; u, F [k][3][n] FP64): the gradient of a loss of the k-RHS
- * matvec of Sec. 2.1, summed over the pairs on the device.  Each pair block
- * and its derivative are formed once for all k (FP32: in passes of up to four
- * pairs).  dtype RPBD_F64 or RPBD_F32 selects the pair arithmetic as in the
- * two calls above; sums are FP64. */
+ * matvec of Sec. 2.1, summed over the pairs on the device, in passes of up to
+ * four right-hand-side pairs that share each blob pair's block and derivatives.
+ * dtype RPBD_F64 or RPBD_F32 selects the pair arithmetic as in the two calls
+ * above; sums across tiles are FP64, in a fixed order.  The workspace is at most
+ * about 4 GiB, less where device memory is short. */
 int rpbd_mobility_adjoint_multi(rpbd_handle* h, int64_t n, const double* r, const double* u,
                                 const double* F, int k, double* grad, int dtype, void* stream);
 
@@ -362,7 +365,8 @@ int rpbd_blob_forces(rpbd_handle* h, int64_t n, int nper, const double* r, const
  * (M_ji = M_ij^T, Sec. 2.1); 0: the one-direction kernel for every k.  Sets
  * every right-hand-side class (see rpbd_autotune). */
 #define RPBD_OPT_SYMMETRIC 1
-/* -1 (default): per-k default; 0..5: loop-unroll / occupancy variant of the
+/* -1 (default): per-k default for the size (small systems: the whole matvec in
+ * one launch); 0..5: loop-unroll / occupancy variant of the
  * symmetric kernel, for every right-hand-side class (4, 5: the packed kernel
  * with four home blobs per thread; the one-home kernel has 0..3 and runs 4, 5
  * as 0). */
@@ -386,7 +390,8 @@ int rpbd_blob_forces(rpbd_handle* h, int64_t n, int nper, const double* r, const
  * the kernel records the timeout, lets its other copies land and exits, and
  * the synchronising calls (Lanczos, GMRES, steps, batched Lanczos with iters)
  * return RPBD_TIMEOUT.  The kernel-only calls then return garbage without a
- * status.  For tests of the error path only; set it back to 0 afterwards. */
+ * status.  Small FP32 systems, whose default kernel has no waits, run on the
+ * kernels above while it is set.  For tests of the error path only; set it back to 0 afterwards. */
 #define RPBD_OPT_TEST_STALL 5
 /* value != 0 (default 0): FP32 matvecs of one system with the wall form each
  * pair block with the direct-minus-image differences written without
@@ -413,8 +418,8 @@ int rpbd_blob_forces(rpbd_handle* h, int64_t n, int nper, const double* r, const
  * finite FP32 forces).  Integer addition does not depend on its order, so
  * both are deterministic; they differ by FP32 output rounding.  Batches on
  * the packed symmetric kernel follow the same option (one maximum force per
- * system); the FP64 kernels and the batched one-direction tiles always keep
- * their partials. */
+ * system); the FP64 kernels, the gradients and the batched one-direction tiles
+ * always keep their partials. */
 #define RPBD_OPT_SYM_PARTIALS 7
 int rpbd_set_option(rpbd_handle* h, int option, int value);
 
@@ -422,7 +427,9 @@ int rpbd_set_option(rpbd_handle* h, int option, int value);
  * forces): the one-direction kernel and, for k <= 4, every symmetric variant;
  * keeps the fastest in the handle for k's class (k = 1, k = 2, 3..4; other
  * classes keep their setting) and returns its index (0: one-direction,
- * 1 + v: symmetric variant v) or a negative status.  *best_ms (host, may be
+ * 1 + v: symmetric variant v; where a small system's one-launch default is the
+ * fastest it is kept, and the index is that of the larger systems' default) or a
+ * negative status.  *best_ms (host, may be
  * NULL) receives its time per launch.  Synchronises the stream. */
 int rpbd_autotune(rpbd_handle* h, int64_t n, const double* r, int k, double* best_ms, void* stream);
 

@@ -15,6 +15,10 @@
 //              in FP64, FP32 partials as compensated float pairs, about
 //              48 bits; the result is deterministic), multiplies by
 //              s_i / (8 pi eta) and writes U in the caller's type.
+// This one-direction form serves FP32 without the wall or without packing, FP64 with
+// many right-hand sides or very many blobs, and the allocation-free call; the
+// dispatch below sends the rest to sym.cu (k <= 4), direct.cu (small systems),
+// sym64.cu (FP64) and, with 5-16 right-hand sides, namespace wide.
 // FP32 applies through the handle accumulate in fixed point instead
 // (fixed_point.cuh): each CTA adds its chunk sums to one 64-bit integer per
 // blob and component, so memory is O(n k) rather than O(n^2 k / 2048), and a
@@ -832,8 +836,7 @@ int mobility_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* 
         }
         return RPBD_OK;
     }
-    // the packed symmetric kernel takes any n (past the partials' limit it sums in FP64
-    // atomics); the one-home kernel only while its partials fit
+    // the packed symmetric kernel takes any n (it sums in fixed point per blob); the one-home kernel only while its partials fit
     const bool packed_sym = h->use_packed && h->p.wall;
     // a small system on the default settings: one launch (the failure-path test
     // wants the bounded waits of the ring kernels, the partials option their
