@@ -13,10 +13,15 @@
 // no atomics, no reduction kernel, deterministic.  It does every block twice and
 // converts every source in every CTA, so it stops paying off where that counts.
 //
-// Device time of a call, sym.cu -> here, open cell: 60 blobs 13.3 -> 3.5 us, 240
-// 13.9 -> 4.3, 600 14.3 -> 8.5, 960 14.3 -> 11.9 (k = 1), 17.1 -> 17.1 (k = 2),
-// 22.1 -> 26.4 (k = 4; 600: 21.9 -> 18.8); 1,440 18.4 -> 21.5.  Periodic: 240 31.2 ->
-// 5.2, 960 33.5 -> 25.2 (k = 1), 40.4 -> 40.0 (k = 4); 1,440 48.3 -> 61.2.
+// What bounds it are the loads of the conversion (every thread has two to four
+// sources in flight at once: with single ones where fewer are left 300 blobs took
+// 5.9 us, now 4.6, 840 15.7, now 9.8) and the few FP64 instructions left.
+//
+// Device time of a call, sym.cu -> here, open cell, k = 1: 240 blobs 11.9 -> 3.8 us,
+// 600 12.7 -> 6.6, 960 12.2 -> 10.2; k = 2: 13.4 -> 4.7, 14.1 -> 9.3, 14.3 -> 13.9;
+// k = 4: 16.3 -> 7.1, 600 18.4 -> 14.4.  Periodic, against sym.cu's 25.5 (k = 1),
+// 27.2 and 33.8 us at 1,080 blobs: 240 4.7, 5.7 and 7.9, 600 10.9, 13.7 and 19.0, 960
+// 22.9 and 27.5.
 #include <cuda_runtime.h>
 
 #include "rpbd_internal.cuh"
@@ -53,31 +58,44 @@ __global__ void __launch_bounds__(NT) direct_kernel(int n, int k, int tp, const 
     pdl_trigger();
     float* f = sm + 5 * n;
     bool bad = false;
-#pragma unroll(K == 1 ? 4 : 2)
-    for (int i = tid; i < n; i += NT) {
-        float h, l;
-        split(r[i], h, l);
-        sm[i] = h;
-        sm[2 * n + i] = l;
-        split(r[n + i], h, l);
-        sm[n + i] = h;
-        sm[3 * n + i] = l;
-        const double z = r[2 * n + i];
-        sm[4 * n + i] = (float)((z > a ? z : a) * ia);
-        double s = 1.0;
-        if (!(z >= a)) {  // overlaps the wall, or NaN (stays NaN)
-            const double t = z / a;
-            s = t >= 1.0 ? 1.0 : (t <= s_min ? s_min : t);
+    constexpr int U4 = K == 1 ? 4 : 2;  // sources a thread has in flight, also at the end
+    for (int i0 = tid; i0 < n; i0 += U4 * NT) {
+        double x[U4], y[U4], zs[U4];
+        In g[U4][3 * K];
+#pragma unroll
+        for (int u = 0; u < U4; ++u) {
+            const int i = min(i0 + u * NT, n - 1);
+            x[u] = r[i];
+            y[u] = r[n + i];
+            zs[u] = r[2 * n + i];
+#pragma unroll
+            for (int q = 0; q < 3 * K; ++q) g[u][q] = q < 3 * k ? F[(int64_t)q * n + i] : In(0);
         }
 #pragma unroll
-        for (int q = 0; q < 3 * K; ++q) {
-            float v = 0.0f;
-            if (q < 3 * k) {
-                const In x = F[(int64_t)q * n + i];
-                v = s == 1.0 ? (float)x : (float)(s * (double)x);
-                bad = bad || !isfinite(v);
+        for (int u = 0; u < U4; ++u) {
+            const int i = i0 + u * NT;
+            if (i >= n) break;
+            float h, l;
+            split(x[u], h, l);
+            sm[i] = h;
+            sm[2 * n + i] = l;
+            split(y[u], h, l);
+            sm[n + i] = h;
+            sm[3 * n + i] = l;
+            const double z = zs[u];
+            const bool below = !(z >= a);  // overlaps the wall, or NaN (stays NaN)
+            sm[4 * n + i] = (float)((below ? a : z) * ia);
+            double s = 1.0;
+            if (below) {
+                const double t = z * ia;  // (an FP64 divide is ~40 instructions)
+                s = t >= 1.0 ? 1.0 : (t <= s_min ? s_min : t);
             }
-            f[q * n + i] = v;
+#pragma unroll
+            for (int q = 0; q < 3 * K; ++q) {
+                const float v = below ? (float)(s * (double)g[u][q]) : (float)g[u][q];
+                bad = bad || !isfinite(v);
+                f[q * n + i] = v;
+            }
         }
     }
     bad = __syncthreads_or(bad);  // a force that is not finite: U is NaN everywhere, as in sym.cu
@@ -151,7 +169,7 @@ __global__ void __launch_bounds__(NT) direct_kernel(int n, int k, int tp, const 
     const double z = r[2 * (int64_t)n + t];
     double s = 1.0;
     if (!(z >= a)) {
-        const double u = z / a;
+        const double u = z * ia;
         s = u >= 1.0 ? 1.0 : (u <= s_min ? s_min : u);
     }
     U[(int64_t)q * n + t] = (Out)(bad || !isfinite(v) ? __longlong_as_double(0x7ff8000000000000LL) : s * inv8pieta * (double)v);

@@ -580,8 +580,8 @@ __global__ void __launch_bounds__(HT2) pack2_kernel(int n_sys, const SymSys* __r
         y = r[n_tot + i];
         zt = r[2 * n_tot + i];
         below = wall && !(zt >= a);
-        if (below) {  // (the FP64 divide is ~40 instructions)
-            const double t = zt / a;
+        if (below) {  // (not z / a: an FP64 divide is ~40 instructions)
+            const double t = zt * ia;
             s = t >= 1.0 ? 1.0 : (t <= s_min ? s_min : t);
             zt = a;
         }
