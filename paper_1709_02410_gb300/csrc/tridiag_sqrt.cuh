@@ -11,12 +11,12 @@
 // Each node is one tridiagonal solve (T + t^2) z = T e_1 (no cancellation), so the
 // chain is ~2 m steps; Jacobi needs 5-6 sweeps of ~m dependent rounds (129 us per
 // call, mean over the iterations of a time step, against 39 for the quadrature
-// with everything on the device, and 1e-15 instead of 1e-16 off at condition 1e4).  hi is Gershgorin's bound; lo the largest of 32
-// trial shifts hi 2^{-47 j/32} with T - shift positive definite.  The shifts' and
-// weights' ratios to hi and sqrt(hi) depend on j alone: a table of 32 KB that the
-// host fills once (sqrt_nodes), since one FP64 operation after another takes the
-// warp ~0.04 us (with the elliptic functions on the device 21.6 us of a Lanczos
-// iteration at 7 vectors, now 10.3).
+// with everything on the device, and 1e-15 instead of 1e-16 off at condition 1e4).
+// hi is Gershgorin's bound; lo the largest of 32 trial shifts hi 2^{-47 j/32} with
+// T - shift positive definite.  The shifts' and weights' ratios to hi and sqrt(hi)
+// depend on j alone: a table of 33 KB that the host fills once (sqrt_nodes), since
+// one FP64 operation after another takes the warp ~0.04 us (with the elliptic
+// functions on the device 21.6 us of a Lanczos iteration at 7 vectors, now 10.3).
 //
 // Otherwise (an eigenvalue below ~1e-14 of the largest, or negative) T is
 // diagonalised by cyclic Jacobi, T = Q diag(lambda) Q^T, and
