@@ -154,6 +154,7 @@ int rpbd_destroy(rpbd_handle* h)
     }
     for (auto e : h->ev_pool) cudaEventDestroy(e);
     batched_free_graphs(h);
+    batched_free_tables(h);
     batched_free_plans(h);
     for (int b = 0; b < BUF_COUNT; ++b)
         if (h->buf[b]) cudaFree(h->buf[b]);

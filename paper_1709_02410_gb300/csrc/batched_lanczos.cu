@@ -276,15 +276,68 @@ void batched_free_graphs(rpbd_handle* h)
     h->bgraphs.clear();
 }
 
+// The chunks of one batch layout on the device, written once when the handle first
+// meets these offsets: later calls' kernels and the captured graphs, possibly still
+// queued when another layout comes, read it where it is.
+struct BlzTable {
+    std::vector<int64_t> off;
+    void* mem = nullptr;
+    BlzChunk* chunks;
+    int2* sys;  // first chunk and chunks of each system
+    int64_t* doff;
+    int nch, chunk;
+};
+
+void batched_free_tables(rpbd_handle* h)
+{
+    for (BlzTable* t : h->blz_tables) {
+        cudaFree(t->mem);
+        delete t;
+    }
+    h->blz_tables.clear();
+}
+
+static int blz_table(rpbd_handle* h, int n_sys, const int64_t* off, const BlzTable** out)
+{
+    for (const BlzTable* t : h->blz_tables)
+        if ((int)t->off.size() == n_sys + 1 && std::equal(t->off.begin(), t->off.end(), off)) {
+            *out = t;
+            return RPBD_OK;
+        }
+    const std::vector<BlzChunk> ch = blz_chunks(n_sys, off);
+    std::vector<char> host(ch.size() * sizeof(BlzChunk) + n_sys * sizeof(int2) + (n_sys + 1) * sizeof(int64_t));
+    char* q = host.data();
+    if (!ch.empty()) std::memcpy(q, ch.data(), ch.size() * sizeof(BlzChunk));
+    int2* hs = reinterpret_cast<int2*>(q + ch.size() * sizeof(BlzChunk));
+    for (int s = 0; s < n_sys; ++s) hs[s] = make_int2(0, 0);
+    for (const BlzChunk& c : ch) hs[c.s] = make_int2(c.c0, c.nc);
+    std::memcpy(hs + n_sys, off, (n_sys + 1) * sizeof(int64_t));
+    BlzTable* t = new BlzTable();
+    t->off.assign(off, off + n_sys + 1);
+    t->nch = (int)ch.size();
+    t->chunk = blz_chunk_size(off[n_sys]);
+    // (the copy has to have arrived before kernels of a stream that does not wait for the legacy one)
+    if (cudaMalloc(&t->mem, host.size()) != cudaSuccess ||
+        cudaMemcpy(t->mem, q, host.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+        cudaFree(t->mem);
+        delete t;
+        return set_error(h, RPBD_NO_MEM, "batched lanczos: chunk table upload failed");
+    }
+    t->chunks = static_cast<BlzChunk*>(t->mem);
+    t->sys = reinterpret_cast<int2*>(t->chunks + ch.size());
+    t->doff = reinterpret_cast<int64_t*>(t->sys + n_sys);
+    h->blz_tables.push_back(t);
+    *out = t;
+    return RPBD_OK;
+}
+
 struct BlzBufs {
     double *V, *z, *y, *w, *Win, *rin, *out, *Fin, *Uout;
     double *H, *part;
     BlzState S;
     int* active[2];  // of even and odd iterations
-    int64_t* doff;
-    BlzChunk* chunks;
-    int2* sys;  // first chunk and chunks of each system
-    int nch, chunk;
+    const BlzTable* T;
 };
 
 // every kernel of one batched Lanczos (+ optional matvec), no host sync
@@ -292,25 +345,26 @@ static int blz_body(rpbd_handle* h, int n_sys, const int64_t* off, int64_t n, co
                     int max_iter, int use_precond, bool with_apply, cudaStream_t st)
 {
     const int64_t len = 3 * n;
-    const int ldh = B.S.mdim + 1, threads = 3 * B.chunk > 512 ? 512 : 256;
-    const unsigned g = (unsigned)std::max(1, B.nch), gs = (unsigned)(B.nch + n_sys);
-    const int elems = 3 * B.chunk;
+    const BlzTable& T = *B.T;
+    const int ldh = B.S.mdim + 1, threads = 3 * T.chunk > 512 ? 512 : 256;
+    const unsigned g = (unsigned)std::max(1, T.nch), gs = (unsigned)(T.nch + n_sys);
+    const int elems = 3 * T.chunk;
     auto ortho = [&](auto kernel, int nv, double* w, const int* active) {
-        launch_pdl(kernel, g, threads, (size_t)(elems + nv) * sizeof(double), st, n, B.nch, (const BlzChunk*)B.chunks,
+        launch_pdl(kernel, g, threads, (size_t)(elems + nv) * sizeof(double), st, n, T.nch, (const BlzChunk*)T.chunks,
                    (const double*)B.V, nv, w, B.part, B.H, ldh, active);
         count_launch();
     };
     ortho(blz_ortho_kernel<3>, 0, B.Win, nullptr);
-    launch_pdl(blz_start_kernel, gs, 256, 0, st, n, B.nch, (const BlzChunk*)B.chunks, (const int2*)B.sys, (const double*)B.Win,
+    launch_pdl(blz_start_kernel, gs, 256, 0, st, n, T.nch, (const BlzChunk*)T.chunks, (const int2*)T.sys, (const double*)B.Win,
                (const double*)B.part, B.V, B.S, B.active[0]);
     count_launch();
     for (int m = 0; m < max_iter; ++m) {
         const double* vm = B.V + (int64_t)m * len;
         const int* act = B.active[m & 1];
         if (use_precond) {
-            RPBD_TRY(precond_apply_impl(h, 2, vm, B.z, st, act, B.doff, n_sys));
+            RPBD_TRY(precond_apply_impl(h, 2, vm, B.z, st, act, T.doff, n_sys));
             RPBD_TRY(batched_apply_impl(h, n_sys, off, B.rin, B.z, B.y, 1, true, act, st));
-            RPBD_TRY(precond_apply_impl(h, 1, B.y, B.w, st, act, B.doff, n_sys));
+            RPBD_TRY(precond_apply_impl(h, 1, B.y, B.w, st, act, T.doff, n_sys));
         } else {
             RPBD_TRY(batched_apply_impl(h, n_sys, off, B.rin, vm, B.w, 1, true, act, st));
         }
@@ -318,13 +372,13 @@ static int blz_body(rpbd_handle* h, int n_sys, const int64_t* off, int64_t n, co
         ortho(blz_ortho_kernel<0>, nv, B.w, act);
         ortho(blz_ortho_kernel<1>, nv, B.w, act);
         ortho(blz_ortho_kernel<2>, nv, B.w, act);
-        launch_pdl(blz_finish_kernel, gs, 256, tridiag_sqrt_smem_doubles(nv) * sizeof(double), st, n, B.nch,
-                   (const BlzChunk*)B.chunks, (const int2*)B.sys, m, max_iter, tol, (const SqrtNode*)h->sqrt_nodes,
-                   (const double*)B.H, (const double*)B.w, (const double*)(B.part + 2 * (int64_t)nv * B.nch),
+        launch_pdl(blz_finish_kernel, gs, 256, tridiag_sqrt_smem_doubles(nv) * sizeof(double), st, n, T.nch,
+                   (const BlzChunk*)T.chunks, (const int2*)T.sys, m, max_iter, tol, (const SqrtNode*)h->sqrt_nodes,
+                   (const double*)B.H, (const double*)B.w, (const double*)(B.part + 2 * (int64_t)nv * T.nch),
                    B.V + (int64_t)(m + 1) * len, B.S, act, B.active[(m + 1) & 1]);
         count_launch();
     }
-    launch_pdl(blz_combine_kernel, g, 256, 0, st, n, B.nch, (const BlzChunk*)B.chunks, (const double*)B.V, B.S,
+    launch_pdl(blz_combine_kernel, g, 256, 0, st, n, T.nch, (const BlzChunk*)T.chunks, (const double*)B.V, B.S,
                use_precond ? B.y : B.out);
     count_launch();
     if (use_precond) RPBD_TRY(precond_apply_impl(h, 0, B.y, B.out, st));
@@ -349,27 +403,10 @@ static int blz_bufs(rpbd_handle* h, int n_sys, const int64_t* off, int64_t n, in
     B->out = p; p += len;
     B->Fin = p; p += len;
     B->Uout = p; p += len;
-    const std::vector<BlzChunk> ch = blz_chunks(n_sys, off);
-    B->nch = (int)ch.size();
-    B->chunk = blz_chunk_size(n);
-    // the layout on the device: chunk table, systems' chunks, offsets (one copy), then the state
-    const size_t tab = ch.size() * sizeof(BlzChunk) + n_sys * sizeof(int2) + (n_sys + 1) * sizeof(int64_t);
+    RPBD_TRY(blz_table(h, n_sys, off, &B->T));
     double* sm;
-    const size_t nsm = tab / sizeof(double) + (size_t)n_sys * (mdim + 1 + 4 * mdim + 2) + (size_t)2 * n_sys +
-                       ch.size() * (2 * (size_t)max_iter + 1);
+    const size_t nsm = (size_t)n_sys * (mdim + 1 + 4 * mdim + 2) + (size_t)2 * n_sys + B->T->nch * (2 * (size_t)max_iter + 1);
     RPBD_TRY(ensure_t(h, BUF_BLZ_SMALL, nsm, &sm));
-    std::vector<char> host(tab);
-    char* q = host.data();
-    if (!ch.empty()) std::memcpy(q, ch.data(), ch.size() * sizeof(BlzChunk));
-    int2* hs = reinterpret_cast<int2*>(q + ch.size() * sizeof(BlzChunk));
-    for (int s = 0; s < n_sys; ++s) hs[s] = make_int2(0, 0);
-    for (const BlzChunk& c : ch) hs[c.s] = make_int2(c.c0, c.nc);
-    std::memcpy(hs + n_sys, off, (n_sys + 1) * sizeof(int64_t));
-    RPBD_CU(h, cudaMemcpy(sm, q, tab, cudaMemcpyHostToDevice));
-    B->chunks = reinterpret_cast<BlzChunk*>(sm);
-    B->sys = reinterpret_cast<int2*>(B->chunks + ch.size());
-    B->doff = reinterpret_cast<int64_t*>(B->sys + n_sys);
-    sm += tab / sizeof(double);
     B->H = sm; sm += (size_t)n_sys * (mdim + 1);
     B->S.mdim = mdim;
     B->S.alpha = sm; sm += (size_t)n_sys * mdim;
@@ -378,7 +415,7 @@ static int blz_bufs(rpbd_handle* h, int n_sys, const int64_t* off, int64_t n, in
     B->S.cprev = sm; sm += (size_t)n_sys * mdim;
     B->S.W2 = sm; sm += n_sys;
     B->S.change = sm; sm += n_sys;
-    B->part = sm; sm += ch.size() * (2 * (size_t)max_iter + 1);
+    B->part = sm; sm += B->T->nch * (2 * (size_t)max_iter + 1);
     B->S.iters = reinterpret_cast<int*>(sm);
     B->active[0] = B->S.iters + n_sys;
     B->active[1] = B->active[0] + n_sys;

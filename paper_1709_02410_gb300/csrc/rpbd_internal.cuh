@@ -73,6 +73,7 @@ enum Buf {
 
 struct BatchPlan;
 struct BatchGraph;
+struct BlzTable;
 struct Sym2Plan;
 
 struct ProfRec {
@@ -118,6 +119,7 @@ struct rpbd_handle {
     std::vector<rpbd::BatchPlan*> bplans;
     int batch_variant = -1;
     std::vector<rpbd::BatchGraph*> bgraphs;
+    std::vector<rpbd::BlzTable*> blz_tables;  // chunks of the batched Lanczos, per offsets
     rpbd::BatchPlan* mv_plan = nullptr;  // work list of the single-system packed matvec
     std::vector<rpbd::Sym2Plan*> sym2_plans;  // work lists of the packed symmetric kernel, per offsets
     // symmetric FP32 kernel (k <= 4): on by default, work list cached per n
@@ -294,5 +296,6 @@ int sym_batched_apply_impl(rpbd_handle* h, int n_sys, const int64_t* off, const 
 void free_sym2_plans(rpbd_handle* h);
 void batched_free_plans(rpbd_handle* h);
 void batched_free_graphs(rpbd_handle* h);
+void batched_free_tables(rpbd_handle* h);
 
 }  // namespace rpbd

@@ -1,0 +1,57 @@
+"""Calls that once went wrong: each test states what it was."""
+import ctypes as C
+
+import numpy as np
+import pytest
+import torch
+
+from paper_1709_02410_gb300 import Handle, synth
+
+from gpu_util import to_dev
+
+pytestmark = pytest.mark.gpu
+
+A = synth.A_BOOMERANG
+
+
+def cloud(n, seed):
+    """n blobs at the boomerang suspensions' density, overlapping pairs and blobs below the wall height a among them."""
+    rng = np.random.default_rng(seed)
+    r = np.empty((3, n))
+    r[:2] = rng.uniform(0.0, 40.0 * np.sqrt(max(n, 60) / 1920), (2, n))
+    r[2] = 0.7 * A + rng.exponential(3.0 * A, n)
+    return r
+
+
+def lanczos_batched(h, off, r, W, out, use_graph, stream, iters=None):
+    """The C entry; without iters it returns while its work is queued."""
+    return h.lib.rpbd_lanczos_sqrt_apply_batched(h.h, off.size - 1, off.ctypes.data_as(C.c_void_p), C.c_void_p(r.data_ptr()),
+                                                 C.c_void_p(W.data_ptr()), C.c_void_p(out.data_ptr()), None, None, 1e-30, 7, 0,
+                                                 use_graph, iters, C.c_void_p(stream.cuda_stream))
+
+
+@pytest.mark.parametrize("use_graph", [0, 1])
+def test_batched_lanczos_layouts_in_flight(use_graph):
+    """Calls with other offsets queued behind one another on a stream of their own: one call's chunk table was written
+    over by the next call's while it was read."""
+    h = Handle(synth.ETA, A, synth.KT)
+    layouts = [np.concatenate([[0], np.cumsum(s)]).astype(np.int64) for s in ((9000, 1, 20_000, 3001), (700,) * 40, (31, 25_000))]
+    st = torch.cuda.Stream()
+    calls = []
+    for i, off in enumerate(layouts):
+        n = int(off[-1])
+        r, W = to_dev(cloud(n, 900 + i)), to_dev(synth.gaussian(910 + i, (3, n)))
+        ref = torch.empty_like(W)
+        torch.cuda.synchronize()
+        iters = (C.c_int * (off.size - 1))()
+        assert lanczos_batched(h, off, r, W, ref, use_graph, st, iters) == 0  # waits; workspaces and graphs exist from here on
+        calls.append((off, r, W, ref))
+    outs = []
+    for off, r, W, ref in calls + calls[::-1]:
+        outs.append((torch.zeros_like(W), ref))
+    torch.cuda.synchronize()
+    for (off, r, W, _), (out, _) in zip(calls + calls[::-1], outs):
+        assert lanczos_batched(h, off, r, W, out, use_graph, st) == 0
+    st.synchronize()
+    for out, ref in outs:
+        assert torch.equal(out, ref)
