@@ -694,16 +694,22 @@ static int get_plan(rpbd_handle* h, int n_sys, const int64_t* off, int k, int va
     return RPBD_OK;
 }
 
+int batched_check_offsets(rpbd_handle* h, int n_sys, const int64_t* off)
+{
+    for (int s = 0; s < n_sys; ++s)
+        if (off[s + 1] < off[s] || (off[s + 1] - off[s]) > (int64_t)1 << 30)
+            return set_error(h, RPBD_BAD_ARG, "batched: offsets must be non-decreasing");
+    if (off[0] != 0) return set_error(h, RPBD_BAD_ARG, "batched: offsets must start at 0");
+    return RPBD_OK;
+}
+
 int batched_apply_impl(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, const void* F, void* U, int k,
                        bool io_double, const int* active, cudaStream_t st)
 {
     if (n_sys <= 0) return set_error(h, RPBD_BAD_ARG, "batched: n_sys <= 0");
     if (h->p.Lx > 0.0) return set_error(h, RPBD_BAD_ARG, "batched: systems are open in x, y (no periodic cell)");
     if (k < 1 || k > 16) return set_error(h, RPBD_BAD_ARG, "batched: k must be in 1..16");
-    for (int s = 0; s < n_sys; ++s)
-        if (off[s + 1] < off[s] || (off[s + 1] - off[s]) > (int64_t)1 << 30)
-            return set_error(h, RPBD_BAD_ARG, "batched: offsets must be non-decreasing");
-    if (off[0] != 0) return set_error(h, RPBD_BAD_ARG, "batched: offsets must start at 0");
+    RPBD_TRY(batched_check_offsets(h, n_sys, off));
     if (off[n_sys] == 0) return RPBD_OK;
     // variant 4: the packed symmetric kernel over the batch (k <= 4 with the wall;
     // the default there: 7.7 vs 11.7 ms for the 64-system boomerang batch)

@@ -437,7 +437,7 @@ int rpbd_lanczos_sqrt_apply_batched(rpbd_handle* h, int n_sys, const int64_t* of
         return set_error(h, RPBD_BAD_ARG, "batched lanczos: bad arguments");
     if (!(tol > 0) || max_iter < 1 || max_iter > BLZ_MAX)
         return set_error(h, RPBD_BAD_ARG, "batched lanczos: need tol > 0 and 1 <= max_iter <= 64");
-    if (offsets[0] != 0) return set_error(h, RPBD_BAD_ARG, "batched lanczos: offsets must start at 0");
+    RPBD_TRY(batched_check_offsets(h, n_sys, offsets));  // (before chunks are cut from them)
     const int64_t n = offsets[n_sys];
     if (use_precond && (!h->prec_valid || h->prec_nb * h->prec_nper != n))
         return set_error(h, RPBD_BAD_ARG, "batched lanczos: preconditioner not built for these blobs");

@@ -284,6 +284,7 @@ int adjoint64_impl(rpbd_handle* h, int64_t n, const double* r, const double* u, 
                    cudaStream_t st);
 
 // batched systems (concatenated SoA; host offsets)
+int batched_check_offsets(rpbd_handle* h, int n_sys, const int64_t* off);
 int batched_apply_impl(rpbd_handle* h, int n_sys, const int64_t* off, const double* r, const void* F, void* U,
                        int k, bool io_double, const int* active, cudaStream_t st);
 // one system through the packed batched tile (two targets per thread): the

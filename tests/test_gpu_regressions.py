@@ -55,3 +55,15 @@ def test_batched_lanczos_layouts_in_flight(use_graph):
     st.synchronize()
     for out, ref in outs:
         assert torch.equal(out, ref)
+
+
+def test_batched_lanczos_refuses_offsets():
+    """Offsets that decrease or do not start at 0 are refused before anything is launched: chunks beyond the last
+    offset were cut from them."""
+    h = Handle(synth.ETA, A, synth.KT)
+    r, W = to_dev(cloud(40, 920)), to_dev(synth.gaussian(921, (3, 40)))
+    out = torch.full_like(W, 5.0)
+    before = h.lib.rpbd_launch_count()
+    for off in ((0, 60, 40), (0, 40, 30, 40), (5, 40), (0, -1, 40)):
+        assert lanczos_batched(h, np.array(off, np.int64), r, W, out, 0, torch.cuda.current_stream()) == -1
+    assert h.lib.rpbd_launch_count() == before and (out == 5.0).all()
