@@ -27,6 +27,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 
 #include "accum.cuh"
 #include "fixed_point.cuh"
@@ -808,6 +809,13 @@ static int apply_typed(rpbd_handle* h, int64_t n, const double* r, const In* F, 
                       : apply_dispatch<double, false, false>(h, n, r, F, U, k, st);
 }
 
+// whether [a, a + na) and [b, b + nb) share bytes
+static bool overlaps(const void* a, size_t na, const void* b, size_t nb)
+{
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + nb && y < x + na;
+}
+
 int mobility_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* F, void* U, int k, int dtype,
                         bool io_double, cudaStream_t st)
 {
@@ -838,10 +846,14 @@ int mobility_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* 
     }
     // the packed symmetric kernel takes any n (it sums in fixed point per blob); the one-home kernel only while its partials fit
     const bool packed_sym = h->use_packed && h->p.wall;
+    // U may lie over F or r: the kernels that pack their inputs first allow it,
+    // the one-launch kernel and a second pass over the right-hand sides do not
+    const size_t vec = (size_t)k * 3 * n * (io_double || dtype == RPBD_F64 ? sizeof(double) : sizeof(float));
+    const bool in_place = overlaps(U, vec, F, vec) || overlaps(U, vec, r, sizeof(double) * 3 * n);
     // a small system on the default settings: one launch (the failure-path test
     // wants the bounded waits of the ring kernels, the partials option their
     // partials, a chosen variant that variant)
-    if (dtype == RPBD_F32 && packed_sym && k <= 4 && h->use_sym[sym_class(k)] && h->sym_variant[sym_class(k)] < 0 &&
+    if (!in_place && dtype == RPBD_F32 && packed_sym && k <= 4 && h->use_sym[sym_class(k)] && h->sym_variant[sym_class(k)] < 0 &&
         !h->sym_partials && !h->test_stall && direct_takes(h, n, k))
         return direct_apply_impl(h, n, r, F, U, k, io_double, st);
     if (dtype == RPBD_F32 && k <= 4 && h->use_sym[sym_class(k)] && (packed_sym || sym_bytes <= 16.0 * (1ull << 30)))
@@ -856,7 +868,7 @@ int mobility_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* 
     }
     // FP64: the symmetric kernel; the one-direction kernel for many right-hand
     // sides and for systems whose partials would not fit
-    if (dtype == RPBD_F64 && sym64_takes(h, n, k))
+    if (dtype == RPBD_F64 && !(in_place && k > 4) && sym64_takes(h, n, k))
         return sym64_apply_impl(h, n, r, (const double*)F, (double*)U, k, st);
     if (io_double || dtype == RPBD_F64)
         return apply_typed<double, double>(h, n, r, (const double*)F, (double*)U, k, dtype, st);

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_1709_02410_gb300 import Handle, synth
+from paper_1709_02410_gb300 import F32, Handle, synth
 
 from gpu_util import to_dev
 
@@ -67,3 +67,28 @@ def test_batched_lanczos_refuses_offsets():
     for off in ((0, 60, 40), (0, 40, 30, 40), (5, 40), (0, -1, 40)):
         assert lanczos_batched(h, np.array(off, np.int64), r, W, out, 0, torch.cuda.current_stream()) == -1
     assert h.lib.rpbd_launch_count() == before and (out == 5.0).all()
+
+
+# 960 / 961: one launch, three launches (FP32, k <= 2); FP64 k = 6: two passes
+@pytest.mark.parametrize("n", [33, 960, 961, 2000])
+@pytest.mark.parametrize("cell", [0.0, 45.3])
+def test_matvec_in_place(n, cell):
+    """U over F, over the positions, and shifted against F by one right-hand side: the one-launch kernel read forces that
+    other blocks had overwritten, and later passes of an FP64 matvec read what the first had written."""
+    h = Handle(synth.ETA, A, synth.KT, Lx=cell, Ly=cell)
+    r = to_dev(cloud(n, 930 + n))
+    for dtype, mode in ((torch.float32, None), (torch.float64, None), (torch.float64, F32)):
+        for k in (1, 2, 4, 6):
+            F = to_dev(synth.gaussian(931 + k, (k, 3, n)), dtype)
+            tol = 1e-12 if dtype == torch.float64 and mode is None else 1e-5  # (the other kernel's rounding)
+            ref = h.mobility_apply(r, F, dtype=mode)
+            near = lambda U: float((U - ref).norm() / ref.norm()) <= tol
+            for _ in range(3):
+                G = F.clone()
+                assert h.mobility_apply(r, G, dtype=mode, out=G) is G and near(G)
+                B = torch.zeros((k + 1, 3, n), dtype=dtype, device=r.device)
+                B[:k] = F
+                assert near(h.mobility_apply(r, B[:k], dtype=mode, out=B[1:]))
+                if dtype == torch.float64:
+                    B[0] = r
+                    assert near(h.mobility_apply(B[0], F, dtype=mode, out=B[:k]))
