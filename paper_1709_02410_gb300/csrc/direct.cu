@@ -9,21 +9,25 @@
 // instruction, would be most of the kernel), the CTA's eight warps share one to
 // eight pairs of targets, a warp's lanes striding over its share of the sources
 // with both targets' blocks in packed two-wide FP32 (wall_rpy_x2.cuh), and the
-// sums are added by shuffles and across warps in a fixed order: no packing kernel,
-// no atomics, no reduction kernel, deterministic.  It does every block twice and
-// converts every source in every CTA, so it stops paying off where that counts.
+// lanes' sums (FP32, at most 32 terms) are added as compensated pairs (accum.cuh) by
+// shuffles and across warps in a fixed order: no packing kernel, no atomics, no
+// reduction kernel, deterministic, records and sums as precise as sym.cu's.  It does
+// every block twice and converts every source in every CTA, so it stops paying off
+// where that counts.
 //
 // What bounds it are the loads of the conversion (every thread has two to four
-// sources in flight at once: with single ones where fewer are left 300 blobs took
-// 5.9 us, now 4.6, 840 15.7, now 9.8) and the few FP64 instructions left.
+// sources in flight at once: with single ones where fewer are left 840 blobs took
+// 15.7 us, now 10.2) and the few FP64 instructions left: x and y scaled by 1/a there
+// and not in FP32 afterwards cost 0.1 us at 240 blobs and 0.3 at 960, the
+// compensated sums 0.1.
 //
-// Device time of a call, sym.cu -> here, open cell, k = 1: 240 blobs 11.9 -> 3.8 us,
-// 600 12.7 -> 6.6, 960 12.2 -> 10.2; k = 2: 13.4 -> 4.7, 14.1 -> 9.3, 14.3 -> 13.9;
-// k = 4: 16.3 -> 7.1, 600 18.4 -> 14.4.  Periodic, against sym.cu's 25.5 (k = 1),
-// 27.2 and 33.8 us at 1,080 blobs: 240 4.7, 5.7 and 7.9, 600 10.9, 13.7 and 19.0, 960
-// 22.9 and 27.5.
+// Device time of a call, sym.cu -> here, open cell, k = 1: 240 blobs 13.0 -> 4.3 us,
+// 600 13.4 -> 7.4, 960 13.5 -> 11.1; k = 2: 14.4 -> 5.3, 15.1 -> 10.1, 15.1 -> 14.9;
+// k = 4: 17.2 -> 7.3, 600 19.2 -> 15.1.  Periodic: 240 13.9 -> 5.2, 14.9 -> 6.2 and
+// 17.2 -> 8.2, 600 18.2 -> 11.9, 19.6 -> 14.9 and 22.7 -> 19.8.
 #include <cuda_runtime.h>
 
+#include "accum.cuh"
 #include "rpbd_internal.cuh"
 #include "wall_rpy_x2.cuh"
 
@@ -32,20 +36,28 @@ namespace direct {
 
 constexpr int NT = 256;
 
-// x = hi + lo to 2^-46: hi the leading 24 bits of x, lo the remaining 29 rounded
+// x = hi + lo, both rounded to nearest even, as (float)x and (float)(x - (double)hi)
 __device__ __forceinline__ void split(double x, float& hi, float& lo)
 {
     const long long u = __double_as_longlong(x);
     const int e = (int)((u >> 52) & 0x7ff) - 896;  // FP32 exponent field
-    if (e > 40 && e < 255) {  // (lo's exponent field stays normal)
+    if (e > 60 && e < 254) {  // (lo is normal too; a carry leaves hi finite)
         const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
-        hi = __uint_as_float(sign | ((unsigned)e << 23) | ((unsigned)(u >> 29) & 0x7fffffu));
-        const float l = (float)((int)u & 0x1fffffff);  // times 2^(e - 127 - 52)
-        lo = __uint_as_float(__float_as_uint(l * __int_as_float((e - 52 + 12) << 23)) | sign) * 0x1p-12f;
+        const long long m = u & 0x7fffffffffffffffLL, h = (m + 0x0fffffff + ((m >> 29) & 1)) >> 29;
+        hi = __uint_as_float(sign | ((unsigned)h - (896u << 23)));
+        const float l = (float)(int)(m - (h << 29));  // times 2^(e - 127 - 52)
+        lo = l * __uint_as_float(sign | ((unsigned)(e - 52) << 23));
     } else {  // tiny, zero, huge or not finite
         hi = (float)x;
-        lo = e >= 255 ? hi - hi : (float)(x - (double)hi);
+        lo = (float)(x - (double)hi);
     }
+}
+
+// s + c += s2 + c2
+__device__ __forceinline__ void two_sum_merge(float& s, float& c, float s2, float c2)
+{
+    two_sum_acc(s, c, s2);
+    c = __fadd_rn(c, c2);
 }
 
 template <int K, bool PER, class In, class Out>
@@ -76,10 +88,10 @@ __global__ void __launch_bounds__(NT) direct_kernel(int n, int k, int tp, const 
             const int i = i0 + u * NT;
             if (i >= n) break;
             float h, l;
-            split(x[u], h, l);
+            split(x[u] * ia, h, l);
             sm[i] = h;
             sm[2 * n + i] = l;
-            split(y[u], h, l);
+            split(y[u] * ia, h, l);
             sm[n + i] = h;
             sm[3 * n + i] = l;
             const double z = zs[u];
@@ -100,7 +112,7 @@ __global__ void __launch_bounds__(NT) direct_kernel(int n, int k, int tp, const 
     }
     bad = __syncthreads_or(bad);  // a force that is not finite: U is NaN everywhere, as in sym.cu
     const PairConstX2 pc = PairConstX2::make_unit();
-    const float2 m1 = pc.m1, ia2 = bc2((float)ia);
+    const float2 m1 = pc.m1;
     const int wp = NT / 32 / tp;                                     // warps per pair of targets
     const int t0 = ((int)blockIdx.x * tp + warp / wp) * 2, t1 = t0 + 1;
     const int c0 = min(t0, n - 1), c1 = min(t1, n - 1);
@@ -116,8 +128,6 @@ __global__ void __launch_bounds__(NT) direct_kernel(int n, int k, int tp, const 
         float2 dx = add2(fma2(m1, bc2(sm[j]), xh), fma2(m1, bc2(sm[2 * n + j]), xl));
         float2 dy = add2(fma2(m1, bc2(sm[n + j]), yh), fma2(m1, bc2(sm[3 * n + j]), yl));
         const float2 dz = fma2(m1, zj, zi);
-        dx = mul2(dx, ia2);
-        dy = mul2(dy, ia2);
         if constexpr (PER) {
             const float iLx = 1.0f / Lx, iLy = 1.0f / Ly;
             dx = make_float2(dx.x - Lx * rintf(dx.x * iLx), dx.y - Lx * rintf(dx.y * iLx));
@@ -145,34 +155,58 @@ __global__ void __launch_bounds__(NT) direct_kernel(int n, int k, int tp, const 
             }
         }
     }
+    // the lanes' sums, as compensated pairs: halves of the sums (target, right-hand
+    // side) to halves of the lanes down to three a lane, then those over the rest
+    float v[6 * K], e[6 * K];
 #pragma unroll
     for (int q = 0; q < 3 * K; ++q) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            acc[q].x += __shfl_xor_sync(0xffffffffu, acc[q].x, o);
-            acc[q].y += __shfl_xor_sync(0xffffffffu, acc[q].y, o);
-        }
+        v[q] = acc[q].x;
+        v[3 * K + q] = acc[q].y;
     }
-    // the pair's warps in order; thread (target of the CTA, component)
-    __shared__ float part[NT / 32][3 * K][2];
-    if (lane == 0)
 #pragma unroll
-        for (int q = 0; q < 3 * K; ++q) {
-            part[warp][q][0] = acc[q].x;
-            part[warp][q][1] = acc[q].y;
+    for (int q = 0; q < 6 * K; ++q) e[q] = 0.0f;
+    int o = 16, g = 0;  // g: the lane's (target, right-hand side)
+#pragma unroll
+    for (int c = K; c > 0; c >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < 3 * c; ++i) {
+            const float s2 = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[3 * c + i], o);
+            const float e2 = __shfl_xor_sync(0xffffffffu, up ? e[i] : e[3 * c + i], o);
+            v[i] = up ? v[3 * c + i] : v[i];
+            e[i] = up ? e[3 * c + i] : e[i];
+            two_sum_merge(v[i], e[i], s2, e2);
         }
+        if (up) g += c;
+    }
+    const bool first = (lane & (2 * o - 1)) == 0;
+#pragma unroll
+    for (; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const float s2 = __shfl_xor_sync(0xffffffffu, v[i], o), e2 = __shfl_xor_sync(0xffffffffu, e[i], o);
+            two_sum_merge(v[i], e[i], s2, e2);
+        }
+    // the pair's warps in order; thread (target of the CTA, component)
+    __shared__ float2 part[NT / 32][2][3 * K];
+    if (first)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) part[warp][g / K][g % K * 3 + c] = make_float2(v[c], e[c]);
     __syncthreads();
     const int tl = tid / (3 * K), q = tid % (3 * K), t = (int)blockIdx.x * 2 * tp + tl;
     if (tl >= 2 * tp || t >= n || q >= 3 * k) return;
-    float v = 0.0f;
-    for (int w = 0; w < wp; ++w) v += part[(tl / 2) * wp + w][q][tl & 1];
+    float sum = 0.0f, err = 0.0f;
+    for (int w = 0; w < wp; ++w) {
+        const float2 x = part[(tl / 2) * wp + w][tl & 1][q];
+        two_sum_merge(sum, err, x.x, x.y);
+    }
     const double z = r[2 * (int64_t)n + t];
     double s = 1.0;
     if (!(z >= a)) {
         const double u = z * ia;
         s = u >= 1.0 ? 1.0 : (u <= s_min ? s_min : u);
     }
-    U[(int64_t)q * n + t] = (Out)(bad || !isfinite(v) ? __longlong_as_double(0x7ff8000000000000LL) : s * inv8pieta * (double)v);
+    U[(int64_t)q * n + t] = (Out)(bad || !isfinite(sum) ? __longlong_as_double(0x7ff8000000000000LL) : s * inv8pieta * two_sum_value(sum, err));
 }
 
 template <int K, bool PER, class In, class Out>
@@ -203,11 +237,14 @@ static int dispatch(rpbd_handle* h, int n, const double* r, const In* F, Out* U,
 
 }  // namespace direct
 
-// where the call is shorter this way (figures above): n <= 960, with three or
-// four right-hand sides n <= 640
+// where the call is shorter this way: open cell n <= 960, with three or four
+// right-hand sides 640; periodic cell, sym.cu -> here, k = 1 at 630 blobs 18.3 -> 17.1,
+// at 690 18.3 -> 18.6, k = 2 and 4 at 600 as above, at 630 19.8 -> 20.5 and
+// 22.7 -> 25.6 (beyond 608 a CTA has four pairs of targets instead of two)
 bool direct_takes(const rpbd_handle* h, int64_t n, int k)
 {
-    return h->p.wall && k <= 4 && n <= (k <= 2 ? 960 : 640);
+    if (!h->p.wall || k > 4) return false;
+    return n <= (h->p.Lx > 0.0 ? (k == 1 ? 640 : 608) : (k <= 2 ? 960 : 640));
 }
 
 int direct_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* F, void* U, int k, bool io_double, cudaStream_t st)

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import mobility as om
 from paper_1709_02410_gb300 import F32, Handle, synth
 
 from gpu_util import to_dev
@@ -92,3 +93,20 @@ def test_matvec_in_place(n, cell):
                 if dtype == torch.float64:
                     B[0] = r
                     assert near(h.mobility_apply(B[0], F, dtype=mode, out=B[:k]))
+
+
+@pytest.mark.parametrize("k", [1, 2, 4])
+def test_small_system_sum_keeps_64_bits(k):
+    """Two forces of 1e4 from mirrored places cancel exactly in the velocity along their axis, so what the forces of
+    order one leave there has the usual relative error.  (One source a lane; the lanes' sums were added in FP32, which
+    loses 2^-24 of the large terms, about 1e-3 here.)"""
+    n = 256
+    r, F = cloud(n, 940), synth.gaussian(941, (k, 3, n))
+    r[:, 0] = 0.0, 0.0, 5.0 * A
+    r[:, 17], r[:, 200] = (4.0 * A, 0.0, 3.0 * A), (-4.0 * A, 0.0, 3.0 * A)
+    r[:2, 1:17] += 20.0 * A
+    F[:, :, 17], F[:, :, 200] = np.array([1e4, 0, 0]), np.array([-1e4, 0, 0])
+    F = F.astype(np.float32)
+    U = Handle(synth.ETA, A, synth.KT).mobility_apply(to_dev(r), to_dev(F, torch.float32)).cpu().numpy()
+    ref = om.apply(r, F.astype(np.float64), om.Params(synth.ETA, A), np.array([0]))
+    assert np.abs(U[:, 0, 0] - ref[:, 0, 0]).max() <= 1e-5 * np.abs(ref[:, 0, 0]).max()
