@@ -84,20 +84,33 @@ __device__ __forceinline__ void overlap(S r2, S ri, const C& c, S& c1, S& c2, S&
 {
     if (r2 < c.template get<FOUR, S>()) {
         const S ks = c.template get<KSELF, S>(), ko = c.template get<KOVL, S>(), i8 = c.template get<I8, S>();
-        const bool apart = r2 > (sizeof(S) == 8 ? S(1e-290) : S(0));  // (closer: the self block to rounding)
+        const bool apart = r2 > (sizeof(S) == 8 ? S(1e-200) : S(4e-26));  // (r^-3 finite; closer: coincident)
         c1 = apart ? ks - ko * (r2 * ri) : ks;
         c2 = apart ? ri * i8 : S(0);
         c1p = apart ? S(-0.5) * ko * ri : S(0);
         c2p = apart ? S(-0.5) * i8 * (ri * ri * ri) : S(0);
     }
 }
+// (closer than 1e-90 r^-3 would overflow: the gradient depends on the direction of the
+// separation only, which a factor 2^200 keeps)
 template <class C>
-__device__ __forceinline__ void overlap_(double r2, double ri, const C& c, double& c1, double& c2, double& c1p, double& c2p)
+__device__ __forceinline__ void overlap_(double r2, double ri, const C& c, double& dx, double& dy, double& dz, double& c1,
+                                         double& c2, double& c1p, double& c2p)
 {
-    overlap<double>(r2, ri, c, c1, c2, c1p, c2p);
+    if (r2 < c.template get<FOUR, double>()) {
+        if (r2 < 1e-180) {
+            dx *= 0x1p200;
+            dy *= 0x1p200;
+            dz *= 0x1p200;
+            r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+            ri = rsq_(r2);
+        }
+        overlap<double>(r2, ri, c, c1, c2, c1p, c2p);
+    }
 }
 template <class C>
-__device__ __forceinline__ void overlap_(float2 r2, float2 ri, const C& c, float2& c1, float2& c2, float2& c1p, float2& c2p)
+__device__ __forceinline__ void overlap_(float2 r2, float2 ri, const C& c, float2&, float2&, float2&, float2& c1, float2& c2,
+                                         float2& c1p, float2& c2p)
 {
     if (r2.x < 4.0f || r2.y < 4.0f) {
         overlap<float>(r2.x, ri.x, c, c1.x, c2.x, c1p.x, c2p.x);
@@ -115,7 +128,7 @@ struct PairGrad {
 template <bool WALL, int K, class V, class C, class Src>
 __device__ __forceinline__ void pair_grad(V dx, V dy, V zi, V zj, const C& c, const V* A, const V* B, Src ce, PairGrad<V>& g)
 {
-    const V dz = sub_(zi, zj);
+    V dz = sub_(zi, zj);
     const V rho2 = fma_(dy, dy, mul_(dx, dx));
     const V r2 = fma_(dz, dz, rho2);
     const V ri = rsq_(r2), ri2 = mul_(ri, ri), ri3 = mul_(ri, ri2);
@@ -123,7 +136,7 @@ __device__ __forceinline__ void pair_grad(V dx, V dy, V zi, V zj, const C& c, co
     V c2 = mul_(ri3, fma_(c.template get<CM2, V>(), ri2, num_<V>(1.0)));
     V c1p = mul_(ri3, fma_(c.template get<CM1, V>(), ri2, num_<V>(-0.5)));
     V c2p = mul_(mul_(ri3, ri2), fma_(c.template get<C5, V>(), ri2, num_<V>(-1.5)));
-    overlap_(r2, ri, c, c1, c2, c1p, c2p);
+    overlap_(r2, ri, c, dx, dy, dz, c1, c2, c1p, c2p);
     // contractions, summed over the right-hand sides
     V S1, S3, Q, R, Z, T1x, T1y, T2x, T2y, qx, qy;
 #pragma unroll

@@ -62,10 +62,10 @@ __device__ __forceinline__ void free_space(double r2, const Const& c, double& ri
     c1 = fma(c.c23, rinv3, rinv);
     g = fma(c.m2, rinv2, 1.0);
     if (__double_as_longlong(r2) < c.four_a2) {  // overlapping or self: rare
-        if (r2 > 1e-290) {
+        if (r2 > 1e-180) {  // (r^-3 is finite)
             c1 = c.k_self - c.k_ovl * (r2 * rinv);
             g = r2 * c.i8;
-        } else {  // (closer than 1e-145: the self block to rounding)
+        } else {  // (closer than 1e-90: the self block to rounding)
             c1 = c.k_self;
             rinv3 = g = 0.0;
         }

@@ -110,3 +110,27 @@ def test_small_system_sum_keeps_64_bits(k):
     U = Handle(synth.ETA, A, synth.KT).mobility_apply(to_dev(r), to_dev(F, torch.float32)).cpu().numpy()
     ref = om.apply(r, F.astype(np.float64), om.Params(synth.ETA, A), np.array([0]))
     assert np.abs(U[:, 0, 0] - ref[:, 0, 0]).max() <= 1e-5 * np.abs(ref[:, 0, 0]).max()
+
+
+@pytest.mark.parametrize("wall,cell", [(True, 0.0), (True, 45.3), (False, 0.0)])
+def test_almost_coincident_blobs(wall, cell):
+    """Blobs so close that r^-3 overflows: velocities as at the smallest separation whose r^-3 is finite, gradients too
+    (they depend on the direction of the separation, however small it is).  The FP64 block and the gradients were
+    infinite or NaN between 1e-145 and 1e-103; in FP32 the gradient counts blobs within 2e-13 a as coincident."""
+    h = Handle(synth.ETA, A, synth.KT, wall=wall, Lx=cell, Ly=cell)
+    r = cloud(40, 950)
+    u, F = synth.gaussian(951, (2, 3, 40))
+    r[0, :2], r[1:, 1] = 0.0, r[1:, 0]
+    calls = [lambda x: h.mobility_apply(x, to_dev(F)), lambda x: h.mobility_adjoint(x, to_dev(u), to_dev(F)),
+             lambda x: h.mobility_adjoint(x, to_dev(u), to_dev(F), dtype=F32)]
+
+    def at(gap):
+        r[0, 1] = gap
+        return [f(to_dev(r)) for f in calls]
+
+    coincident, ref = at(0.0), at(1e-60)
+    for gap in (1e-85, 1e-92, 1e-104, 1e-120, 1e-140, 1e-150):
+        for i, (g, v, tol) in enumerate(zip(at(gap), (coincident[0], ref[1], coincident[2]), (1e-14, 1e-13, 1e-6))):
+            assert float((g - v).norm() / v.norm()) <= tol, (gap, i)
+    for gap in (1e-14 * A, 1e-155, 1e-165, 1e-200, 1e-310):
+        assert all(torch.isfinite(g).all() for g in at(gap)), gap
