@@ -185,7 +185,8 @@ int rpbd_mobility_adjoint_f32(rpbd_handle* h, int64_t n, const double* r, const 
  * four right-hand-side pairs that share each blob pair's block and derivatives.
  * dtype RPBD_F64 or RPBD_F32 selects the pair arithmetic as in the two calls
  * above; sums across tiles are FP64, in a fixed order.  The workspace is at most
- * about 4 GiB, less where device memory is short. */
+ * about 4.5 GiB (from about 5 million blobs in FP64 and 11 in FP32 on, 24 times
+ * the size of a blob's four sums), less where device memory is short. */
 int rpbd_mobility_adjoint_multi(rpbd_handle* h, int64_t n, const double* r, const double* u,
                                 const double* F, int k, double* grad, int dtype, void* stream);
 
@@ -421,6 +422,9 @@ int rpbd_blob_forces(rpbd_handle* h, int64_t n, int nper, const double* r, const
  * system); the FP64 kernels, the gradients and the batched one-direction tiles
  * always keep their partials. */
 #define RPBD_OPT_SYM_PARTIALS 7
+/* value > 0 (default 0: off): workspace buffers larger than value KiB are
+ * refused as if device memory had run out.  For tests of what calls do then. */
+#define RPBD_OPT_TEST_MEMORY 8
 int rpbd_set_option(rpbd_handle* h, int option, int value);
 
 /* Times the FP32 matvec kernels on n blobs at r (k right-hand sides, zero

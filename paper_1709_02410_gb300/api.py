@@ -109,6 +109,11 @@ class Handle:
         (RPBD_TIMEOUT from the synchronising calls) until this is set back off."""
         self._check(self.lib.rpbd_set_option(self.h, 5, int(bool(on))), "set_option")
 
+    def set_test_memory(self, kib: int):
+        """Failure-path test only: workspace buffers above this size (KiB; 0: no limit) are refused as if
+        device memory had run out."""
+        self._check(self.lib.rpbd_set_option(self.h, 8, int(kib)), "set_option")
+
     def set_far_field(self, on: bool):
         """FP32 matvecs with the wall: form every pair block with the cancellation-free
         direct-minus-image differences (FP32 accuracy at any separation, ~9% slower)."""

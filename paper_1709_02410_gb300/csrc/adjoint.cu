@@ -145,7 +145,7 @@ static void pack(rpbd_handle* h, const adj::Cut& c, int kc, const double* r, con
 static int run(rpbd_handle* h, int64_t n, const double* r, const double* u, const double* F, int nr, double* grad,
                cudaStream_t st)
 {
-    const adj::Cut c = adj::cut(n, 2, SMALL_N, MAX_CHUNK, 4 * sizeof(float), h->sm_count);
+    const adj::Cut c = adj::cut(n, 2, SMALL_N, MAX_CHUNK, h->sm_count);
     float4* rec;
     RPBD_TRY(ensure_t(h, BUF_PACK, (size_t)c.n_pad * Rec32<4>::NCH, &rec));
     const double ie = 1.0 / (8.0 * 3.14159265358979323846 * h->p.eta * h->p.a), ig = ie / h->p.a;

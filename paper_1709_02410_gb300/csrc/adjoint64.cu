@@ -35,7 +35,7 @@ int adjoint64_impl(rpbd_handle* h, int64_t n, const double* r, const double* u, 
                    cudaStream_t st)
 {
     using namespace adj64;
-    const adj::Cut c = adj::cut(n, 1, SMALL_N, MAX_CHUNK, 4 * sizeof(double), h->sm_count);
+    const adj::Cut c = adj::cut(n, 1, SMALL_N, MAX_CHUNK, h->sm_count);
     const double i8 = 1.0 / (8.0 * 3.14159265358979323846 * h->p.eta);
     auto launch = [&](const adj::Cut& g, int kc, int m0, double* partial, const adj::Out& o) -> int {
         const double *um = u + (int64_t)m0 * 3 * n, *Fm = F + (int64_t)m0 * 3 * n;

@@ -20,8 +20,11 @@
 //
 // Cutting as in sym64.cu: CTAs of one warp for small n, four beyond, items of
 // `chunk` visitor tiles, the 32 steps of a tile over `parts` items for very
-// small n.  Home tiles run in groups whose partials stay under GROUP_BYTES, so
-// any n takes bounded memory.
+// small n.  The partials stay under GROUP_BYTES (or MIN_ROWS rows, from 5 million
+// blobs in FP64 and 11 in FP32): home tiles run in groups, for the visitors' rows;
+// for the homes' rows, one per item, FP64 takes longer items and FP32, whose sums
+// should not get longer, groups of items.  At 10^6 blobs the homes' rows alone
+// would be 14.6 and 29 GiB.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -37,6 +40,7 @@ namespace adj {
 
 constexpr int VT = 32;                            // visitor tile
 constexpr double GROUP_BYTES = 4.0 * (1ull << 30);
+constexpr int64_t MIN_ROWS = 24;  // 12 home tiles x 12 items a launch
 
 // how one launch (a group of home tiles) is cut
 struct Cut {
@@ -45,8 +49,8 @@ struct Cut {
     int vpw, vph;      // visitor tiles per warp's home blobs, per home tile
     int tiles;         // visitor tiles
     int chunk, parts;  // visitor tiles per item (a power of two), items per tile's steps
-    int h0, hg;        // first home tile, home tiles of the group
-    int items;         // chunks of the longest home tile
+    int h0, hg;        // first home tile, home tiles of the launch
+    int i0, items;     // first item of every home tile, items of the launch
 };
 
 // one launch's outputs: G [4][n_pad] carries the sums between groups and passes
@@ -150,17 +154,24 @@ __global__ void __launch_bounds__(32 * RS) adjoint_reduce_kernel(Cut c, Out o, c
     pdl_wait();
     pdl_trigger();
     const int lane = threadIdx.x & 31, y = threadIdx.x >> 5;
-    const int tile = blockIdx.x, home = tile / c.vph, sub = tile % c.vph, q0 = blockIdx.y, nq = q0 == 2 ? 2 : 1;
+    const int vb = __ffs(c.vph) - 1, cb = __ffs(c.chunk) - 1;  // (powers of two)
+    const int tile = blockIdx.x, home = tile >> vb, sub = tile - (home << vb), q0 = blockIdx.y, nq = q0 == 2 ? 2 : 1;
     if (home < c.h0) return;  // complete already
     const bool own = home < c.h0 + c.hg;
     const int64_t i = (int64_t)tile * VT + lane;
-    const int vis = (min(c.h0 + c.hg, home) - c.h0 + (own && sub >= c.vpw ? 1 : 0)) * c.parts;
-    const int rows = vis + (own ? (c.tiles - home * c.vph + c.chunk - 1) / c.chunk * c.parts : 0);
-    const int shift = c.hg * c.parts - vis;
+    // home tiles lo..hi of the launch met this tile in its items' range, the tile's own past its warps' own blobs
+    const int beg = c.i0 << cb, end = beg + (c.items << cb);
+    const int lo = max(c.h0, tile >= end ? ((tile - end) >> vb) + 1 : 0);
+    int hi = min(c.h0 + c.hg - 1, own && sub >= c.vpw ? home : home - 1);
+    hi = tile >= beg ? min(hi, (tile - beg) >> vb) : -1;
+    const int vis = max(0, hi - lo + 1) * c.parts;
+    const int its = (c.tiles - (home << vb) + c.chunk - 1) >> cb;
+    const int rows = vis + (own ? max(0, min(its - c.i0, c.items)) * c.parts : 0);
+    const int skip = (lo - c.h0) * c.parts, shift = c.hg * c.parts - vis;
     const int64_t ld = 4 * c.n_pad;
     for (int q = 0; q < nq; ++q) {
         const S* p = partial + (q0 + q) * c.n_pad + i;
-        sm[q][y][lane] = sum_rows<S>(y, RS, rows, [&](int e) { return p + (e < vis ? e : e + shift) * ld; });
+        sm[q][y][lane] = sum_rows<S>(y, RS, rows, [&](int e) { return p + (e < vis ? e + skip : e + shift) * ld; });
     }
     __syncthreads();
     if (y || i >= c.n) return;
@@ -222,7 +233,7 @@ __global__ void __launch_bounds__(128) adjoint_kernel(Cut c, int nr, const doubl
     extern __shared__ __align__(128) unsigned char smem_raw[];
     S* red = reinterpret_cast<S*>(smem_raw + 2 * STAGE);  // [2 buffers][nw][4][VT]
     const int home = c.h0 + blockIdx.x, item = blockIdx.y, part = blockIdx.z;
-    const int tile0 = home * c.vph + item * c.chunk;  // visitors: the home tile's own blobs and all after them
+    const int tile0 = home * c.vph + (c.i0 + item) * c.chunk;  // visitors: the home tile's own blobs and all after them
     const int ntile = min(c.chunk, c.tiles - tile0);
     pdl_wait();
     pdl_trigger();
@@ -388,7 +399,7 @@ __global__ void __launch_bounds__(128) adjoint_kernel(Cut c, int nr, const doubl
 }
 
 // cuts n blobs; vpw: visitor tiles per warp's home blobs (1: FP64, 2: packed FP32)
-inline Cut cut(int64_t n, int vpw, int64_t small_n, int max_chunk, size_t row_bytes, int sm_count)
+inline Cut cut(int64_t n, int vpw, int64_t small_n, int max_chunk, int sm_count)
 {
     Cut c;
     c.n = n;
@@ -412,19 +423,27 @@ inline Cut cut(int64_t n, int vpw, int64_t small_n, int max_chunk, size_t row_by
     const bool few = count(c.chunk) * c.parts <= 4 * (int64_t)sm_count;
     if (few && vpw == 1) c.parts *= 2;
     c.threads = few && vpw == 1 ? 128 : 32 * c.nw;
-    // (past 65,535 items, the grid's limit, longer chunks)
-    while ((c.tiles + c.chunk - 1) / c.chunk > 65535) c.chunk *= 2;
-    const int64_t fit = (int64_t)(GROUP_BYTES / ((double)row_bytes * c.n_pad * c.parts));
-    const int64_t items = (c.tiles + c.chunk - 1) / c.chunk;
-    c.h0 = 0;
-    c.hg = (int)std::max<int64_t>(1, std::min<int64_t>(T, fit - items));
-    c.items = (int)items;
+    c.h0 = c.i0 = 0;
+    c.hg = T;
+    c.items = (c.tiles + c.chunk - 1) / c.chunk;
     return c;
 }
 
+// home tiles and items of a launch, half of the rows that fit for the items;
+// longer: items may not be split into groups but take more visitor tiles
+inline void group(Cut& c, int64_t rows, bool longer)
+{
+    const int T = c.tiles / c.vph;
+    const int64_t most = std::min<int64_t>(65535, std::max(std::max<int64_t>(1, rows / 2), rows - T));
+    if (longer)
+        while ((c.tiles + c.chunk - 1) / c.chunk > most) c.chunk *= 2;
+    c.items = (int)std::min<int64_t>((c.tiles + c.chunk - 1) / c.chunk, most);
+    c.hg = (int)std::max<int64_t>(1, std::min<int64_t>(T, rows - c.items));
+}
+
 // all launches of one call: passes of up to four right-hand sides, groups of
-// home tiles.  pass(m0, kc): prepares pass m0 (FP32: packs its records);
-// launch(c, kc, m0, out): one launch.
+// home tiles and of items.  pass(m0, kc): prepares pass m0 (FP32: packs its
+// records); launch(c, kc, m0, out): one launch.
 template <class S, class Pass, class Launch>
 static int run_all(rpbd_handle* h, Cut c, int nr, double* grad, double ig, double ie, Pass pass, Launch launch, cudaStream_t st)
 {
@@ -432,13 +451,21 @@ static int run_all(rpbd_handle* h, Cut c, int nr, double* grad, double ig, doubl
     const int T = c.tiles / c.vph;
     unsigned char* base;
     const size_t g_bytes = sizeof(double) * 4 * c.n_pad, t_bytes = ((size_t)T * sizeof(int) + 15) / 16 * 16;
-    for (;;) {  // smaller groups where the memory left is short
-        const size_t words = (size_t)((int64_t)c.hg + c.items) * c.parts * 4 * c.n_pad;
-        const int s = ensure_t(h, BUF_PARTIAL, words * sizeof(S) + g_bytes + t_bytes, &base);
-        if (s == RPBD_OK) break;
-        if (s != RPBD_NO_MEM || c.hg == 1) return s;
-        cudaGetLastError();
-        c.hg = (c.hg + 1) / 2;
+    const double row_bytes = 4.0 * sizeof(S) * (double)c.n_pad * c.parts;
+    const Cut whole = c;
+    double limit = GROUP_BYTES;
+    for (;;) {  // smaller groups where device memory is short
+        c = whole;
+        group(c, std::max((int64_t)(limit / row_bytes), limit < GROUP_BYTES ? 2 : MIN_ROWS), tickets);
+        const size_t part = (size_t)((int64_t)c.hg + c.items) * (size_t)row_bytes, bytes = part + g_bytes + t_bytes;
+        const bool least = c.hg + c.items <= 2;
+        if (least || worth_trying(h, BUF_PARTIAL, bytes, st)) {
+            const int s = ensure_t(h, BUF_PARTIAL, bytes, &base);
+            if (s == RPBD_OK) break;
+            if (s != RPBD_NO_MEM || least) return s;
+            cudaGetLastError();
+        }
+        limit = 0.5 * (double)part;
     }
     Out o;
     o.G = reinterpret_cast<double*>(base);
@@ -447,20 +474,24 @@ static int run_all(rpbd_handle* h, Cut c, int nr, double* grad, double ig, doubl
     o.grad = grad;
     o.ig = ig;
     o.ie = ie;
-    const int hg = c.hg;
+    const int hg = c.hg, items = c.items;
     for (int m0 = 0; m0 < nr; m0 += 4) {
         const int kc = std::min(4, nr - m0);
-        if (tickets) RPBD_CU(h, cudaMemsetAsync(o.ticket, 0, t_bytes, st));
         RPBD_TRY(pass(m0, kc));
         for (int h0 = 0; h0 < T; h0 += hg) {
-            if (tickets && h0) RPBD_CU(h, cudaMemsetAsync(o.ticket, 0, t_bytes, st));
             c.h0 = h0;
             c.hg = std::min(hg, T - h0);
-            o.first = m0 == 0 && h0 == 0;
-            o.last = m0 + 4 >= nr;
-            RPBD_TRY(launch(c, kc, m0, partial, o));
-            count_launch();
-            RPBD_LAUNCH_CHECK(h);
+            const int own = (c.tiles - h0 * c.vph + c.chunk - 1) / c.chunk;  // items of the first home tile, the most
+            for (int i0 = 0; i0 < own; i0 += items) {
+                if (tickets) RPBD_CU(h, cudaMemsetAsync(o.ticket, 0, t_bytes, st));
+                c.i0 = i0;
+                c.items = std::min(items, own - i0);
+                o.first = m0 == 0 && h0 == 0 && i0 == 0;
+                o.last = m0 + 4 >= nr && i0 + items >= own;
+                RPBD_TRY(launch(c, kc, m0, partial, o));
+                count_launch();
+                RPBD_LAUNCH_CHECK(h);
+            }
         }
     }
     return RPBD_OK;

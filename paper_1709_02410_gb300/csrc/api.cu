@@ -71,15 +71,29 @@ int ensure(rpbd_handle* h, Buf b, size_t bytes, void** out)
             if (e != cudaSuccess) return set_error(h, RPBD_CUDA, std::string("cudaFree: ") + cudaGetErrorString(e));
         }
         size_t want = bytes + bytes / 8;  // headroom for slowly growing sizes
-        cudaError_t e = cudaMalloc(&h->buf[b], want);
+        cudaError_t e = h->test_memory && bytes > h->test_memory ? cudaErrorMemoryAllocation : cudaMalloc(&h->buf[b], want);
         if (e != cudaSuccess) {
             h->buf[b] = nullptr;
+            h->no_mem = bytes < h->no_mem ? bytes : h->no_mem;
             return set_error(h, RPBD_NO_MEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
         }
         h->cap[b] = want;
+        if (bytes >= h->no_mem) h->no_mem = SIZE_MAX;
     }
     *out = h->buf[b];
     return RPBD_OK;
+}
+
+bool worth_trying(rpbd_handle* h, Buf b, size_t bytes, cudaStream_t st)
+{
+    if (h->cap[b] >= bytes || bytes < h->no_mem) return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (h->no_mem_skipped < 255 || cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        h->no_mem_skipped += h->no_mem_skipped < 255;
+        return false;
+    }
+    h->no_mem_skipped = 0;
+    return true;
 }
 
 }  // namespace rpbd
@@ -312,6 +326,10 @@ int rpbd_set_option(rpbd_handle* h, int option, int value)
         for (int c = 0; c < 3; ++c) h->sym_variant[c] = value;
         return RPBD_OK;
     case RPBD_OPT_TEST_STALL: h->test_stall = value != 0; return RPBD_OK;
+    case RPBD_OPT_TEST_MEMORY:
+        if (value < 0) return set_error(h, RPBD_BAD_ARG, "test memory limit must not be negative");
+        h->test_memory = (size_t)value * 1024;
+        return RPBD_OK;
     case RPBD_OPT_FARFIELD: h->far_field = value != 0; return RPBD_OK;
     case RPBD_OPT_SYM_PARTIALS: h->sym_partials = value != 0; return RPBD_OK;
     default: return set_error(h, RPBD_BAD_ARG, "unknown option");

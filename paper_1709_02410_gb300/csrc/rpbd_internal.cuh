@@ -134,6 +134,12 @@ struct rpbd_handle {
     // first source stage's barrier without a copy, so its bounded wait runs
     // out after a short limit and the kernel reports RPBD_TIMEOUT
     int test_stall = 0;
+    // failure-path test (RPBD_OPT_TEST_MEMORY): larger workspace buffers are refused (0: none)
+    size_t test_memory = 0;
+    // the smallest buffer that device memory did not have lately, and how often
+    // one of at least that size was not tried again since (worth_trying)
+    size_t no_mem = SIZE_MAX;
+    int no_mem_skipped = 0;
     // RPBD_OPT_FARFIELD: single-system FP32 matvecs with the wall form every
     // block with the cancellation-free direct-minus-image differences
     int far_field = 0;
@@ -175,6 +181,10 @@ inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 }
 
 int set_error(rpbd_handle* h, int code, const std::string& msg);
+// whether to ask for a buffer of this size where a smaller one would do too: not
+// while an allocation no larger has failed, but for every 256th time (a failing
+// attempt frees the buffer that is there, synchronises the device and breaks a capture)
+bool worth_trying(rpbd_handle* h, Buf b, size_t bytes, cudaStream_t st);
 // true the first time it is called for (h's device, key), false afterwards;
 // guards per-device one-time settings such as a kernel's shared-memory limit
 bool once_per_device(rpbd_handle* h, const void* key);

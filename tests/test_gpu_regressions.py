@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from oracle import mobility as om
-from paper_1709_02410_gb300 import F32, Handle, synth
+from paper_1709_02410_gb300 import F32, F64, Handle, synth
 
 from gpu_util import to_dev
 
@@ -134,3 +134,39 @@ def test_almost_coincident_blobs(wall, cell):
             assert float((g - v).norm() / v.norm()) <= tol, (gap, i)
     for gap in (1e-14 * A, 1e-155, 1e-165, 1e-200, 1e-310):
         assert all(torch.isfinite(g).all() for g in at(gap)), gap
+
+
+# home tiles of one and four warps; the last: one home tile and one item of every step part a launch
+@pytest.mark.parametrize("n,kib", [(3000, 1000), (9000, 3000), (700, 200)])
+@pytest.mark.parametrize("wall,cell", [(True, 0.0), (True, 45.3), (False, 0.0)])
+def test_adjoint_with_little_memory(n, kib, wall, cell):
+    """Partials cut into groups of home tiles and, in FP32, of items give the sums of the whole."""
+    r = to_dev(cloud(n, 960))
+    new = lambda: Handle(synth.ETA, A, synth.KT, wall=wall, Lx=cell, Ly=cell)
+    h, g = new(), new()
+    h.set_test_memory(kib)
+    for k in (1, 6):
+        u, F = (to_dev(synth.gaussian(961 + i, (k, 3, n))) for i in range(2))
+        for dtype in (F64, F32):
+            if dtype == F32 and n == 700:
+                h.set_test_memory(300)  # (its records)
+            before = h.lib.rpbd_launch_count()
+            a = h.mobility_adjoint(r, u, F, dtype=dtype)
+            launches = h.lib.rpbd_launch_count() - before
+            b = g.mobility_adjoint(r, u, F, dtype=dtype)
+            assert launches > 2 * (h.lib.rpbd_launch_count() - before - launches)
+            assert float((a - b).norm() / b.norm()) <= 1e-12
+
+
+def test_adjoint_workspace_is_bounded():
+    """The homes' partial rows, one per item, grew with the square of n: 11 GiB at this size."""
+    n = 600_000
+    args = [to_dev(x) for x in (cloud(n, 970), *synth.gaussian(971, (2, 3, n)))]
+    h = Handle(synth.ETA, A, synth.KT)
+    out = torch.empty_like(args[0])
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    h.mobility_adjoint(*args, out=out, dtype=F32)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] <= 5 << 30  # 4 GiB of partials, an eighth of headroom, records, sums
+    assert torch.isfinite(out).all()
