@@ -868,7 +868,7 @@ int mobility_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* 
     }
     // FP64: the symmetric kernel; the one-direction kernel for many right-hand
     // sides and for systems whose partials would not fit
-    if (dtype == RPBD_F64 && !(in_place && k > 4) && sym64_takes(h, n, k))
+    if (dtype == RPBD_F64 && !(in_place && k > 4) && sym64_takes(h, n, k, st))
         return sym64_apply_impl(h, n, r, (const double*)F, (double*)U, k, st);
     if (io_double || dtype == RPBD_F64)
         return apply_typed<double, double>(h, n, r, (const double*)F, (double*)U, k, dtype, st);

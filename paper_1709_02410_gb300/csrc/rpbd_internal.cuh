@@ -286,7 +286,7 @@ bool direct_takes(const rpbd_handle* h, int64_t n, int k);
 int direct_apply_impl(rpbd_handle* h, int64_t n, const double* r, const void* F, void* U, int k, bool io_double, cudaStream_t st);
 
 // symmetric FP64 matvec: whether it takes (n, k), and the matvec itself
-bool sym64_takes(rpbd_handle* h, int64_t n, int k);
+bool sym64_takes(rpbd_handle* h, int64_t n, int k, cudaStream_t st);
 int sym64_apply_impl(rpbd_handle* h, int64_t n, const double* r, const double* F, double* U, int k, cudaStream_t st);
 
 // FP64 gradient of sum_m u_m^T M F_m

@@ -331,19 +331,33 @@ static int run(rpbd_handle* h, const Cut& c, int64_t n, const double* r, const d
 // Whether the symmetric FP64 kernel takes n blobs with k right-hand sides.
 // Instructions per ordered pair (above): passes of up to four right-hand sides
 // cost 36, 46 or 66 each, the one-direction kernel 66 + 9 K with K = 8 or 16:
-// fewer up to k = 8.  The partials, about n^2/128 rows beyond SMALL_N, have to
-// stay under PARTIAL_LIMIT (n about 145,000 for k = 1), and fit the memory left:
-// where they do not, the one-direction kernel, which needs a tenth of it, runs.
-bool sym64_takes(rpbd_handle* h, int64_t n, int k)
+// fewer up to k = 8.  The partials, 3 K n^2/128 doubles beyond SMALL_N, have to
+// stay under PARTIAL_LIMIT (n about 145,000 for k = 1), and everything has to fit
+// the memory left: where it does not, the one-direction kernel, which needs a tenth
+// of it, runs, and later calls of the handle go straight there (worth_trying).
+bool sym64_takes(rpbd_handle* h, int64_t n, int k, cudaStream_t st)
 {
     if (k > 8 || n > (int64_t)1 << 20) return false;
     const sym64::Cut c = sym64::cut(n, h->sm_count);
-    const double bytes = c.rows() * 3.0 * (k <= 2 ? k : 4) * (double)c.n_pad * sizeof(double);
+    const int K = k <= 2 ? k : 4;
+    const double bytes = c.rows() * 3.0 * K * (double)c.n_pad * sizeof(double);
     if (c.items > 65535 || bytes > sym64::PARTIAL_LIMIT) return false;
-    void* p;
-    if (ensure(h, BUF_PARTIAL, (size_t)bytes, &p) == RPBD_OK) return true;
-    cudaGetLastError();  // (the failed allocation is not the one-direction kernel's)
-    return false;
+    const struct { Buf b; size_t bytes; } need[] = {{BUF_PACK, (size_t)c.n_pad * (3 + 3 * K) * sizeof(double)},
+                                                    {BUF_SCALE, (size_t)c.n_pad * sizeof(double)},
+                                                    {BUF_PARTIAL, (size_t)bytes}};
+    for (const auto& q : need)
+        if (!worth_trying(h, q.b, q.bytes, st)) return false;
+    for (const auto& q : need) {
+        void* p;
+        if (ensure(h, q.b, q.bytes, &p) != RPBD_OK) {
+            cudaGetLastError();  // (the failed allocation is not the one-direction kernel's)
+            cudaFree(h->buf[BUF_PARTIAL]);  // (nor does that kernel need partials of this size)
+            h->buf[BUF_PARTIAL] = nullptr;
+            h->cap[BUF_PARTIAL] = 0;
+            return false;
+        }
+    }
+    return true;
 }
 
 int sym64_apply_impl(rpbd_handle* h, int64_t n, const double* r, const double* F, double* U, int k, cudaStream_t st)

@@ -170,3 +170,34 @@ def test_adjoint_workspace_is_bounded():
     torch.cuda.synchronize()
     assert free - torch.cuda.mem_get_info()[0] <= 5 << 30  # 4 GiB of partials, an eighth of headroom, records, sums
     assert torch.isfinite(out).all()
+
+
+@pytest.mark.parametrize("k", [1, 3, 6])
+def test_short_memory_is_remembered(k):
+    """Where the symmetric FP64 matvec's or the gradients' partials do not fit, the smaller way is taken without asking
+    for the memory again: repeated calls can be captured, and one in 256 asks again without harm."""
+    n = 3000
+    r = to_dev(cloud(n, 980))
+    u, F = (to_dev(synth.gaussian(981 + i, (k, 3, n))) for i in range(2))
+    h, g = Handle(synth.ETA, A, synth.KT), Handle(synth.ETA, A, synth.KT)
+    limits = {1: 4000, 3: 16_000, 6: 32_000}[k], 4000  # KiB: room for the one-direction kernel's partials; a few rows
+    calls = [lambda q, out: q.mobility_apply(r, F, out=out), lambda q, out: q.mobility_adjoint(r, u, F, out=out, dtype=F64)]
+    for f, like, limit in zip(calls, (F, r), limits):
+        h.set_test_memory(limit)
+        ref, out = f(g, torch.empty_like(like)), torch.empty_like(like)
+        st = torch.cuda.Stream()
+        st.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(st):
+            f(h, out)
+            assert float((out - ref).norm() / ref.norm()) <= 1e-12
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=st):
+                f(h, out)
+            out.zero_()
+            graph.replay()
+            assert float((out - ref).norm() / ref.norm()) <= 1e-12
+            for _ in range(300):
+                out.zero_()
+                f(h, out)
+            assert float((out - ref).norm() / ref.norm()) <= 1e-12
+        st.synchronize()
