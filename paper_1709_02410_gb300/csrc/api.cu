@@ -130,7 +130,7 @@ static bool put_sqrt_nodes(rpbd_handle* h)
 {
     static const SqrtTable t;
     return cudaMalloc(&h->sqrt_nodes, sizeof(t)) == cudaSuccess &&
-           cudaMemcpy(h->sqrt_nodes, &t, sizeof(t), cudaMemcpyHostToDevice) == cudaSuccess;
+           upload(h->sqrt_nodes, &t, sizeof(t)) == cudaSuccess;
 }
 
 int rpbd_create(rpbd_handle** out, const rpbd_params* p)

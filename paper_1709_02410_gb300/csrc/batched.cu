@@ -546,8 +546,9 @@ static int build_plan(rpbd_handle* h, const int64_t* off_host, int n_sys, int k,
     p->n_items = (int)items.size();
     auto up = [&](void** d, const void* src, size_t bytes) -> int {
         if (cudaMalloc(d, bytes ? bytes : 16) != cudaSuccess) return RPBD_NO_MEM;
-        if (bytes && src && cudaMemcpy(*d, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) return RPBD_CUDA;
-        if (bytes && !src && cudaMemset(*d, 0, bytes) != cudaSuccess) return RPBD_CUDA;
+        if (bytes && src && upload(*d, src, bytes) != cudaSuccess) return RPBD_CUDA;
+        if (bytes && !src && (cudaMemset(*d, 0, bytes) != cudaSuccess || cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess))
+            return RPBD_CUDA;
         return RPBD_OK;
     };
     int st = RPBD_OK;

@@ -316,10 +316,7 @@ static int blz_table(rpbd_handle* h, int n_sys, const int64_t* off, const BlzTab
     t->off.assign(off, off + n_sys + 1);
     t->nch = (int)ch.size();
     t->chunk = blz_chunk_size(off[n_sys]);
-    // (the copy has to have arrived before kernels of a stream that does not wait for the legacy one)
-    if (cudaMalloc(&t->mem, host.size()) != cudaSuccess ||
-        cudaMemcpy(t->mem, q, host.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+    if (cudaMalloc(&t->mem, host.size()) != cudaSuccess || upload(t->mem, q, host.size()) != cudaSuccess) {
         cudaFree(t->mem);
         delete t;
         return set_error(h, RPBD_NO_MEM, "batched lanczos: chunk table upload failed");

@@ -181,6 +181,14 @@ inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 }
 
 int set_error(rpbd_handle* h, int code, const std::string& msg);
+// copies a table to the device and waits until it is there: cudaMemcpy from pageable
+// memory returns once the data is staged, and streams made with
+// cudaStreamNonBlocking do not wait for the legacy stream it runs on
+inline cudaError_t upload(void* dst, const void* src, size_t bytes)
+{
+    const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(cudaStreamLegacy);
+}
 // whether to ask for a buffer of this size where a smaller one would do too: not
 // while an allocation no larger has failed, but for every 256th time (a failing
 // attempt frees the buffer that is there, synchronises the device and breaks a capture)

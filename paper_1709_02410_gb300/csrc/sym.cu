@@ -413,7 +413,7 @@ static int get_items(rpbd_handle* h, int64_t n, int64_t n_pad, SymItem** d_items
         std::stable_sort(items.begin(), items.end(), [](const SymItem& a, const SymItem& b) { return a.ntile > b.ntile; });
         void* d = nullptr;
         RPBD_TRY(ensure(h, BUF_SYM_ITEMS, items.size() * sizeof(SymItem), &d));
-        RPBD_CU(h, cudaMemcpy(d, items.data(), items.size() * sizeof(SymItem), cudaMemcpyHostToDevice));
+        RPBD_CU(h, upload(d, items.data(), items.size() * sizeof(SymItem)));
         pl.n = n;
         pl.n_items = (int)items.size();
         pl.n_home = T;
@@ -1148,8 +1148,8 @@ static int get_plan2(rpbd_handle* h, int n_sys, const int64_t* off, Sym2Plan** o
                                             cudaSuccess ||
         cudaMalloc(&p->d_sys, sizeof(SymSys) * n_sys) != cudaSuccess ||
         (!items.empty() &&
-         cudaMemcpy(p->d_items, items.data(), sizeof(SymItem) * items.size(), cudaMemcpyHostToDevice) != cudaSuccess) ||
-        cudaMemcpy(p->d_sys, p->sys.data(), sizeof(SymSys) * n_sys, cudaMemcpyHostToDevice) != cudaSuccess) {
+         upload(p->d_items, items.data(), sizeof(SymItem) * items.size()) != cudaSuccess) ||
+        upload(p->d_sys, p->sys.data(), sizeof(SymSys) * n_sys) != cudaSuccess) {
         cudaFree(p->d_items);
         cudaFree(p->d_sys);
         delete p;
