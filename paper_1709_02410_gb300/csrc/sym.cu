@@ -386,7 +386,7 @@ __global__ void reduce_kernel(int64_t n, int64_t n_pad, int k, int kt, int n_hom
 // Cached per n (the one-home kernel; the packed kernel's lists are Sym2Plan).
 template <int TILE>
 static int get_items(rpbd_handle* h, int64_t n, int64_t n_pad, SymItem** d_items, int* n_items, int* n_home,
-                     int* max_slots, int* chunk_out)
+                     int* max_slots, int* chunk_out, cudaStream_t st)
 {
     SymPlan& pl = h->sym_plan;
     if (pl.n != n) {
@@ -411,6 +411,8 @@ static int get_items(rpbd_handle* h, int64_t n, int64_t n_pad, SymItem** d_items
         }
         // longest items first so the hardware scheduler fills the tail with short ones
         std::stable_sort(items.begin(), items.end(), [](const SymItem& a, const SymItem& b) { return a.ntile > b.ntile; });
+        if (pl.n >= 0) RPBD_CU(h, cudaStreamSynchronize(st));  // a queued call may still read the list of the other n
+        pl.n = -1;
         void* d = nullptr;
         RPBD_TRY(ensure(h, BUF_SYM_ITEMS, items.size() * sizeof(SymItem), &d));
         RPBD_CU(h, upload(d, items.data(), items.size() * sizeof(SymItem)));
@@ -436,7 +438,7 @@ static int run(rpbd_handle* h, int64_t n, const double* r, const In* F, Out* U, 
     SymItem* items;
     int n_items, n_home, max_slots;
     int chunk;
-    RPBD_TRY(get_items<HT>(h, n, n_pad, &items, &n_items, &n_home, &max_slots, &chunk));
+    RPBD_TRY(get_items<HT>(h, n, n_pad, &items, &n_items, &n_home, &max_slots, &chunk, st));
     float* rec;
     double* scale;
     float* partial;

@@ -201,3 +201,23 @@ def test_short_memory_is_remembered(k):
                 f(h, out)
             assert float((out - ref).norm() / ref.norm()) <= 1e-12
         st.synchronize()
+
+
+def test_one_home_list_in_flight():
+    """Matvecs without the wall, of other sizes queued behind one another on a stream of their own: the work list was
+    rewritten for the next size while the last call read it."""
+    h = Handle(synth.ETA, A, synth.KT, wall=False)
+    st = torch.cuda.Stream()
+    calls = []
+    for n in (30_000, 300, 12_001):
+        r, F = to_dev(cloud(n, 990)), to_dev(synth.gaussian(991, (3, n)), torch.float32)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(st):
+            ref = h.mobility_apply(r, F)
+            st.synchronize()
+            calls.append((r, F, ref))
+    with torch.cuda.stream(st):
+        outs = [(h.mobility_apply(r, F), ref) for r, F, ref in calls * 3]
+        st.synchronize()
+    for out, ref in outs:
+        assert torch.equal(out, ref)
