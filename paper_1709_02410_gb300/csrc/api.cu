@@ -381,7 +381,10 @@ int rpbd_autotune(rpbd_handle* h, int64_t n, const double* r, int k, double* bes
     RPBD_CU(h, cudaMemsetAsync(F, 0, sizeof(float) * k * 3 * n, st));
     cudaEvent_t e0, e1;
     RPBD_CU(h, cudaEventCreate(&e0));
-    RPBD_CU(h, cudaEventCreate(&e1));
+    if (cudaEventCreate(&e1) != cudaSuccess) {
+        cudaEventDestroy(e0);
+        return set_error(h, RPBD_CUDA, "autotune: no event");
+    }
     // candidates: one-direction kernel (-1) and, for k <= 4, the symmetric variants (0..5 of the
     // packed kernel with the wall, 0..3 of the one-home kernel otherwise)
     const int nsym = (h->use_packed && h->p.wall) ? 6 : 4;
@@ -391,38 +394,39 @@ int rpbd_autotune(rpbd_handle* h, int64_t n, const double* r, int k, double* bes
     const bool prof = h->profile;
     h->profile = false;
     const int cls = sym_class(k);
-    for (int c = -1; c < ncand - 1; ++c) {
-        h->use_sym[cls] = c >= 0;
-        if (c >= 0) h->sym_variant[cls] = c;
-        int s = mobility_apply_impl(h, n, r, F, U, k, RPBD_F32, false, st);
-        if (s != RPBD_OK) { h->profile = prof; return s; }
+    const int use0 = h->use_sym[cls], variant0 = h->sym_variant[cls];
+    // ms per launch as the handle is set now
+    auto measure = [&](double* t) -> int {
+        RPBD_TRY(mobility_apply_impl(h, n, r, F, U, k, RPBD_F32, false, st));
         RPBD_CU(h, cudaEventRecord(e0, st));
         for (int rep = 0; rep < 2; ++rep) RPBD_TRY(mobility_apply_impl(h, n, r, F, U, k, RPBD_F32, false, st));
         RPBD_CU(h, cudaEventRecord(e1, st));
         RPBD_CU(h, cudaEventSynchronize(e1));
         float ms = 0.0f;
         RPBD_CU(h, cudaEventElapsedTime(&ms, e0, e1));
-        if (ms / 2.0 < best) {
-            best = ms / 2.0;
+        *t = ms / 2.0;
+        return RPBD_OK;
+    };
+    int s = RPBD_OK;
+    double t = 0.0;
+    for (int c = -1; c < ncand - 1 && s == RPBD_OK; ++c) {
+        h->use_sym[cls] = c >= 0;
+        if (c >= 0) h->sym_variant[cls] = c;
+        s = measure(&t);
+        if (s == RPBD_OK && t < best) {
+            best = t;
             best_c = c;
         }
     }
     // a small system's default is a kernel of its own (direct.cu), not one of the variants: kept
     // where it is the fastest, as the variant that the default would be for larger systems
     bool keep_default = false;
-    if (nsym == 6 && direct_takes(h, n, k) && !h->sym_partials && !h->far_field) {
+    if (s == RPBD_OK && nsym == 6 && direct_takes(h, n, k) && !h->sym_partials && !h->far_field) {
         h->use_sym[cls] = 1;
         h->sym_variant[cls] = -1;
-        int s = mobility_apply_impl(h, n, r, F, U, k, RPBD_F32, false, st);
-        if (s != RPBD_OK) { h->profile = prof; return s; }
-        RPBD_CU(h, cudaEventRecord(e0, st));
-        for (int rep = 0; rep < 2; ++rep) RPBD_TRY(mobility_apply_impl(h, n, r, F, U, k, RPBD_F32, false, st));
-        RPBD_CU(h, cudaEventRecord(e1, st));
-        RPBD_CU(h, cudaEventSynchronize(e1));
-        float ms = 0.0f;
-        RPBD_CU(h, cudaEventElapsedTime(&ms, e0, e1));
-        if (ms / 2.0 < best) {
-            best = ms / 2.0;
+        s = measure(&t);
+        if (s == RPBD_OK && t < best) {
+            best = t;
             best_c = h->p.Lx > 0.0 ? 1 : 3;
             keep_default = true;
         }
@@ -430,8 +434,9 @@ int rpbd_autotune(rpbd_handle* h, int64_t n, const double* r, int k, double* bes
     h->profile = prof;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    h->use_sym[cls] = best_c >= 0;
-    h->sym_variant[cls] = best_c >= 0 && !keep_default ? best_c : -1;
+    h->use_sym[cls] = s == RPBD_OK ? best_c >= 0 : use0;
+    h->sym_variant[cls] = s != RPBD_OK ? variant0 : best_c >= 0 && !keep_default ? best_c : -1;
+    if (s != RPBD_OK) return s;
     if (best_ms) *best_ms = best;
     return best_c + 1;
 }

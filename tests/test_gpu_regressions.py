@@ -7,6 +7,7 @@ import torch
 
 from oracle import mobility as om
 from paper_1709_02410_gb300 import F32, F64, Handle, synth
+from paper_1709_02410_gb300.api import RpbdError
 
 from gpu_util import to_dev
 
@@ -221,3 +222,20 @@ def test_one_home_list_in_flight():
         st.synchronize()
     for out, ref in outs:
         assert torch.equal(out, ref)
+
+
+def test_failed_autotune_changes_nothing():
+    """An autotuning run that ends in an error leaves the handle's kernel choice as it was (the one-direction kernel
+    stayed chosen, and profiling off)."""
+    n = 3000
+    r, F = to_dev(cloud(n, 995)), to_dev(synth.gaussian(996, (3, n)), torch.float32)
+    h, g = Handle(synth.ETA, A, synth.KT), Handle(synth.ETA, A, synth.KT)
+    h.set_test_memory(80)  # KiB: room for the vectors (70), not for records
+    h.lib.rpbd_profile_enable(h.h, 1)
+    with pytest.raises(RpbdError, match="memory"):
+        h.autotune(r)
+    h.set_test_memory(0)
+    assert torch.equal(h.mobility_apply(r, F), g.mobility_apply(r, F))
+    ms, launches, pairs = C.c_double(), C.c_longlong(), C.c_double()
+    h.lib.rpbd_profile_read(h.h, 4, 1, C.byref(ms), C.byref(launches), C.byref(pairs), 1)
+    assert launches.value == 1
