@@ -1,5 +1,6 @@
 """Calls that once went wrong: each test states what it was."""
 import ctypes as C
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -239,3 +240,45 @@ def test_failed_autotune_changes_nothing():
     ms, launches, pairs = C.c_double(), C.c_longlong(), C.c_double()
     h.lib.rpbd_profile_read(h.h, 4, 1, C.byref(ms), C.byref(launches), C.byref(pairs), 1)
     assert launches.value == 1
+
+
+# 4,096 / 4,097: 16 and 64 sources a stage; 4,159 / 4,161: around a whole number of stages of 64
+@pytest.mark.parametrize("n", [4096, 4097, 4159, 4161])
+@pytest.mark.parametrize("cell", [0.0, 45.3])
+def test_many_right_hand_sides_by_stage_length(n, cell):
+    r = cloud(n, 1000 + n)
+    h = Handle(synth.ETA, A, synth.KT, Lx=cell, Ly=cell)
+    rows = np.unique(np.concatenate([[0, 63, 64, 255, 256, n - 66, n - 65, n - 2, n - 1], np.linspace(0, n - 1, 25).astype(int)]))
+    for k in (5, 8, 9, 16):
+        F = synth.gaussian(1001 + k, (k, 3, n), np.float32)
+        U = h.mobility_apply(to_dev(r), to_dev(F, torch.float32)).cpu().numpy()
+        ref = om.apply(r, F.astype(np.float64), om.Params(synth.ETA, A, Lx=cell, Ly=cell), rows)
+        assert np.linalg.norm(U[:, :, rows] - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
+def test_fp64_reciprocal_root():
+    """Velocities along z of far blobs on the x axis, pulled by one at the origin: 1/r + 2 a^2 / (3 r^3), r from 2.1 a to
+    1e100.  The root may be two units of 2^-52 off (one from CUDA's, which may be one off), r^2, the sum and the three
+    factors of 1/(8 pi eta) round by half a unit each."""
+    n = 2049
+    x = np.exp(np.linspace(np.log(2.1 * A), np.log(1e100), n - 1)) * (1 + 0.3 * np.random.default_rng(1010).uniform(size=n - 1))
+    r, F = np.zeros((3, n)), np.zeros((3, n))
+    r[0, 1:], F[2, 0] = x, 1.0
+    eta = 1.0 / (8.0 * np.pi)
+    U = Handle(eta, A, synth.KT, wall=False).mobility_apply(to_dev(r), to_dev(F)).cpu().numpy()
+    inv8pieta = Fraction(1.0 / (8.0 * np.pi * eta))
+    for xi, u in zip(x, U[2, 1:]):
+        f = Fraction(float(xi))
+        ref = inv8pieta * (1 / f + Fraction(2, 3) * Fraction(float(A)) ** 2 / f ** 3)
+        assert abs(Fraction(float(u)) / ref - 1) <= 5 * Fraction(1, 2 ** 52)
+
+
+def test_square_root_of_one_number():
+    """M^(1/2) W of a lone unbounded blob, over two octaves of its mobility: sqrt(1 / (6 pi eta a)) W.  Nodes and weights
+    are good to 5e-15, 64 rounded terms add 7e-15, the pivots' reciprocals and the norms a few units of 2^-52."""
+    W = to_dev(synth.gaussian(1011, (3, 1)))
+    r = torch.zeros_like(W)
+    for eta in np.geomspace(1e-3, 4e-3, 65):
+        out, _ = Handle(eta, A, synth.KT, wall=False).lanczos_sqrt_apply(r, W, tol=1e-14, use_precond=False)
+        ref = np.sqrt(1.0 / (6.0 * np.pi * eta * A)) * W
+        assert float((out - ref).norm() / ref.norm()) <= 2e-14
