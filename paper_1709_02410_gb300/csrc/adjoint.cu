@@ -22,7 +22,6 @@
 
 namespace rpbd {
 
-
 struct RegBlob {
     double x, y, zt, s, dzt, ds;
 };
@@ -46,20 +45,19 @@ __device__ __forceinline__ RegBlob reg_blob(const double* r, int64_t n, int64_t 
 }
 
 // block of target t (dual: partials w.r.t. t's regularised coordinates) and
-// source s; out[9] row-major.  Differences are taken in FP64, then the block
-// is evaluated in S (double, or float for the FP32 variant).
-template <bool WALL, bool PER, class S>
-__device__ __forceinline__ void dual_block(const RegBlob& t, const RegBlob& s, const PairConst<S>& pc,
-                                           Dual<3, S> M[9])
+// source s, FP64; out[9] row-major
+template <bool WALL, bool PER>
+__device__ __forceinline__ void dual_block(const RegBlob& t, const RegBlob& s, const PairConst<double>& pc,
+                                           Dual<3> M[9])
 {
-    using D3 = Dual<3, S>;
-    D3 dx(S(t.x - s.x)), dy(S(t.y - s.y)), dz(S(t.zt - s.zt)), zi(S(t.zt)), zj(S(s.zt));
-    dx.g[0] = S(1);
-    dy.g[1] = S(1);
-    dz.g[2] = S(1);
-    zi.g[2] = S(1);
+    using D3 = Dual<3>;
+    D3 dx(t.x - s.x), dy(t.y - s.y), dz(t.zt - s.zt), zi(t.zt), zj(s.zt);
+    dx.g[0] = 1.0;
+    dy.g[1] = 1.0;
+    dz.g[2] = 1.0;
+    zi.g[2] = 1.0;
     D3 Mxx, Mxy, Mxz, Myy, Myz, Mzx, Mzy, Mzz;
-    pair_block_images<D3, S, WALL, PER>(dx, dy, dz, zi, zj, pc, Mxx, Mxy, Mxz, Myy, Myz, Mzx, Mzy, Mzz);
+    pair_block_images<D3, double, WALL, PER>(dx, dy, dz, zi, zj, pc, Mxx, Mxy, Mxz, Myy, Myz, Mzx, Mzy, Mzz);
     M[0] = Mxx; M[1] = Mxy; M[2] = Mxz;
     M[3] = Mxy; M[4] = Myy; M[5] = Myz;
     M[6] = Mzx; M[7] = Mzy; M[8] = Mzz;
@@ -173,12 +171,12 @@ __global__ void divergence_kernel(int64_t n, const double* __restrict__ r, doubl
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const PairConst<double> pc = PairConst<double>::make(a, Lx, Ly);
-    const RegBlob bi = reg_blob(r, n, i, a, WALL, s_min);  // divergence: FP64 only
+    const RegBlob bi = reg_blob(r, n, i, a, WALL, s_min);
     double acc[3] = {0.0, 0.0, 0.0};
     for (int64_t j = 0; j < n; ++j) {
-        Dual<3, double> T[9];
+        Dual<3> T[9];
         if (j == i) {
-            dual_block<WALL, PER, double>(bi, bi, pc, T);
+            dual_block<WALL, PER>(bi, bi, pc, T);
 #pragma unroll
             for (int aa = 0; aa < 3; ++aa) {
                 double v = 2.0 * bi.s * bi.ds * T[aa * 3 + 2].v;
@@ -191,7 +189,7 @@ __global__ void divergence_kernel(int64_t n, const double* __restrict__ r, doubl
             }
         } else {
             const RegBlob bj = reg_blob(r, n, j, a, WALL, s_min);
-            dual_block<WALL, PER, double>(bj, bi, pc, T);  // target j, source i
+            dual_block<WALL, PER>(bj, bi, pc, T);  // target j, source i
 #pragma unroll
             for (int aa = 0; aa < 3; ++aa) {
                 double v = bi.s * bj.ds * T[2 * 3 + aa].v;

@@ -2,9 +2,8 @@
 //
 //  Lanczos M^{1/2} W (Sec. 2.2): Lanczos on G = L^-1 M L^-T (L the block
 //    Cholesky preconditioner) from v_1 = W/|W| with full (classical, twice)
-//    reorthogonalisation; f(G) W ~ |W| V_m T_m^{1/2} e_1, T_m^{1/2} e_1 from a
-//    one-warp (round-robin parallel) Jacobi eigendecomposition of T_m; stop
-//    when |y_m - y_{m-1}| / |y_m| < tol (evaluated in the small space, V is
+//    reorthogonalisation; f(G) W ~ |W| V_m T_m^{1/2} e_1, T_m^{1/2} e_1 by one
+//    warp (contour-integral quadrature, tridiag_sqrt.cuh); stop when |y_m - y_{m-1}| / |y_m| < tol (evaluated in the small space, V is
 //    orthonormal); output L y_m.
 //  GMRES (Sec. 2.1, eq. saddle): right-preconditioned restarted GMRES(m) on
 //    [M -K; -K^T 0] with the exact body-block solve of Sec. 2.2 as
@@ -55,9 +54,8 @@ __global__ void multidot_kernel(int64_t n, const double* __restrict__ V, int64_t
     }
 }
 
-// out[i] (+)= sum_b partial[i * nb + b]; one block per i
-__global__ void reduce_partials_kernel(int nblocks, const double* __restrict__ partial, double* __restrict__ out,
-                                       int accumulate)
+// out[i] = sum_b partial[i * nb + b]; one block per i
+__global__ void reduce_partials_kernel(int nblocks, const double* __restrict__ partial, double* __restrict__ out)
 {
     const int i = blockIdx.x;
     double s = 0.0;
@@ -71,20 +69,18 @@ __global__ void reduce_partials_kernel(int nblocks, const double* __restrict__ p
         s = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (threadIdx.x == 0) out[i] = accumulate ? out[i] + s : s;
+        if (threadIdx.x == 0) out[i] = s;
     }
 }
 
-// out = scale * sum_i y[i] V_i   (scale = *scale_dev when scale_dev != NULL)
+// out = scale * sum_i y[i] V_i
 __global__ void lincomb_kernel(int64_t n, const double* __restrict__ V, int64_t ld, int nv,
-                               const double* __restrict__ y, double scale, const double* __restrict__ scale_dev,
-                               double* __restrict__ out)
+                               const double* __restrict__ y, double scale, double* __restrict__ out)
 {
-    const double sc = scale_dev ? scale * scale_dev[0] : scale;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         double s = 0.0;
         for (int i = 0; i < nv; ++i) s += y[i] * V[(int64_t)i * ld + e];
-        out[e] = sc * s;
+        out[e] = scale * s;
     }
 }
 
@@ -157,12 +153,12 @@ static unsigned vgrid(int64_t n)
     return (unsigned)(g < 1 ? 1 : g);
 }
 
-// h[0..nv) = V^T w (accumulate != 0: h += V^T w)
+// out[0..nv) = V^T w
 static int multidot(rpbd_handle* h, int64_t n, const double* V, int64_t ld, int nv, const double* w, double* out,
-                    int accumulate, double* partial, cudaStream_t st)
+                    double* partial, cudaStream_t st)
 {
     multidot_kernel<<<dim3(DOT_BLOCKS, nv), 256, 0, st>>>(n, V, ld, w, partial); count_launch();
-    reduce_partials_kernel<<<nv, 256, 0, st>>>(DOT_BLOCKS, partial, out, accumulate); count_launch();
+    reduce_partials_kernel<<<nv, 256, 0, st>>>(DOT_BLOCKS, partial, out); count_launch();
     RPBD_LAUNCH_CHECK(h);
     return RPBD_OK;
 }
@@ -532,7 +528,7 @@ int lanczos_multi_impl(rpbd_handle* h, int64_t n, const double* r, int nsys, con
         p.cprev = p.cvec + mdim;
         p.sc = p.S.scal();
         RPBD_CU(h, cudaMemsetAsync(p.cprev, 0, sizeof(double) * mdim, st));
-        RPBD_TRY(multidot(h, len, p.W, 0, 1, p.W, &p.sc[0], 0, p.S.partial(), st));
+        RPBD_TRY(multidot(h, len, p.W, 0, 1, p.W, &p.sc[0], p.S.partial(), st));
         normalize_kernel<<<g, 256, 0, st>>>(len, p.W, &p.sc[0], p.V); count_launch();
         RPBD_CU(h, cudaMemcpyAsync(h->host_small + s, &p.sc[0], sizeof(double), cudaMemcpyDeviceToHost, st));
     }
@@ -608,7 +604,7 @@ int lanczos_multi_impl(rpbd_handle* h, int64_t n, const double* r, int nsys, con
                 p.active = false;
                 // y = |W| V c, out = L y
                 const int nv = p.m + 1;
-                lincomb_kernel<<<g, 256, 0, st>>>(len, p.V, len, nv, p.cvec, std::sqrt(p.W2), nullptr,
+                lincomb_kernel<<<g, 256, 0, st>>>(len, p.V, len, nv, p.cvec, std::sqrt(p.W2),
                                                   use_precond ? p.y : p.out);
                 count_launch();
                 if (use_precond) RPBD_TRY(precond_apply_impl(h, 0, p.y, p.out, st));
@@ -686,7 +682,7 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
 
     // r0 = w: |r0|, g, residual estimate, v_0 (first: |b| = |r0|)
     auto begin_cycle = [&](GmresProc& p, int first) -> int {
-        RPBD_TRY(multidot(h, len, p.w, 0, 1, p.w, &p.sc[0], 0, p.S.partial(), st));
+        RPBD_TRY(multidot(h, len, p.w, 0, 1, p.w, &p.sc[0], p.S.partial(), st));
         gmres_start_kernel<<<1, 64, 0, st>>>(mdim, &p.sc[0], p.S.g(), p.sc, first, h->host_small + 2 * (&p - P));
         count_launch();
         normalize_kernel<<<g, 256, 0, st>>>(len, p.w, &p.sc[0], p.V); count_launch();
@@ -697,7 +693,7 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
     // x += P^-1 V y over the cycle's jn Arnoldi vectors
     auto end_cycle = [&](GmresProc& p, int jn) -> int {
         gmres_backsolve_kernel<<<1, 64, jn * sizeof(double), st>>>(jn, mdim, p.S.H(), p.S.g(), p.S.y()); count_launch();
-        lincomb_kernel<<<g, 256, 0, st>>>(len, p.V, len, jn, p.S.y(), 1.0, nullptr, p.w); count_launch();
+        lincomb_kernel<<<g, 256, 0, st>>>(len, p.V, len, jn, p.S.y(), 1.0, p.w); count_launch();
         const PrecSaddle ps{p.w, p.w + 3 * n, p.zl, p.zU};
         p.z_ready = false;
         RPBD_TRY(precond_saddle_impl(h, 1, &ps, st));
@@ -733,7 +729,7 @@ int gmres_multi_impl(rpbd_handle* h, int64_t nb, int nper, const double* r, cons
             // x0 = [lambda; U] as given; |b| is the scale of the stopping test, as for x0 = 0
             RPBD_CU(h, cudaMemcpyAsync(p.x, p.pb.lambda, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, st));
             RPBD_CU(h, cudaMemcpyAsync(p.x + 3 * n, p.pb.U, sizeof(double) * 6 * nb, cudaMemcpyDeviceToDevice, st));
-            RPBD_TRY(multidot(h, len, p.b, 0, 1, p.b, &p.sc[0], 0, p.S.partial(), st));
+            RPBD_TRY(multidot(h, len, p.b, 0, 1, p.b, &p.sc[0], p.S.partial(), st));
             gmres_start_kernel<<<1, 64, 0, st>>>(mdim, &p.sc[0], p.S.g(), p.sc, 1, h->host_small + 2 * s); count_launch();
             want_resid(p);
         } else {
