@@ -81,7 +81,7 @@ struct PairConst {
 
 __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
-// 1/sqrt(x) for normal positive x (0, infinities and subnormals give NaN or
+// 1/sqrt(x) for normal positive x and infinity (0 and subnormals give NaN or
 // infinity: callers treat coinciding blobs themselves): PTX's approximate seed
 // y, then Householder's third-order iteration y (1 + e/2 + 3/8 e^2), e = 1 - x y^2,
 // measured |e| < 2^-19 over [1, 4); the next term, 5/16 e^3, is below 2^-57.  Five
@@ -91,7 +91,8 @@ __device__ __forceinline__ double rsqrt3(double x)
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = fma(-x * y, y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
+    const double z = fma(y * e, fma(0.375, e, 0.5), y);
+    return __double2hiint(x) == 0x7ff00000 ? 0.0 : z;  // (an integer comparison: not the FP64 pipe's)
 }
 // 1/x for normal x, the same way: y (1 + e + e^2), e = 1 - x y
 __device__ __forceinline__ double rcp3(double x)

@@ -282,3 +282,15 @@ def test_square_root_of_one_number():
         out, _ = Handle(eta, A, synth.KT, wall=False).lanczos_sqrt_apply(r, W, tol=1e-14, use_precond=False)
         ref = np.sqrt(1.0 / (6.0 * np.pi * eta * A)) * W
         assert float((out - ref).norm() / ref.norm()) <= 2e-14
+
+
+@pytest.mark.parametrize("wall", [True, False])
+def test_blobs_beyond_the_square_root_of_the_range(wall):
+    """Blobs so far apart that r^2 overflows do not feel one another (1/r was NaN there, in FP64)."""
+    h = Handle(synth.ETA, A, synth.KT, wall=wall)
+    r, F = cloud(80, 1020), synth.gaussian(1021, (3, 80))
+    near = [h.mobility_apply(to_dev(r[:, s]), to_dev(F[:, s])) for s in (slice(0, 40), slice(40, 80))]
+    r[0, 40:] = 1e160  # (all of them on one line along y)
+    far = h.mobility_apply(to_dev(r), to_dev(F))
+    assert torch.allclose(far[:, :40], near[0], rtol=1e-13, atol=1e-13 * float(near[0].abs().max()))
+    assert torch.isfinite(far).all()
