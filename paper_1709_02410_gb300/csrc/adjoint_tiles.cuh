@@ -15,7 +15,7 @@
 // Bound by arithmetic: the FP64 pipe, or packed FP32 issue (~160 operations per
 // unordered pair).  Before, one thread per blob walked all sources with the block
 // on dual numbers, so 1,920 blobs filled 15 of 152 SMs: FP64 gradient with its two
-// matvecs 29.3 -> 1.31 ms at 1,920 blobs (FP64 pipe 85% busy); FP32 2.99 -> 0.78 ms
+// matvecs 29.3 -> 1.30 ms at 1,920 blobs (FP64 pipe 85% busy); FP32 2.99 -> 0.78 ms
 // at 16,380 (FMA pipe 78%).
 //
 // Cutting as in sym64.cu: CTAs of one warp for small n, four beyond, items of

@@ -23,7 +23,7 @@
 // partials; items of `chunk` visitor tiles; and for very small systems the 32
 // steps of a tile are split over `parts` items.
 //
-// Measured, boomerangs, k = 1, whole call: 1,920 blobs 541 -> 274 us (its FP64
+// Measured, boomerangs, k = 1, whole call: 1,920 blobs 541 -> 282 us (its FP64
 // instructions at the measured rate: 253 us).
 #include <cuda_runtime.h>
 
